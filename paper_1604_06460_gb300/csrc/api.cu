@@ -1094,6 +1094,7 @@ int qe_batch_create(int count, const int* nqubits, int layers, const double* ang
     b->n.assign(nqubits, nqubits + count);
     b->angles.assign(angles, angles + nang);
     b->plan.T = dtype == QE_C64 ? 13 : 12;
+    b->plan.tiles_per_item = dtype == QE_C64 ? 2 : 4;
     int nbig = 0;
     for (int v : b->n) nbig = std::max(nbig, v);
     while (2 * b->plan.T - 1 < nbig) ++b->plan.T;   // cannot happen within the limits above

@@ -4,31 +4,58 @@
 // RZ(phi) on every qubit, then CZ on (q, q+1) for q = 0..n-2), started from
 // |0...0>, and returns the energy of the transverse-field Ising Hamiltonian
 // sum_i Z_i Z_{i+1} + h sum_i X_i (open chain), the expectation evaluated
-// directly (Sec. III-D).  The RY/RZ pair of a qubit is fused on the host into
-// one 2x2 matrix; the CZ ladder of a layer is one diagonal phase
-// (-1)^popcount(x & x>>1).
+// directly (Sec. III-D).
+//
+// Arithmetic of a layer.  Every RZ and CZ is diagonal, so a layer is n real
+// rotations followed by one diagonal.
+//   - A rotation is applied without its scale: with a, b the two amplitudes,
+//       p = a + kappa b,  q = b - kappa a,
+//     kappa = -tan(theta/2) when |tan| <= 1, leaving (p, q) = (out0, out1) / c;
+//     else kappa = cot(theta/2), leaving (p, q) = (out1, -out0) / s: the two
+//     outputs trade places, which is kept as a flip bit of that qubit ("slot
+//     bit = logical bit ^ flip") instead of being moved.  |kappa| <= 1, and
+//     two real multiply-adds an amplitude and gate replace the eight of the
+//     complex 2 x 2 matrix RZ RY.
+//   - The diagonal of the layer is the product over the qubits of a factor for
+//     each slot bit (the scale, the sign of the flip and the RZ phase) times
+//     (-1)^popcount(x & x >> 1) for logical x.  Two tables of at most 64 and
+//     128 partial products (and one scalar for the bits outside a tile) give
+//     an amplitude's factor with one complex product.
+//   - Layer 0 acts on |0...0>, so its result is a product state: the same
+//     tables with the factors (1, -kappa) folded in write it directly.
+// Double-float values keep (re, im) of the high and of the low words in packed
+// pairs, so that one f32x2 instruction serves both components.
+// 512 circuits of 10..22 qubits, 8 layers: complex128 double-float 242 ms with
+// the complex matrices, 72 ms so; FP64 1030 and 215 ms (its pipe's rate);
+// complex64 66 and 25 ms.
 //
 // Work decomposition (one work queue, claimed in order with an atomic head):
 //   - a circuit with n <= T qubits is one item: its whole state lives in one
 //     CTA's shared memory, HBM is never touched;
 //   - a circuit with n > T qubits keeps its state in HBM and is processed in
-//     2*layers + 1 passes over tiles of 2^T amplitudes: per layer a "low"
-//     pass (contiguous tiles, gates on qubits < T) and a "high" pass (tiles
-//     of 2^(2T-n)-amplitude chunks, gates on qubits >= T, then the CZ phase);
-//     the last high pass also accumulates the ZZ terms and the X terms of the
-//     high qubits; a final read-only low pass adds the X terms of the low
-//     qubits.  Each pass is split into items of a few tiles.
+//     2*(layers-1) + 1 passes over tiles of 2^T amplitudes: per layer from
+//     layer 1 on a "low" pass (contiguous tiles, rotations of qubits < T) and
+//     a "high" pass (tiles of 2^(2T-n)-amplitude chunks, rotations of qubits
+//     >= T, then the diagonal); the first pass starts from the product state
+//     instead of reading; the last high pass also accumulates the ZZ terms and
+//     the X terms of the high qubits; a final read-only low pass adds the X
+//     terms of the low qubits (layers = 1: one high pass writes the product
+//     state).  The states are internal, so double-float pairs are stored as
+//     they are.  Each pass is split into items of a few tiles.
+//   - rotations are done a few at a time in registers: a thread owns the 2^G
+//     amplitudes that differ in G bits.  The first such group of a pass reads
+//     global memory and the last one writes it, so a pass makes one
+//     shared-memory round trip fewer than it has groups.
 // An item may start only when every item of the circuit's earlier passes has
 // finished: CTAs wait on a per-circuit completion counter.  Large circuits
-// are queued in waves of at most 64 MiB of state (half the L2 cache),
-// pass-major inside a wave, with the small circuits spread between the
+// are queued in waves of at most 64 or 256 MiB of state, pass-major inside a wave, with the small circuits spread between the
 // passes; the dependencies of any claimed item were claimed earlier by
 // running CTAs; waits are bounded and report a timeout.
 #include <algorithm>
 #include <cmath>
+#include <cstring>
 #include <vector>
 
-#include "qe_arith.cuh"
 #include "qe_batch.h"
 #include "qe_internal.h"
 
@@ -38,12 +65,13 @@ namespace {
 
 struct Item {
     int circuit;
-    int kind;          // 0 small, 1 low layer pass, 2 high layer pass, 3 energy low pass
-    int layer;
     uint32_t tile0, tile1;
     uint32_t dep;      // completed items of this circuit required before starting
     int slot;          // energy partial slot (or -1)
-    int last_energy;   // 1: high pass of the last layer (accumulates energy)
+    uint32_t kind : 2;    // 0 small, 1 low layer pass, 2 high layer pass, 3 energy low pass
+    uint32_t first : 1;   // the circuit's first pass (starts from the product state)
+    uint32_t last : 1;    // its last high pass (energy)
+    uint32_t layer : 28;
 };
 
 struct Circ {
@@ -51,13 +79,251 @@ struct Circ {
     int nitems;        // items of this circuit
     int slot0, nslots; // energy partial slots
     uint64_t state_off; // amplitude offset of its HBM state (large circuits)
-    uint64_t u_off;     // offset of its matrices (layers * n * 4 entries)
+    uint64_t u_off;     // offset of its rotations (layers * n entries)
+    uint64_t f_off;     // offset of its flip masks (layers entries)
+};
+
+// ------------------------------------------------- packed pairs of floats
+using f2 = unsigned long long;   // (x, y) in the low, high word
+__device__ __forceinline__ f2 pack2(float x, float y) {
+    f2 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(x), "f"(y));
+    return r;
+}
+__device__ __forceinline__ float2 unpack2(f2 a) {
+    float2 r;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(a));
+    return r;
+}
+__device__ __forceinline__ f2 dup2(float x) { return pack2(x, x); }
+__device__ __forceinline__ f2 swap2(f2 a) {
+    const float2 v = unpack2(a);
+    return pack2(v.y, v.x);
+}
+__device__ __forceinline__ f2 neg2(f2 a) { return a ^ 0x8000000080000000ull; }
+__device__ __forceinline__ f2 add2(f2 a, f2 b) {
+    f2 r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ f2 sub2(f2 a, f2 b) {
+    f2 r;
+    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ f2 mul2(f2 a, f2 b) {
+    f2 r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ f2 fma2(f2 a, f2 b, f2 c) {
+    f2 r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+
+// Each policy: V one amplitude (also its memory form), K a rotation's kappa,
+// R kappa expanded for the device, rot the unscaled rotation, norm the
+// renormalisation after a group of rotations, cmul, neg, and the energy sums.
+struct BF32 {
+    using V = f2;
+    using K = float;
+    static constexpr int kGroup = 4;         // bits per register group
+    static constexpr int kSw = 4;            // swizzle: 16 8-byte slots a row
+    struct R { f2 k, nk; };
+    static K make_k(double k) { return (float)k; }
+    static double value(K k) { return (double)k; }
+    static V make_v(double re, double im) {
+        const float2 v = make_float2((float)re, (float)im);
+        V r;
+        std::memcpy(&r, &v, 8);
+        return r;
+    }
+    __device__ __forceinline__ static R expand(K k) { return R{dup2(k), dup2(-k)}; }
+    __device__ __forceinline__ static V one() { return pack2(1.f, 0.f); }
+    __device__ __forceinline__ static void rot(V& a, V& b, const R& r) {
+        const V p = fma2(r.k, b, a);
+        b = fma2(r.nk, a, b);
+        a = p;
+    }
+    __device__ __forceinline__ static void norm(V&) {}
+    __device__ __forceinline__ static V cmul(const V& w, const V& v) {
+        const float2 f = unpack2(w);
+        return fma2(dup2(f.x), v, mul2(pack2(-f.y, f.y), swap2(v)));
+    }
+    __device__ __forceinline__ static V neg(const V& v, uint32_t odd) {
+        const uint32_t s = odd << 31;
+        return v ^ (((f2)s << 32) | s);
+    }
+    __device__ __forceinline__ static void ld(V& v, const V* p) { v = __ldcg(p); }
+};
+
+// unnormalised double-float pairs (h + l), |l| a few units of h's last place
+__device__ __forceinline__ void two_sum(f2 a, f2 b, f2& s, f2& e) {
+    s = add2(a, b);
+    const f2 bb = sub2(s, a);
+    e = add2(sub2(a, sub2(s, bb)), sub2(b, bb));
+}
+
+struct BDF {
+    struct alignas(16) V { f2 h, l; };
+    using K = float2;                        // (high, low)
+    static constexpr int kGroup = 3;
+    static constexpr int kSw = 3;            // 8 16-byte slots a row
+    struct R { f2 h, l; };
+    static K make_k(double k) {
+        const float h = (float)k;
+        return make_float2(h, (float)(k - (double)h));
+    }
+    static double value(K k) { return (double)k.x + (double)k.y; }
+    static V make_v(double re, double im) {
+        const K a = make_k(re), b = make_k(im);
+        const float2 h = make_float2(a.x, b.x), l = make_float2(a.y, b.y);
+        V r;
+        std::memcpy(&r.h, &h, 8);
+        std::memcpy(&r.l, &l, 8);
+        return r;
+    }
+    __device__ __forceinline__ static R expand(K k) { return R{dup2(k.x), dup2(k.y)}; }
+    __device__ __forceinline__ static V one() { return V{pack2(1.f, 0.f), 0ull}; }
+    // v + k u: the product's high part exactly (its negative n, so that the
+    // residual is one fused multiply-add), the cross terms in FP32, TwoSum
+    __device__ __forceinline__ static V madd(const V& v, f2 kh, f2 kl, f2 nkh, const V& u) {
+        const f2 n = mul2(nkh, u.h);
+        f2 pl = fma2(kh, u.h, n);
+        pl = fma2(kh, u.l, pl);
+        pl = fma2(kl, u.h, pl);
+        const f2 s = sub2(v.h, n);
+        const f2 bb = sub2(s, v.h);
+        const f2 e = sub2(sub2(v.h, sub2(s, bb)), add2(n, bb));
+        return V{s, add2(v.l, add2(e, pl))};
+    }
+    __device__ __forceinline__ static void rot(V& a, V& b, const R& r) {
+        const f2 nh = neg2(r.h), nl = neg2(r.l);
+        const V p = madd(a, r.h, r.l, nh, b);
+        b = madd(b, nh, nl, r.h, a);
+        a = p;
+    }
+    __device__ __forceinline__ static void norm(V& v) {
+        const f2 h = add2(v.h, v.l);
+        v.l = sub2(v.l, sub2(h, v.h));
+        v.h = h;
+    }
+    __device__ __forceinline__ static V cmul(const V& w, const V& v) {
+        const float2 wh = unpack2(w.h), wl = unpack2(w.l);
+        const f2 rh = dup2(wh.x), rl = dup2(wl.x);
+        V t;
+        t.h = mul2(rh, v.h);
+        t.l = fma2(rh, v.h, neg2(t.h));
+        t.l = fma2(rh, v.l, t.l);
+        t.l = fma2(rl, v.h, t.l);
+        const f2 ih = pack2(-wh.y, wh.y), il = pack2(-wl.y, wl.y);
+        V r = madd(t, ih, il, neg2(ih), V{swap2(v.h), swap2(v.l)});
+        norm(r);
+        return r;
+    }
+    __device__ __forceinline__ static V neg(const V& v, uint32_t odd) {
+        const uint32_t s = odd << 31;
+        const f2 m = ((f2)s << 32) | s;
+        return V{v.h ^ m, v.l ^ m};
+    }
+    __device__ __forceinline__ static void ld(V& v, const V* p) {
+        const ulonglong2 t = __ldcg(reinterpret_cast<const ulonglong2*>(p));
+        v.h = t.x;
+        v.l = t.y;
+    }
+};
+
+struct BF64 {
+    using V = double2;
+    using K = double;
+    static constexpr int kGroup = 3;
+    static constexpr int kSw = 3;
+    using R = double;
+    static K make_k(double k) { return k; }
+    static double value(K k) { return k; }
+    static V make_v(double re, double im) { return make_double2(re, im); }
+    __device__ __forceinline__ static R expand(K k) { return k; }
+    __device__ __forceinline__ static V one() { return make_double2(1.0, 0.0); }
+    __device__ __forceinline__ static void rot(V& a, V& b, R k) {
+        const V p = make_double2(__fma_rn(k, b.x, a.x), __fma_rn(k, b.y, a.y));
+        b = make_double2(__fma_rn(-k, a.x, b.x), __fma_rn(-k, a.y, b.y));
+        a = p;
+    }
+    __device__ __forceinline__ static void norm(V&) {}
+    __device__ __forceinline__ static V cmul(const V& w, const V& v) {
+        return make_double2(__fma_rn(w.x, v.x, -__dmul_rn(w.y, v.y)), __fma_rn(w.x, v.y, __dmul_rn(w.y, v.x)));
+    }
+    __device__ __forceinline__ static V neg(const V& v, uint32_t odd) {
+        const int s = (int)(odd << 31);
+        return make_double2(__hiloint2double(__double2hiint(v.x) ^ s, __double2loint(v.x)),
+                            __hiloint2double(__double2hiint(v.y) ^ s, __double2loint(v.y)));
+    }
+    __device__ __forceinline__ static void ld(V& v, const V* p) { v = __ldcg(p); }
+};
+
+// Energy sums of one thread: z += f |v|^2 (f a small integer), x += Re(conj(w) v).
+// Packed float pairs with exact products (one lane of the pair per component)
+// for FP32 and double-float, plain FP64 fused multiply-adds for FP64.
+template <class P>
+struct EAcc {
+    f2 zs = 0, ze = 0, xs = 0, xe = 0;
+    __device__ __forceinline__ static void high_low(const f2& v, f2& h, f2& l) { h = v; l = 0; }
+    __device__ __forceinline__ static void high_low(const BDF::V& v, f2& h, f2& l) { h = v.h; l = v.l; }
+    __device__ __forceinline__ static void prod(const typename P::V& w, const typename P::V& v, f2& h, f2& l) {
+        f2 wh, wl, vh, vl;
+        high_low(w, wh, wl);
+        high_low(v, vh, vl);
+        h = mul2(wh, vh);
+        l = fma2(wh, vh, neg2(h));
+        if (sizeof(typename P::V) == 16) {
+            l = fma2(wh, vl, l);
+            l = fma2(wl, vh, l);
+        }
+    }
+    __device__ __forceinline__ void add_z(const typename P::V& v, float f) {
+        f2 h, l, s, e;
+        prod(v, v, h, l);
+        const f2 ff = dup2(f);
+        const f2 p = mul2(h, ff);
+        const f2 pe = fma2(l, ff, fma2(h, ff, neg2(p)));
+        two_sum(zs, p, s, e);
+        zs = s;
+        ze = add2(ze, add2(e, pe));
+    }
+    __device__ __forceinline__ void add_x(const typename P::V& w, const typename P::V& v) {
+        f2 h, l, s, e;
+        prod(w, v, h, l);
+        two_sum(xs, h, s, e);
+        xs = s;
+        xe = add2(xe, add2(e, l));
+    }
+    __device__ __forceinline__ static double total(f2 s, f2 e) {
+        const float2 a = unpack2(s), b = unpack2(e);
+        return ((double)a.x + (double)b.x) + ((double)a.y + (double)b.y);
+    }
+    __device__ double z() const { return total(zs, ze); }
+    __device__ double x() const { return total(xs, xe); }
+};
+template <>
+struct EAcc<BF64> {
+    double zs = 0.0, xs = 0.0;
+    __device__ __forceinline__ void add_z(const double2& v, float f) {
+        zs = __fma_rn(__fma_rn(v.x, v.x, __dmul_rn(v.y, v.y)), (double)f, zs);
+    }
+    __device__ __forceinline__ void add_x(const double2& w, const double2& v) {
+        xs = __fma_rn(w.x, v.x, __fma_rn(w.y, v.y, xs));
+    }
+    __device__ double z() const { return zs; }
+    __device__ double x() const { return xs; }
 };
 
 template <class P>
 struct BatchArgs {
-    typename P::S* states;
-    const typename P::M* U;
+    typename P::V* states;
+    const typename P::K* kap;      // kappa per (circuit, layer, qubit)
+    const typename P::V* fac;      // factors per (circuit, layer, qubit, slot bit)
+    const uint32_t* flips;         // per (circuit, layer): slot ^ logical
     const Item* items;
     const Circ* circ;
     int nitems;
@@ -70,149 +336,245 @@ struct BatchArgs {
     double2* partials;     // (zz sum, x sum) per energy slot
     double* energies;
     long long spin_limit;
-    int gmax;              // single-qubit gates per register group
+};
+
+// Shared-memory slot of tile element i: the lowest bits XORed with the next
+// ones, so that both unit strides and the strides of the lowest register
+// groups reach distinct banks (2^kSw elements fill the 32 banks).
+template <class P>
+__device__ __forceinline__ uint32_t slot(uint32_t i) {
+    return i ^ ((i >> P::kSw) & ((1u << P::kSw) - 1u));
+}
+
+constexpr int kTabA = 64, kTabB = 128;   // table entries: local bits 0..5 and 6..12
+
+// One tile as a pass sees it: local bits [0, nb) are qubits [0, L) and
+// [hq, hq + nb - L); the tile index t holds the nt qubits from tq on.
+struct Layout {
+    int nb, L, hq, nt, tq;
+    __device__ __forceinline__ int qubit(int j) const { return j < L ? j : hq + (j - L); }
+    __device__ __forceinline__ uint32_t index(uint32_t l, uint32_t t) const {
+        return (l & ((1u << L) - 1u)) | ((l >> L) << hq) | (t << tq);
+    }
+};
+
+// Where a group's amplitudes come from and go to.
+enum { kFromTile = 0, kFromGlobal = 1, kFromProduct = 2 };
+enum { kToTile = 1, kToGlobal = 2 };
+
+template <class P>
+struct Group {
+    typename P::V* tile;
+    typename P::V* st;              // the circuit's HBM state (large circuits)
+    const typename P::V *tabA, *tabB;   // the diagonal's (or product state's) tables
+    const typename P::V* tf;        // factor of the tile's bits (null: none)
+    Layout lay;
+    uint32_t t;
+    uint32_t flip;                  // slot ^ logical of the diagonal
+    int src, dst;
+    int diag;                       // multiply by the diagonal before writing
 };
 
 template <class P>
-__device__ __forceinline__ typename P::V outv(const typename P::A& a);
-template <>
-__device__ __forceinline__ F32::V outv<F32>(const F32::A& a) { return make_float2(a.re, a.im); }
-template <>
-__device__ __forceinline__ F64::V outv<F64>(const F64::A& a) { return make_double2(a.re, a.im); }
-template <>
-__device__ __forceinline__ DF::V outv<DF>(const DF::A& a) {
-    return DF::V{df_norm(a.rs, a.re_), df_norm(a.is, a.ie)};
-}
+__device__ __forceinline__ uint32_t cz_odd(uint32_t x) { return (uint32_t)__popc(x & (x >> 1)) & 1u; }
 
-// |v|^2 and Re(conj(w) v) as double-float pairs.
-__device__ __forceinline__ void sq(const float2& v, float& h, float& l) {
-    df_first(h, l, df{v.x, 0.f}, df{v.x, 0.f});
-    df_acc(h, l, df{v.y, 0.f}, df{v.y, 0.f});
-}
-__device__ __forceinline__ void sq(const DF::V& v, float& h, float& l) {
-    df_first(h, l, v.re, v.re);
-    df_acc(h, l, v.im, v.im);
-}
-__device__ __forceinline__ void sq(const double2& v, float& h, float& l) { sq(DF::load(v), h, l); }
-__device__ __forceinline__ void re_dot(const float2& w, const float2& v, float& h, float& l) {
-    df_first(h, l, df{w.x, 0.f}, df{v.x, 0.f});
-    df_acc(h, l, df{w.y, 0.f}, df{v.y, 0.f});
-}
-__device__ __forceinline__ void re_dot(const DF::V& w, const DF::V& v, float& h, float& l) {
-    df_first(h, l, w.re, v.re);
-    df_acc(h, l, w.im, v.im);
-}
-__device__ __forceinline__ void re_dot(const double2& w, const double2& v, float& h, float& l) {
-    re_dot(DF::load(w), DF::load(v), h, l);
-}
-__device__ __forceinline__ void acc2(float& s, float& e, float ph, float pl) {
-    float t = fadd(s, ph);
-    float bb = fsub(t, s);
-    float err = fadd(fsub(s, fsub(t, bb)), fsub(ph, bb));
-    s = t;
-    e = fadd(e, fadd(err, pl));
-}
-
+// The factor of slot index l: tables, the tile's scalar and the CZ sign.
 template <class P>
-__device__ __forceinline__ typename P::V zero_v();
-template <>
-__device__ __forceinline__ float2 zero_v<F32>() { return make_float2(0.f, 0.f); }
-template <>
-__device__ __forceinline__ double2 zero_v<F64>() { return make_double2(0.0, 0.0); }
-template <>
-__device__ __forceinline__ DF::V zero_v<DF>() { return DF::V{df{0.f, 0.f}, df{0.f, 0.f}}; }
+__device__ __forceinline__ typename P::V factor(const Group<P>& g, const typename P::V& w, uint32_t l) {
+    const uint32_t x = g.lay.index(l, g.t) ^ g.flip;
+    return P::neg(P::cmul(w, g.tabB[l >> 6]), cz_odd<P>(x));
+}
 template <class P>
-__device__ __forceinline__ typename P::V one_v();
-template <>
-__device__ __forceinline__ float2 one_v<F32>() { return make_float2(1.f, 0.f); }
-template <>
-__device__ __forceinline__ double2 one_v<F64>() { return make_double2(1.0, 0.0); }
-template <>
-__device__ __forceinline__ DF::V one_v<DF>() { return DF::V{df{1.f, 0.f}, df{0.f, 0.f}}; }
-template <class P>
-__device__ __forceinline__ typename P::V neg_v(const typename P::V& v);
-template <>
-__device__ __forceinline__ float2 neg_v<F32>(const float2& v) { return make_float2(-v.x, -v.y); }
-template <>
-__device__ __forceinline__ double2 neg_v<F64>(const double2& v) { return make_double2(-v.x, -v.y); }
-template <>
-__device__ __forceinline__ DF::V neg_v<DF>(const DF::V& v) {
-    return DF::V{df{-v.re.h, -v.re.l}, df{-v.im.h, -v.im.l}};
+__device__ __forceinline__ typename P::V factor_low(const Group<P>& g, uint32_t l) {
+    const typename P::V a = g.tabA[l & 63u];
+    return g.tf ? P::cmul(*g.tf, a) : a;
 }
 
-// Shared-memory slot of tile element i (one pad slot per 16 elements keeps
-// the 16-element strides of register groups on distinct banks).
-__device__ __forceinline__ uint32_t pad16(uint32_t i) { return i + (i >> 4); }
-
-// Apply the G single-qubit matrices of tile-local bits b0 .. b0+G-1
-// (U + 4*t for bit b0+t) in registers: a thread owns the 2^G elements that
-// differ in those bits, so G gates cost one shared-memory round trip.
+// The rotations of local bits b0 .. b0 + G - 1 (kappas k[0..G-1]; null: none)
+// on the tile, in registers.
 template <class P, int G>
-__device__ void tile_gates_reg(typename P::V* tile, int T, int b0, const typename P::M* U) {
+__device__ void run_group(const Group<P>& g, int b0, const typename P::K* k) {
     using V = typename P::V;
     constexpr int E = 1 << G;
-    typename P::M u[G][4];
+    typename P::R r[G];
+    if (k) {
 #pragma unroll
-    for (int t = 0; t < G; ++t)
-#pragma unroll
-        for (int k = 0; k < 4; ++k) u[t][k] = U[4 * t + k];
+        for (int t = 0; t < G; ++t) r[t] = P::expand(k[t]);
+    }
     const uint32_t below = (1u << b0) - 1u;
-    const int nbase = 1 << (T - G);
+    const int nbase = 1 << (g.lay.nb - G);
+    for (int b = threadIdx.x; b < nbase; b += blockDim.x) {
+        const uint32_t base = (((uint32_t)b & ~below) << G) | ((uint32_t)b & below);
+        V v[E];
+        if (g.src == kFromTile) {
+#pragma unroll
+            for (int j = 0; j < E; ++j) v[j] = g.tile[slot<P>(base | ((uint32_t)j << b0))];
+        } else if (g.src == kFromGlobal) {
+#pragma unroll
+            for (int j = 0; j < E; ++j) P::ld(v[j], g.st + g.lay.index(base | ((uint32_t)j << b0), g.t));
+        } else {
+#pragma unroll
+            for (int j = 0; j < E; ++j) {
+                const uint32_t l = base | ((uint32_t)j << b0);
+                v[j] = factor<P>(g, factor_low<P>(g, l), l);
+            }
+        }
+        if (k) {
+#pragma unroll
+            for (int t = 0; t < G; ++t)
+#pragma unroll
+                for (int j = 0; j < E; ++j)
+                    if (!(j & (1 << t))) P::rot(v[j], v[j | (1 << t)], r[t]);
+#pragma unroll
+            for (int j = 0; j < E; ++j) P::norm(v[j]);
+        }
+        if (g.diag) {
+            V w = factor_low<P>(g, base);
+#pragma unroll
+            for (int j = 0; j < E; ++j) {
+                const uint32_t l = base | ((uint32_t)j << b0);
+                if (j > 0 && b0 < 6) w = factor_low<P>(g, l);
+                v[j] = P::cmul(factor<P>(g, w, l), v[j]);
+            }
+        }
+        if (g.dst & kToTile) {
+#pragma unroll
+            for (int j = 0; j < E; ++j) g.tile[slot<P>(base | ((uint32_t)j << b0))] = v[j];
+        }
+        if (g.dst & kToGlobal) {
+#pragma unroll
+            for (int j = 0; j < E; ++j) g.st[g.lay.index(base | ((uint32_t)j << b0), g.t)] = v[j];
+        }
+    }
+}
+
+template <class P>
+__device__ void run_group_n(const Group<P>& g, int size, int b0, const typename P::K* k) {
+    switch (size) {
+        case 4:
+            if constexpr (P::kGroup >= 4) run_group<P, 4>(g, b0, k);
+            break;
+        case 3: run_group<P, 3>(g, b0, k); break;
+        case 2: run_group<P, 2>(g, b0, k); break;
+        default: run_group<P, 1>(g, b0, k); break;
+    }
+}
+
+// The rotations of local bits [b0, b0 + cnt) (kappa k[i] for bit b0 + i), cnt
+// >= 1, as register groups of at most kGroup bits.  top_first: the topmost
+// group first (it reads global memory in contiguous runs), then the others
+// upwards; else upwards.  `g` describes the first group's source and the last
+// group's destination and diagonal; the groups in between use the tile.
+template <class P>
+__device__ void run_groups(Group<P> g, int b0, int cnt, const typename P::K* k, bool top_first) {
+    const int ng = (cnt + P::kGroup - 1) / P::kGroup;
+    const int dst = g.dst, diag = g.diag;
+    for (int i = 0; i < ng; ++i) {
+        const int m = top_first ? (i == 0 ? ng - 1 : i - 1) : i;
+        // sizes cnt / ng, one more for the topmost ones
+        const int q = cnt / ng, rem = cnt % ng;
+        const int size = q + (m >= ng - rem ? 1 : 0);
+        const int off = m * q + max(0, m - (ng - rem));
+        g.dst = i == ng - 1 ? dst : kToTile;
+        g.diag = i == ng - 1 ? diag : 0;
+        run_group_n<P>(g, size, b0 + off, k + off);
+        g.src = kFromTile;
+        if (g.dst & kToTile) __syncthreads();
+    }
+}
+
+// X terms of local bits [b0, b0 + G), and with `z` the ZZ terms.
+template <class P, int G>
+__device__ void energy_group(const Group<P>& g, int b0, bool z, int n, EAcc<P>& acc) {
+    using V = typename P::V;
+    constexpr int E = 1 << G;
+    const uint32_t below = (1u << b0) - 1u;
+    const uint32_t zmask = (n > 1) ? ((1u << (n - 1)) - 1u) : 0u;
+    const int nbase = 1 << (g.lay.nb - G);
     for (int b = threadIdx.x; b < nbase; b += blockDim.x) {
         const uint32_t base = (((uint32_t)b & ~below) << G) | ((uint32_t)b & below);
         V v[E];
 #pragma unroll
-        for (int j = 0; j < E; ++j) v[j] = tile[pad16(base | ((uint32_t)j << b0))];
+        for (int j = 0; j < E; ++j) {
+            const uint32_t l = base | ((uint32_t)j << b0);
+            if (g.src == kFromTile) v[j] = g.tile[slot<P>(l)];
+            else P::ld(v[j], g.st + g.lay.index(l, g.t));
+            if (g.dst & kToTile) g.tile[slot<P>(l)] = v[j];
+        }
+        if (z) {
+#pragma unroll
+            for (int j = 0; j < E; ++j) {
+                const uint32_t x = g.lay.index(base | ((uint32_t)j << b0), g.t) ^ g.flip;
+                acc.add_z(v[j], (float)((n - 1) - 2 * __popc((x ^ (x >> 1)) & zmask)));
+            }
+        }
 #pragma unroll
         for (int t = 0; t < G; ++t)
 #pragma unroll
-            for (int j = 0; j < E; ++j) {
-                if (j & (1 << t)) continue;
-                const int j2 = j | (1 << t);
-                typename P::A a0, a1;
-                P::mac_first(a0, u[t][0], v[j]);
-                P::mac(a0, u[t][1], v[j2]);
-                P::mac_first(a1, u[t][2], v[j]);
-                P::mac(a1, u[t][3], v[j2]);
-                v[j] = outv<P>(a0);
-                v[j2] = outv<P>(a1);
-            }
-#pragma unroll
-        for (int j = 0; j < E; ++j) tile[pad16(base | ((uint32_t)j << b0))] = v[j];
+            for (int j = 0; j < E; ++j)
+                if (!(j & (1 << t))) acc.add_x(v[j | (1 << t)], v[j]);
     }
-    __syncthreads();
 }
 
-// Gates on the tile-local bits [b0, b0 + cnt), whose matrices are U + 4*i.
+// X terms of local bits [b0, b0 + cnt), cnt >= 1; the topmost group first
+// (from g.src, into the tile when other groups follow).
 template <class P>
-__device__ void tile_gates(typename P::V* tile, int T, int b0, int cnt, const typename P::M* U, int gmax_arg) {
-    // register budget: 16 complex64 or 8 double-float values per thread
-    // double-float groups hold at most 2 gates: wider groups are not even
-    // instantiated for it (their registers would spill)
-    constexpr bool wide = sizeof(typename P::V) < 16;
-    const int gmax = wide ? gmax_arg : (gmax_arg < 2 ? gmax_arg : 2);
-    while (cnt > 0) {
-        const int g = cnt >= gmax ? gmax : cnt;
-        if constexpr (wide) {
-            switch (g) {
-                case 4: tile_gates_reg<P, 4>(tile, T, b0, U); break;
-                case 3: tile_gates_reg<P, 3>(tile, T, b0, U); break;
-                case 2: tile_gates_reg<P, 2>(tile, T, b0, U); break;
-                default: tile_gates_reg<P, 1>(tile, T, b0, U); break;
-            }
-        } else {
-            if (g == 2) tile_gates_reg<P, 2>(tile, T, b0, U);
-            else tile_gates_reg<P, 1>(tile, T, b0, U);
+__device__ void run_energy(Group<P> g, int b0, int cnt, bool z, int n, EAcc<P>& acc) {
+    const int ng = (cnt + 2) / 3;
+    for (int m = ng - 1; m >= 0; --m) {
+        const int q = cnt / ng, rem = cnt % ng;
+        const int size = q + (m >= ng - rem ? 1 : 0);
+        const int off = m * q + max(0, m - (ng - rem));
+        g.dst = (m == ng - 1 && ng > 1 && g.src != kFromTile) ? kToTile : 0;
+        switch (size) {
+            case 3: energy_group<P, 3>(g, b0 + off, z, n, acc); break;
+            case 2: energy_group<P, 2>(g, b0 + off, z, n, acc); break;
+            default: energy_group<P, 1>(g, b0 + off, z, n, acc); break;
         }
-        b0 += g;
-        cnt -= g;
-        U += 4 * g;
+        z = false;
+        if (g.dst & kToTile) __syncthreads();
+        g.src = kFromTile;
     }
 }
 
-// Block-wide double-float sum of (s, e) pairs; result valid in thread 0.
-__device__ double block_sum(float s, float e, double* sh) {
-    double d = df2d(s, e);
+// Partial products of the factors (2 per qubit) over the local bits 0..5 and
+// 6..nb-1, and (by the last warp) the product over the tile's bits into *tf.
+template <class P>
+__device__ void build_tables(const Layout& lay, const typename P::V* fac, typename P::V* tabA, typename P::V* tabB) {
+    const int na = lay.nb < 6 ? lay.nb : 6;
+    const int ta = 1 << na, tb = 1 << (lay.nb - na);
+    for (int i = threadIdx.x; i < ta + tb; i += blockDim.x) {
+        const bool low = i < ta;
+        const uint32_t e = low ? i : i - ta;
+        const int j0 = low ? 0 : na, cnt = low ? na : lay.nb - na;
+        typename P::V w = P::one();
+        for (int j = 0; j < cnt; ++j) {
+            const typename P::V f = fac[2 * lay.qubit(j0 + j) + ((e >> j) & 1u)];
+            w = j == 0 ? f : P::cmul(f, w);
+        }
+        if (low) tabA[e] = w;
+        else tabB[e] = w;
+    }
+}
+template <class P>
+__device__ void build_tile_factor(const Layout& lay, const typename P::V* fac, uint32_t t, typename P::V* tf) {
+    const int last = (blockDim.x >> 5) - 1;
+    if ((int)(threadIdx.x >> 5) != last) return;
+    const int lane = threadIdx.x & 31;
+    typename P::V w = lane < lay.nt ? fac[2 * (lay.tq + lane) + ((t >> lane) & 1u)] : P::one();
+    for (int o = 1; o < lay.nt; o <<= 1) {
+        typename P::V u;
+        const uint32_t* s = reinterpret_cast<const uint32_t*>(&w);
+        uint32_t* d = reinterpret_cast<uint32_t*>(&u);
+#pragma unroll
+        for (int k = 0; k < (int)(sizeof(w) / 4); ++k) d[k] = __shfl_xor_sync(0xffffffffu, s[k], o);
+        w = P::cmul(u, w);
+    }
+    if (lane == 0) *tf = w;
+}
+
+// Block-wide sum; result valid in thread 0.
+__device__ double block_sum(double d, double* sh) {
     for (int o = 16; o > 0; o >>= 1) d += __shfl_down_sync(0xffffffffu, d, o);
     __syncthreads();
     if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = d;
@@ -222,58 +584,15 @@ __device__ double block_sum(float s, float e, double* sh) {
         for (int w = 0; w < (int)(blockDim.x >> 5); ++w) tot += sh[w];
     return tot;
 }
-// ... of FP64 values; result valid in thread 0
-__device__ double block_sum_d(double d, double* sh) {
-    for (int o = 16; o > 0; o >>= 1) d += __shfl_down_sync(0xffffffffu, d, o);
-    __syncthreads();
-    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = d;
-    __syncthreads();
-    double tot = 0.0;
-    if (threadIdx.x == 0)
-        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) tot += sh[w];
-    return tot;
-}
-
-// Energy sums of one CTA: float pairs (s, e) with exact products for the
-// FP32 and double-float policies, plain FP64 fused multiply-adds for FP64.
-template <class P>
-struct EAcc {
-    float zs = 0.f, ze = 0.f, xs = 0.f, xe = 0.f;
-    // z += |v|^2 f (f a small integer), x += Re(conj(w) v)
-    __device__ __forceinline__ void add_z(const typename P::V& v, float f) {
-        float h, l;
-        sq(v, h, l);
-        const float p = fmul(h, f);
-        const float pe = __fmaf_rn(h, f, -p);
-        acc2(zs, ze, p, __fmaf_rn(l, f, pe));
-    }
-    __device__ __forceinline__ void add_x(const typename P::V& w, const typename P::V& v) {
-        float h, l;
-        re_dot(w, v, h, l);
-        acc2(xs, xe, h, l);
-    }
-    __device__ double z_total(double* sh) { return block_sum(zs, ze, sh); }
-    __device__ double x_total(double* sh) { return block_sum(xs, xe, sh); }
-};
-template <>
-struct EAcc<F64> {
-    double z = 0.0, x = 0.0;
-    __device__ __forceinline__ void add_z(const double2& v, float f) {
-        z = __fma_rn(__fma_rn(v.x, v.x, __dmul_rn(v.y, v.y)), (double)f, z);
-    }
-    __device__ __forceinline__ void add_x(const double2& w, const double2& v) {
-        x = __fma_rn(w.x, v.x, __fma_rn(w.y, v.y, x));
-    }
-    __device__ double z_total(double* sh) { return block_sum_d(z, sh); }
-    __device__ double x_total(double* sh) { return block_sum_d(x, sh); }
-};
-
 
 template <class P>
-__global__ void __launch_bounds__(512) k_batch(const __grid_constant__ BatchArgs<P> a) {
+__global__ void __maxnreg__(128) k_batch(const __grid_constant__ BatchArgs<P> a) {
     using V = typename P::V;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     V* tile = reinterpret_cast<V*>(smem_raw);
+    V* tabA = tile + (1u << a.T);
+    V* tabB = tabA + kTabA;
+    V* s_tf = tabB + kTabB;
     __shared__ double shred[32];
     __shared__ int s_item;
     __shared__ int s_ok;
@@ -307,83 +626,85 @@ __global__ void __launch_bounds__(512) k_batch(const __grid_constant__ BatchArgs
         }
         __syncthreads();
         if (!s_ok) continue;
-        const typename P::M* U = a.U + cc.u_off;
+        const typename P::K* kap = a.kap + cc.u_off;
+        const V* fac = a.fac + 2 * cc.u_off;
+        const uint32_t* flips = a.flips + cc.f_off;
         EAcc<P> acc;
+        Group<P> g;
+        g.tile = tile;
+        g.st = a.states + cc.state_off;
+        g.tabA = tabA;
+        g.tabB = tabB;
+        g.tf = nullptr;
+        g.t = 0;
         if (it.kind == 0) {
             // ------------------------------------------------ small circuit
-            const uint32_t N = 1u << n;
-            for (uint32_t i = threadIdx.x; i < N; i += blockDim.x)
-                tile[pad16(i)] = (i == 0) ? one_v<P>() : zero_v<P>();
+            g.lay = Layout{n, n, n, 0, 0};
+            build_tables<P>(g.lay, fac, tabA, tabB);
             __syncthreads();
-            for (int l = 0; l < a.layers; ++l) {
-                tile_gates<P>(tile, n, 0, n, U + (size_t)l * n * 4, a.gmax);
-                for (uint32_t i = threadIdx.x; i < N; i += blockDim.x)
-                    if (__popc(i & (i >> 1)) & 1) tile[pad16(i)] = neg_v<P>(tile[pad16(i)]);
+            g.flip = flips[0];
+            g.src = kFromProduct;
+            g.dst = kToTile;
+            g.diag = 0;
+            run_group<P, 1>(g, 0, nullptr);
+            __syncthreads();
+            g.src = kFromTile;
+            g.diag = 1;
+            for (int l = 1; l < a.layers; ++l) {
+                build_tables<P>(g.lay, fac + (size_t)l * 2 * n, tabA, tabB);
                 __syncthreads();
+                g.flip = flips[l];
+                run_groups<P>(g, 0, n, kap + (size_t)l * n, false);
             }
-            const uint32_t zmask = (n > 1) ? ((1u << (n - 1)) - 1u) : 0u;
-            for (uint32_t i = threadIdx.x; i < N; i += blockDim.x) {
-                acc.add_z(tile[pad16(i)], (float)((n - 1) - 2 * __popc((i ^ (i >> 1)) & zmask)));
-                for (int q = 0; q < n; ++q)
-                    if (!((i >> q) & 1u)) acc.add_x(tile[pad16(i | (1u << q))], tile[pad16(i)]);
-            }
-            const double z = acc.z_total(shred);
-            const double x = acc.x_total(shred);
+            run_energy<P>(g, 0, n, true, n, acc);
+            const double z = block_sum(acc.z(), shred);
+            const double x = block_sum(acc.x(), shred);
             if (threadIdx.x == 0) a.energies[it.circuit] = z + 2.0 * a.hx * x;
             __syncthreads();
             continue;
         }
         // ---------------------------------------------------- large circuit
-        typename P::S* st = a.states + cc.state_off;
         const int L = 2 * T - n;                 // chunk bits of the high layout
-        const uint32_t lowmask = (1u << L) - 1u;
-        const uint64_t zmask = (n > 1) ? ((1ull << (n - 1)) - 1ull) : 0ull;
+        const bool high = it.kind == 2;
+        g.lay = high ? Layout{T, L, T, T - L, L} : Layout{T, T, T, n - T, T};
+        g.flip = flips[it.first ? 0 : it.layer];
+        // the diagonal of a high pass, or layer 0's product state
+        const int tab_layer = it.first ? 0 : it.layer;
+        const bool tables = it.first || high;
+        if (tables) build_tables<P>(g.lay, fac + (size_t)tab_layer * 2 * n, tabA, tabB);
         for (uint32_t t = it.tile0; t < it.tile1; ++t) {
-            const bool high = it.kind == 2;
-            auto gidx = [&](uint32_t l) -> uint64_t {
-                if (!high) return ((uint64_t)t << T) | l;
-                return (uint64_t)(l & lowmask) | ((uint64_t)t << L) | ((uint64_t)(l >> L) << T);
-            };
-            const uint32_t TN = 1u << T;
-            if (it.kind == 1 && it.layer == 0) {
-                for (uint32_t l = threadIdx.x; l < TN; l += blockDim.x)
-                    tile[pad16(l)] = (t == 0 && l == 0) ? one_v<P>() : zero_v<P>();
-            } else {
-                for (uint32_t l = threadIdx.x; l < TN; l += blockDim.x) tile[pad16(l)] = P::load(st[gidx(l)]);
-            }
-            __syncthreads();
-            if (it.kind == 1) {
-                tile_gates<P>(tile, T, 0, T, U + (size_t)it.layer * n * 4, a.gmax);
-            } else if (it.kind == 2) {
-                tile_gates<P>(tile, T, L, n - T, U + ((size_t)it.layer * n + T) * 4, a.gmax);
-                for (uint32_t l = threadIdx.x; l < TN; l += blockDim.x) {
-                    const uint64_t x = gidx(l);
-                    if (__popcll(x & (x >> 1)) & 1) tile[pad16(l)] = neg_v<P>(tile[pad16(l)]);
-                }
+            g.t = t;
+            if (tables) {
+                build_tile_factor<P>(g.lay, fac + (size_t)tab_layer * 2 * n, t, s_tf);
                 __syncthreads();
+                g.tf = s_tf;
             }
-            if (it.kind == 2 && it.last_energy) {
-                for (uint32_t l = threadIdx.x; l < TN; l += blockDim.x) {
-                    const uint64_t x = gidx(l);
-                    acc.add_z(tile[pad16(l)], (float)((n - 1) - 2 * __popcll((x ^ (x >> 1)) & zmask)));
-                    for (int q = T; q < n; ++q) {
-                        const int b = L + (q - T);
-                        if (!((l >> b) & 1u)) acc.add_x(tile[pad16(l | (1u << b))], tile[pad16(l)]);
-                    }
+            g.src = it.first ? kFromProduct : kFromGlobal;
+            g.dst = kToGlobal;
+            g.diag = 0;
+            if (it.kind == 1) {
+                run_groups<P>(g, 0, T, kap + (size_t)it.layer * n, true);
+            } else if (high) {
+                if (it.last) g.dst |= kToTile;
+                if (it.first) {                  // a single layer: the product state itself
+                    run_group<P, 1>(g, 0, nullptr);
+                    if (it.last) __syncthreads();
+                } else {
+                    g.diag = 1;
+                    run_groups<P>(g, L, n - T, kap + (size_t)it.layer * n + T, false);
                 }
-            }
-            if (it.kind == 3) {
-                for (uint32_t l = threadIdx.x; l < TN; l += blockDim.x)
-                    for (int q = 0; q < T; ++q)
-                        if (!((l >> q) & 1u)) acc.add_x(tile[pad16(l | (1u << q))], tile[pad16(l)]);
+                if (it.last) {
+                    g.src = kFromTile;
+                    run_energy<P>(g, L, n - T, true, n, acc);
+                }
             } else {
-                for (uint32_t l = threadIdx.x; l < TN; l += blockDim.x) st[gidx(l)] = P::store(tile[pad16(l)]);
+                run_energy<P>(g, 0, T, false, n, acc);
             }
             __syncthreads();
         }
         if (it.slot >= 0) {
-            const double z = acc.z_total(shred);
-            const double x = acc.x_total(shred);
+            const double z = block_sum(acc.z(), shred);
+            const double x = block_sum(acc.x(), shred);
             if (threadIdx.x == 0) a.partials[it.slot] = make_double2(z, x);
         }
         // publish completion; the CTA that completes the circuit sums its energy
@@ -415,38 +736,67 @@ namespace qe {
 
 namespace {
 
+// Host side of a layer: kappa, the slot factors and the flips of every
+// rotation (see the top of the file), angles in qe_batch_create's order.
 template <class P>
-void upload_matrices(qe_batch* b, std::vector<uint64_t>& u_off) {
-    std::vector<typename P::M> h;
+void upload_rotations(qe_batch* b, std::vector<uint64_t>& u_off) {
     u_off.resize(b->count);
-    size_t ai = 0;
+    const size_t total = b->angles.size() / 2;
+    std::vector<typename P::K> kap(total);
+    std::vector<typename P::V> fac(2 * total);
+    std::vector<uint32_t> flips((size_t)b->count * b->layers);
+    size_t i = 0;
     for (int c = 0; c < b->count; ++c) {
         const int n = b->n[c];
-        u_off[c] = h.size();
-        for (int l = 0; l < b->layers; ++l)
-            for (int q = 0; q < n; ++q) {
-                const double th = b->angles[ai++], ph = b->angles[ai++];
-                // RZ(ph) * RY(th)
-                const double c2 = std::cos(0.5 * th), s2 = std::sin(0.5 * th);
-                const cd em = std::polar(1.0, -0.5 * ph), ep = std::polar(1.0, 0.5 * ph);
-                const cd m[4] = {em * c2, -em * s2, ep * s2, ep * c2};
-                for (int k = 0; k < 4; ++k) h.push_back(P::mat(m[k].real(), m[k].imag()));
+        u_off[c] = i;
+        uint32_t flip = 0;
+        for (int l = 0; l < b->layers; ++l) {
+            for (int q = 0; q < n; ++q, ++i) {
+                const double th = b->angles[2 * i], ph = b->angles[2 * i + 1];
+                const double cs = std::cos(0.5 * th);
+                // in the slot basis a flipped qubit turns the other way
+                const double sn = ((flip >> q) & 1u) ? -std::sin(0.5 * th) : std::sin(0.5 * th);
+                const bool trade = std::fabs(sn) > std::fabs(cs);
+                kap[i] = P::make_k(trade ? cs / sn : -sn / cs);
+                const double k = P::value(kap[i]);
+                const double mag = 1.0 / std::sqrt(1.0 + k * k);
+                if (trade) flip ^= 1u << q;
+                // scales of slots 0 and 1: (c, c), or (s, -s) when traded
+                double f0 = std::copysign(mag, trade ? sn : cs), f1 = trade ? -f0 : f0;
+                if (l == 0) f1 *= -k;            // the product state: (p, q) of (1, 0)
+                const double pc = std::cos(0.5 * ph), ps = std::sin(0.5 * ph);
+                const double s0 = ((flip >> q) & 1u) ? ps : -ps;   // slot 0's logical bit is the flip
+                fac[2 * i] = P::make_v(f0 * pc, f0 * s0);
+                fac[2 * i + 1] = P::make_v(f1 * pc, -f1 * s0);
             }
+            flips[(size_t)c * b->layers + l] = flip;
+        }
     }
-    if (b->U) cudaFree(b->U);
-    QE_CUDA(cudaMalloc(&b->U, h.size() * sizeof(typename P::M)));
-    QE_CUDA(cudaMemcpy(b->U, h.data(), h.size() * sizeof(typename P::M), cudaMemcpyHostToDevice));
+    const size_t fb = fac.size() * sizeof(fac[0]), kb = kap.size() * sizeof(kap[0]);
+    if (b->fac) cudaFree(b->fac);
+    b->fac = nullptr;
+    QE_CUDA(cudaMalloc(&b->fac, fb + kb + flips.size() * sizeof(uint32_t)));
+    b->kap = (char*)b->fac + fb;
+    b->flips = (uint32_t*)((char*)b->kap + kb);
+    QE_CUDA(cudaMemcpy(b->fac, fac.data(), fb, cudaMemcpyHostToDevice));
+    QE_CUDA(cudaMemcpy(b->kap, kap.data(), kb, cudaMemcpyHostToDevice));
+    QE_CUDA(cudaMemcpy(b->flips, flips.data(), flips.size() * sizeof(uint32_t), cudaMemcpyHostToDevice));
 }
 
-// States of the large circuits of one wave: together at most this many bytes
-// (half the 129 MB L2 cache).
-constexpr uint64_t kWaveBytes = 64ull << 20;
+// States of the large circuits of one wave: together at most this many bytes.
+// complex64 passes are short enough to want their states in L2 (half of its
+// 129 MB: 25 ms for 512 circuits of 10..22 qubits, 28 ms with 256 MiB); the
+// complex128 passes are bound by arithmetic and gain more from several large
+// circuits that fill the gaps at the ends of each other's passes (with four
+// tiles an item, double-float 72 against 92 ms, FP64 215 against 281 ms).
+template <class P>
+constexpr uint64_t kWaveBytes = (sizeof(typename P::V) == 16 ? 256ull : 64ull) << 20;
 
 template <class P>
 void build_plan(qe_batch* b) {
     const int T = b->plan.T;
     std::vector<uint64_t> u_off;
-    upload_matrices<P>(b, u_off);
+    upload_rotations<P>(b, u_off);
     std::vector<Circ> circ(b->count);
     std::vector<Item> items;
     uint64_t state_off = 0;
@@ -456,6 +806,7 @@ void build_plan(qe_batch* b) {
         Circ& cc = circ[c];
         cc.n = b->n[c];
         cc.u_off = u_off[c];
+        cc.f_off = (uint64_t)c * b->layers;
         cc.state_off = 0;
         if (cc.n <= T) {
             cc.nitems = 1;
@@ -469,7 +820,8 @@ void build_plan(qe_batch* b) {
     }
     // large circuits largest first
     std::stable_sort(large.begin(), large.end(), [&](int x, int y) { return circ[x].n > circ[y].n; });
-    const int P_ = 2 * b->layers + 1;
+    // layer 0 is the product state that the first pass starts from
+    const int P_ = b->layers > 1 ? 2 * (b->layers - 1) + 1 : 2;
     std::vector<std::vector<int>> per_pass_count(b->count, std::vector<int>(P_, 0));
     for (int c : large) {
         Circ& cc = circ[c];
@@ -481,6 +833,9 @@ void build_plan(qe_batch* b) {
         cc.nslots = 2 * nper;   // last high pass + energy low pass
         slots += cc.nslots;
     }
+    size_t total_items = b->count;
+    for (int c : large) total_items += circ[c].nitems;
+    items.reserve(total_items);
     auto push_pass = [&](int c, int p) {
         const Circ& cc = circ[c];
         const uint32_t tiles = 1u << (cc.n - T);
@@ -489,12 +844,13 @@ void build_plan(qe_batch* b) {
         for (int j = 0; j < nper; ++j) {
             Item it{};
             it.circuit = c;
-            it.kind = (p == P_ - 1) ? 3 : (p % 2 == 0 ? 1 : 2);
-            it.layer = p / 2;
+            it.kind = (p == P_ - 1) ? 3 : (b->layers > 1 && p % 2 == 0) ? 1 : 2;
+            it.layer = b->layers > 1 ? 1 + p / 2 : 0;
+            it.first = p == 0;
             it.tile0 = j * per;
             it.tile1 = std::min(tiles, (uint32_t)(j + 1) * per);
             it.dep = (uint32_t)(p * nper);
-            it.last_energy = (p == P_ - 2) ? 1 : 0;
+            it.last = p == P_ - 2;
             it.slot = (p == P_ - 2) ? cc.slot0 + j : (p == P_ - 1) ? cc.slot0 + nper + j : -1;
             items.push_back(it);
         }
@@ -521,8 +877,8 @@ void build_plan(qe_batch* b) {
     std::vector<std::vector<int>> waves;
     uint64_t in_wave = 0;
     for (int c : large) {
-        const uint64_t bytes = (1ull << circ[c].n) * sizeof(typename P::S);
-        if (waves.empty() || in_wave + bytes > kWaveBytes) {
+        const uint64_t bytes = (1ull << circ[c].n) * sizeof(typename P::V);
+        if (waves.empty() || in_wave + bytes > kWaveBytes<P>) {
             waves.emplace_back();
             in_wave = 0;
         }
@@ -540,7 +896,7 @@ void build_plan(qe_batch* b) {
     for (; si < small.size(); ++si) push_small(small[si]);
     b->nitems = (int)items.size();
     // device buffers
-    const size_t need_states = state_off * sizeof(typename P::S);
+    const size_t need_states = state_off * sizeof(typename P::V);
     if (b->state_bytes < need_states) {
         if (b->states) cudaFree(b->states);
         b->states = nullptr;
@@ -561,7 +917,7 @@ void build_plan(qe_batch* b) {
     // writes its state, the energy pass only reads it, the others do both:
     // 1 + 2 (P - 2) + 1 = 2 (P - 1) state sizes
     double bytes = 0.0;
-    for (int c : large) bytes += 2.0 * (P_ - 1) * (double)((1ull << circ[c].n) * sizeof(typename P::S));
+    for (int c : large) bytes += 2.0 * (P_ - 1) * (double)((1ull << circ[c].n) * sizeof(typename P::V));
     b->hbm_bytes = bytes;
 }
 
@@ -572,8 +928,10 @@ void capture(qe_batch* b) {
     b->exec = nullptr;
     b->graph = nullptr;
     static thread_local BatchArgs<P> a;
-    a.states = reinterpret_cast<typename P::S*>(b->states);
-    a.U = reinterpret_cast<const typename P::M*>(b->U);
+    a.states = reinterpret_cast<typename P::V*>(b->states);
+    a.kap = reinterpret_cast<const typename P::K*>(b->kap);
+    a.fac = reinterpret_cast<const typename P::V*>(b->fac);
+    a.flips = b->flips;
     a.items = reinterpret_cast<const Item*>(b->items);
     a.circ = reinterpret_cast<const Circ*>(b->circ);
     a.nitems = b->nitems;
@@ -586,9 +944,7 @@ void capture(qe_batch* b) {
     a.partials = b->partials;
     a.energies = b->energies;
     a.spin_limit = 1ll << 24;   // ~4 s of 256 ns sleeps
-    // gates per register group, measured best on GB300: 2 (double-float), 4 (FP32)
-    a.gmax = sizeof(typename P::V) >= 16 ? 2 : 4;
-    const size_t smem = (sizeof(typename P::V) << b->plan.T) + (sizeof(typename P::V) << b->plan.T) / 16;
+    const size_t smem = sizeof(typename P::V) * (((size_t)1 << b->plan.T) + kTabA + kTabB + 1);
     auto fn = k_batch<P>;
     QE_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     int occ = 0;
@@ -610,14 +966,14 @@ void capture(qe_batch* b) {
 
 void prepare(qe_batch* b) {
     if (b->dtype == QE_C64) {
-        build_plan<F32>(b);
-        capture<F32>(b);
+        build_plan<BF32>(b);
+        capture<BF32>(b);
     } else if (b->arith == QE_ARITH_FP64) {
-        build_plan<F64>(b);
-        capture<F64>(b);
+        build_plan<BF64>(b);
+        capture<BF64>(b);
     } else {
-        build_plan<DF>(b);
-        capture<DF>(b);
+        build_plan<BDF>(b);
+        capture<BDF>(b);
     }
 }
 
@@ -660,7 +1016,7 @@ void batch_set_plan(qe_batch* b, int T, int tiles_per_item, int threads) {
 void batch_destroy(qe_batch* b) {
     if (b->exec) cudaGraphExecDestroy(b->exec);
     if (b->graph) cudaGraphDestroy(b->graph);
-    for (void* p : {b->states, b->U, b->items, b->circ, (void*)b->sync, (void*)b->partials, (void*)b->energies})
+    for (void* p : {b->states, b->fac, b->items, b->circ, (void*)b->sync, (void*)b->partials, (void*)b->energies})
         if (p) cudaFree(p);
     if (b->host_energies) cudaFreeHost(b->host_energies);
     if (b->host_status) cudaFreeHost(b->host_status);
