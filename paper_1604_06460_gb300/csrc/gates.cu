@@ -399,30 +399,30 @@ void launch_gate_dense(qe_state* s, int k, const int* qubits, const cd* U) {
     // and in native FP64 arithmetic)
     const int kmin = tc64 ? 4 : c128_tc_kmin(s);
     if ((tc64 || tc128) && s->tensor_cores && !s->force_tile && s->n >= 12 && k >= kmin) {
-        auto run = [&](const int* q5, const cd* U5) {
-            if (tc64) launch_gate_tc5(s, q5, U5);
-            else launch_gate_tc5_c128(s, q5, U5);
-        };
-        if (k == 5) {
-            run(qubits, U);
-            return;
-        }
-        // widen the block by 5 - k idle qubits (the lowest ones not in the
-        // block): U5 = 1 (x) U, the idle qubits as the high matrix bits
-        int q5[5];
+        // Widen the block by 5 - k idle qubits (U5 = 1 (x) U on them) and order
+        // the matrix bits by qubit, as the kernels' memory access wants them.
+        // The idle qubits are the lowest ones from 5 on: qubits 0..4 as row
+        // bits let a warp touch whole lines.
+        int q5[5], w = k;
         for (int j = 0; j < k; ++j) q5[j] = qubits[j];
-        int w = k;
-        for (int c = 0; c < s->n && w < 5; ++c) {
-            bool used = false;
-            for (int j = 0; j < k; ++j) used |= qubits[j] == c;
-            if (!used) q5[w++] = c;
-        }
+        for (int c = 5; w < 5; c = c + 1 < s->n ? c + 1 : 0)
+            if (std::find(q5, q5 + w, c) == q5 + w) q5[w++] = c;
+        int order[5] = {0, 1, 2, 3, 4};
+        std::sort(order, order + 5, [&](int x, int y) { return q5[x] < q5[y]; });
         const int d = 1 << k;
-        std::vector<cd> U5(32 * 32, cd(0.0));
-        for (int hb = 0; hb < (32 >> k); ++hb)
-            for (int r = 0; r < d; ++r)
-                for (int c = 0; c < d; ++c) U5[(r | (hb << k)) * 32 + (c | (hb << k))] = U[r * d + c];
-        run(q5, U5.data());
+        int of[32];   // matrix index in (q5) bit order of the ordered index
+        for (int r = 0; r < 32; ++r) {
+            of[r] = 0;
+            for (int j = 0; j < 5; ++j) of[r] |= ((r >> j) & 1) << order[j];
+        }
+        static thread_local std::vector<cd> U5(32 * 32);
+        for (int r = 0; r < 32; ++r)
+            for (int c = 0; c < 32; ++c)
+                U5[r * 32 + c] = (of[r] >> k) == (of[c] >> k) ? U[(of[r] & (d - 1)) * d + (of[c] & (d - 1))] : cd(0.0);
+        int qs[5];
+        for (int j = 0; j < 5; ++j) qs[j] = q5[order[j]];
+        if (tc64) launch_gate_tc5(s, qs, U5.data());
+        else launch_gate_tc5_c128(s, qs, U5.data());
         return;
     }
     QE_DISPATCH(s, dense_k, s, k, qubits, U);

@@ -120,6 +120,48 @@ __device__ __forceinline__ void mbar_arrive(uint64_t* mbar) {
     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(mbar)) : "memory");
 }
 
+// 2^VEC neighbouring columns moved by one instruction: VEC = 2 when matrix bits
+// 0 and 1 are qubits 0 and 1 (four columns are 32 contiguous bytes), 1 when
+// matrix bit 0 is qubit 0 and bit 1 is not qubit 1, else 0 (one lane a row,
+// lanes contiguous).  A pass at n = 28 on qubits 0..4: 1.06 ms, 2.67 ms
+// with a row a lane throughout; on 0, 1, 2, 20, 27: 0.70 and 1.52 ms.
+template <int VEC>
+__device__ __forceinline__ void load_cols(const float2* g, const uint64_t* off, float2* dst) {
+    if constexpr (VEC == 2) {
+        asm volatile("ld.global.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                     : "=f"(dst[0].x), "=f"(dst[0].y), "=f"(dst[1].x), "=f"(dst[1].y), "=f"(dst[2].x), "=f"(dst[2].y),
+                       "=f"(dst[3].x), "=f"(dst[3].y)
+                     : "l"(g + off[0]));
+    } else if constexpr (VEC == 1) {
+#pragma unroll
+        for (int u = 0; u < 4; u += 2) {
+            const float4 v = *reinterpret_cast<const float4*>(g + off[u]);
+            dst[u] = make_float2(v.x, v.y);
+            dst[u + 1] = make_float2(v.z, v.w);
+        }
+    } else {
+#pragma unroll
+        for (int u = 0; u < 4; ++u) dst[u] = g[off[u]];
+    }
+}
+template <int VEC>
+__device__ __forceinline__ void store_cols(float2* g, const uint64_t* off, const uint32_t* re, const uint32_t* im) {
+    if constexpr (VEC == 2) {
+        asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(g + off[0]), "r"(re[0]), "r"(im[0]),
+                     "r"(re[1]), "r"(im[1]), "r"(re[2]), "r"(im[2]), "r"(re[3]), "r"(im[3])
+                     : "memory");
+    } else if constexpr (VEC == 1) {
+#pragma unroll
+        for (int u = 0; u < 4; u += 2)
+            *reinterpret_cast<uint4*>(g + off[u]) = make_uint4(re[u], im[u], re[u + 1], im[u + 1]);
+    } else {
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+            *reinterpret_cast<uint2*>(g + off[u]) = make_uint2(re[u], im[u]);
+    }
+}
+
+template <int VEC>
 __global__ void __maxnreg__(72) k_gate_tc5(const __grid_constant__ TcArgs a) {
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     // 1024-byte aligned regions: W_hi, W_lo (64 x 64 x 4 B), then per operand
@@ -253,22 +295,23 @@ __global__ void __maxnreg__(72) k_gate_tc5(const __grid_constant__ TcArgs a) {
         auto load_tile = [&](uint64_t t, float2* dst) {
             const float2* g = a.x + insert_zero_bits(t << a.L, a.hq, a.kh) + rowoff;
 #pragma unroll
-            for (int j = 0; j < 2; ++j)
-#pragma unroll
-                for (int u = 0; u < 4; ++u) dst[4 * j + u] = g[coloff[4 * (qbase + 4 * j) + u]];
+            for (int j = 0; j < 2; ++j) load_cols<VEC>(g, coloff + 4 * (qbase + 4 * j), dst + 4 * j);
         };
         uint64_t t = blockIdx.x;
         if (t < a.ntiles) load_tile(t, cur);
         for (int i = 0; t < a.ntiles; t += gridDim.x, ++i) {
             const int b = i & 1;
             // the next tile's loads are in flight while this one is split; the
-            // tile after it is prefetched into L2 (its 2^kh contiguous runs of
-            // 2^L amplitudes, >= 1 KB, one bulk prefetch each)
+            // tile after it is prefetched into L2, 1 KB by one lane of every
+            // half-warp (its runs are at least 1 KB; one prefetch a run, all
+            // from the first warp, held that warp up: 1.15 ms against 0.76 ms
+            // a pass on qubits 23..27 at n = 28)
             const uint64_t tn = t + gridDim.x, tn2 = tn + gridDim.x;
             if (tn < a.ntiles) load_tile(tn, nxt);
-            if (tn2 < a.ntiles && st < (1 << a.kh)) {
-                const float2* g2 = a.x + insert_zero_bits(tn2 << a.L, a.hq, a.kh) + hoff[st];
-                asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(g2), "r"(8u << a.L) : "memory");
+            if (tn2 < a.ntiles && (st & 15) == 0) {
+                const int run = (st >> 4) >> (a.L - 7), piece = (st >> 4) & ((1 << (a.L - 7)) - 1);
+                const float2* g2 = a.x + insert_zero_bits(tn2 << a.L, a.hq, a.kh) + hoff[run] + (piece << 7);
+                asm volatile("cp.async.bulk.prefetch.L2.global [%0], 1024;" ::"l"(g2) : "memory");
             }
             // the MMAs two tiles back have read this operand buffer
             if (i >= 2 && !wait_warp(&mbDone[b], (uint32_t)((i - 2) >> 1) & 1u, a.spin_limit, &s_abort)) {
@@ -338,8 +381,7 @@ __global__ void __maxnreg__(72) k_gate_tc5(const __grid_constant__ TcArgs a) {
                     mbar_arrive(&mbAccFree[b]);
                 }
 #pragma unroll
-                for (int c = 0; c < 8; ++c)
-                    gout[coloff[ehalf + 8 * h + c]] = make_float2(__uint_as_float(re[c]), __uint_as_float(im[c]));
+                for (int c = 0; c < 8; c += 4) store_cols<VEC>(gout, coloff + ehalf + 8 * h + c, re + c, im + c);
             }
         }
     }
@@ -398,12 +440,13 @@ void launch_gate_tc5(qe_state* s, const int* qubits, const cd* U) {
     a.stall_test = (stall != nullptr && stall[0] == '1') ? 1 : 0;
     if (a.stall_test) a.spin_limit = 1ll << 12;
     const size_t smem = 1024 + (size_t)2 * kN * kK * 4 + (size_t)2 * 2 * kRows * kK * 4;
-    QE_CUDA(cudaFuncSetAttribute(k_gate_tc5, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    QE_CUDA(cudaFuncSetAttribute(k_gate_tc5, cudaFuncAttributePreferredSharedMemoryCarveout, 100));
+    auto fn = qubits[0] != 0 ? k_gate_tc5<0> : qubits[1] != 1 ? k_gate_tc5<1> : k_gate_tc5<2>;
+    QE_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    QE_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributePreferredSharedMemoryCarveout, 100));
     const uint64_t grid = std::min<uint64_t>(a.ntiles, (uint64_t)num_sms());
     {
         Launch Lc(s, "gate_tc_k5", 2.0 * dim(s) * amp_bytes(s));
-        k_gate_tc5<<<(unsigned)grid, kTcThreads, smem, s->stream>>>(a);
+        fn<<<(unsigned)grid, kTcThreads, smem, s->stream>>>(a);
         QE_CUDA(cudaGetLastError());
     }
     // checked before the next tensor-core launch or at the end of the flush,
