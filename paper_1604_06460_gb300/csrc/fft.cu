@@ -225,26 +225,18 @@ __global__ void __launch_bounds__(kFftThreads) k_fft_pass(const __grid_constant_
 }
 
 // --------------------------------------------------------------- bitrev
-// In-place reversal of the order of the register value's D-bit digits (D = 1:
-// the bit reversal).  Work item = (outer bits, middle value Mv <= rev(Mv));
-// tiles X(Mv) and Y(rev Mv) hold elements [b][a][w] (b: top c register bits,
-// a: bottom c register bits, c a multiple of D, w: the lo qubits below the
-// register) and are exchanged transposed and digit-reversed.
+// In-place reversal of the register value's bits.  Work item = (outer bits,
+// middle value Mv <= rev(Mv)); tiles X(Mv) and Y(rev Mv) hold elements
+// [b][a][w] (b: top c register bits, a: bottom c register bits, w: the lo
+// qubits below the register) and are exchanged transposed and bit-reversed.
 template <class P>
 struct RevArgs {
     typename P::S* x;
     uint64_t items;
-    int lo, m, c, D;
+    int lo, m, c;
 };
 
-// v (bits bits, a multiple of D) with the order of its D-bit digits reversed.
-__device__ __forceinline__ uint64_t digit_rev(uint64_t v, int bits, int D) {
-    if (D == 1) return bits > 0 ? (__brevll(v) >> (64 - bits)) : 0ull;
-    uint64_t r = 0;
-    const uint64_t dm = (1ull << D) - 1ull;
-    for (int i = 0; i < bits; i += D) r = (r << D) | ((v >> i) & dm);
-    return r;
-}
+__device__ __forceinline__ uint64_t bit_rev(uint64_t v, int bits) { return bits > 0 ? (__brevll(v) >> (64 - bits)) : 0ull; }
 
 template <class P>
 __global__ void __launch_bounds__(256) k_bitrev(const __grid_constant__ RevArgs<P> a) {
@@ -257,9 +249,15 @@ __global__ void __launch_bounds__(256) k_bitrev(const __grid_constant__ RevArgs<
     const int mid_bits = a.m - 2 * a.c;
     const uint64_t nmid = 1ull << mid_bits;
     for (uint64_t item = blockIdx.x; item < a.items; item += gridDim.x) {
-        const uint64_t mv = item & (nmid - 1ull);
+        // the middle value's low and high bits vary first, so that the tiles in
+        // flight, and their partners, are neighbours in memory a few at a time
+        uint64_t mv = item & (nmid - 1ull);
+        if (mid_bits >= 8) {
+            const uint64_t h = (mv >> 4) & 15ull;
+            mv = (mv & 15ull) | ((mv >> 8) << 4) | (h << (mid_bits - 4));
+        }
         const uint64_t outer = item >> mid_bits;
-        const uint64_t mr = digit_rev(mv, mid_bits, a.D);
+        const uint64_t mr = bit_rev(mv, mid_bits);
         if (mv > mr) continue;
         const bool self = (mv == mr);
         const uint64_t obase = outer << (a.lo + a.m);
@@ -278,8 +276,8 @@ __global__ void __launch_bounds__(256) k_bitrev(const __grid_constant__ RevArgs<
         for (int i = threadIdx.x; i < n; i += blockDim.x) {
             const int b2 = i / (C * W), aw = i % (C * W);
             const int a2 = aw / W, w = aw % W;
-            const int rb = (int)digit_rev((uint64_t)a2, a.c, a.D);   // source b
-            const int ra = (int)digit_rev((uint64_t)b2, a.c, a.D);   // source a
+            const int rb = (int)bit_rev((uint64_t)a2, a.c);   // source b
+            const int ra = (int)bit_rev((uint64_t)b2, a.c);   // source a
             const uint64_t off = ((uint64_t)b2 << shb) | (uint64_t)aw;
             a.x[bx + off] = srcX[rb * row + ra * W + w];
             if (!self) a.x[by + off] = X[rb * row + ra * W + w];
@@ -409,12 +407,12 @@ void fft_impl(qe_state* s, int lo, int m, int inverse, int pol) {
 }
 
 template <class S>
-__global__ void __launch_bounds__(256) k_bitrev_chunks(S* __restrict__ x, uint64_t count, int lo, int m, int D) {
+__global__ void __launch_bounds__(256) k_bitrev_chunks(S* __restrict__ x, uint64_t count, int lo, int m) {
     const uint64_t rmask = ((1ull << m) - 1ull) << lo;
     for (uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i < count;
          i += (uint64_t)gridDim.x * blockDim.x) {
         const uint64_t k = (i & rmask) >> lo;
-        const uint64_t kr = digit_rev(k, m, D);
+        const uint64_t kr = bit_rev(k, m);
         if (k < kr) {
             const uint64_t j = (i & ~rmask) | (kr << lo);
             S t = x[i];
@@ -425,23 +423,22 @@ __global__ void __launch_bounds__(256) k_bitrev_chunks(S* __restrict__ x, uint64
 }
 
 template <class P>
-void bitrev_impl(qe_state* s, int lo, int m, int D = 1) {
-    if (m <= D) return;
+void bitrev_impl(qe_state* s, int lo, int m, const char* tag = "bitrev") {
+    if (m <= 1) return;
     using S = typename P::S;
-    Launch L(s, D == 1 ? "bitrev" : "digitrev", 2.0 * dim(s) * amp_bytes(s));
-    // end blocks of c bits (a multiple of D, 2c <= m) in tiles of 2^(2c + lo) <= 2^11
-    const int c = D * std::min(m / (2 * D), std::max(0, (11 - lo) / 2) / D);
+    Launch L(s, tag, 2.0 * dim(s) * amp_bytes(s));
+    // end blocks of c bits (2c <= m) in tiles of 2^(2c + lo) <= 2^11
+    const int c = std::min(m / 2, std::max(0, (11 - lo) / 2));
     if (lo >= 5 || c == 0) {
         // chunks of >= 32 contiguous amplitudes move as units: coalesced pair swaps
         const uint64_t count = dim(s);
         unsigned grid = (unsigned)std::min<uint64_t>((count + 255) / 256, (uint64_t)num_sms() * 8);
-        k_bitrev_chunks<S><<<grid, 256, 0, s->stream>>>(reinterpret_cast<S*>(s->d), count, lo, m, D);
+        k_bitrev_chunks<S><<<grid, 256, 0, s->stream>>>(reinterpret_cast<S*>(s->d), count, lo, m);
     } else {
         static thread_local RevArgs<P> a;
         a.x = reinterpret_cast<S*>(s->d);
         a.lo = lo;
         a.m = m;
-        a.D = D;
         a.c = c;
         a.items = (1ull << (s->n - lo - m)) << (m - 2 * a.c);
         const int C = 1 << a.c, W = 1 << lo;
@@ -457,59 +454,61 @@ void bitrev_impl(qe_state* s, int lo, int m, int D = 1) {
 }
 
 // ------------------------------------------------ tensor-core digit passes
-// The QFT of a register of m = G d bits as G dense d-qubit blocks on the
-// tensor cores (the 2^d-point DFT, the same matrix for every group of the
-// other qubits) with diagonal twiddles between them (Cooley-Tukey, digits
-// from the top): with k = k0 2^(m-d) + k' and l = l0 + 2^d l',
-//   y_l = sum_k' w_(2^(m-d))^(k' l') [ w_(2^m)^(k' l0) sum_k0 x_(k0, k') w_(2^d)^(k0 l0) ],
-// so a pass applies the DFT to the top digit (output l0 left in its qubits),
-// a twiddle pass multiplies by w_(2^m)^(k' l0), and the rest is the QFT of
-// the lower m - d bits; at the end the digits sit in reversed order and one
-// digit-reversal pass restores the natural order.  Scale 2^(-d/2) per block.
-template <class P>
+// The QFT of a register of m qubits as G = ceil(m / 5) dense blocks of 3..5
+// qubits on the tensor cores (Cooley-Tukey, digits from the top).  With the
+// digits of the register value from the top k_0, k_1, ... (k = k_0 2^(m-d_0) + k')
+// and the outputs so far l = l_0 + 2^(d_0) l_1 + ..., digit j is
+//   y = sum_(k_j) x(k_j) 2^(-d_j/2) w_(2^(P+d_j))^(k_j (l + 2^P l_j)),
+// P = d_0 + .. + d_(j-1): its 2^(d_j)-point transform with the twiddle
+// w_(2^(P+d_j))^(k_j l) folded into the matrix, which then depends on the
+// outputs l (qubits outside the block).  What is left of the twiddles, by the
+// lower bits k' that no digit of this group will meet, is w_(2^m)^(k' l) for l
+// all the outputs of the group: one diagonal pass for each group of digits
+// instead of one for each digit.  Every digit leaves its output bit-reversed in
+// its own qubits, so one bit reversal of the register restores the natural
+// order for any split into digits (a single digit writes it directly).
+//
+// A digit joins the group while a matrix still serves at least 16 tiles
+// (P <= n - 16: rebuilding it costs a segment of the pipeline, about two tiles)
+// and its roots fit a direct table (P + d <= 20); the digits are then spread
+// evenly over that number of groups.  Measured on complex128 in the FP64 mode,
+// against dense blocks with a twiddle pass after each (m a multiple of its
+// digit) or the shared-memory transform: the 30-qubit QFT 121 -> 79 ms (six
+// digits 54, one twiddle pass 15.4, reversal 9), 29 qubits 161 -> 39.5 ms, 17
+// qubits from qubit 5 of 27 on 24.9 -> 5.9 ms.
 struct TwArgs {
-    typename P::S* x;
-    const typename P::M* fine;
-    const typename P::M* coarse;
-    const typename P::M* direct;   // w_(2^(top + d))^j for all j, when the order is at most 2^20 (else null)
+    double2* x;
+    const double2* fine;
+    const double2* coarse;
+    const double2* direct;   // w_(2^(base + S))^j for all j, when that order is at most 2^20 (else null)
     uint64_t count;
-    int lo, m, h;
-    int top;      // the digit just transformed: register bits [top, top + d)
-    int d;
+    int lo, h;
+    int base, S;  // the group just transformed: register bits [base, base + S)
     int shift;    // the twiddle exponent's scale to the 2^m table: 2^shift
 };
 
-// x *= w_(2^(top + d))^(k' l0), k' = register bits [0, top), l0 = bits [top, top + d)
-template <class P>
-__global__ void __launch_bounds__(256) k_digit_twiddle(const __grid_constant__ TwArgs<P> a) {
-    const uint64_t rmask = (1ull << a.m) - 1ull;
+// x *= w_(2^(base + S))^(k' l), k' = register bits [0, base), l = bits
+// [base, base + S) read from the top down
+__global__ void __launch_bounds__(256) k_digit_twiddle(const __grid_constant__ TwArgs a) {
     const uint64_t hmask = (1ull << a.h) - 1ull;
     for (uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i < a.count;
          i += (uint64_t)gridDim.x * blockDim.x) {
-        const uint64_t r = (i >> a.lo) & rmask;
-        const uint64_t kp = r & ((1ull << a.top) - 1ull);
-        const uint64_t l0 = (r >> a.top) & ((1ull << a.d) - 1ull);
-        if (kp == 0 || l0 == 0) continue;
-        // exponent over 2^(top + d): one table entry when the order is small
+        const uint64_t r = i >> a.lo;
+        const uint64_t kp = r & ((1ull << a.base) - 1ull);
+        const uint64_t l = __brevll(r >> a.base) >> (64 - a.S);
+        if (kp == 0 || l == 0) continue;
+        // exponent over 2^(base + S): one table entry when the order is small
         // enough for a direct table, else the product of the two 2^m tables
-        const uint64_t e0 = (kp * l0) & ((1ull << (a.top + a.d)) - 1ull);
-        typename P::M w;
+        const uint64_t e0 = (kp * l) & ((1ull << (a.base + a.S)) - 1ull);
+        double2 w;
         if (a.direct) {
             w = a.direct[e0];
         } else {
             const uint64_t e = e0 << a.shift;
-            w = P::cmul(a.coarse[e >> a.h], a.fine[e & hmask]);
+            w = F64::cmul(a.coarse[e >> a.h], a.fine[e & hmask]);
         }
-        a.x[i] = P::store(P::cmul(w, P::load(a.x[i])));
+        a.x[i] = F64::cmul(w, a.x[i]);
     }
-}
-
-// Digit size for the tensor-core QFT of an m-bit register: the largest of
-// 5, 4, 3 dividing m (0: none).
-int qft_digit(int m) {
-    for (int d : {5, 4, 3})
-        if (m % d == 0) return d;
-    return 0;
 }
 
 // Direct table of the 2^k roots of unity w_(2^k)^j (FP64-generated, stored in
@@ -539,67 +538,82 @@ const typename P::M* get_direct(qe_state* s, int k, int sign, int pol) {
     const unsigned grid = (unsigned)std::min<uint64_t>(((1ull << k) + 255) / 256, 4096);
     k_roots_direct<P><<<grid, 256, 0, s->stream>>>((typename P::M*)t, k, sign);
     QE_CUDA(cudaGetLastError());
+    QE_CUDA(cudaStreamSynchronize(s->stream));   // once a table: later callers may be on other streams
     g_direct[key] = t;
     return (const typename P::M*)t;
 }
 
-template <class P>
-void qft_tc_impl(qe_state* s, int lo, int m, int inverse, int pol, int d) {
+void qft_tc(qe_state* s, int lo, int m, int inverse) {
     const int sign = inverse ? -1 : 1;
-    Table tb = get_tables<P>(s, m, sign, pol);
-    const int D = 1 << d;
-    std::vector<cd> F((size_t)D * D);
-    const double sc = 1.0 / std::sqrt((double)D);
-    for (int l = 0; l < D; ++l)
-        for (int k = 0; k < D; ++k) {
-            const double t = sign * 2.0 * ((double)((k * l) % D) / D);   // angle in units of pi
-            F[(size_t)l * D + k] = cd(sc * std::cos(M_PI * t), sc * std::sin(M_PI * t));
-        }
-    // exact values at the quarter turns (cos/sin of multiples of pi/2)
-    for (auto& v : F) {
-        if (std::fabs(v.real()) < 1e-17) v = cd(0.0, v.imag());
-        if (std::fabs(v.imag()) < 1e-17) v = cd(v.real(), 0.0);
-    }
-    static thread_local TwArgs<P> a;
-    a.x = reinterpret_cast<typename P::S*>(s->d);
-    a.fine = (const typename P::M*)tb.fine;
-    a.coarse = (const typename P::M*)tb.coarse;
+    const int G = (m + 4) / 5;
+    int digit[7];
+    for (int j = 0; j < G; ++j) digit[j] = m / G + (j >= G - m % G ? 1 : 0);   // wider ones lowest: longer runs
+    // the fewest groups, then as even as possible
+    auto fits = [&](int P, int d) { return P == 0 || (P <= s->n - 16 && P + d <= 20); };
+    int groups = 0;
+    for (int j = 0; j < G; ++groups)
+        for (int P = 0; j < G && fits(P, digit[j]); P += digit[j++]) {}
+    static thread_local TwArgs a;
+    a.x = reinterpret_cast<double2*>(s->d);
     a.count = dim(s);
     a.lo = lo;
-    a.m = m;
     a.h = (m + 1) / 2;
-    a.d = d;
-    const int G = m / d;
-    for (int t = 0; t < G; ++t) {
-        const int top = m - d * (t + 1);
-        int q[5];
-        for (int j = 0; j < d; ++j) q[j] = lo + top + j;
-        launch_gate_dense(s, d, q, F.data());
+    int top = m, j = 0;
+    uint32_t* const status = dft_digits_begin(s);
+    for (int g = 0; g < groups; ++g) {
+        const int last = G * (g + 1) / groups;
+        int P = 0;
+        for (; j < last; ++j) {
+            const int d = digit[j];
+            top -= d;
+            launch_dft_digit_c128(s, lo + top, d, P, G > 1, get_direct<F64>(s, P + d, sign, 1), status);
+            P += d;
+        }
         if (top == 0) break;
-        a.top = top;
-        a.shift = m - (top + d);
-        a.direct = (top + d <= 20) ? get_direct<P>(s, top + d, sign, pol) : nullptr;
+        a.base = top;
+        a.S = P;
+        a.shift = m - (top + P);
+        a.direct = (top + P <= 20) ? get_direct<F64>(s, top + P, sign, 1) : nullptr;
+        if (!a.direct) {
+            const Table tb = get_tables<F64>(s, m, sign, 1);
+            a.fine = (const double2*)tb.fine;
+            a.coarse = (const double2*)tb.coarse;
+        }
         const unsigned grid = (unsigned)std::min<uint64_t>((a.count + 255) / 256, (uint64_t)num_sms() * 8);
         Launch L(s, "fft_twiddle", 2.0 * dim(s) * amp_bytes(s));
-        k_digit_twiddle<P><<<grid, 256, 0, s->stream>>>(a);
+        k_digit_twiddle<<<grid, 256, 0, s->stream>>>(a);
         QE_CUDA(cudaGetLastError());
     }
-    bitrev_impl<F64>(s, lo, m, d);
+    dft_digits_end(s, status);
+    if (G > 1) bitrev_impl<F64>(s, lo, m, "digitrev");
 }
 
 }  // namespace
 
-// Tensor-core digit passes in the FP64 mode where a dense block of 3-5
-// qubits runs on the tensor cores (n >= 12) and a digit size divides m;
-// otherwise the radix-2 shared-memory FFT.
+// Digit passes on the tensor cores or the radix-2 shared-memory transform, for
+// complex128 registers of at least 3 qubits on states of at least 12.  A digit
+// pass takes about 15 us on a small state and 1/0.24 of the copy time on a large
+// one; a shared-memory pass (11 stages, 8 to 10 above low qubits) costs the
+// arithmetic of its stages.  Measured (ms, shared memory / digits):
+//   FP64 mode, one shared-memory pass: n = 18, m = 11 0.041 / 0.088, n = 20
+//   0.127 / 0.105, n = 24 1.52 / 0.63; n = 20, m = 5 0.06 / 0.038;
+//   several passes: n = 17, m = 17 0.077 / 0.106, n = 19 0.141 / 0.120, n = 24,
+//   m = 23 3.96 / 1.30 (registers of whole five-qubit digits above one pass
+//   take the digits at every size);
+//   double-float mode: n = 24, m = 5 0.294 / 0.195 (n = 20 0.031 / 0.038),
+//   m = 10 0.439 / 0.483, m = 24 1.48 / 1.34, n = 20, m = 20 0.120 / 0.160,
+//   n = 30, m = 30 118 / 79.
+static bool qft_on_tensor_cores(const qe_state* s, int lo, int m) {
+    if (s->dtype != QE_C128 || !s->c128_tc || !s->tensor_cores || s->force_tile || s->n < 12 || m < 3) return false;
+    const bool one_pass = m <= 11 - std::min(lo, 3);
+    if (s->arith == QE_ARITH_FP64) return one_pass ? s->n >= 20 : s->n >= 19 || m % 5 == 0;
+    return m <= 5 ? s->n >= 22 : !one_pass && s->n >= 23;
+}
+
 void launch_qft_fft(qe_state* s, int lo, int m, int inverse) {
-    const int d = qft_digit(m);
-    // (in the double-float mode the shared-memory FFT is the faster: its
-    // twiddle joins cost as much FP64 work as the digit passes save)
-    const bool tc = s->dtype == QE_C128 && s->arith == QE_ARITH_FP64 && s->c128_tc && s->tensor_cores &&
-                    !s->force_tile && s->n >= 12 && d >= c128_tc_kmin(s) && m > 1;
+    const bool tc = qft_on_tensor_cores(s, lo, m);
     if (tc) {
-        qft_tc_impl<F64>(s, lo, m, inverse, 1, d);
+        qft_tc(s, lo, m, inverse);
         return;
     }
     if (s->dtype == QE_C64) fft_impl<F32>(s, lo, m, inverse, 0);

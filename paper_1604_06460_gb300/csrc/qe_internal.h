@@ -127,9 +127,16 @@ void launch_gate_dense(qe_state* s, int k, const int* qubits, const cd* U);
 // waits for the stream and raises QE_ERR_TIMEOUT if a launch reported one.
 uint32_t* status_word_host(qe_state* s);
 void complete_pending(qe_state* s);
-// 5-qubit block on a complex64 state with tcgen05 tensor cores (n >= 12)
+// 5-qubit block on a complex64 / complex128 state with tcgen05 tensor cores
+// (n >= 12, qubits ascending)
 void launch_gate_tc5(qe_state* s, const int* qubits, const cd* U);
 void launch_gate_tc5_c128(qe_state* s, const int* qubits, const cd* U);
+// one digit [q0, q0 + d) of a Fourier transform on a complex128 state, its
+// matrix chosen by the P qubits above it; begin and end bracket a run of digits
+// that share a status word (tc_c128.cu)
+uint32_t* dft_digits_begin(qe_state* s);
+void launch_dft_digit_c128(qe_state* s, int q0, int d, int P, bool reversed, const double2* roots, uint32_t* status);
+void dft_digits_end(qe_state* s, const uint32_t* status);
 // diagonal gate: amplitude x *= d[row(x)] for all x
 void launch_gate_diag(qe_state* s, int k, const int* qubits, const cd* d);
 // amplitudes with (x & mask) == value are multiplied by phase

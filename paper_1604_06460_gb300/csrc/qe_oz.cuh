@@ -29,6 +29,32 @@ __device__ __forceinline__ void mma_f16(uint32_t d_tmem, uint64_t a, uint64_t b,
         "l"(a), "l"(b), "r"(idesc), "r"(accumulate));
 }
 
+// The same, issued by the lanes with `elected` set of a converged warp: the
+// operands stay warp-uniform values, which the compiler can keep in uniform
+// registers (where the instruction wants them).
+__device__ __forceinline__ void mma_f16_elected(uint32_t elected, uint32_t d_tmem, uint64_t a, uint64_t b, uint32_t idesc,
+                                                uint32_t accumulate) {
+    asm volatile(
+        "{\n\t.reg .pred p, q;\n\t"
+        "setp.ne.b32 p, %4, 0;\n\t"
+        "setp.ne.b32 q, %5, 0;\n\t"
+        "@q tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}\n" ::"r"(d_tmem),
+        "l"(a), "l"(b), "r"(idesc), "r"(accumulate), "r"(elected));
+}
+__device__ __forceinline__ void mma_commit_elected(uint32_t elected, uint64_t* mbar) {
+    asm volatile(
+        "{\n\t.reg .pred q;\n\t"
+        "setp.ne.b32 q, %1, 0;\n\t"
+        "@q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}\n" ::"r"(smem_u32(mbar)),
+        "r"(elected));
+}
+// 1 on one lane of a converged warp.
+__device__ __forceinline__ uint32_t elect_lane() {
+    uint32_t e;
+    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xFFFFFFFF;\n\tselp.b32 %0, 1, 0, p;\n\t}\n" : "=r"(e));
+    return e;
+}
+
 __device__ __forceinline__ void cp_async16(uint32_t dst, const void* src) {
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src));
 }
@@ -66,13 +92,6 @@ __device__ __forceinline__ bool wait_or_abort(uint32_t mbar, uint32_t phase, lon
     *reinterpret_cast<volatile uint32_t*>(abort_flag) = 1u;
     return false;
 }
-
-// Bulk prefetch of `bytes` (a multiple of 16) at a 16-byte aligned global
-// address into L2.
-__device__ __forceinline__ void l2_prefetch(const void* p, uint32_t bytes) {
-    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p), "r"(bytes) : "memory");
-}
-
 
 // The balanced-offset integer Z of v (as two words) for a row whose largest
 // biased exponent is em: X = round(|v| 2^(8D - E_r)) = round(M53 2^(e - em + 8D - 54))

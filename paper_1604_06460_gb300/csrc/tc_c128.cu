@@ -68,8 +68,10 @@
 // buffers for D = 6, one for D = 7 (whose digit slices take the room of the
 // second); the load warps refill a buffer with cp.async as soon as the
 // splitters have read its half into registers (completion is signalled on the
-// half's mbarrier), and prefetch the next tile into L2 (one bulk prefetch per
-// contiguous run).  The splitters derive each row's largest exponent from the
+// half's mbarrier), and prefetch the next tile into L2, a 128-byte line a
+// lane (one bulk prefetch per contiguous run, 32 of them from one warp where
+// all five qubits are high, held the loads up: 2.38 against 2.01 ms a pass on
+// qubits 23..27 at n = 28).  The splitters derive each row's largest exponent from the
 // values they hold.  Every hand-off is an mbarrier (count-based arrivals by
 // threads, tcgen05.commit for MMA completion); waits suspend the thread until
 // the phase completes, have an iteration limit, and on a timeout raise a
@@ -78,6 +80,7 @@
 #include <cmath>
 #include <cstdlib>
 #include <cstring>
+#include <type_traits>
 
 #include "qe_arith.cuh"
 #include "qe_internal.h"
@@ -115,13 +118,28 @@ struct OzArgs {
     double2* x;
     uint64_t ntiles;
     int L, kh;
-    uint8_t hq[8];
-    uint8_t gpos[5];
+    uint8_t hq[12];
+    uint8_t gpos[5];        // tile-local positions of the matrix bits, ascending
     uint32_t* status;
     long long spin_limit;
     const uint16_t* B;      // [D][64][64] fp16 digits of W': slice j, row n', column k
     const int* F;           // [64] row scale exponents of W (original row order)
     int stall_test;         // failure-path test: the first staged half is never announced
+};
+
+// One digit of a Fourier transform as a block whose matrix is built on the
+// device and depends on `P` index bits outside the tile (see build_dft).
+struct DftArgs {
+    OzArgs z;               // z.B, z.F unused; z.hq the tile's bits at or above L
+    int nskip;              // bits left out of a tile's index: the tile's and the P matrix bits, ascending
+    uint8_t skip[32];
+    int lt;                 // 2^lt tiles share a matrix
+    int teams;              // CTAs i, i + teams, ... form team i; the matrices go to the teams in turn
+    int P, vlo;             // the matrix bits [vlo, vlo + P)
+    int d, below;           // the digit's bits, the idle matrix bits below them
+    int reversed;           // leave the output bit-reversed in its qubits
+    double scale;           // 2^(-d/2)
+    const double2* roots;   // exp(+-2 pi i j / 2^(P + d)), j < 2^(P + d)
 };
 
 // mbarriers of the kernel
@@ -143,7 +161,10 @@ enum Bar {
     kBars
 };
 
-// The MMA-issuing thread.  The accumulators of one half lie side by side,
+// The MMA-issuing warp: all lanes compute the (warp-uniform) operands, one
+// elected lane issues, so that the descriptors come from uniform registers
+// (2.47 against 2.40 ms a pass at n = 28 with one divergent lane doing both:
+// the kernel's period runs through this warp).  The accumulators of one half lie side by side,
 // C_d at column 32 (d - 2), and each half's W' digit slices are stacked along
 // N (rows 32 (j - 1) + m), so one MMA of A_i against the stacked slices
 // j0..j1 writes C_{i + j0} .. C_{i + j1} at once: the digit products form a
@@ -151,10 +172,14 @@ enum Bar {
 // 8).  Per tile: both halves' K-steps over the real parts (each half once
 // its set is free), a commit that releases the real-part digits, then the
 // imaginary-part K-steps of X (committed: X full) and of Y (committed: Y
-// full and every digit consumed).  False when a wait ran out.
+// full and every digit consumed).
+// `ph` holds the barrier phases across calls (bit 0 digits ready, bit 1 sets
+// free, bit 2 no tile yet: 4 before the first call), bit 3 of the result that
+// a wait ran out.
 template <int D>
-__device__ __noinline__ bool issue_mmas(const OzArgs& a, uint32_t tmem, uint32_t a0, uint32_t b0, uint64_t* bars,
-                                        uint32_t* abort_flag) {
+__device__ __forceinline__ uint32_t issue_mmas(uint32_t elected, const OzArgs& a, uint32_t t0, uint32_t t1,
+                                               uint32_t step, uint32_t tmem, uint32_t a0, uint32_t b0, uint64_t* bars,
+                                               uint32_t* abort_flag, uint32_t ph) {
     constexpr MmaTable<D> tab;
     constexpr uint32_t kStackB = (uint32_t)D * kStackSlice;
     const uint64_t da0 = tc::sdesc_sw128(a0);      // an offset of b bytes adds b >> 4
@@ -171,33 +196,78 @@ __device__ __noinline__ bool issue_mmas(const OzArgs& a, uint32_t tmem, uint32_t
                 const uint64_t da = da0 + (((uint32_t)(i - 1) * kSliceA + 32u * ks) >> 4);
                 const uint64_t db = db0 + (((uint32_t)(j0 - 1) * kStackSlice + 32u * ks) >> 4);
                 const uint32_t dt = set + (uint32_t)(i + j0 - 2) * kNH;
-                mma_f16(dt, da, db, tc::idesc(0u, nn, kRows), (ks > 0 || m > 1) ? 1u : 0u);
+                mma_f16_elected(elected, dt, da, db, tc::idesc(0u, nn, kRows), (ks > 0 || m > 1) ? 1u : 0u);
             }
         }
     };
     auto wait = [&](Bar b, uint32_t& ph) {
-        if (!wait_or_abort(smem_u32(&bars[b]), ph, a.spin_limit, abort_flag)) return false;
+        const bool ok = wait_or_abort(smem_u32(&bars[b]), ph, a.spin_limit, abort_flag);
+        if (__any_sync(0xFFFFFFFFu, !ok)) return false;
         ph ^= 1u;
         asm volatile("tcgen05.fence::after_thread_sync;");
         return true;
     };
-    uint32_t pre = 0, pim = 0, pxf = 0, pyf = 0;
-    bool first = true;
-    for (uint64_t t = blockIdx.x; t < a.ntiles; t += gridDim.x) {
-        if (!wait(kReReady, pre)) return false;
-        if (!first && !wait(kXFree, pxf)) return false;
+    uint32_t pre = ph & 1u, pim = pre, pxf = (ph >> 1) & 1u, pyf = pxf;
+    bool first = ph & 4u;
+    for (uint32_t t = t0; t < t1; t += step) {
+        if (!wait(kReReady, pre)) return 8u;
+        if (!first && !wait(kXFree, pxf)) return 8u;
         issue(0, 0, 2);
-        if (!first && !wait(kYFree, pyf)) return false;
+        if (!first && !wait(kYFree, pyf)) return 8u;
         issue(1, 0, 2);
-        tc::mma_commit(&bars[kReFree]);
-        if (!wait(kImReady, pim)) return false;
+        mma_commit_elected(elected, &bars[kReFree]);
+        if (!wait(kImReady, pim)) return 8u;
         issue(0, 2, 4);
-        tc::mma_commit(&bars[kXFull]);
+        mma_commit_elected(elected, &bars[kXFull]);
         issue(1, 2, 4);
-        tc::mma_commit(&bars[kYFull]);
+        mma_commit_elected(elected, &bars[kYFull]);
         first = false;
     }
-    return true;
+    return pre | (pxf << 1) | (first ? 4u : 0u);
+}
+
+// W of a transform digit, built in shared memory by all warps.  With l_prior
+// the P-bit value of the transform's outputs so far (the matrix bits, which
+// hold it bit-reversed),
+//   U[l][k] = 2^(-d/2) w_(2^(P + d))^(k (l_prior + 2^P l)):
+// the digit's 2^d-point transform with the twiddle by the earlier outputs
+// folded into the columns.  With several digits, output l is left at the
+// bit-reversed position, so that one bit reversal of the register restores the
+// natural order whatever the digits are.  One warp per complex row, lane <->
+// column; entries split like the inputs (scale from the row's largest
+// component).
+template <int D>
+__device__ __noinline__ void build_dft(const DftArgs& f, uint32_t v, unsigned char* sB, int* sF20) {
+    constexpr uint32_t kStackB = (uint32_t)D * kStackSlice;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const uint32_t lp = f.P ? (__brev(v) >> (32 - f.P)) : 0u;
+    const uint32_t dm = (1u << f.d) - 1u;
+    for (int r = warp; r < 32; r += kOzThreads / 32) {
+        const uint32_t lr = ((uint32_t)r >> f.below) & dm, k = ((uint32_t)lane >> f.below) & dm;
+        const uint32_t l = f.reversed ? __brev(lr) >> (32 - f.d) : lr;
+        const uint32_t e = (k * (lp + (l << f.P))) & ((1u << (f.P + f.d)) - 1u);
+        const bool inside = (((uint32_t)lane ^ (uint32_t)r) & ~(dm << f.below)) == 0;   // idle qubits: the identity
+        const double2 w = f.roots[e];
+        const double re = inside ? w.x * f.scale : 0.0, im = inside ? w.y * f.scale : 0.0;
+        uint32_t em = max((uint32_t)__double2hiint(re) << 1, (uint32_t)__double2hiint(im) << 1);
+        for (int o = 16; o > 0; o >>= 1) em = max(em, __shfl_xor_sync(0xFFFFFFFFu, em, o));
+        em >>= 21;
+        const uint32_t base_s = D == 7 ? em : em + 5u;
+        uint32_t dg[D];   // (re, im) digits as fp16 pairs
+        digit_pairs<D>(split_z<D>(re, base_s), split_z<D>(im, base_s), dg);
+        const int hh = r >> 4, m = r & 15;
+        unsigned char* const b = sB + hh * kStackB + 2 * (lane & 7);
+        const int c0 = lane >> 3, c1 = 4 + (lane >> 3);
+#pragma unroll
+        for (int j = 0; j < D; ++j) {
+            const uint16_t dr = (uint16_t)dg[j], di = (uint16_t)(dg[j] >> 16);
+            *reinterpret_cast<uint16_t*>(b + sw128_chunk(j * kNH + m, c0)) = dr;
+            *reinterpret_cast<uint16_t*>(b + sw128_chunk(j * kNH + m, c1)) = di ^ 0x8000u;
+            *reinterpret_cast<uint16_t*>(b + sw128_chunk(j * kNH + m + 16, c0)) = di;
+            *reinterpret_cast<uint16_t*>(b + sw128_chunk(j * kNH + m + 16, c1)) = dr;
+        }
+        if (lane == 0) sF20[r] = sF20[32 + r] = ((int)em - 1021) * (1 << 20);
+    }
 }
 
 // Dynamic shared memory: D digit slices of In, D of W' (two stacked halves),
@@ -208,10 +278,35 @@ constexpr size_t oz_smem() {
 }
 static_assert(oz_smem<6>() <= 227 * 1024 && oz_smem<7>() <= 227 * 1024, "shared memory per CTA");
 
+// Blocks with qubit 0 (PAIR: matrix bit 0 is qubit 0, so that columns 2j and
+// 2j + 1 are neighbours in memory) load along memory instead of along rows and
+// store 32 bytes at a time: qubits 0, 1, 2, 20, 27 at n = 28 took 3.43 ms a pass
+// with a row a lane and 16-byte stores, 2.53 ms so; the other blocks do without
+// the index arithmetic (2.04 against 2.08 ms).
+// Byte offset of amplitude (row of 64, column c) in a staged half with PAIR:
+// column-major, the rows of a column XORed with the reversal of the column's low three bits,
+// so that the eight lanes of a 16-byte access reach different banks whether
+// their index bits are row bits (low ones), column bits or some of each.  XOR
+// linear in (row, column).
+__host__ __device__ constexpr uint32_t stage_swizzle(uint32_t c) { return ((c & 1u) << 2) | (c & 2u) | ((c >> 2) & 1u); }
+__device__ __forceinline__ uint32_t stage_off(uint32_t row, uint32_t c) {
+    return 16u * (kHalfRows * c + (row ^ stage_swizzle(c)));
+}
+
+__device__ __forceinline__ const OzArgs& oz_args(const OzArgs& a) { return a; }
+__device__ __forceinline__ const OzArgs& oz_args(const DftArgs& a) { return a.z; }
+
 // 19 warps of 96 registers a thread: a sub-partition holding five of the warps
 // uses 15,360 of its 16,384 registers (104 would exceed them).
-template <int D>
-__global__ void __maxnreg__(96) k_gate_tc5_c128(const __grid_constant__ OzArgs a) {
+//
+// Without DFT, one matrix for all tiles, tile t = block, block + grid, ...
+// With it, the 2^lt tiles of one matrix are a segment of a team of CTAs, each
+// of which takes every step-th tile; between segments all roles meet at a
+// barrier, build the next matrix and go on with their barrier phases.
+template <int D, bool PAIR, class Args>
+__global__ void __maxnreg__(96) k_gate_tc5_c128(const __grid_constant__ Args arg) {
+    constexpr bool kDft = std::is_same<Args, DftArgs>::value;
+    const OzArgs& a = oz_args(arg);
     constexpr int kAcc = D + 1;                  // accumulators C_2 .. C_{D+2}
     constexpr bool kOneStage = D == 7;           // one staging buffer for both halves of a tile
     constexpr uint32_t kStackB = (uint32_t)D * kStackSlice;
@@ -222,22 +317,25 @@ __global__ void __maxnreg__(96) k_gate_tc5_c128(const __grid_constant__ OzArgs a
     unsigned char* stage = sB + D * kSliceB;                    // raw amplitudes of one or two tile halves
     __shared__ __align__(8) uint64_t bars[kBars];
     __shared__ uint32_t tmem_base, abort_flag;
-    __shared__ uint64_t hoff[32];
+    __shared__ uint64_t hoff[kDft ? 512 : 32];
     __shared__ uint32_t cpos[32];
     __shared__ uint64_t coloff[32];
+    __shared__ ulonglong2 k_off[32];           // the loaders' k-th copy: offsets in memory and in the staging buffer
     __shared__ int sF20[kN];
     __shared__ int s_eterm[2][kRows];          // (E_r - 56) << 20 of the rows of two tiles in flight
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
 
     // W' digits into their swizzled operand layout; W row scales
+    if constexpr (!kDft) {
 #pragma unroll 1
-    for (int i = tid; i < D * kN * 8; i += blockDim.x) {
-        const int j = i / (kN * 8), n = (i / 8) % kN, ch = i % 8;
-        const uint4 v = *reinterpret_cast<const uint4*>(a.B + ((size_t)(j * kN + n) * kK + ch * 8));
-        const int hh = n / kNH, m = n % kNH;
-        *reinterpret_cast<uint4*>(sB + hh * kStackB + sw128_chunk(j * kNH + m, ch)) = v;
+        for (int i = tid; i < D * kN * 8; i += blockDim.x) {
+            const int j = i / (kN * 8), n = (i / 8) % kN, ch = i % 8;
+            const uint4 v = *reinterpret_cast<const uint4*>(a.B + ((size_t)(j * kN + n) * kK + ch * 8));
+            const int hh = n / kNH, m = n % kNH;
+            *reinterpret_cast<uint4*>(sB + hh * kStackB + sw128_chunk(j * kNH + m, ch)) = v;
+        }
     }
-    if (tid < kN) sF20[tid] = a.F[tid] * (1 << 20);
+    if (!kDft && tid < kN) sF20[tid] = a.F[tid] * (1 << 20);
     if (tid < (1 << a.kh)) {
         uint64_t o = 0;
         for (int j = 0; j < a.kh; ++j)
@@ -287,8 +385,68 @@ __global__ void __maxnreg__(96) k_gate_tc5_c128(const __grid_constant__ OzArgs a
         const uint32_t l = row_bits(r);
         return 16ull * ((l & ((1u << a.L) - 1u)) + hoff[l >> a.L]);
     };
+    // row (of 64) and column of the half's index whose lowest six bits in memory
+    // order are i and whose others are k
+    auto half_index = [&](uint32_t i, uint32_t k, uint32_t& row, uint32_t& col) {
+        uint32_t rest = i | (k << 6), rb = 0, cb = 0;
+        row = col = 0;
+        for (int b = 0; b < 12 && rb + cb < 11; ++b) {
+            if ((gmask >> b) & 1u) col |= (rest & 1u) << cb++;
+            else if (rb < 6) row |= (rest & 1u) << rb++;
+            else continue;
+            rest >>= 1;
+        }
+    };
+    if (PAIR && tid < 32) {
+        uint32_t r, c;
+        half_index(0, tid, r, c);
+        k_off[tid] = make_ulonglong2(row_off(r) + coloff[c], stage_off(r, c));
+    }
+    __syncthreads();
     char* const xb = reinterpret_cast<char*>(a.x);
-    auto tile_ptr = [&](uint64_t t) { return xb + 16ull * insert_zero_bits(t << a.L, a.hq, a.kh); };
+    auto tile_ptr = [&](uint32_t t) {
+        if constexpr (kDft) {
+            const uint64_t u = t & ((1u << arg.lt) - 1u), v = t >> arg.lt;
+            return xb + 16ull * (insert_zero_bits(u << a.L, arg.skip, arg.nskip) | (v << arg.vlo));
+        } else {
+            return xb + 16ull * insert_zero_bits((uint64_t)t << a.L, a.hq, a.kh);
+        }
+    };
+    // The CTA's current segment: tiles [begin, end) in steps of `step` (32 bits
+    // hold any tile index).  With kDft they live in shared memory, where they
+    // cost the roles no registers (the digit kernel spilled with them in
+    // registers: 12.3 against 11.3 ms a pass at n = 30).
+    __shared__ uint32_t s_begin, s_end, s_step;
+    auto seg_begin = [&]() -> uint32_t { return kDft ? s_begin : blockIdx.x; };
+    auto seg_end = [&]() -> uint32_t { return kDft ? s_end : (uint32_t)a.ntiles; };
+    auto seg_step = [&]() -> uint32_t { return kDft ? s_step : gridDim.x; };
+    // Starts the next segment (all threads): false when there is none or a
+    // wait has run out.  The barrier before the rebuild follows the
+    // recombination of the segment's last tile, hence all its MMAs.
+    auto next_segment = [&](bool begin) {
+        if constexpr (!kDft) {
+            return begin;
+        } else {
+            const uint32_t team = blockIdx.x % arg.teams;
+            uint32_t v = team;
+            if (!begin) {
+                __syncthreads();
+                if (*reinterpret_cast<volatile uint32_t*>(&abort_flag)) return false;
+                v = (s_begin >> arg.lt) + arg.teams;
+                __syncthreads();
+            }
+            if (v >> arg.P) return false;
+            if (tid == 0) {
+                s_begin = (v << arg.lt) + blockIdx.x / arg.teams;
+                s_end = (v + 1) << arg.lt;
+                s_step = (gridDim.x - team + arg.teams - 1) / arg.teams;    // CTAs of the team
+            }
+            build_dft<D>(arg, v, sB, sF20);
+            asm volatile("fence.proxy.async.shared::cta;");
+            __syncthreads();
+            return true;
+        }
+    };
     // wait (all lanes of a warp) for a phase of barrier b; on a timeout or an
     // abort raise the status word.  The outcome is the same on every lane,
     // so the warp stays converged for its .sync.aligned instructions.
@@ -303,25 +461,39 @@ __global__ void __maxnreg__(96) k_gate_tc5_c128(const __grid_constant__ OzArgs a
     };
     if (warp == kMmaWarp) {
         // ---------------------------------------------------- MMA issuer
+        uint32_t ph = 4u;
+        const uint32_t elected = elect_lane();
+        for (bool more = next_segment(true); more; more = next_segment(false)) {
+            ph = issue_mmas<D>(elected, a, seg_begin(), seg_end(), seg_step(), tmem, smem_u32(sA), smem_u32(sB), bars,
+                               &abort_flag, ph);
+            if (ph & 8u) atomicExch(a.status, 1u);
+            __syncwarp();
+        }
+        mma_commit_elected(elected, &bars[kDrain]);    // by the lane that issued the MMAs
         if (lane == 0) {
-            if (!issue_mmas<D>(a, tmem, smem_u32(sA), smem_u32(sB), bars, &abort_flag)) atomicExch(a.status, 1u);
             // every MMA issued has completed before tensor memory is freed
-            tc::mma_commit(&bars[kDrain]);
             if (!tc::mbar_wait(smem_u32(&bars[kDrain]), 0u, a.spin_limit)) atomicExch(a.status, 1u);
         }
         __syncwarp();
     } else if (warp >= kLoadWarp0) {
         // ------------------------------------------------------- tile loads
-        // thread <-> group row i of each staged half: per half, once the
-        // splitters have read it, 32 16-byte copies into the column-major
-        // staging buffer (a warp's copies of one column fill 512 contiguous
-        // bytes) and an arrival on the half's stage barrier when they land
+        // per half, once the splitters have read it, 32 16-byte copies a thread
+        // into the column-major staging buffer and an arrival on the half's
+        // stage barrier when they land.  Thread <-> group row i of the half and
+        // copy <-> column; with PAIR the half's 11 index bits (6 of the row, 5
+        // of the column) are taken in the order of their place in memory, the
+        // thread index holding the lowest six, so that a warp copies whole
+        // lines where a row a lane would take 16-byte pieces
         const int i = tid - kLoadWarp0 * 32;
-        const uint64_t ro[2] = {row_off(i), row_off(kHalfRows + i)};
-        const uint32_t d = smem_u32(stage) + 16u * (uint32_t)i;
+        uint32_t ri = i, ci = 0;
+        if constexpr (PAIR) half_index(i, 0, ri, ci);
+        const uint64_t go = row_off(ri) + coloff[ci], go_half = row_off(kHalfRows);
+        const uint32_t so = PAIR ? stage_off(ri, ci) : 16u * ri;
+        const uint32_t d = smem_u32(stage);
         uint32_t pf[2] = {0u, 0u};
         bool first = true, ok = true;
-        for (uint64_t t = blockIdx.x; t < a.ntiles && ok; t += gridDim.x) {
+        for (bool more = next_segment(true); more; more = next_segment(false))
+        for (uint32_t t = seg_begin(); t < seg_end() && ok; t += seg_step()) {
             const char* g = tile_ptr(t);
 #pragma unroll
             for (int h = 0; h < 2; ++h) {
@@ -333,19 +505,32 @@ __global__ void __maxnreg__(96) k_gate_tc5_c128(const __grid_constant__ OzArgs a
                     ok = false;
                     break;
                 }
-                const char* gr = g + ro[h];
+                const char* gr = g + go + (h ? go_half : 0ull);
                 const uint32_t dh = d + (kOneStage ? 0u : (uint32_t)h * kHalfStage);
+                if constexpr (PAIR) {
 #pragma unroll 8
-                for (int c = 0; c < 32; ++c) cp_async16(dh + 16u * kHalfRows * c, gr + coloff[c]);
+                    for (int k = 0; k < 32; ++k) {
+                        const ulonglong2 o = k_off[k];
+                        cp_async16(dh + (so ^ (uint32_t)o.y), gr + o.x);
+                    }
+                } else {
+#pragma unroll 8
+                    for (int c = 0; c < 32; ++c) cp_async16(dh + so + 16u * kHalfRows * c, gr + coloff[c]);
+                }
                 if (!(a.stall_test && first && h == 0)) cp_async_arrive(&bars[h ? kStage1 : kStage0]);
             }
             first = false;
-            // the tile after this one into L2 meanwhile: its 2^kh contiguous
-            // runs of 2^L amplitudes (>= 2 KB), one bulk prefetch each
-            const uint64_t tn = t + gridDim.x;
-            if (ok && tn < a.ntiles) {
+            // the tile after this one into L2 meanwhile, a 128-byte line at a time
+            // (2^(L-3) lines in each of its 2^kh runs)
+            const uint32_t tn = t + seg_step();
+            if (ok && tn < seg_end()) {
                 const char* gn = tile_ptr(tn);
-                for (int h = i; h < (1 << a.kh); h += 32 * kLoadWarps) l2_prefetch(gn + 16ull * hoff[h], 16u << a.L);
+#pragma unroll
+                for (int k = 0; k < 512 / (32 * kLoadWarps); ++k) {
+                    const int l = i + 32 * kLoadWarps * k;
+                    const char* gl = gn + 16ull * hoff[l >> (a.L - 3)] + 128u * (uint32_t)(l & ((1 << (a.L - 3)) - 1));
+                    asm volatile("prefetch.global.L2 [%0];" ::"l"(gl) : "memory");
+                }
             }
         }
         asm volatile("cp.async.wait_all;" ::: "memory");
@@ -359,11 +544,12 @@ __global__ void __maxnreg__(96) k_gate_tc5_c128(const __grid_constant__ OzArgs a
         // then the imaginary-part digits (chunk 4 + qq).
         const int sw = warp - kSplitWarp0;
         const int ri = 8 * sw + (lane & 7), qq = lane >> 3;
-        const unsigned char* const srow = stage + 16u * (kHalfRows * 8 * qq + ri);   // (row ri, column 8 qq)
+        const unsigned char* const scol = stage + 16u * kHalfRows * 8 * qq;   // column 8 qq
         uint32_t prf = 0, pyf = 0;
         bool first = true, ok = true;
         int it = 0;
-        for (uint64_t t = blockIdx.x; t < a.ntiles && ok; t += gridDim.x, ++it) {
+        for (bool more = next_segment(true); more; more = next_segment(false))
+        for (uint32_t t = seg_begin(); t < seg_end() && ok; t += seg_step(), ++it) {
             const uint32_t ph = (uint32_t)it & 1u;    // each stage barrier completes once per tile
 #pragma unroll 1
             for (int h = 0; h < 2; ++h) {
@@ -375,9 +561,9 @@ __global__ void __maxnreg__(96) k_gate_tc5_c128(const __grid_constant__ OzArgs a
                 const int r = kHalfRows * h + ri;
                 double2 v[8];
                 const double2* src =
-                    reinterpret_cast<const double2*>(srow + (kOneStage ? 0u : (uint32_t)h * kHalfStage));
+                    reinterpret_cast<const double2*>(scol + (kOneStage ? 0u : (uint32_t)h * kHalfStage));
 #pragma unroll
-                for (int k = 0; k < 8; ++k) v[k] = src[kHalfRows * k];
+                for (int k = 0; k < 8; ++k) v[k] = src[kHalfRows * k + (PAIR ? ri ^ (int)stage_swizzle(k) : ri)];
                 mbar_arrive(&bars[h ? kStageFree1 : kStageFree0]);
                 uint32_t em = 0;    // largest (high word << 1): the biased exponent in the top 11 bits
 #pragma unroll
@@ -494,16 +680,27 @@ __global__ void __maxnreg__(96) k_gate_tc5_c128(const __grid_constant__ OzArgs a
             }
         };
         auto store = [&](char* gb, int c0, const long long y[8], int eterm) {
+            // whole 32-byte sectors where neighbouring columns share one
 #pragma unroll
-            for (int u = 0; u < 4; ++u) {
+            for (int u = 0; u < 4; u += 2) {
                 const int c = c0 + u;
-                *reinterpret_cast<double2*>(gb + coloff[c]) =
-                    make_double2(finish_y(y[2 * u], eterm + sF20[c]), finish_y(y[2 * u + 1], eterm + sF20[32 + c]));
+                const double re0 = finish_y(y[2 * u], eterm + sF20[c]), im0 = finish_y(y[2 * u + 1], eterm + sF20[32 + c]);
+                const double re1 = finish_y(y[2 * u + 2], eterm + sF20[c + 1]);
+                const double im1 = finish_y(y[2 * u + 3], eterm + sF20[32 + c + 1]);
+                if constexpr (PAIR) {
+                    asm volatile("st.global.v4.f64 [%0], {%1, %2, %3, %4};" ::"l"(gb + coloff[c]), "d"(re0), "d"(im0),
+                                 "d"(re1), "d"(im1)
+                                 : "memory");
+                } else {
+                    *reinterpret_cast<double2*>(gb + coloff[c]) = make_double2(re0, im0);
+                    *reinterpret_cast<double2*>(gb + coloff[c + 1]) = make_double2(re1, im1);
+                }
             }
         };
         uint32_t px = 0, py = 0;
         int it = 0;
-        for (uint64_t t = blockIdx.x; t < a.ntiles; t += gridDim.x, ++it) {
+        for (bool more = next_segment(true); more; more = next_segment(false))
+        for (uint32_t t = seg_begin(); t < seg_end(); t += seg_step(), ++it) {
             char* gb = tile_ptr(t) + rowoff;
             const int slot = it & 1;
             uint32_t pet = (uint32_t)(it >> 1) & 1u;     // each slot completes every other tile
@@ -573,7 +770,7 @@ void launch_impl(qe_state* s, const int* qubits, const cd* U, const char* tag) {
     a.x = reinterpret_cast<double2*>(s->d);
     a.L = g.L;
     a.kh = g.kh;
-    std::memcpy(a.hq, g.hq, sizeof(a.hq));
+    std::memcpy(a.hq, g.hq, sizeof(g.hq));
     std::memcpy(a.gpos, g.gpos, sizeof(a.gpos));
     a.ntiles = 1ull << (s->n - 12);
     // W = [[Re U, -Im U], [Im U, Re U]], row n (output), column k (input)
@@ -615,11 +812,12 @@ void launch_impl(qe_state* s, const int* qubits, const cd* U, const char* tag) {
     a.stall_test = (stall != nullptr && stall[0] == '1') ? 1 : 0;
     if (a.stall_test) a.spin_limit = 1ll << 12;
     const size_t smem = oz_smem<D>();
-    QE_CUDA(cudaFuncSetAttribute(k_gate_tc5_c128<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    auto fn = qubits[0] == 0 ? k_gate_tc5_c128<D, true, OzArgs> : k_gate_tc5_c128<D, false, OzArgs>;
+    QE_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     const uint64_t grid = std::min<uint64_t>(a.ntiles, (uint64_t)num_sms());
     {
         Launch Lc(s, tag, 2.0 * dim(s) * amp_bytes(s));
-        k_gate_tc5_c128<D><<<(unsigned)grid, kOzThreads, smem, s->stream>>>(a);
+        fn<<<(unsigned)grid, kOzThreads, smem, s->stream>>>(a);
         QE_CUDA(cudaGetLastError());
     }
     // checked before the next tensor-core launch or at the end of the flush,
@@ -636,6 +834,97 @@ void launch_impl(qe_state* s, const int* qubits, const cd* U, const char* tag) {
 void launch_gate_tc5_c128(qe_state* s, const int* qubits, const cd* U) {
     if (s->arith == QE_ARITH_DF64) launch_impl<6>(s, qubits, U, "gate_tc_k5_c128_df");
     else launch_impl<7>(s, qubits, U, "gate_tc_k5_c128");
+}
+
+// The status word of a run of transform digits: cleared before the first and
+// read back after the last (the digits only ever raise it, so no host wait
+// separates them: one digit alone took 38 us at n = 12 with a wait before each
+// launch).
+uint32_t* dft_digits_begin(qe_state* s) {
+    complete_pending(s);   // the previous tensor-core launch, before the status word is reused
+    uint32_t* status = (uint32_t*)ensure_scratch(s, 256);
+    QE_CUDA(cudaMemsetAsync(status, 0, sizeof(uint32_t), s->stream));
+    return status;
+}
+void dft_digits_end(qe_state* s, const uint32_t* status) {
+    QE_CUDA(cudaMemcpyAsync(status_word_host(s), status, sizeof(uint32_t), cudaMemcpyDeviceToHost, s->stream));
+    s->status_pending = true;
+}
+
+// One digit of a Fourier transform on a complex128 state (n >= 12): the qubits
+// [q0, q0 + d), 3 <= d <= 5, whose matrix depends on the P qubits above them
+// (P + d <= 20, n - 12 - P >= 0).  `roots` holds the 2^(P + d) roots of unity
+// of the transform's sign; `reversed`: leave the output bit-reversed.  56-bit
+// splitting in both arithmetic modes (the seventh digit costs 3 %).
+void launch_dft_digit_c128(qe_state* s, int q0, int d, int P, bool reversed, const double2* roots, uint32_t* status) {
+    constexpr int D = 7;
+    if (s->n < 12 + P) fail(QE_ERR_UNSUPPORTED, "transform digits need n >= 12 + P");
+    static thread_local DftArgs f;
+    std::memset(&f, 0, sizeof(f));
+    OzArgs& a = f.z;
+    a.x = reinterpret_cast<double2*>(s->d);
+    a.ntiles = 1ull << (s->n - 12);
+    f.P = P;
+    f.vlo = q0 + d;
+    f.d = d;
+    f.reversed = reversed;
+    f.scale = std::pow(2.0, -0.5 * d);
+    f.roots = roots;
+    f.lt = s->n - 12 - P;
+    // The tile: the digit, the lowest qubits outside it and the matrix bits.
+    // Gate bits are the digit and, for d < 5, the lowest other tile qubits.
+    bool matrix[64] = {}, local[64] = {};
+    for (int j = 0; j < P; ++j) matrix[f.vlo + j] = true;
+    for (int j = 0; j < d; ++j) local[q0 + j] = true;
+    int nlocal = d;
+    for (int q = 0; nlocal < 12; ++q)
+        if (!local[q] && !matrix[q]) {
+            local[q] = true;
+            ++nlocal;
+        }
+    // idle matrix bits (d < 5): tile bits next to the digit, so that qubit 0
+    // stays a row bit where it can
+    int gate[5], ng = 0;
+    for (int j = 0; j < d; ++j) gate[ng++] = q0 + j;
+    for (int q = q0 + d; q < s->n && ng < 5; ++q)
+        if (local[q]) gate[ng++] = q;
+    for (int q = q0 - 1; q >= 0 && ng < 5; --q)
+        if (local[q]) {
+            gate[ng++] = q;
+            ++f.below;
+        }
+    std::sort(gate, gate + 5);
+    const bool pair = gate[0] == 0;
+    while (local[a.L]) ++a.L;
+    if (a.L > 12) a.L = 12;
+    int pos[64];
+    for (int q = 0; q < s->n; ++q) {
+        pos[q] = q < a.L ? q : a.L + a.kh;
+        if (q >= a.L && local[q]) a.hq[a.kh++] = (uint8_t)q;
+        if (q >= a.L && (local[q] || matrix[q])) f.skip[f.nskip++] = (uint8_t)q;
+    }
+    for (int j = 0; j < 5; ++j) a.gpos[j] = (uint8_t)pos[gate[j]];
+    a.status = status;
+    a.spin_limit = 1ll << 21;
+    const size_t smem = oz_smem<D>();
+    auto fn = pair ? k_gate_tc5_c128<D, true, DftArgs> : k_gate_tc5_c128<D, false, DftArgs>;
+    QE_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    const uint64_t grid = std::min<uint64_t>(a.ntiles, (uint64_t)num_sms());
+    // The number of teams that makes the longest CTA's work the shortest: its
+    // segments, each a share of the matrix's tiles and about 1.6 tiles' time to
+    // drain, rebuild and refill the pipeline.
+    double best = 1e300;
+    for (int teams = 1; teams <= (int)std::min<uint64_t>(grid, 1ull << P); ++teams) {
+        const double segs = std::ceil((double)(1ull << P) / teams);
+        const double time = segs * (std::ceil((double)(1ull << f.lt) / (double)(grid / teams)) + 1.6);
+        if (time < best) {
+            best = time;
+            f.teams = teams;
+        }
+    }
+    Launch Lc(s, "gate_tc_k5_c128", 2.0 * dim(s) * amp_bytes(s));
+    fn<<<(unsigned)grid, kOzThreads, smem, s->stream>>>(f);
+    QE_CUDA(cudaGetLastError());
 }
 
 }  // namespace qe
