@@ -12,11 +12,16 @@
 //
 // Each map is closed on "planes": the multiplication permutes the 2^N values
 // of c for fixed a, b and the other qubits; the division permutes the 2^(2N)
-// values of (a, c) for fixed b and the other qubits.  A plane that fits one
-// CTA's shared memory is loaded, then every output slot is written from the
-// slot of its preimage (one read and one write of every amplitude).  Larger
-// planes go through a scratch buffer in batches: a gather of the preimages
-// into the buffer, then a copy back.
+// values of (a, c) for fixed b and the other qubits.  Planes of at most 64 KB
+// go through shared-memory tiles of 64 KB (several planes a tile, filled up
+// with the lowest other qubits so that memory is touched in long runs): one
+// read and one write of every amplitude.  Larger planes are scattered into a
+// scratch buffer in batches small enough to stay in L2 and copied back.  In
+// both, a thread works on many amplitudes of one tile or chunk, so that the
+// index arithmetic with the plane's qubits is done once for them, and values
+// fit 32 bits: nine-qubit registers at n = 28 in complex128, multiplication
+// 2.46 -> 1.48 ms, division (planes of 4 MB; a gather into a buffer of 1 GB
+// and a copy back before) 9.4 -> 3.7 ms; one pass over the state is 1.27 ms.
 #include <algorithm>
 #include <cstring>
 
@@ -50,87 +55,192 @@ __device__ __forceinline__ uint64_t reg_put(const RegArg& r, int N, uint32_t v) 
 
 enum { kMul = 0, kDiv = 1 };
 
+// The inverse map on register values: the preimage of (a, b, c) in *a, *c.
+// Multiplication: c - a b mod 2^N (products wrap mod 2^32 alike).  Division: the
+// restoring steps undone in reverse order (i = 0 .. N-1): if c_i, a += b 2^i;
+// then c_i ^= [b != 0 and a >= b 2^i] (b 2^i < 2^32).
+template <int OP>
+__device__ __forceinline__ void preimage(int N, uint32_t& a, uint32_t b, uint32_t& c) {
+    const uint32_t mask = (1u << N) - 1u;
+    if (OP == kMul) {
+        c = (c - a * b) & mask;
+        return;
+    }
+    if (b == 0u) {       // no step adds or flips anything
+        return;
+    }
+    uint32_t bi = b;
+    for (int i = 0; i < N; ++i, bi <<= 1) {
+        const uint32_t bit = 1u << i;
+        if (c & bit) a = (a + bi) & mask;
+        if (a >= bi) c ^= bit;
+    }
+}
+
+// The map itself: the image of (a, b, c) in a, c.
+template <int OP>
+__device__ __forceinline__ void image(int N, uint32_t& a, uint32_t b, uint32_t& c) {
+    const uint32_t mask = (1u << N) - 1u;
+    if (OP == kMul) {
+        c = (c + a * b) & mask;
+        return;
+    }
+    if (b == 0u) {       // c_i set subtracts nothing
+        return;
+    }
+    uint32_t bi = b << (N - 1);
+    for (int i = N - 1; i >= 0; --i, bi >>= 1) {
+        const uint32_t bit = 1u << i;
+        if (a >= bi) c ^= bit;
+        if (c & bit) a = (a - bi) & mask;
+    }
+}
+
+template <class S>
+struct TileArgs {
+    S* x;
+    uint64_t ntiles;
+    int N, T, L, kh;          // tile of 2^T amplitudes: runs of 2^L, kh bits at or above L
+    uint8_t hq[16];
+    RegArg a, b;              // by global qubits
+    RegArg la, lc;            // by tile-local bits (la: division)
+};
+
+// Whole planes in shared memory: one read and one write per amplitude.
+template <class S, int OP>
+__global__ void __launch_bounds__(kArithThreads) k_arith_plane(const __grid_constant__ TileArgs<S> a) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    S* buf = reinterpret_cast<S*>(smem_raw);
+    __shared__ uint64_t offA[64], offB[256];
+    if (threadIdx.x < 256) {
+        uint64_t oa = 0, ob = 0;
+        for (int j = 0; j < a.kh; ++j)
+            if (j < 6) oa |= ((uint64_t)(threadIdx.x >> j) & 1ull) << a.hq[j];
+            else ob |= ((uint64_t)(threadIdx.x >> (j - 6)) & 1ull) << a.hq[j];
+        if (threadIdx.x < 64) offA[threadIdx.x] = oa;
+        offB[threadIdx.x] = ob;
+    }
+    __syncthreads();
+    const uint32_t E = 1u << a.T, lowmask = (1u << a.L) - 1u;
+    const uint32_t cmask = (uint32_t)reg_put(a.lc, a.N, (1u << a.N) - 1u);
+    const uint32_t amask = OP == kDiv ? (uint32_t)reg_put(a.la, a.N, (1u << a.N) - 1u) : 0u;
+    for (uint64_t t = blockIdx.x; t < a.ntiles; t += gridDim.x) {
+        const uint64_t base = insert_zero_bits(t << a.L, a.hq, a.kh);
+        auto at = [&](uint32_t i) { return base + (i & lowmask) + offA[(i >> a.L) & 63u] + offB[i >> a.L >> 6]; };
+#pragma unroll 8
+        for (uint32_t i = threadIdx.x; i < E; i += kArithThreads) buf[i] = a.x[at(i)];
+        __syncthreads();
+#pragma unroll 4
+        for (uint32_t i = threadIdx.x; i < E; i += kArithThreads) {
+            const uint64_t x = at(i);
+            const uint32_t bv = reg_get(a.b, a.N, x);
+            uint32_t av = OP == kDiv ? reg_get(a.la, a.N, i) : reg_get(a.a, a.N, x);
+            uint32_t cv = reg_get(a.lc, a.N, i);
+            preimage<OP>(a.N, av, bv, cv);
+            uint32_t src = (i & ~(cmask | amask)) | (uint32_t)reg_put(a.lc, a.N, cv);
+            if (OP == kDiv) src |= (uint32_t)reg_put(a.la, a.N, av);
+            a.x[x] = buf[src];
+        }
+        __syncthreads();
+    }
+}
+
+// Larger planes.  A block is 2^w planes that differ in the lowest w <= 3 qubits
+// (those below every plane qubit), its value e = (plane value y) 2^w + (low
+// bits l), so that a warp touches whole lines of the state wherever the
+// registers lie.
 template <class S>
 struct ArithArgs {
     S* x;
-    S* scratch;
-    uint64_t plane0, nplanes;   // planes [plane0, plane0 + nplanes) of this launch
-    int N, P, op;               // register width, plane bits (N or 2N), operation
+    S* scratch;                 // blocks [blk0, blk0 + nblk) are scattered into scratch,
+    const S* back;              // [back0, back0 + nback) copied back from `back`
+    uint64_t blk0, nblk, back0, nback;
+    int N, P, w;                // register width, plane bits (N or 2N), low bits
     RegArg a, b, c;
-    int nsorted;
-    uint8_t plane_sorted[32];   // the plane's qubits ascending (to enumerate plane bases)
+    int nruns;                  // the block's qubits as runs of consecutive ones, ascending
+    uint8_t run_lo[34], run_len[34];
 };
 
-// Offset of plane-local value y: the c register holds its low N bits, and for
-// the division the a register its high N bits.
+// Index of the first amplitude of block p: the runs' bits inserted as zeros.
 template <class S>
-__device__ __forceinline__ uint64_t plane_offset(const ArithArgs<S>& a, uint32_t y) {
-    const uint32_t mask = (1u << a.N) - 1u;
-    if (a.op == kMul) return reg_put(a.c, a.N, y);
-    return reg_put(a.c, a.N, y & mask) | reg_put(a.a, a.N, y >> a.N);
+__device__ __forceinline__ uint64_t block_base(const ArithArgs<S>& a, uint64_t p) {
+    for (int j = 0; j < a.nruns; ++j) {
+        const uint64_t low = p & ((1ull << a.run_lo[j]) - 1ull);
+        p = ((p >> a.run_lo[j]) << (a.run_lo[j] + a.run_len[j])) | low;
+    }
+    return p;
 }
 
-// Plane-local value of the preimage of output y, in the plane whose other
-// qubits are those of base (the inverse map).
-template <class S>
-__device__ __forceinline__ uint32_t preimage(const ArithArgs<S>& a, uint64_t base, uint32_t y) {
-    const uint32_t mask = (1u << a.N) - 1u;
-    const uint32_t bv = reg_get(a.b, a.N, base);
-    if (a.op == kMul) {
-        const uint32_t av = reg_get(a.a, a.N, base);
-        return (y - av * bv) & mask;        // c - a b mod 2^N (products wrap mod 2^32 alike)
-    }
-    // the restoring steps undone in reverse order (i = 0 .. N-1): if c_i,
-    // a += b 2^i; then c_i ^= [b != 0 and a >= b 2^i]
-    uint32_t cv = y & mask;
-    uint64_t av = y >> a.N;
-    for (int i = 0; i < a.N; ++i) {
-        const uint64_t bi = (uint64_t)bv << i;
-        if ((cv >> i) & 1u) av = (av + bi) & mask;
-        const uint32_t t = (bv != 0u && av >= bi) ? 1u : 0u;
-        cv ^= t << i;
-    }
-    return cv | ((uint32_t)av << a.N);
+// Offset of block value e in the state: the c register holds y's low N bits,
+// and for the division the a register its high N bits.
+template <class S, int OP>
+__device__ __forceinline__ uint64_t block_offset(const ArithArgs<S>& a, uint32_t e) {
+    const uint32_t mask = (1u << a.N) - 1u, l = e & ((1u << a.w) - 1u), y = e >> a.w;
+    if (OP == kMul) return l | reg_put(a.c, a.N, y);
+    return l | reg_put(a.c, a.N, y & mask) | reg_put(a.a, a.N, y >> a.N);
 }
 
-// Whole planes in shared memory: one read and one write per amplitude.
-template <class S>
-__global__ void __launch_bounds__(kArithThreads) k_arith_plane(const __grid_constant__ ArithArgs<S> a) {
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    S* buf = reinterpret_cast<S*>(smem_raw);
-    const uint32_t E = 1u << a.P;
-    for (uint64_t p = blockIdx.x; p < a.nplanes; p += gridDim.x) {
-        const uint64_t base = insert_zero_bits(a.plane0 + p, a.plane_sorted, a.nsorted);
-        for (uint32_t i = threadIdx.x; i < E; i += blockDim.x) buf[i] = a.x[base | plane_offset(a, i)];
-        __syncthreads();
-        for (uint32_t y = threadIdx.x; y < E; y += blockDim.x)
-            a.x[base | plane_offset(a, y)] = buf[preimage(a, base, y)];
-        __syncthreads();
-    }
-}
+// Bytes of a batch of blocks, and block values of one CTA pass.  Two batches of
+// 16 MB (one scattered, one copied back) stay in L2: nine-qubit registers at
+// n = 28 with batches of 8, 16, 32, 64 MB: 4.4, 3.7, 4.3, 5.4 ms.
+constexpr uint64_t kBatch = 1ull << 24;
+constexpr int kChunk = 1024;
 
-// Larger planes, a batch at a time: gather the preimages into scratch ...
-template <class S>
-__global__ void __launch_bounds__(256) k_arith_gather(const __grid_constant__ ArithArgs<S> a) {
-    const uint64_t total = a.nplanes << a.P;
-    const uint32_t emask = (1u << a.P) - 1u;
-    for (uint64_t e = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; e < total;
-         e += (uint64_t)gridDim.x * blockDim.x) {
-        const uint64_t base = insert_zero_bits(a.plane0 + (e >> a.P), a.plane_sorted, a.nsorted);
-        const uint32_t y = (uint32_t)e & emask;
-        a.scratch[e] = a.x[base | plane_offset(a, preimage(a, base, y))];
+// A chunk of a batch scattered into the scratch buffer, each amplitude to the
+// place of its image ...  The state is read in order; the scattered writes stay
+// within the block's part of the buffer, 16 bytes each but complete in L2.
+// (The reverse, a gather of the preimages, scatters its reads over the block's
+// places in the state, 512 runs 4 MB apart for nine-qubit registers a b c, and
+// read DRAM four times over: 6.6 ms for the gather alone.)
+template <class S, int OP>
+__device__ __forceinline__ void scatter_chunk(const ArithArgs<S>& a, uint64_t k) {
+    constexpr int kAtOnce = kChunk / 256;   // independent loads in flight a thread
+    const int bits = a.P + a.w;
+    const uint32_t emask = (1u << bits) - 1u, mask = (1u << a.N) - 1u, wmask = (1u << a.w) - 1u;
+    const uint64_t e0 = k * kChunk;
+    const uint64_t base = block_base(a, a.blk0 + (e0 >> bits));
+    S* const out = a.scratch + (e0 & ~(uint64_t)emask);
+    S v[kAtOnce];
+#pragma unroll
+    for (int j = 0; j < kAtOnce; ++j)
+        v[j] = a.x[base | block_offset<S, OP>(a, (uint32_t)(e0 + 256 * j + threadIdx.x) & emask)];
+#pragma unroll
+    for (int j = 0; j < kAtOnce; ++j) {
+        const uint32_t e = (uint32_t)(e0 + 256 * j + threadIdx.x) & emask, l = e & wmask, y = e >> a.w;
+        const uint32_t bv = reg_get(a.b, a.N, base | l);
+        uint32_t av = OP == kMul ? reg_get(a.a, a.N, base | l) : y >> a.N, cv = y & mask;
+        image<OP>(a.N, av, bv, cv);
+        out[((OP == kMul ? cv : cv | (av << a.N)) << a.w) | l] = v[j];
     }
 }
 
-// ... then copy the batch back to its planes.
-template <class S>
-__global__ void __launch_bounds__(256) k_arith_copy_back(const __grid_constant__ ArithArgs<S> a) {
-    const uint64_t total = a.nplanes << a.P;
-    const uint32_t emask = (1u << a.P) - 1u;
-    for (uint64_t e = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; e < total;
-         e += (uint64_t)gridDim.x * blockDim.x) {
-        const uint64_t base = insert_zero_bits(a.plane0 + (e >> a.P), a.plane_sorted, a.nsorted);
-        a.x[base | plane_offset(a, (uint32_t)e & emask)] = a.scratch[e];
+// ... and a chunk copied back to its places in the state.
+template <class S, int OP>
+__device__ __forceinline__ void copy_back_chunk(const ArithArgs<S>& a, uint64_t k) {
+    const int bits = a.P + a.w;
+    const uint32_t emask = (1u << bits) - 1u;
+    const uint64_t e0 = k * kChunk;
+    const uint64_t base = block_base(a, a.back0 + (e0 >> bits));
+    S v[kChunk / 256];
+#pragma unroll
+    for (int j = 0; j < kChunk / 256; ++j) v[j] = a.back[e0 + 256 * j + threadIdx.x];
+#pragma unroll
+    for (int j = 0; j < kChunk / 256; ++j)
+        a.x[base | block_offset<S, OP>(a, (uint32_t)(e0 + 256 * j + threadIdx.x) & emask)] = v[j];
+}
+
+// One launch copies a batch back and scatters the next one (other blocks, the
+// other half of the buffer): half as many launches, reads and writes mixed.
+template <class S, int OP>
+__global__ void __launch_bounds__(256) k_arith_batch(const __grid_constant__ ArithArgs<S> a) {
+    const uint64_t backs = (a.nback << (a.P + a.w)) / kChunk, scatters = (a.nblk << (a.P + a.w)) / kChunk;
+    const uint64_t both = backs < scatters ? backs : scatters, all = backs + scatters;
+    for (uint64_t k = blockIdx.x; k < all; k += gridDim.x) {
+        // alternately while both last, then what is left of either
+        const bool back = k < 2 * both ? (k & 1) : backs > scatters;
+        const uint64_t i = k < 2 * both ? k >> 1 : k - both;
+        if (back) copy_back_chunk<S, OP>(a, i);
+        else scatter_chunk<S, OP>(a, i);
     }
 }
 
@@ -145,59 +255,102 @@ RegArg make_reg(int N, const int* q) {
     return r;
 }
 
-template <class S>
-void arith_impl(qe_state* s, int op, int N, const int* qa, const int* qb, const int* qc) {
+template <class S, int OP>
+void arith_tiles(qe_state* s, int N, const int* qa, const int* qb, const int* qc, int P, const char* tag) {
+    static thread_local TileArgs<S> a;
+    std::memset(&a, 0, sizeof(a));
+    a.x = reinterpret_cast<S*>(s->d);
+    a.N = N;
+    a.a = make_reg(N, qa);
+    a.b = make_reg(N, qb);
+    // the tile's bits: the plane's qubits and the lowest others, 64 KB in all
+    // (less on small states, for at least 256 tiles)
+    a.T = std::min(s->n, std::max({P, std::min(sizeof(S) == 16 ? 12 : 13, s->n - 8), 5}));
+    bool local[64] = {};
+    for (int j = 0; j < N; ++j) {
+        local[qc[j]] = true;
+        if (OP == kDiv) local[qa[j]] = true;
+    }
+    for (int q = 0, left = a.T - P; left > 0; ++q)
+        if (!local[q]) {
+            local[q] = true;
+            --left;
+        }
+    while (a.L < a.T && local[a.L]) ++a.L;
+    int pos[64];
+    for (int q = 0; q < s->n; ++q) {
+        pos[q] = q < a.L ? q : a.L + a.kh;
+        if (q >= a.L && local[q]) a.hq[a.kh++] = (uint8_t)q;
+    }
+    int lc[16], la[16];
+    for (int j = 0; j < N; ++j) {
+        lc[j] = pos[qc[j]];
+        la[j] = pos[qa[j]];
+    }
+    a.lc = make_reg(N, lc);
+    if (OP == kDiv) a.la = make_reg(N, la);
+    a.ntiles = 1ull << (s->n - a.T);
+    const size_t smem = sizeof(S) << a.T;
+    auto fn = k_arith_plane<S, OP>;
+    QE_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    int occ = 0;
+    QE_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fn, kArithThreads, smem));
+    const uint64_t grid = std::min<uint64_t>(a.ntiles, (uint64_t)num_sms() * std::max(occ, 1));
+    Launch L(s, tag, 2.0 * dim(s) * amp_bytes(s));
+    fn<<<(unsigned)grid, kArithThreads, smem, s->stream>>>(a);
+    QE_CUDA(cudaGetLastError());
+}
+
+template <class S, int OP>
+void arith_impl(qe_state* s, int N, const int* qa, const int* qb, const int* qc) {
+    const int P = OP == kMul ? N : 2 * N;
+    const char* tag = OP == kMul ? "mul_emulated" : "div_emulated";
+    const size_t plane_bytes = sizeof(S) << P;
+    if (plane_bytes <= 64 * 1024) {
+        arith_tiles<S, OP>(s, N, qa, qb, qc, P, tag);
+        return;
+    }
     static thread_local ArithArgs<S> a;
     std::memset(&a, 0, sizeof(a));
     a.x = reinterpret_cast<S*>(s->d);
     a.N = N;
-    a.op = op;
-    a.P = op == kMul ? N : 2 * N;
+    a.P = P;
     a.a = make_reg(N, qa);
     a.b = make_reg(N, qb);
     a.c = make_reg(N, qc);
-    int pq[32], np = 0;
-    for (int j = 0; j < N; ++j) pq[np++] = qc[j];
-    if (op == kDiv)
-        for (int j = 0; j < N; ++j) pq[np++] = qa[j];
-    std::sort(pq, pq + np);
-    a.nsorted = np;
-    for (int j = 0; j < np; ++j) a.plane_sorted[j] = (uint8_t)pq[j];
-    const uint64_t planes = 1ull << (s->n - a.P);
-    const size_t plane_bytes = sizeof(S) << a.P;
-    const char* tag = op == kMul ? "mul_emulated" : "div_emulated";
-    if (plane_bytes <= 64 * 1024) {
-        a.plane0 = 0;
-        a.nplanes = planes;
-        const size_t smem = plane_bytes;
-        auto fn = k_arith_plane<S>;
-        QE_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-        int occ = 0;
-        QE_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fn, kArithThreads, smem));
-        const uint64_t grid = std::min<uint64_t>(planes, (uint64_t)num_sms() * std::max(occ, 1));
-        Launch L(s, tag, 2.0 * dim(s) * amp_bytes(s));
-        fn<<<(unsigned)grid, kArithThreads, smem, s->stream>>>(a);
+    int bq[35], nq = 0;
+    for (int j = 0; j < N; ++j) bq[nq++] = qc[j];
+    if (OP == kDiv)
+        for (int j = 0; j < N; ++j) bq[nq++] = qa[j];
+    a.w = std::min(3, *std::min_element(bq, bq + nq));
+    for (int q = 0; q < a.w; ++q) bq[nq++] = q;
+    std::sort(bq, bq + nq);
+    for (int j = 0; j < nq; ++j)
+        if (a.nruns && bq[j] == a.run_lo[a.nruns - 1] + a.run_len[a.nruns - 1]) {
+            ++a.run_len[a.nruns - 1];
+        } else {
+            a.run_lo[a.nruns] = (uint8_t)bq[j];
+            a.run_len[a.nruns++] = 1;
+        }
+    const uint64_t blocks = 1ull << (s->n - P - a.w);
+    const size_t block_bytes = plane_bytes << a.w;
+    // batches of whole blocks through the two halves of a scratch buffer
+    const uint64_t per_batch = std::max<uint64_t>(1, std::min<uint64_t>(blocks, kBatch / block_bytes));
+    S* const scratch = reinterpret_cast<S*>(ensure_scratch(s, (blocks > per_batch ? 2 : 1) * per_batch * block_bytes));
+    int half = 0;
+    for (uint64_t p0 = 0; p0 < blocks || a.nblk; p0 += per_batch) {
+        a.back = a.scratch;
+        a.back0 = a.blk0;
+        a.nback = a.nblk;
+        a.scratch = scratch + (half ? per_batch << (P + a.w) : 0);
+        half ^= 1;
+        a.blk0 = p0;
+        a.nblk = p0 < blocks ? std::min<uint64_t>(per_batch, blocks - p0) : 0;
+        const uint64_t total = (a.nblk + a.nback) << (P + a.w);
+        const unsigned grid = (unsigned)std::min<uint64_t>(total / kChunk, (uint64_t)num_sms() * 8);
+        Launch L(s, tag, 1.0 * (double)total * amp_bytes(s), false);
+        k_arith_batch<S, OP><<<grid, 256, 0, s->stream>>>(a);
         QE_CUDA(cudaGetLastError());
-        return;
-    }
-    // batches of whole planes through a scratch buffer of at most 1 GiB
-    const uint64_t per_batch = std::max<uint64_t>(1, std::min<uint64_t>(planes, (1ull << 30) / plane_bytes));
-    a.scratch = reinterpret_cast<S*>(ensure_scratch(s, per_batch * plane_bytes));
-    for (uint64_t p0 = 0; p0 < planes; p0 += per_batch) {
-        a.plane0 = p0;
-        a.nplanes = std::min<uint64_t>(per_batch, planes - p0);
-        const uint64_t total = a.nplanes << a.P;
-        const unsigned grid = (unsigned)std::min<uint64_t>((total + 255) / 256, (uint64_t)num_sms() * 16);
-        {
-            Launch L(s, tag, 2.0 * (double)total * amp_bytes(s), false);
-            k_arith_gather<S><<<grid, 256, 0, s->stream>>>(a);
-            QE_CUDA(cudaGetLastError());
-        }
-        {
-            Launch L(s, "arith_copy_back", 2.0 * (double)total * amp_bytes(s), false);
-            k_arith_copy_back<S><<<grid, 256, 0, s->stream>>>(a);
-            QE_CUDA(cudaGetLastError());
-        }
     }
     s->stats.passes += 2;   // two full passes in total over the batches
 }
@@ -205,13 +358,13 @@ void arith_impl(qe_state* s, int op, int N, const int* qa, const int* qb, const 
 }  // namespace
 
 void launch_mul(qe_state* s, int N, const int* qa, const int* qb, const int* qc) {
-    if (s->dtype == QE_C128) arith_impl<double2>(s, kMul, N, qa, qb, qc);
-    else arith_impl<float2>(s, kMul, N, qa, qb, qc);
+    if (s->dtype == QE_C128) arith_impl<double2, kMul>(s, N, qa, qb, qc);
+    else arith_impl<float2, kMul>(s, N, qa, qb, qc);
 }
 
 void launch_div(qe_state* s, int N, const int* qa, const int* qb, const int* qc) {
-    if (s->dtype == QE_C128) arith_impl<double2>(s, kDiv, N, qa, qb, qc);
-    else arith_impl<float2>(s, kDiv, N, qa, qb, qc);
+    if (s->dtype == QE_C128) arith_impl<double2, kDiv>(s, N, qa, qb, qc);
+    else arith_impl<float2, kDiv>(s, N, qa, qb, qc);
 }
 
 }  // namespace qe
