@@ -242,7 +242,7 @@ int qe_norm2(qe_state* s, double* out);
 /* Apply queued gates / wait for all work on the state's stream.  qe_flush
  * launches the fused passes as they are planned and, before returning, waits
  * for the last tensor-core pass: QE_ERR_TIMEOUT if one of them reported a
- * bounded wait that ran out (the remaining queued gates are then dropped). */
+ * bounded wait that ran out (the state's contents are then undefined). */
 int qe_flush(qe_state* s);
 int qe_sync(qe_state* s);
 

@@ -421,11 +421,12 @@ std::vector<Planned> plan_fusion_list(const std::vector<PendingGate>& q, int max
 // blocks in all (never more on any of them).
 bool plan_lookahead(int n) { return n >= 30; }
 
-uint32_t* status_word_host(qe_state* s) {
+uint32_t* status_word(qe_state* s) {
     if (!s->status_host) {
         QE_CUDA(cudaMallocHost(&s->status_host, sizeof(uint32_t)));
         *s->status_host = 0u;
     }
+    s->status_pending = true;
     return s->status_host;
 }
 
@@ -433,7 +434,7 @@ void complete_pending(qe_state* s) {
     if (!s->status_pending) return;
     s->status_pending = false;
     QE_CUDA(cudaStreamSynchronize(s->stream));
-    const uint32_t st = *s->status_host;
+    const uint32_t st = *(volatile uint32_t*)s->status_host;
     *s->status_host = 0u;
     if (st) fail(QE_ERR_TIMEOUT, "tensor-core gate: an mbarrier wait exceeded its limit");
 }

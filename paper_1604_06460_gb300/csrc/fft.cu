@@ -559,14 +559,13 @@ void qft_tc(qe_state* s, int lo, int m, int inverse) {
     a.lo = lo;
     a.h = (m + 1) / 2;
     int top = m, j = 0;
-    uint32_t* const status = dft_digits_begin(s);
     for (int g = 0; g < groups; ++g) {
         const int last = G * (g + 1) / groups;
         int P = 0;
         for (; j < last; ++j) {
             const int d = digit[j];
             top -= d;
-            launch_dft_digit_c128(s, lo + top, d, P, G > 1, get_direct<F64>(s, P + d, sign, 1), status);
+            launch_dft_digit_c128(s, lo + top, d, P, G > 1, get_direct<F64>(s, P + d, sign, 1));
             P += d;
         }
         if (top == 0) break;
@@ -584,7 +583,6 @@ void qft_tc(qe_state* s, int lo, int m, int inverse) {
         k_digit_twiddle<<<grid, 256, 0, s->stream>>>(a);
         QE_CUDA(cudaGetLastError());
     }
-    dft_digits_end(s, status);
     if (G > 1) bitrev_impl<F64>(s, lo, m, "digitrev");
 }
 

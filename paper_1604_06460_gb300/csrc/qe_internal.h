@@ -67,8 +67,8 @@ struct qe_state {
     // pinned host mirror of small results
     double* host_result = nullptr;
     qe::Stats stats;
-    // status word of the last tensor-core launch (pinned host copy), checked
-    // before the next such launch and at the end of every flush
+    // status word of the tensor-core launches (pinned host memory), checked at
+    // the end of every flush
     uint32_t* status_host = nullptr;
     bool status_pending = false;
     // optional per-launch event timing
@@ -122,21 +122,19 @@ void launch_scale(qe_state* s, double factor);
 
 // dense k-qubit gate (1 <= k <= 5) through shared-memory tiles
 void launch_gate_dense(qe_state* s, int k, const int* qubits, const cd* U);
-// The tensor-core launchers copy their device status word into the state's
-// pinned host word after the kernel and mark it pending; complete_pending()
-// waits for the stream and raises QE_ERR_TIMEOUT if a launch reported one.
-uint32_t* status_word_host(qe_state* s);
+// The tensor-core kernels raise the state's status word (pinned host memory the
+// device writes to) when one of their waits runs out; status_word() marks it as
+// to be looked at, complete_pending() waits for the stream and raises
+// QE_ERR_TIMEOUT if a launch reported one.
+uint32_t* status_word(qe_state* s);
 void complete_pending(qe_state* s);
 // 5-qubit block on a complex64 / complex128 state with tcgen05 tensor cores
 // (n >= 12, qubits ascending)
 void launch_gate_tc5(qe_state* s, const int* qubits, const cd* U);
 void launch_gate_tc5_c128(qe_state* s, const int* qubits, const cd* U);
 // one digit [q0, q0 + d) of a Fourier transform on a complex128 state, its
-// matrix chosen by the P qubits above it; begin and end bracket a run of digits
-// that share a status word (tc_c128.cu)
-uint32_t* dft_digits_begin(qe_state* s);
-void launch_dft_digit_c128(qe_state* s, int q0, int d, int P, bool reversed, const double2* roots, uint32_t* status);
-void dft_digits_end(qe_state* s, const uint32_t* status);
+// matrix chosen by the P qubits above it (tc_c128.cu)
+void launch_dft_digit_c128(qe_state* s, int q0, int d, int P, bool reversed, const double2* roots);
 // diagonal gate: amplitude x *= d[row(x)] for all x
 void launch_gate_diag(qe_state* s, int k, const int* qubits, const cd* d);
 // amplitudes with (x & mask) == value are multiplied by phase

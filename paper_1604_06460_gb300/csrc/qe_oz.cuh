@@ -213,17 +213,6 @@ struct MmaTable {
     }
 };
 
-// IEEE binary16 bits of an integer of magnitude below 2048 (exact).
-inline uint16_t fp16_bits(int d) {
-    if (d == 0) return 0;
-    const uint16_t sign = d < 0 ? 0x8000u : 0u;
-    unsigned m = (unsigned)(d < 0 ? -d : d);
-    int e = 0;
-    while ((m >> (e + 1)) != 0) ++e;                     // m in [2^e, 2^(e+1))
-    const unsigned frac = (m << (10 - e)) & 0x3FFu;
-    return (uint16_t)(sign | ((unsigned)(e + 15) << 10) | frac);
-}
-
 // The executing thread's arrival on the mbarrier, announcing `bytes` of
 // asynchronous copies that complete on it.
 __device__ __forceinline__ void mbar_expect_tx(uint64_t* mbar, uint32_t bytes) {

@@ -60,6 +60,14 @@ __device__ __forceinline__ void mma_commit(uint64_t* mbar) {
         smem_u32(mbar)));
 }
 
+// Report a wait that ran out: the status word is in pinned host memory, read
+// after the stream has been waited for, so a launch needs no copy to clear it
+// or to bring it back.
+__device__ __forceinline__ void raise_status(uint32_t* status) {
+    *reinterpret_cast<volatile uint32_t*>(status) = 1u;
+    __threadfence_system();
+}
+
 // Tile geometry of a 5-qubit block: 12 tile-local index bits, the low bits
 // [0, L) (contiguous chunks of 2^L amplitudes) plus the kh gate qubits >= L;
 // the five gate qubits sit at tile-local positions gpos[] and the other

@@ -19,7 +19,7 @@
 // balanced digits: X = sum_i a_i 256^(D - i), a_1 in [0, 128], a_2..a_D in
 // [-128, 127]; the value's sign multiplies every digit.  Digit i thus weighs
 // 2^(E_r - 8 i) whatever D is.  W's rows get scales 2^F_n and digits b_j the
-// same way on the host.  Every digit is an integer of magnitude <= 128 and
+// same way (by every CTA at its start).  Every digit is an integer of magnitude <= 128 and
 // exact in FP16.
 //
 // Products.  C_d = sum_{i + j = d} A_i B_j^T for d = 2..D+2 (26 digit pairs
@@ -93,6 +93,7 @@ namespace {
 
 using namespace oz;
 using tc::mbar_wait;
+using tc::raise_status;
 using tc::smem_u32;
 
 constexpr int kEpiWarps = 8;                 // warps [0, 8): recombination, two per TMEM lane quarter
@@ -122,15 +123,20 @@ struct OzArgs {
     uint8_t gpos[5];        // tile-local positions of the matrix bits, ascending
     uint32_t* status;
     long long spin_limit;
-    const uint16_t* B;      // [D][64][64] fp16 digits of W': slice j, row n', column k
-    const int* F;           // [64] row scale exponents of W (original row order)
     int stall_test;         // failure-path test: the first staged half is never announced
 };
 
-// One digit of a Fourier transform as a block whose matrix is built on the
-// device and depends on `P` index bits outside the tile (see build_dft).
+// A block with its matrix (row-major), split into digits by every CTA.
+struct GateArgs {
+    OzArgs z;
+    const double2* U;       // [32][32] in device memory (as a kernel parameter, read by lanes at different
+                            // addresses, it cost 40 us a launch)
+};
+
+// One digit of a Fourier transform as a block whose matrix depends on `P` index
+// bits outside the tile (see matrix_entry).
 struct DftArgs {
-    OzArgs z;               // z.B, z.F unused; z.hq the tile's bits at or above L
+    OzArgs z;               // z.hq the tile's bits at or above L
     int nskip;              // bits left out of a tile's index: the tile's and the P matrix bits, ascending
     uint8_t skip[32];
     int lt;                 // 2^lt tiles share a matrix
@@ -226,35 +232,42 @@ __device__ __forceinline__ uint32_t issue_mmas(uint32_t elected, const OzArgs& a
     return pre | (pxf << 1) | (first ? 4u : 0u);
 }
 
-// W of a transform digit, built in shared memory by all warps.  With l_prior
-// the P-bit value of the transform's outputs so far (the matrix bits, which
-// hold it bit-reversed),
+// Entry (row, column) of the block's complex matrix.
+__device__ __forceinline__ double2 matrix_entry(const GateArgs& g, uint32_t, uint32_t row, uint32_t col) {
+    return g.U[32 * row + col];
+}
+// Of a transform digit: with l_prior the P-bit value of the transform's outputs
+// so far (the matrix bits v, which hold it bit-reversed),
 //   U[l][k] = 2^(-d/2) w_(2^(P + d))^(k (l_prior + 2^P l)):
 // the digit's 2^d-point transform with the twiddle by the earlier outputs
 // folded into the columns.  With several digits, output l is left at the
 // bit-reversed position, so that one bit reversal of the register restores the
-// natural order whatever the digits are.  One warp per complex row, lane <->
-// column; entries split like the inputs (scale from the row's largest
-// component).
-template <int D>
-__device__ __noinline__ void build_dft(const DftArgs& f, uint32_t v, unsigned char* sB, int* sF20) {
+// natural order whatever the digits are.
+__device__ __forceinline__ double2 matrix_entry(const DftArgs& f, uint32_t v, uint32_t row, uint32_t col) {
+    const uint32_t lp = f.P ? (__brev(v) >> (32 - f.P)) : 0u, dm = (1u << f.d) - 1u;
+    const uint32_t lr = (row >> f.below) & dm, k = (col >> f.below) & dm;
+    const uint32_t l = f.reversed ? __brev(lr) >> (32 - f.d) : lr;
+    const double2 w = f.roots[(k * (lp + (l << f.P))) & ((1u << (f.P + f.d)) - 1u)];
+    const bool inside = ((col ^ row) & ~(dm << f.below)) == 0;    // idle qubits: the identity
+    return inside ? make_double2(w.x * f.scale, w.y * f.scale) : make_double2(0.0, 0.0);
+}
+
+// The digits and row scales of W = [[Re U, -Im U], [Im U, Re U]] in shared
+// memory, by all warps: one warp per complex row, lane <-> column, every entry
+// split like the inputs with the scale of its row's largest component (real
+// rows n and n + 32 share it); rows below 2^-920 are flushed to zero.
+template <int D, class Args>
+__device__ __noinline__ void build_w(const Args& g, uint32_t v, unsigned char* sB, int* sF20) {
     constexpr uint32_t kStackB = (uint32_t)D * kStackSlice;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const uint32_t lp = f.P ? (__brev(v) >> (32 - f.P)) : 0u;
-    const uint32_t dm = (1u << f.d) - 1u;
     for (int r = warp; r < 32; r += kOzThreads / 32) {
-        const uint32_t lr = ((uint32_t)r >> f.below) & dm, k = ((uint32_t)lane >> f.below) & dm;
-        const uint32_t l = f.reversed ? __brev(lr) >> (32 - f.d) : lr;
-        const uint32_t e = (k * (lp + (l << f.P))) & ((1u << (f.P + f.d)) - 1u);
-        const bool inside = (((uint32_t)lane ^ (uint32_t)r) & ~(dm << f.below)) == 0;   // idle qubits: the identity
-        const double2 w = f.roots[e];
-        const double re = inside ? w.x * f.scale : 0.0, im = inside ? w.y * f.scale : 0.0;
-        uint32_t em = max((uint32_t)__double2hiint(re) << 1, (uint32_t)__double2hiint(im) << 1);
+        const double2 u = matrix_entry(g, v, (uint32_t)r, (uint32_t)lane);
+        uint32_t em = max((uint32_t)__double2hiint(u.x) << 1, (uint32_t)__double2hiint(u.y) << 1);
         for (int o = 16; o > 0; o >>= 1) em = max(em, __shfl_xor_sync(0xFFFFFFFFu, em, o));
         em >>= 21;
-        const uint32_t base_s = D == 7 ? em : em + 5u;
+        const uint32_t base_s = em < (uint32_t)kFlushExp ? 0x10000u : (D == 7 ? em : em + 5u);
         uint32_t dg[D];   // (re, im) digits as fp16 pairs
-        digit_pairs<D>(split_z<D>(re, base_s), split_z<D>(im, base_s), dg);
+        digit_pairs<D>(split_z<D>(u.x, base_s), split_z<D>(u.y, base_s), dg);
         const int hh = r >> 4, m = r & 15;
         unsigned char* const b = sB + hh * kStackB + 2 * (lane & 7);
         const int c0 = lane >> 3, c1 = 4 + (lane >> 3);
@@ -266,7 +279,7 @@ __device__ __noinline__ void build_dft(const DftArgs& f, uint32_t v, unsigned ch
             *reinterpret_cast<uint16_t*>(b + sw128_chunk(j * kNH + m + 16, c0)) = di;
             *reinterpret_cast<uint16_t*>(b + sw128_chunk(j * kNH + m + 16, c1)) = dr;
         }
-        if (lane == 0) sF20[r] = sF20[32 + r] = ((int)em - 1021) * (1 << 20);
+        if (lane == 0) sF20[r] = sF20[32 + r] = em < (uint32_t)kFlushExp ? 0 : ((int)em - 1021) * (1 << 20);
     }
 }
 
@@ -293,7 +306,7 @@ __device__ __forceinline__ uint32_t stage_off(uint32_t row, uint32_t c) {
     return 16u * (kHalfRows * c + (row ^ stage_swizzle(c)));
 }
 
-__device__ __forceinline__ const OzArgs& oz_args(const OzArgs& a) { return a; }
+__device__ __forceinline__ const OzArgs& oz_args(const GateArgs& a) { return a.z; }
 __device__ __forceinline__ const OzArgs& oz_args(const DftArgs& a) { return a.z; }
 
 // 19 warps of 96 registers a thread: a sub-partition holding five of the warps
@@ -325,17 +338,7 @@ __global__ void __maxnreg__(96) k_gate_tc5_c128(const __grid_constant__ Args arg
     __shared__ int s_eterm[2][kRows];          // (E_r - 56) << 20 of the rows of two tiles in flight
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
 
-    // W' digits into their swizzled operand layout; W row scales
-    if constexpr (!kDft) {
-#pragma unroll 1
-        for (int i = tid; i < D * kN * 8; i += blockDim.x) {
-            const int j = i / (kN * 8), n = (i / 8) % kN, ch = i % 8;
-            const uint4 v = *reinterpret_cast<const uint4*>(a.B + ((size_t)(j * kN + n) * kK + ch * 8));
-            const int hh = n / kNH, m = n % kNH;
-            *reinterpret_cast<uint4*>(sB + hh * kStackB + sw128_chunk(j * kNH + m, ch)) = v;
-        }
-    }
-    if (!kDft && tid < kN) sF20[tid] = a.F[tid] * (1 << 20);
+    if constexpr (!kDft) build_w<D>(arg, 0u, sB, sF20);
     if (tid < (1 << a.kh)) {
         uint64_t o = 0;
         for (int j = 0; j < a.kh; ++j)
@@ -441,7 +444,7 @@ __global__ void __maxnreg__(96) k_gate_tc5_c128(const __grid_constant__ Args arg
                 s_end = (v + 1) << arg.lt;
                 s_step = (gridDim.x - team + arg.teams - 1) / arg.teams;    // CTAs of the team
             }
-            build_dft<D>(arg, v, sB, sF20);
+            build_w<D>(arg, v, sB, sF20);
             asm volatile("fence.proxy.async.shared::cta;");
             __syncthreads();
             return true;
@@ -453,7 +456,7 @@ __global__ void __maxnreg__(96) k_gate_tc5_c128(const __grid_constant__ Args arg
     auto wait = [&](Bar b, uint32_t& ph) {
         const bool ok = wait_or_abort(smem_u32(&bars[b]), ph, a.spin_limit, &abort_flag);
         if (__any_sync(0xFFFFFFFFu, !ok)) {
-            if (!ok) atomicExch(a.status, 1u);
+            if (!ok) raise_status(a.status);
             return false;
         }
         ph ^= 1u;
@@ -466,13 +469,13 @@ __global__ void __maxnreg__(96) k_gate_tc5_c128(const __grid_constant__ Args arg
         for (bool more = next_segment(true); more; more = next_segment(false)) {
             ph = issue_mmas<D>(elected, a, seg_begin(), seg_end(), seg_step(), tmem, smem_u32(sA), smem_u32(sB), bars,
                                &abort_flag, ph);
-            if (ph & 8u) atomicExch(a.status, 1u);
+            if (ph & 8u) raise_status(a.status);
             __syncwarp();
         }
         mma_commit_elected(elected, &bars[kDrain]);    // by the lane that issued the MMAs
         if (lane == 0) {
             // every MMA issued has completed before tensor memory is freed
-            if (!tc::mbar_wait(smem_u32(&bars[kDrain]), 0u, a.spin_limit)) atomicExch(a.status, 1u);
+            if (!tc::mbar_wait(smem_u32(&bars[kDrain]), 0u, a.spin_limit)) raise_status(a.status);
         }
         __syncwarp();
     } else if (warp >= kLoadWarp0) {
@@ -732,77 +735,26 @@ __global__ void __maxnreg__(96) k_gate_tc5_c128(const __grid_constant__ Args arg
     }
 }
 
-// Balanced base-256 digits of one row of W (host side, same rule as the
-// device splitting): returns the scale exponent F and fills digits[j][k].
-template <int D>
-int split_row_host(const double* w, int16_t digits[D][kK]) {
-    int emax = 0;
-    for (int k = 0; k < kK; ++k) {
-        uint64_t b;
-        std::memcpy(&b, &w[k], 8);
-        emax = std::max(emax, (int)((b >> 52) & 0x7FF));
-    }
-    if (emax < kFlushExp) {
-        std::memset(digits, 0, sizeof(int16_t) * D * kK);
-        return 0;
-    }
-    const int F = emax - 1021;
-    uint64_t off = 0;   // D - 1 bytes of 0x80
-    for (int j = 1; j < D; ++j) off = (off << 8) | 0x80u;
-    for (int k = 0; k < kK; ++k) {
-        // <= 2^(8D - 1), exact scaling, one rounding
-        const uint64_t X = (uint64_t)std::llround(std::ldexp(std::fabs(w[k]), 8 * D - F));
-        const uint64_t Z = X + off;
-        const int sg = std::signbit(w[k]) ? -1 : 1;
-        digits[0][k] = (int16_t)(sg * (int)(Z >> (8 * (D - 1))));
-        for (int j = 1; j < D; ++j)
-            digits[j][k] = (int16_t)(sg * ((int)((Z >> (8 * (D - 1 - j))) & 0xFF) - 128));
-    }
-    return F;
-}
-
 template <int D>
 void launch_impl(qe_state* s, const int* qubits, const cd* U, const char* tag) {
     if (s->dtype != QE_C128) fail(QE_ERR_UNSUPPORTED, "this tensor-core path is for complex128 states");
     if (s->n < 12) fail(QE_ERR_UNSUPPORTED, "tensor-core gates need n >= 12");
     const tc::Geometry g = tc::tile_geometry(qubits);
-    OzArgs a;
+    GateArgs arg{};
+    OzArgs& a = arg.z;
     a.x = reinterpret_cast<double2*>(s->d);
     a.L = g.L;
     a.kh = g.kh;
     std::memcpy(a.hq, g.hq, sizeof(g.hq));
     std::memcpy(a.gpos, g.gpos, sizeof(a.gpos));
     a.ntiles = 1ull << (s->n - 12);
-    // W = [[Re U, -Im U], [Im U, Re U]], row n (output), column k (input)
-    struct HostW {
-        uint16_t B[D * kN * kK];
-        int F[kN];
-    };
-    static thread_local HostW hw;
-    for (int n = 0; n < kN; ++n) {
-        double w[kK];
-        for (int k = 0; k < kK; ++k) {
-            const cd u = U[(n & 31) * 32 + (k & 31)];
-            w[k] = (n < 32) ? ((k < 32) ? u.real() : -u.imag()) : ((k < 32) ? u.imag() : u.real());
-        }
-        int16_t dg[D][kK];
-        hw.F[n] = split_row_host<D>(w, dg);
-        // operand row n' of W' (two halves of 32 rows, see the epilogue)
-        const int c = n & 31, hh = c >> 4, m = (c & 15) + ((n >> 5) << 4);
-        const int np = hh * kNH + m;
-        for (int j = 0; j < D; ++j)
-            for (int k = 0; k < kK; ++k) {
-                hw.B[((size_t)j * kN + np) * kK + k] = fp16_bits(dg[j][k]);
-            }
-    }
-    complete_pending(s);   // the previous tensor-core launch, before the scratch is reused
-    char* scr = (char*)ensure_scratch(s, 256 + sizeof(HostW));
-    uint32_t* status = (uint32_t*)scr;
-    QE_CUDA(cudaMemsetAsync(status, 0, sizeof(uint32_t), s->stream));
-    QE_CUDA(cudaMemcpyAsync(scr + 256, &hw, sizeof(HostW), cudaMemcpyHostToDevice, s->stream));
-    a.status = status;
-    a.B = reinterpret_cast<const uint16_t*>(scr + 256);
-    a.F = reinterpret_cast<const int*>(scr + 256 + sizeof(hw.B));
+    // the copy is ordered after the previous block on the stream and returns
+    // once U is staged: no wait between blocks, and nothing to split on the host
+    static_assert(sizeof(cd) == sizeof(double2), "interleaved complex");
+    double2* const dU = reinterpret_cast<double2*>(ensure_scratch(s, 32 * 32 * sizeof(double2)));
+    QE_CUDA(cudaMemcpyAsync(dU, U, 32 * 32 * sizeof(double2), cudaMemcpyHostToDevice, s->stream));
+    arg.U = dU;
+    a.status = status_word(s);
     a.spin_limit = 1ll << 21;   // polls of up to kSuspendNs each
     // Failure-path test (QE_TEST_STALL_TC128=1): the load warps withhold the
     // arrival for the first staged half, so the splitters' wait runs out after
@@ -812,18 +764,12 @@ void launch_impl(qe_state* s, const int* qubits, const cd* U, const char* tag) {
     a.stall_test = (stall != nullptr && stall[0] == '1') ? 1 : 0;
     if (a.stall_test) a.spin_limit = 1ll << 12;
     const size_t smem = oz_smem<D>();
-    auto fn = qubits[0] == 0 ? k_gate_tc5_c128<D, true, OzArgs> : k_gate_tc5_c128<D, false, OzArgs>;
+    auto fn = qubits[0] == 0 ? k_gate_tc5_c128<D, true, GateArgs> : k_gate_tc5_c128<D, false, GateArgs>;
     QE_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     const uint64_t grid = std::min<uint64_t>(a.ntiles, (uint64_t)num_sms());
-    {
-        Launch Lc(s, tag, 2.0 * dim(s) * amp_bytes(s));
-        fn<<<(unsigned)grid, kOzThreads, smem, s->stream>>>(a);
-        QE_CUDA(cudaGetLastError());
-    }
-    // checked before the next tensor-core launch or at the end of the flush,
-    // so that the host plans the next block while this one runs
-    QE_CUDA(cudaMemcpyAsync(status_word_host(s), status, sizeof(uint32_t), cudaMemcpyDeviceToHost, s->stream));
-    s->status_pending = true;
+    Launch Lc(s, tag, 2.0 * dim(s) * amp_bytes(s));
+    fn<<<(unsigned)grid, kOzThreads, smem, s->stream>>>(arg);
+    QE_CUDA(cudaGetLastError());
 }
 
 }  // namespace
@@ -836,27 +782,12 @@ void launch_gate_tc5_c128(qe_state* s, const int* qubits, const cd* U) {
     else launch_impl<7>(s, qubits, U, "gate_tc_k5_c128");
 }
 
-// The status word of a run of transform digits: cleared before the first and
-// read back after the last (the digits only ever raise it, so no host wait
-// separates them: one digit alone took 38 us at n = 12 with a wait before each
-// launch).
-uint32_t* dft_digits_begin(qe_state* s) {
-    complete_pending(s);   // the previous tensor-core launch, before the status word is reused
-    uint32_t* status = (uint32_t*)ensure_scratch(s, 256);
-    QE_CUDA(cudaMemsetAsync(status, 0, sizeof(uint32_t), s->stream));
-    return status;
-}
-void dft_digits_end(qe_state* s, const uint32_t* status) {
-    QE_CUDA(cudaMemcpyAsync(status_word_host(s), status, sizeof(uint32_t), cudaMemcpyDeviceToHost, s->stream));
-    s->status_pending = true;
-}
-
 // One digit of a Fourier transform on a complex128 state (n >= 12): the qubits
 // [q0, q0 + d), 3 <= d <= 5, whose matrix depends on the P qubits above them
 // (P + d <= 20, n - 12 - P >= 0).  `roots` holds the 2^(P + d) roots of unity
 // of the transform's sign; `reversed`: leave the output bit-reversed.  56-bit
 // splitting in both arithmetic modes (the seventh digit costs 3 %).
-void launch_dft_digit_c128(qe_state* s, int q0, int d, int P, bool reversed, const double2* roots, uint32_t* status) {
+void launch_dft_digit_c128(qe_state* s, int q0, int d, int P, bool reversed, const double2* roots) {
     constexpr int D = 7;
     if (s->n < 12 + P) fail(QE_ERR_UNSUPPORTED, "transform digits need n >= 12 + P");
     static thread_local DftArgs f;
@@ -904,7 +835,7 @@ void launch_dft_digit_c128(qe_state* s, int q0, int d, int P, bool reversed, con
         if (q >= a.L && (local[q] || matrix[q])) f.skip[f.nskip++] = (uint8_t)q;
     }
     for (int j = 0; j < 5; ++j) a.gpos[j] = (uint8_t)pos[gate[j]];
-    a.status = status;
+    a.status = status_word(s);
     a.spin_limit = 1ll << 21;
     const size_t smem = oz_smem<D>();
     auto fn = pair ? k_gate_tc5_c128<D, true, DftArgs> : k_gate_tc5_c128<D, false, DftArgs>;

@@ -61,7 +61,7 @@ struct TcArgs {
     uint8_t gpos[5];          // tile-local bit positions of the matrix bits
     uint32_t* status;
     long long spin_limit;
-    const float* W;           // [2][kN * kK]: hi, lo parts of W, row n, column k
+    const float2* U;          // [32][32]: the block's matrix
     int stall_test;           // failure-path test: the first tile's operand is never announced
 };
 
@@ -182,11 +182,15 @@ __global__ void __maxnreg__(72) k_gate_tc5(const __grid_constant__ TcArgs a) {
     __shared__ int s_abort;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
 
-    // W into its swizzled operand layout
+    // W = [[Re U, -Im U], [Im U, Re U]] (row n: output, column k: input) split
+    // into TF32 parts, in its swizzled operand layout
     for (int i = tid; i < kN * kK; i += blockDim.x) {
         const int n = i / kK, k = i % kK;
-        *reinterpret_cast<float*>(sW_hi + sw128_offset(n, k, kN)) = a.W[i];
-        *reinterpret_cast<float*>(sW_lo + sw128_offset(n, k, kN)) = a.W[kN * kK + i];
+        const float2 u = a.U[(n & 31) * 32 + (k & 31)];
+        const float w = (n < 32) ? ((k < 32) ? u.x : -u.y) : ((k < 32) ? u.y : u.x);
+        const float hi = tf32_hi(w);
+        *reinterpret_cast<float*>(sW_hi + sw128_offset(n, k, kN)) = hi;
+        *reinterpret_cast<float*>(sW_lo + sw128_offset(n, k, kN)) = __fsub_rn(w, hi);
     }
     if (tid < (1 << a.kh)) {
         uint64_t o = 0;
@@ -234,7 +238,7 @@ __global__ void __maxnreg__(72) k_gate_tc5(const __grid_constant__ TcArgs a) {
         return l;
     };
     auto goff = [&](uint32_t l) -> uint64_t { return (l & lowmask) + hoff[l >> a.L]; };
-    auto fail_status = [&]() { atomicExch(a.status, 1u); };
+    auto fail_status = [&]() { tc::raise_status(a.status); };
 
     if (warp == kMmaWarp) {
         // ------------------------------------------------------ MMA issuer
@@ -399,7 +403,7 @@ __global__ void __maxnreg__(72) k_gate_tc5(const __grid_constant__ TcArgs a) {
 void launch_gate_tc5(qe_state* s, const int* qubits, const cd* U) {
     if (s->dtype != QE_C64) fail(QE_ERR_UNSUPPORTED, "tensor-core gates are complex64 only");
     if (s->n < 12) fail(QE_ERR_UNSUPPORTED, "tensor-core gates need n >= 12");
-    TcArgs a;
+    TcArgs a{};
     const tc::Geometry g = tc::tile_geometry(qubits);
     a.x = reinterpret_cast<float2*>(s->d);
     a.L = g.L;
@@ -407,31 +411,14 @@ void launch_gate_tc5(qe_state* s, const int* qubits, const cd* U) {
     std::memcpy(a.hq, g.hq, sizeof(a.hq));
     std::memcpy(a.gpos, g.gpos, sizeof(a.gpos));
     a.ntiles = 1ull << (s->n - 12);
-    // W = [[Re U, -Im U], [Im U, Re U]], row n (output), column k (input)
-    static thread_local float W[2 * kN * kK];
-    for (int n = 0; n < kN; ++n)
-        for (int k = 0; k < kK; ++k) {
-            const cd u = U[(n & 31) * 32 + (k & 31)];
-            double w;
-            if (n < 32) w = (k < 32) ? u.real() : -u.imag();
-            else w = (k < 32) ? u.imag() : u.real();
-            const float f = (float)w;
-            // TF32 high part: round to 10 mantissa bits (nearest, ties away)
-            uint32_t bits;
-            std::memcpy(&bits, &f, 4);
-            bits = (bits + 0x1000u) & 0xFFFFE000u;
-            float hi;
-            std::memcpy(&hi, &bits, 4);
-            W[n * kK + k] = hi;
-            W[kN * kK + n * kK + k] = f - hi;
-        }
-    complete_pending(s);   // the previous tensor-core launch, before the scratch is reused
-    char* scr = (char*)ensure_scratch(s, 256 + sizeof(W));
-    uint32_t* status = (uint32_t*)scr;
-    QE_CUDA(cudaMemsetAsync(status, 0, sizeof(uint32_t), s->stream));
-    QE_CUDA(cudaMemcpyAsync(scr + 256, W, sizeof(W), cudaMemcpyHostToDevice, s->stream));
-    a.status = status;
-    a.W = (const float*)(scr + 256);
+    // the copy is ordered after the previous block on the stream and returns
+    // once the matrix is staged: no wait between blocks
+    static thread_local float2 hU[32 * 32];
+    for (int i = 0; i < 32 * 32; ++i) hU[i] = make_float2((float)U[i].real(), (float)U[i].imag());
+    float2* const dU = reinterpret_cast<float2*>(ensure_scratch(s, sizeof(hU)));
+    QE_CUDA(cudaMemcpyAsync(dU, hU, sizeof(hU), cudaMemcpyHostToDevice, s->stream));
+    a.U = dU;
+    a.status = status_word(s);
     a.spin_limit = 1ll << 21;   // polls of up to kSuspendNs each
     // Failure-path test (QE_TEST_STALL_TC64=1): the splitters withhold the
     // first tile's operand arrival, so the MMA thread's wait runs out after a
@@ -444,15 +431,9 @@ void launch_gate_tc5(qe_state* s, const int* qubits, const cd* U) {
     QE_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     QE_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributePreferredSharedMemoryCarveout, 100));
     const uint64_t grid = std::min<uint64_t>(a.ntiles, (uint64_t)num_sms());
-    {
-        Launch Lc(s, "gate_tc_k5", 2.0 * dim(s) * amp_bytes(s));
-        fn<<<(unsigned)grid, kTcThreads, smem, s->stream>>>(a);
-        QE_CUDA(cudaGetLastError());
-    }
-    // checked before the next tensor-core launch or at the end of the flush,
-    // so that the host plans the next block while this one runs
-    QE_CUDA(cudaMemcpyAsync(status_word_host(s), status, sizeof(uint32_t), cudaMemcpyDeviceToHost, s->stream));
-    s->status_pending = true;
+    Launch Lc(s, "gate_tc_k5", 2.0 * dim(s) * amp_bytes(s));
+    fn<<<(unsigned)grid, kTcThreads, smem, s->stream>>>(a);
+    QE_CUDA(cudaGetLastError());
 }
 
 }  // namespace qe
