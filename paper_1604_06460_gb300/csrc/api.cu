@@ -190,25 +190,26 @@ void apply_in_place(std::vector<cd>& U, int D, int gk, const int* pos, const std
         }
         return;
     }
-    double xr[32], xi[32];
+    // a whole row at a time, zero entries of G skipped (a CNOT moves two rows)
+    double x[32][64];
     for (int r0 = 0; r0 < D; ++r0) {
         if (r0 & gmask) continue;
-        for (int col = 0; col < D; ++col) {
+        for (int c = 0; c < Dg; ++c) std::memcpy(x[c], u + 2 * (size_t)(r0 | dep[c]) * D, 2 * sizeof(double) * D);
+        for (int r = 0; r < Dg; ++r) {
+            double* e = u + 2 * (size_t)(r0 | dep[r]) * D;
+            std::memset(e, 0, 2 * sizeof(double) * D);
             for (int c = 0; c < Dg; ++c) {
-                const double* e = u + 2 * ((size_t)(r0 | dep[c]) * D + col);
-                xr[c] = e[0];
-                xi[c] = e[1];
-            }
-            for (int r = 0; r < Dg; ++r) {
-                double sr = 0.0, si = 0.0;
-                const double* gr = g + 2 * (size_t)r * Dg;
-                for (int c = 0; c < Dg; ++c) {
-                    sr += gr[2 * c] * xr[c] - gr[2 * c + 1] * xi[c];
-                    si += gr[2 * c] * xi[c] + gr[2 * c + 1] * xr[c];
+                const double gr = g[2 * ((size_t)r * Dg + c)], gi = g[2 * ((size_t)r * Dg + c) + 1];
+                const double* v = x[c];
+                if (gr == 0.0 && gi == 0.0) continue;
+                if (gr == 1.0 && gi == 0.0) {
+                    for (int k = 0; k < 2 * D; ++k) e[k] += v[k];
+                    continue;
                 }
-                double* e = u + 2 * ((size_t)(r0 | dep[r]) * D + col);
-                e[0] = sr;
-                e[1] = si;
+                for (int col = 0; col < D; ++col) {
+                    e[2 * col] += gr * v[2 * col] - gi * v[2 * col + 1];
+                    e[2 * col + 1] += gr * v[2 * col + 1] + gi * v[2 * col];
+                }
             }
         }
     }
@@ -235,14 +236,25 @@ void plan_fusion_frontier(const std::vector<PendingGate>& q, int max_k, int nq,
         for (int j = 0; j < q[i].k; ++j) m |= 1ull << q[i].q[j];
         gm[i] = m;
         special[i] = (q[i].cmask != 0 || q[i].k > max_k) ? 1 : 0;
-        for (int b = 0; b < nq; ++b)
-            if ((m >> b) & 1ull) queue[b].push_back(i);
+        for (uint64_t t = m; t; t &= t - 1) queue[__builtin_ctzll(t)].push_back(i);
     }
-    std::vector<int> ptr(nq, 0);
-    auto front = [&](int b, const std::vector<int>& p) { return p[b] < (int)queue[b].size() ? queue[b][p[b]] : -1; };
-    // gates absorbable into a block on S from positions p (p is advanced)
-    auto absorb = [&](uint64_t S, std::vector<int>& p, std::vector<int>* taken) {
-        int count = 0;
+    for (auto& v : queue) v.push_back(-1);   // ends every queue
+    // positions in the queues (n <= 34), cheap to copy
+    struct Pos {
+        int v[36];
+    };
+    auto front = [&](int b, const Pos& p) { return queue[b][p.v[b]]; };
+    auto ready = [&](int gi, const Pos& p) {
+        for (uint64_t t = gm[gi]; t; t &= t - 1)
+            if (front(__builtin_ctzll(t), p) != gi) return false;
+        return true;
+    };
+    auto advance = [&](int gi, Pos& p) {
+        for (uint64_t t = gm[gi]; t; t &= t - 1) ++p.v[__builtin_ctzll(t)];
+    };
+    // gates absorbable into a block on S from positions p (p is advanced), in
+    // the order of taking
+    auto absorb = [&](uint64_t S, Pos& p, std::vector<int>& taken) {
         bool progress = true;
         while (progress) {
             progress = false;
@@ -250,52 +262,65 @@ void plan_fusion_frontier(const std::vector<PendingGate>& q, int max_k, int nq,
                 const int b = __builtin_ctzll(r);
                 for (;;) {
                     const int gi = front(b, p);
-                    if (gi < 0 || special[gi] || (gm[gi] & ~S)) break;
-                    bool at_front = true;
-                    for (uint64_t t = gm[gi]; t; t &= t - 1)
-                        if (front(__builtin_ctzll(t), p) != gi) { at_front = false; break; }
-                    if (!at_front) break;
-                    for (uint64_t t = gm[gi]; t; t &= t - 1) ++p[__builtin_ctzll(t)];
-                    if (taken) taken->push_back(gi);
-                    ++count;
+                    if (gi < 0 || special[gi] || (gm[gi] & ~S) || !ready(gi, p)) break;
+                    advance(gi, p);
+                    taken.push_back(gi);
                     progress = true;
                 }
             }
         }
-        return count;
+    };
+    // their number alone, starting from the qubits `from` of S (the others are
+    // known to be blocked): a gate taken from one qubit's queue puts its other
+    // qubits back on the list
+    auto count = [&](uint64_t S, uint64_t from, Pos& p) {
+        int c = 0;
+        for (uint64_t todo = from; todo;) {
+            const int b = __builtin_ctzll(todo);
+            todo &= todo - 1;
+            for (;;) {
+                const int gi = front(b, p);
+                if (gi < 0 || special[gi] || (gm[gi] & ~S) || !ready(gi, p)) break;
+                advance(gi, p);
+                todo |= gm[gi] & ~(1ull << b);
+                ++c;
+            }
+        }
+        return c;
     };
     // Absorption is confluent (taking a gate never blocks another), so the
     // gates of S | add are those of S plus what absorbing S | add from S's
-    // end positions adds.
-    std::vector<int> pS(nq), scratch(nq);
+    // end positions adds; a gate that S alone could not take is at the front
+    // of an added qubit, so only those are looked at.
+    Pos pS, scratch, ptr{};
     // grow a candidate set from S up to max_k qubits with the queues at
     // positions base; returns its gate count
-    auto grow = [&](uint64_t& S, const std::vector<int>& base) {
+    auto grow = [&](uint64_t& S, const Pos& base) {
         pS = base;
-        int cS = absorb(S, pS, nullptr);
+        int cS = count(S, S, pS);
         while (__builtin_popcountll(S) < max_k) {
             int best = -1, best_add = 0;
             uint64_t best_m = 0;
             auto consider = [&](uint64_t add) {
                 if (!add || __builtin_popcountll(S | add) > max_k) return;
                 scratch = pS;
-                const int sc = cS + absorb(S | add, scratch, nullptr), na = __builtin_popcountll(add);
+                const int sc = cS + count(S | add, add, scratch), na = __builtin_popcountll(add);
                 if (sc > best || (sc == best && na < best_add)) { best = sc; best_add = na; best_m = add; }
             };
             for (int b = 0; b < nq; ++b) {
-                if (((S >> b) & 1ull) || base[b] >= (int)queue[b].size()) continue;
+                const int gi = front(b, base);
+                if (((S >> b) & 1ull) || gi < 0) continue;
                 consider(1ull << b);
-                const int gi = queue[b][base[b]];
-                if (!special[gi]) consider(gm[gi] & ~S);
+                if (!special[gi] && (gm[gi] & ~S) != (1ull << b)) consider(gm[gi] & ~S);
             }
             if (best < 0) break;
             S |= best_m;
-            cS += absorb(S, pS, nullptr);
+            cS += count(S, best_m, pS);
         }
         return cS;
     };
     // (gate count, set) of the set grown from each distinct front gate
-    auto candidates = [&](const std::vector<int>& base, std::vector<std::pair<int, uint64_t>>& out) {
+    auto candidates = [&](const Pos& base, std::vector<std::pair<int, uint64_t>>& out) {
         out.clear();
         for (int b = 0; b < nq; ++b) {
             const int gi = front(b, base);
@@ -312,7 +337,7 @@ void plan_fusion_frontier(const std::vector<PendingGate>& q, int max_k, int nq,
         }
     };
     std::vector<std::pair<int, uint64_t>> cand, next;
-    std::vector<int> after(nq);
+    Pos after;
     int remaining = G;
     std::vector<int> taken;
     while (remaining > 0) {
@@ -321,15 +346,12 @@ void plan_fusion_frontier(const std::vector<PendingGate>& q, int max_k, int nq,
         for (int b = 0; b < nq && !emitted; ++b) {
             const int gi = front(b, ptr);
             if (gi < 0 || !special[gi]) continue;
-            bool ready = true;
-            for (uint64_t t = gm[gi]; t; t &= t - 1)
-                if (front(__builtin_ctzll(t), ptr) != gi) { ready = false; break; }
-            if (!ready) continue;
+            if (!ready(gi, ptr)) continue;
             Planned p;
             p.q.assign(q[gi].q, q[gi].q + q[gi].k);
             if (matrices) p.U = q[gi].U;
             p.cmask = q[gi].cmask;
-            for (uint64_t t = gm[gi]; t; t &= t - 1) ++ptr[__builtin_ctzll(t)];
+            advance(gi, ptr);
             --remaining;
             emitted = true;
             emit(std::move(p));
@@ -354,7 +376,7 @@ void plan_fusion_frontier(const std::vector<PendingGate>& q, int max_k, int nq,
             int best_total = -1;
             for (auto& [c, S] : cand) {
                 after = ptr;
-                absorb(S, after, nullptr);
+                count(S, S, after);
                 candidates(after, next);
                 int nb = 0;
                 for (auto& x : next) nb = std::max(nb, x.first);
@@ -367,7 +389,7 @@ void plan_fusion_frontier(const std::vector<PendingGate>& q, int max_k, int nq,
         }
         if (bestc <= 0) fail(QE_ERR_STATE, "fusion planner made no progress");
         taken.clear();
-        absorb(bestS, ptr, &taken);
+        absorb(bestS, ptr, taken);
         uint64_t used = 0;
         for (int gi : taken) used |= gm[gi];
         Planned p;
@@ -440,19 +462,24 @@ void complete_pending(qe_state* s) {
 }
 
 
+// Plan and launch the queued gates (no wait for the device).
+static void launch_queue(qe_state* s) {
+    std::vector<PendingGate> q;
+    q.swap(s->queue);
+    const int k = choose_fusion_width(s, q);
+    s->stats.gates += q.size();
+    plan_fusion(
+        q, k, s->n, [&](Planned&& b) { apply_block(s, (int)b.q.size(), b.q.data(), b.U, b.cmask); }, true,
+        plan_lookahead(s->n));
+}
+
 void flush(qe_state* s) {
     if (s->queue.empty()) {
         complete_pending(s);   // a tensor-core pass launched outside a flush (QFT digit passes)
         return;
     }
-    std::vector<PendingGate> q;
-    q.swap(s->queue);
-    const int k = choose_fusion_width(s, q);
-    s->stats.gates += q.size();
     try {
-        plan_fusion(
-            q, k, s->n, [&](Planned&& b) { apply_block(s, (int)b.q.size(), b.q.data(), b.U, b.cmask); }, true,
-            plan_lookahead(s->n));
+        launch_queue(s);
     } catch (...) {
         try {
             complete_pending(s);
@@ -747,6 +774,9 @@ int qe_apply_gate(qe_state* s, int k, const int* qubits, const double* matrix) {
         g.U[i] = cd(matrix[2 * i], matrix[2 * i + 1]);
     }
     s->queue.push_back(std::move(g));
+    // without fusion there is nothing to wait for: hand the gates over in small
+    // lots, so that the device works while the caller queues the next ones
+    if (s->max_k == 1 && s->queue.size() >= 16) launch_queue(s);
     QE_API_END
 }
 
