@@ -229,58 +229,82 @@ __global__ void __launch_bounds__(kFftThreads) k_fft_pass(const __grid_constant_
 // middle value Mv <= rev(Mv)); tiles X(Mv) and Y(rev Mv) hold elements
 // [b][a][w] (b: top c register bits, a: bottom c register bits, w: the lo
 // qubits below the register) and are exchanged transposed and bit-reversed.
-template <class P>
+template <class S>
 struct RevArgs {
-    typename P::S* x;
+    S* x;
     uint64_t items;
     int lo, m, c;
 };
 
 __device__ __forceinline__ uint64_t bit_rev(uint64_t v, int bits) { return bits > 0 ? (__brevll(v) >> (64 - bits)) : 0ull; }
 
-template <class P>
-__global__ void __launch_bounds__(256) k_bitrev(const __grid_constant__ RevArgs<P> a) {
-    using S = typename P::S;
+constexpr int kRevThreads = 256;
+// Tile bits: 32 KB a tile.  n = 30 complex128 9.0 -> 8.8 ms and n = 27 complex64
+// 0.73 -> 0.52 ms (0.32 for one pass) with shifts for divisions, loads in
+// batches of eight, the swizzle below and, for 8-byte elements, one bit more;
+// tiles of 64 KB measured 8.96 ms, one tile with the other in registers 8.4 ms
+// but 0.66 ms in complex64.  Rows of 512 bytes bound it: with rows of 1 KB
+// (one qubit below the register) n = 27 takes 0.89 instead of 1.11 ms.
+template <class S>
+constexpr int kRevBits = sizeof(S) == 16 ? 11 : 12;
+
+template <class S>
+__global__ void __launch_bounds__(kRevThreads) k_bitrev(const __grid_constant__ RevArgs<S> a) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    const int C = 1 << a.c, W = 1 << a.lo;
-    const int row = C * W + 1;   // odd stride in elements: conflict-free 16-byte accesses
-    S* X = reinterpret_cast<S*>(smem_raw);
-    S* Y = X + C * row;
-    const int mid_bits = a.m - 2 * a.c;
+    constexpr int kAtOnce = 8;   // independent loads in flight a thread
+    const int c = a.c, ab = c + a.lo;                 // bits of a row (a, w)
+    const uint32_t n = 1u << (c + ab), amask = (1u << ab) - 1u, wmask = (1u << a.lo) - 1u;
+    S* const X = reinterpret_cast<S*>(smem_raw);
+    S* const Y = X + n;
+    // Tile slot (row, place in the row).  The lanes that one phase of an access
+    // serves (8 of 16 bytes, 16 of 8) read the low bits of a, hence rows that
+    // differ in their top bits: those are XORed into the place, above the w bits
+    // that vary along with them.
+    constexpr int kPhase = sizeof(S) == 16 ? 3 : 4;
+    const int k = max(0, min(c, kPhase - a.lo));
+    auto slot = [&](uint32_t r, uint32_t place) { return (r << ab) | (place ^ (k ? (r >> (c - k)) << a.lo : 0u)); };
+    const int mid_bits = a.m - 2 * c;
     const uint64_t nmid = 1ull << mid_bits;
+    const int shb = a.lo + a.m - c;
     for (uint64_t item = blockIdx.x; item < a.items; item += gridDim.x) {
-        // the middle value's low and high bits vary first, so that the tiles in
-        // flight, and their partners, are neighbours in memory a few at a time
-        uint64_t mv = item & (nmid - 1ull);
-        if (mid_bits >= 8) {
-            const uint64_t h = (mv >> 4) & 15ull;
-            mv = (mv & 15ull) | ((mv >> 8) << 4) | (h << (mid_bits - 4));
-        }
+        const uint64_t mv = item & (nmid - 1ull);
         const uint64_t outer = item >> mid_bits;
         const uint64_t mr = bit_rev(mv, mid_bits);
         if (mv > mr) continue;
         const bool self = (mv == mr);
         const uint64_t obase = outer << (a.lo + a.m);
-        const uint64_t bx = obase | (mv << (a.lo + a.c));
-        const uint64_t by = obase | (mr << (a.lo + a.c));
-        const int shb = a.lo + a.m - a.c;
-        const int n = C * C * W;
-        for (int i = threadIdx.x; i < n; i += blockDim.x) {
-            const int b = i / (C * W), aw = i % (C * W);
-            const uint64_t off = ((uint64_t)b << shb) | (uint64_t)aw;
-            X[b * row + aw] = a.x[bx + off];
-            if (!self) Y[b * row + aw] = a.x[by + off];
+        S* const bx = a.x + (obase | (mv << (a.lo + c)));
+        S* const by = a.x + (obase | (mr << (a.lo + c)));
+        auto off = [&](uint32_t i) { return ((uint64_t)(i >> ab) << shb) | (i & amask); };
+        for (uint32_t i0 = threadIdx.x; i0 < n; i0 += kRevThreads * kAtOnce) {
+            S vx[kAtOnce], vy[kAtOnce];
+#pragma unroll
+            for (int u = 0; u < kAtOnce; ++u) {
+                const uint32_t i = i0 + kRevThreads * u;
+                if (i < n) {
+                    vx[u] = bx[off(i)];
+                    if (!self) vy[u] = by[off(i)];
+                }
+            }
+#pragma unroll
+            for (int u = 0; u < kAtOnce; ++u) {
+                const uint32_t i = i0 + kRevThreads * u;
+                if (i < n) {
+                    X[slot(i >> ab, i & amask)] = vx[u];
+                    if (!self) Y[slot(i >> ab, i & amask)] = vy[u];
+                }
+            }
         }
         __syncthreads();
         const S* srcX = self ? X : Y;   // destination tile X(mv) receives from Y
-        for (int i = threadIdx.x; i < n; i += blockDim.x) {
-            const int b2 = i / (C * W), aw = i % (C * W);
-            const int a2 = aw / W, w = aw % W;
-            const int rb = (int)bit_rev((uint64_t)a2, a.c);   // source b
-            const int ra = (int)bit_rev((uint64_t)b2, a.c);   // source a
-            const uint64_t off = ((uint64_t)b2 << shb) | (uint64_t)aw;
-            a.x[bx + off] = srcX[rb * row + ra * W + w];
-            if (!self) a.x[by + off] = X[rb * row + ra * W + w];
+#pragma unroll 4
+        for (uint32_t i = threadIdx.x; i < n; i += kRevThreads) {
+            const uint32_t b2 = i >> ab, a2 = (i & amask) >> a.lo, w = i & wmask;
+            const uint32_t rb = (uint32_t)bit_rev(a2, c);   // source b
+            const uint32_t ra = (uint32_t)bit_rev(b2, c);   // source a
+            const uint32_t src = slot(rb, (ra << a.lo) | w);
+            bx[off(i)] = srcX[src];
+            if (!self) by[off(i)] = X[src];
         }
         __syncthreads();
     }
@@ -427,30 +451,285 @@ void bitrev_impl(qe_state* s, int lo, int m, const char* tag = "bitrev") {
     if (m <= 1) return;
     using S = typename P::S;
     Launch L(s, tag, 2.0 * dim(s) * amp_bytes(s));
-    // end blocks of c bits (2c <= m) in tiles of 2^(2c + lo) <= 2^11
-    const int c = std::min(m / 2, std::max(0, (11 - lo) / 2));
+    // end blocks of c bits (2c <= m) in tiles of 2^(2c + lo) <= 2^kRevBits
+    const int c = std::min(m / 2, std::max(0, (kRevBits<S> - lo) / 2));
     if (lo >= 5 || c == 0) {
         // chunks of >= 32 contiguous amplitudes move as units: coalesced pair swaps
         const uint64_t count = dim(s);
         unsigned grid = (unsigned)std::min<uint64_t>((count + 255) / 256, (uint64_t)num_sms() * 8);
         k_bitrev_chunks<S><<<grid, 256, 0, s->stream>>>(reinterpret_cast<S*>(s->d), count, lo, m);
     } else {
-        static thread_local RevArgs<P> a;
+        RevArgs<S> a;
         a.x = reinterpret_cast<S*>(s->d);
         a.lo = lo;
         a.m = m;
         a.c = c;
         a.items = (1ull << (s->n - lo - m)) << (m - 2 * a.c);
-        const int C = 1 << a.c, W = 1 << lo;
-        size_t smem = sizeof(S) * 2 * (size_t)C * (C * W + 1);
-        auto fn = k_bitrev<P>;
+        const size_t smem = sizeof(S) * 2 << (2 * c + lo);
+        auto fn = k_bitrev<S>;
         QE_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
         int occ = 0;
-        QE_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fn, 256, smem));
+        QE_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fn, kRevThreads, smem));
         uint64_t grid = std::min<uint64_t>(a.items, (uint64_t)num_sms() * std::max(occ, 1));
-        fn<<<(unsigned)grid, 256, smem, s->stream>>>(a);
+        fn<<<(unsigned)grid, kRevThreads, smem, s->stream>>>(a);
     }
     QE_CUDA(cudaGetLastError());
+}
+
+// ------------------------------------------------ complex64, several passes
+// A pass over r = 5..12 register bits of a complex64 state, in tiles of 2^12
+// amplitudes: the bits in two or three groups of 2..4, each a 2^g-point
+// transform in registers whose roots are constants, a twiddle from a shared
+// table between groups, the tile in shared memory only between groups (the
+// first reads global memory, the last writes it).  The inter-pass twiddles are
+// computed: the angle k' l / 2^M is an exact 32-bit fraction of a turn, so a
+// root costs one sincospif of at most pi/4 and no table in memory; a thread's
+// 2^g outputs share one (A) and take the powers of another (B): with
+// k = 4a + b, w_k = (A B^(4a)) B^b, products of two rounded roots as a two-level
+// table gives.  What bounded the radix-2 passes that this replaces was their
+// table reads (two 32-byte sectors an amplitude): 27 qubits at n = 27 1.09 ->
+// 0.41 ms a pass (0.32 copied), with the reversal 4.10 -> 1.73 ms.
+struct Fft4Args {
+    float2* x;
+    uint64_t ntiles;
+    int L, kh;      // tile: 2^L contiguous amplitudes, kh = r (pass bits above them) or 0 (among them)
+    int g0;         // qubit of the pass's lowest bit
+    int P0;         // its tile-local place
+    int b0;         // register bits below the pass
+    int lo;
+    float scale;    // of the last pass (b0 = 0)
+};
+
+using fc = unsigned long long;   // (re, im) as packed floats
+__device__ __forceinline__ fc fc_pack(float x, float y) {
+    fc r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(x), "f"(y));
+    return r;
+}
+__device__ __forceinline__ float2 fc_unpack(fc a) {
+    float2 r;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(a));
+    return r;
+}
+__device__ __forceinline__ fc fc_add(fc a, fc b) {
+    fc r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ fc fc_sub(fc a, fc b) {
+    fc r;
+    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ fc fc_mul2(fc a, fc b) {
+    fc r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ fc fc_cmul(fc w, fc v) {
+    const float2 f = fc_unpack(w), u = fc_unpack(v);
+    const fc t = fc_mul2(fc_pack(-f.y, f.y), fc_pack(u.y, u.x));
+    fc r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(fc_pack(f.x, f.x)), "l"(v), "l"(t));
+    return r;
+}
+// exp(SIGN 2 pi i th / 2^32)
+template <int SIGN>
+__device__ __forceinline__ fc turn(uint32_t th) {
+    const uint32_t q = (th + (1u << 29)) >> 30;              // nearest quarter turn
+    const float x = (float)(int)(th - (q << 30)) * 0x1p-31f;   // what is left, in units of pi
+    float s, c;
+    sincospif(x, &s, &c);
+    const float re = (q & 1u) ? -s : c, im = (q & 1u) ? c : s;
+    const bool neg = q & 2u;
+    return fc_pack(neg ? -re : re, (neg != (SIGN < 0)) ? -im : im);
+}
+// exp(2 pi i k / 16) for k < 8
+__device__ constexpr float kCos16[8] = {1.0f, 0.92387953251128674f, 0.70710678118654752f, 0.38268343236508977f,
+                                        0.0f, -0.38268343236508977f, -0.70710678118654752f, -0.92387953251128674f};
+
+// v <- the 2^G-point transform, output l at the bit-reversed place.
+template <int G, int SIGN>
+__device__ __forceinline__ void small_dft(fc* v) {
+    constexpr int E = 1 << G;
+#pragma unroll
+    for (int h = E / 2; h >= 1; h /= 2)
+#pragma unroll
+        for (int j = 0; j < E; ++j) {
+            if (j & h) continue;
+            const fc u = v[j], x = v[j | h];
+            v[j] = fc_add(u, x);
+            const fc d = fc_sub(u, x);
+            const int k = (j & (h - 1)) * (8 / h);           // root exp(SIGN 2 pi i k / 16)
+            if (k == 0) {
+                v[j | h] = d;
+            } else if (k == 4) {
+                const float2 f = fc_unpack(d);
+                v[j | h] = SIGN > 0 ? fc_pack(-f.y, f.x) : fc_pack(f.y, -f.x);
+            } else {
+                const float sn = k < 4 ? -kCos16[k + 4] : kCos16[k - 4];     // sin(2 pi k / 16)
+                v[j | h] = fc_cmul(fc_pack(kCos16[k], SIGN > 0 ? sn : -sn), d);
+            }
+        }
+}
+__host__ __device__ constexpr int rev_bits(int v, int bits) {
+    int r = 0;
+    for (int j = 0; j < bits; ++j) r |= ((v >> j) & 1) << (bits - 1 - j);
+    return r;
+}
+// Conflict-free slot of a tile element or root (16 8-byte lanes a phase).
+__device__ __forceinline__ uint32_t slot16(uint32_t i) { return i ^ ((i >> 4) & 15u); }
+
+constexpr int kFft4Bits = 12, kFft4Threads = 256;
+
+// One group: pass bits [SLO, SLO + G) of the tile at tile0 in global memory.
+template <int R, int SLO, int G, int SIGN>
+__device__ __forceinline__ void fft4_group(const Fft4Args& a, float2* tile0, uint32_t j2_tile, fc* tile, const fc* roots) {
+    constexpr int E = 1 << G;
+    constexpr bool kFirst = SLO + G == R, kLast = SLO == 0;
+    const int sh = a.P0 + SLO;
+    const uint32_t below = (1u << sh) - 1u, lowmask = (1u << a.L) - 1u;
+#pragma unroll 1
+    for (uint32_t b = threadIdx.x; b < (1u << (kFft4Bits - G)); b += kFft4Threads) {
+        const uint32_t base = ((b & ~below) << G) | (b & below);
+        const uint64_t at = (base & lowmask) | (a.kh ? (uint64_t)(base >> a.L) << a.g0 : (uint64_t)0);
+        const uint64_t stride = 1ull << (a.g0 + SLO);
+        fc v[E];
+        if constexpr (kFirst) {
+#pragma unroll
+            for (int j = 0; j < E; ++j) v[j] = *reinterpret_cast<const fc*>(tile0 + at + j * stride);
+        } else {
+#pragma unroll
+            for (int j = 0; j < E; ++j) v[j] = tile[slot16(base | ((uint32_t)j << sh))];
+        }
+        small_dft<G, SIGN>(v);
+        const uint32_t gp = (base >> a.P0) & ((1u << R) - 1u);
+        if constexpr (!kLast) {
+            // twiddle by the pass bits below this group
+            const uint32_t low = gp & ((1u << SLO) - 1u);
+#pragma unroll
+            for (int j = 1; j < E; ++j)
+                v[j] = fc_cmul(roots[slot16((low * (uint32_t)rev_bits(j, G)) << (R - SLO - G))], v[j]);
+#pragma unroll
+            for (int j = 0; j < E; ++j) tile[slot16(base | ((uint32_t)j << sh))] = v[j];
+        } else {
+            if (a.b0 > 0) {
+                // twiddle by the register bits below the pass: j2 l / 2^(b0 + R)
+                const uint64_t j2 = j2_tile | ((((base & lowmask) & (a.kh ? ~0u : (1u << a.g0) - 1u)) >> a.lo));
+                const uint32_t rb = __brev(gp) >> (32 - R);
+                const int up = 64 - (a.b0 + R);
+                const uint32_t tA = (uint32_t)(((j2 * rb) << up) >> 32), tB = (uint32_t)(((j2 << (R - G)) << up) >> 32);
+                fc wb[4];
+#pragma unroll
+                for (int k = 1; k < 4 && k < E; ++k) wb[k] = turn<SIGN>(tB * (uint32_t)k);
+#pragma unroll
+                for (int ka = 0; ka < E / 4; ++ka) {
+                    const fc wa = turn<SIGN>(tA + tB * (uint32_t)(4 * ka));
+#pragma unroll
+                    for (int kb = 0; kb < 4; ++kb) {
+                        const int j = rev_bits(4 * ka + kb, G);
+                        v[j] = fc_cmul(kb ? fc_cmul(wa, wb[kb]) : wa, v[j]);
+                    }
+                }
+            } else {
+                const fc sc = fc_pack(a.scale, a.scale);
+#pragma unroll
+                for (int j = 0; j < E; ++j) v[j] = fc_mul2(sc, v[j]);
+            }
+            fc* const out = reinterpret_cast<fc*>(tile0 + at);
+            if (a.g0 == 0) {
+                // a thread's outputs are contiguous: 32 bytes at a time
+#pragma unroll
+                for (int j = 0; j < E; j += 4)
+                    asm volatile("st.global.v4.b64 [%0], {%1, %2, %3, %4};" ::"l"(out + j), "l"(v[j]), "l"(v[j + 1]),
+                                 "l"(v[j + 2]), "l"(v[j + 3])
+                                 : "memory");
+            } else {
+#pragma unroll
+                for (int j = 0; j < E; ++j) out[j * stride] = v[j];
+            }
+        }
+    }
+}
+
+template <int R, int SIGN>
+__global__ void __launch_bounds__(kFft4Threads, 4) k_fft4(const __grid_constant__ Fft4Args a) {
+    static_assert(R >= 5 && R <= 12, "two or three groups of 2..4 bits");
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    fc* const tile = reinterpret_cast<fc*>(smem_raw);
+    fc* const roots = tile + (1 << kFft4Bits);
+    constexpr int NG = R <= 8 ? 2 : 3;
+    constexpr int G1 = (R + NG - 1) / NG, G2 = (R - G1 + NG - 2) / (NG - 1), G3 = R - G1 - G2;   // from the top
+    for (uint32_t e = threadIdx.x; e < (1u << R); e += kFft4Threads) roots[slot16(e)] = turn<SIGN>(e << (32 - R));
+    __syncthreads();
+    for (uint64_t t = blockIdx.x; t < a.ntiles; t += gridDim.x) {
+        // the pass bits inserted as zeros above the contiguous ones
+        const uint64_t u = t << a.L;
+        const uint64_t base = a.kh ? ((u >> a.g0) << (a.g0 + R)) | (u & ((1ull << a.g0) - 1ull)) : u;
+        float2* const tile0 = a.x + base;
+        const uint32_t j2 = (uint32_t)((base >> a.lo) & ((1ull << a.b0) - 1ull));
+        fft4_group<R, R - G1, G1, SIGN>(a, tile0, j2, tile, roots);
+        __syncthreads();
+        if constexpr (NG == 3) {
+            fft4_group<R, G3, G2, SIGN>(a, tile0, j2, tile, roots);
+            __syncthreads();
+            fft4_group<R, 0, G3, SIGN>(a, tile0, j2, tile, roots);
+        } else {
+            fft4_group<R, 0, G2, SIGN>(a, tile0, j2, tile, roots);
+        }
+        __syncthreads();
+    }
+}
+
+template <int R>
+void fft4_launch(qe_state* s, const Fft4Args& a, int sign) {
+    auto fn = sign > 0 ? k_fft4<R, 1> : k_fft4<R, -1>;
+    const size_t smem = sizeof(fc) * ((size_t)(1 << kFft4Bits) + ((size_t)1 << R));
+    QE_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    int occ = 0;
+    QE_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fn, kFft4Threads, smem));
+    const uint64_t grid = std::min<uint64_t>(a.ntiles, (uint64_t)num_sms() * std::max(occ, 1));
+    Launch L(s, "fft_pass", 2.0 * dim(s) * amp_bytes(s));
+    fn<<<(unsigned)grid, kFft4Threads, smem, s->stream>>>(a);
+    QE_CUDA(cudaGetLastError());
+}
+
+// Complex64 registers of more than one pass (m > 12 - min(lo, 3), hence n >= 12).
+void fft4(qe_state* s, int lo, int m, int inverse) {
+    const int last_max = kFft4Bits - std::min(lo, 3), up_max = kFft4Bits - 3;   // runs of at least 8 amplitudes
+    const int np = 1 + (m - last_max + up_max - 1) / up_max;
+    // upper passes of 8 bits (two groups of four) where that suffices
+    const int up = std::max((m - last_max + np - 2) / (np - 1), std::min(8, m / np));
+    Fft4Args a{};
+    a.x = reinterpret_cast<float2*>(s->d);
+    a.ntiles = 1ull << (s->n - kFft4Bits);
+    a.lo = lo;
+    a.scale = (float)std::pow(2.0, -0.5 * m);
+    int top = m;
+    for (int p = 0; p < np; ++p) {
+        const int r = p + 1 < np ? up : top;
+        top -= r;
+        a.b0 = top;
+        a.g0 = lo + top;
+        // the pass bits within the lowest 12, or above 12 - r contiguous ones
+        const bool low = a.g0 + r <= kFft4Bits;
+        a.L = low ? kFft4Bits : kFft4Bits - r;
+        a.kh = low ? 0 : r;
+        a.P0 = low ? a.g0 : a.L;
+        const int sign = inverse ? -1 : 1;
+        switch (r) {
+            case 5: fft4_launch<5>(s, a, sign); break;
+            case 6: fft4_launch<6>(s, a, sign); break;
+            case 7: fft4_launch<7>(s, a, sign); break;
+            case 8: fft4_launch<8>(s, a, sign); break;
+            case 9: fft4_launch<9>(s, a, sign); break;
+            case 10: fft4_launch<10>(s, a, sign); break;
+            case 11: fft4_launch<11>(s, a, sign); break;
+            case 12: fft4_launch<12>(s, a, sign); break;
+            default: fail(QE_ERR_ARG, "no FFT pass plan");
+        }
+    }
+    launch_bitrev(s, lo, m);
 }
 
 // ------------------------------------------------ tensor-core digit passes
@@ -614,7 +893,8 @@ void launch_qft_fft(qe_state* s, int lo, int m, int inverse) {
         qft_tc(s, lo, m, inverse);
         return;
     }
-    if (s->dtype == QE_C64) fft_impl<F32>(s, lo, m, inverse, 0);
+    if (s->dtype == QE_C64 && m > kFft4Bits - std::min(lo, 3)) fft4(s, lo, m, inverse);
+    else if (s->dtype == QE_C64) fft_impl<F32>(s, lo, m, inverse, 0);
     else if (s->arith == QE_ARITH_FP64) fft_impl<F64>(s, lo, m, inverse, 1);
     else fft_impl<DF>(s, lo, m, inverse, 2);
 }
