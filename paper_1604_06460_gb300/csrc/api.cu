@@ -699,6 +699,7 @@ int qe_free_state(qe_state* s) {
     if (s->owned && s->d) cudaFree(s->d);
     if (s->scratch) cudaFree(s->scratch);
     if (s->oz_ws) cudaFree(s->oz_ws);
+    if (s->powers) cudaFree(s->powers);
     if (s->status_host) cudaFreeHost(s->status_host);
     profile_clear(s);
     for (auto e : s->event_pool) cudaEventDestroy(e);
@@ -914,6 +915,7 @@ int qe_matmul(qe_state* c, qe_state* a, qe_state* b) {
     if (a->stream != c->stream) QE_CUDA(cudaStreamSynchronize(a->stream));
     if (b->stream != c->stream && b->stream != a->stream) QE_CUDA(cudaStreamSynchronize(b->stream));
     launch_matmul(c, c->d, a->d, b->d, k);
+    complete_pending(c);
     QE_API_END
 }
 
@@ -935,10 +937,31 @@ int qe_qpe_emulate(qe_state* s, int nsys, int b, qe_state* u) {
         apply_block(s, 1, &q, H, 0);
     }
     // ancilla j controls U^(2^j): the powers by repeated squaring in two
-    // temporary matrices
+    // temporary matrices, kept with the state up to kKeptPowers bytes
+    // (allocating and freeing them took 0.3 ms a call) and allocated for the
+    // call above that
+    constexpr size_t kKeptPowers = 64u << 20;
     const size_t mbytes = (size_t)16 << (2 * nsys);
     void* tmp[2] = {nullptr, nullptr};
-    if (b > 1) {
+    const bool kept = 2 * mbytes <= kKeptPowers;
+    if (b > 1 && kept) {
+        if (s->powers_bytes < 2 * mbytes) {
+            if (s->powers) {
+                QE_CUDA(cudaStreamSynchronize(s->stream));
+                QE_CUDA(cudaFree(s->powers));
+                s->powers = nullptr;
+                s->powers_bytes = 0;
+            }
+            if (cudaMalloc(&s->powers, 2 * mbytes) != cudaSuccess) {
+                cudaGetLastError();
+                s->powers = nullptr;
+                fail(QE_ERR_OOM, "no room for the matrix powers");
+            }
+            s->powers_bytes = 2 * mbytes;
+        }
+        tmp[0] = s->powers;
+        tmp[1] = (char*)s->powers + mbytes;
+    } else if (b > 1) {
         for (auto& t : tmp) {
             cudaError_t e = cudaMalloc(&t, mbytes);
             if (e != cudaSuccess) {
@@ -948,26 +971,32 @@ int qe_qpe_emulate(qe_state* s, int nsys, int b, qe_state* u) {
             }
         }
     }
+    auto release = [&] {
+        for (auto t : tmp)
+            if (t && !kept) cudaFree(t);
+    };
     try {
         const void* cur = u->d;
+        const int64_t D = 1ll << nsys, rows = 1ll << (s->n - nsys - 1);
+        if (s->tensor_cores && nsys >= 6 && oz_gemm_available(D, D, D)) oz_zgemm_reserve(s, std::max(D, rows), D, D);
         for (int j = 0; j < b; ++j) {
-            launch_dense_controlled(s, cur, nsys, nsys + j);
+            // the controlled product leaves cur's digits for the squaring
+            const bool split = launch_dense_controlled(s, cur, nsys, nsys + j);
             if (j + 1 < b) {
                 void* next = tmp[j & 1];
-                launch_matmul(s, next, cur, cur, nsys);
+                launch_matmul(s, next, cur, cur, nsys, split);
                 cur = next;
             }
         }
         launch_qft_fft(s, nsys, b, 1);
+        complete_pending(s);
         QE_CUDA(cudaStreamSynchronize(s->stream));
     } catch (...) {
         cudaStreamSynchronize(s->stream);
-        for (auto t : tmp)
-            if (t) cudaFree(t);
+        release();
         throw;
     }
-    for (auto t : tmp)
-        if (t) cudaFree(t);
+    release();
     QE_API_END
 }
 

@@ -21,10 +21,10 @@
 //
 // Product kernel: one CTA per output tile of 128 rows x 16 complex columns,
 // warp-specialised like the gate kernel.  One thread copies each K-stage's
-// (32 values) seven A and seven Bt digit blocks (56 + 14 KB, two stage
+// (32 values) seven A and seven Bt digit blocks (56 + 14 KB, three stage
 // buffers, 64-byte swizzle) with the bulk-copy engine (cp.async.bulk,
 // completion counted in bytes on the buffer's mbarrier), so the copy of a
-// stage overlaps the MMAs of the previous one; one thread issues the 34 digit
+// stage overlaps the MMAs of the previous ones; one thread issues the 34 digit
 // pairs with i + j <= 9 as 8 MMAs per K-step (the Bt digit slices stacked
 // along N, as the gate kernel stacks W's) into one of two tensor-memory
 // accumulator sets (8 accumulators x 32 columns each; a set sums one chunk of
@@ -66,7 +66,10 @@ constexpr int kThreads = 32 * (kLoadWarp + 1);   // 576
 constexpr int kRecThreads = 32 * kRecWarps;
 constexpr uint32_t kStageBytes = kD * (kASlice + kBSlice);   // bulk-copied per stage (70 KB)
 constexpr int kFlushExp = 100;              // biased exponent below which a row is flushed
-constexpr size_t kSmem = 1024 + 2 * (size_t)kStageBytes;      // two stage buffers
+// Stage buffers: a stage's copies take about 1.3 us to arrive and its MMAs half
+// a microsecond, so three in flight (two: 0.346 against 0.293 ms at 1024^3).
+constexpr int kStages = 3;
+constexpr size_t kSmem = 1024 + kStages * (size_t)kStageBytes;
 static_assert(kSmem <= 227 * 1024, "shared memory per CTA");
 
 // ------------------------------------------------------------- splitting
@@ -161,36 +164,55 @@ __global__ void __launch_bounds__(256) k_split_a(const double2* __restrict__ src
     if (threadIdx.x == 0) escale[r] = (int)em - 1021;
 }
 
-// One CTA per tile of 16 complex columns c of B (K x N, row-major): the Bt
-// rows of column c are [Re B[:,c] ; -Im B[:,c]] (real part of C) and
-// [Im B[:,c] ; Re B[:,c]] (imaginary part).  Digits are written through a
-// shared-memory transpose of 32-row blocks of B.
-__global__ void __launch_bounds__(256) k_split_b(const double2* __restrict__ src, int64_t K, int64_t ldb,
-                                                 uint32_t* __restrict__ dig, int* __restrict__ fscale, int64_t Nr) {
-    __shared__ double2 blk[32][17];
+constexpr int kSplitK = 64;   // rows of B a CTA of the two kernels below takes
+
+// Largest biased exponent of every complex column of B (K x N, row-major), into
+// zeroed cmax[N]: one CTA per 16 columns and kSplitK rows.
+__global__ void __launch_bounds__(256) k_colmax(const double2* __restrict__ src, int64_t K, int64_t ldb,
+                                                uint32_t* __restrict__ cmax) {
     __shared__ uint32_t colmax[16][17];
-    __shared__ uint32_t base[16];
-    const int tid = threadIdx.x;
-    const int64_t c0 = (int64_t)blockIdx.x * 16;
-    const int ci = tid & 15, kr = tid >> 4;
+    const int ci = threadIdx.x & 15, kr = threadIdx.x >> 4;
+    const int64_t c0 = (int64_t)blockIdx.x * 16, k0 = (int64_t)blockIdx.y * kSplitK;
     uint32_t em = 0;
-    for (int64_t k = kr; k < K; k += 16) {
-        const double2 v = src[k * ldb + c0 + ci];
-        em = max(em, max(biased_exp(v.x), biased_exp(v.y)));
-    }
+#pragma unroll
+    for (int k = 0; k < kSplitK; k += 16)
+        if (k0 + k + kr < K) {
+            const double2 v = src[(k0 + k + kr) * ldb + c0 + ci];
+            em = max(em, max(biased_exp(v.x), biased_exp(v.y)));
+        }
     colmax[ci][kr] = em;
     __syncthreads();
-    if (tid < 16) {
+    if (threadIdx.x < 16) {
         uint32_t m = 0;
-        for (int j = 0; j < 16; ++j) m = max(m, colmax[tid][j]);
-        base[tid] = m < (uint32_t)kFlushExp ? 0x10000u : m;
-        fscale[32 * blockIdx.x + tid] = (int)m - 1021;
-        fscale[32 * blockIdx.x + 16 + tid] = (int)m - 1021;
+        for (int j = 0; j < 16; ++j) m = max(m, colmax[threadIdx.x][j]);
+        if (m) atomicMax(&cmax[c0 + threadIdx.x], m);
     }
-    __syncthreads();
+}
+
+// The Bt rows of complex column c are [Re B[:,c] ; -Im B[:,c]] (real part of C)
+// and [Im B[:,c] ; Re B[:,c]] (imaginary part).  One CTA per tile of 16 columns
+// and kSplitK rows of B (a CTA per tile and all K, with the column maxima found
+// first, left most SMs idle: 68 us at 1024 x 1024 against 26 us for both
+// kernels).  Digits are written through a shared-memory transpose of 32-row
+// blocks of B.
+__global__ void __launch_bounds__(256) k_split_b(const double2* __restrict__ src, int64_t K, int64_t ldb,
+                                                 const uint32_t* __restrict__ cmax, uint32_t* __restrict__ dig,
+                                                 int* __restrict__ fscale, int64_t Nr) {
+    __shared__ double2 blk[32][17];
+    __shared__ uint32_t base[16];
+    const int tid = threadIdx.x;
+    const int64_t c0 = (int64_t)blockIdx.x * 16, kb = (int64_t)blockIdx.y * kSplitK;
+    if (tid < 16) {
+        const uint32_t m = cmax[c0 + tid];
+        base[tid] = m < (uint32_t)kFlushExp ? 0x10000u : m;
+        if (blockIdx.y == 0) {
+            fscale[32 * blockIdx.x + tid] = (int)m - 1021;
+            fscale[32 * blockIdx.x + 16 + tid] = (int)m - 1021;
+        }
+    }
     const int64_t nt = Nr / kTN, nc = 2 * K / kKS;
     const int q = tid & 15;    // pair within a 32-value segment
-    for (int64_t k0 = 0; k0 < K; k0 += 32) {
+    for (int64_t k0 = kb; k0 < min(K, kb + kSplitK); k0 += 32) {
         for (int e = tid; e < 32 * 16; e += 256) blk[e >> 4][e & 15] = src[(k0 + (e >> 4)) * ldb + c0 + (e & 15)];
         __syncthreads();
         // segments g = (row rho of the tile, half hf of the K range)
@@ -224,7 +246,7 @@ struct GemmOzArgs {
     long long spin_limit;
 };
 
-enum GBar { kReady0, kReady1, kOpFree0, kOpFree1, kFull0, kFull1, kFree0, kFree1, kDrain, kGBars };
+enum GBar { kReady0, kOpFree0 = kReady0 + kStages, kFull0 = kOpFree0 + kStages, kFull1, kFree0, kFree1, kDrain, kGBars };
 
 __device__ __forceinline__ double i128_to_double(long long hi, unsigned long long lo) {
     if ((hi == 0 && (long long)lo >= 0) || (hi == -1 && (long long)lo < 0)) return __ll2double_rn((long long)lo);
@@ -234,7 +256,7 @@ __device__ __forceinline__ double i128_to_double(long long hi, unsigned long lon
 __global__ void __launch_bounds__(kThreads, 1) k_oz_zgemm(const __grid_constant__ GemmOzArgs a) {
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     unsigned char* base = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
-    // stage buffer b (0, 1): 7 digit planes of the A tile, then the 7 of the
+    // stage buffer b: 7 digit planes of the A tile, then the 7 of the
     // Bt tile stacked (row j * 32 + r of the stacked operand)
     auto stageA = [&](int b) { return base + (size_t)b * kStageBytes; };
     auto stageB = [&](int b) { return base + (size_t)b * kStageBytes + kD * kASlice; };
@@ -244,8 +266,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_oz_zgemm(const __grid_constant_
     const int64_t row0 = (int64_t)blockIdx.y * kTM, brow0 = (int64_t)blockIdx.x * kTN;
     const int nchunks = (int)(a.Kr / kKC), nstages = (int)(a.Kr / kKS);
     if (tid == 0) {
-        const uint32_t counts[kGBars] = {1, 1, 1, 1, 1, 1, kRecThreads, kRecThreads, 1};
-        for (int b = 0; b < kGBars; ++b) mbar_init_count(&bars[b], counts[b]);
+        for (int b = 0; b < kGBars; ++b) mbar_init_count(&bars[b], b == kFree0 || b == kFree1 ? kRecThreads : 1);
         abort_flag = 0u;
         asm volatile("fence.mbarrier_init.release.cluster;");
     }
@@ -258,29 +279,26 @@ __global__ void __launch_bounds__(kThreads, 1) k_oz_zgemm(const __grid_constant_
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;");
     const uint32_t tmem = tmem_base;
-    auto wait = [&](GBar b, uint32_t ph) {
+    auto wait = [&](int b, uint32_t ph) {
         const bool ok = wait_or_abort(smem_u32(&bars[b]), ph, a.spin_limit, &abort_flag);
         if (__any_sync(0xFFFFFFFFu, !ok)) {
-            if (!ok) atomicExch(a.status, 1u);
+            if (!ok) tc::raise_status(a.status);
             return false;
         }
         return true;
     };
     if (warp == kMmaWarp) {
         // ---------------------------------------------------- MMA issuer
-        // stage s (32 values of K) from buffer s & 1 into set (s >> 1) & 1;
+        // stage s (32 values of K) from buffer s mod kStages into set (s >> 1) & 1;
         // a set holds one chunk of 64 values (two stages), then is recombined
-        if (lane == 0) {
+        // (all lanes compute the operands, one elected lane issues)
+        {
             constexpr MmaTable<kD> tab;
-            bool ok = true;
-            for (int st = 0; st < nstages && ok; ++st) {
-                const int buf = st & 1, c = st >> 1, set = c & 1;
-                ok = wait_or_abort(smem_u32(&bars[buf ? kReady1 : kReady0]), (uint32_t)(st >> 1) & 1u, a.spin_limit,
-                                   &abort_flag);
-                if (ok && (st & 1) == 0 && c >= 2)
-                    ok = wait_or_abort(smem_u32(&bars[set ? kFree1 : kFree0]), (uint32_t)((c >> 1) - 1) & 1u,
-                                       a.spin_limit, &abort_flag);
-                if (!ok) break;
+            const uint32_t elected = elect_lane();
+            for (int st = 0; st < nstages; ++st) {
+                const int buf = st % kStages, c = st >> 1, set = c & 1;
+                if (!wait(kReady0 + buf, (uint32_t)(st / kStages) & 1u)) break;
+                if ((st & 1) == 0 && c >= 2 && !wait(set ? kFree1 : kFree0, (uint32_t)((c >> 1) - 1) & 1u)) break;
                 asm volatile("tcgen05.fence::after_thread_sync;");
                 const uint32_t dset = tmem + (uint32_t)set * kSetCols;
                 const uint64_t da0 = sdesc_sw64(smem_u32(stageA(buf))), db0 = sdesc_sw64(smem_u32(stageB(buf)));
@@ -292,35 +310,34 @@ __global__ void __launch_bounds__(kThreads, 1) k_oz_zgemm(const __grid_constant_
                         const uint32_t nn = (uint32_t)(j1 - j0 + 1) * kTN;
                         const uint64_t da = da0 + (((uint32_t)(i - 1) * kASlice + 32u * ks) >> 4);
                         const uint64_t db = db0 + (((uint32_t)(j0 - 1) * kBSlice + 32u * ks) >> 4);
-                        mma_f16(dset + (uint32_t)(i + j0 - 2) * kTN, da, db, tc::idesc(0u, nn, kTM),
-                                ((st & 1) || ks > 0 || m > 1) ? 1u : 0u);
+                        mma_f16_elected(elected, dset + (uint32_t)(i + j0 - 2) * kTN, da, db, tc::idesc(0u, nn, kTM),
+                                        ((st & 1) || ks > 0 || m > 1) ? 1u : 0u);
                     }
                 }
-                tc::mma_commit(&bars[buf ? kOpFree1 : kOpFree0]);
-                if (st & 1) tc::mma_commit(&bars[set ? kFull1 : kFull0]);
+                mma_commit_elected(elected, &bars[kOpFree0 + buf]);
+                if (st & 1) mma_commit_elected(elected, &bars[set ? kFull1 : kFull0]);
             }
-            if (!ok) atomicExch(a.status, 1u);
-            tc::mma_commit(&bars[kDrain]);
-            if (!tc::mbar_wait(smem_u32(&bars[kDrain]), 0u, a.spin_limit)) atomicExch(a.status, 1u);
+            mma_commit_elected(elected, &bars[kDrain]);
         }
+        if (lane == 0 && !tc::mbar_wait(smem_u32(&bars[kDrain]), 0u, a.spin_limit)) tc::raise_status(a.status);
         __syncwarp();
     } else if (warp == kLoadWarp) {
         // ------------------------------------------------------- loads
-        // one thread: stage s into buffer s & 1 once that buffer's previous
-        // stage (s - 2) has been consumed by its MMAs: the byte count on the
+        // one thread: stage s into its buffer once that buffer's previous
+        // stage (s - kStages) has been consumed by its MMAs: the byte count on the
         // buffer's ready barrier and 14 bulk copies
         if (lane == 0) {
             const int64_t ntA = a.Mp / kTM, ntB = a.Nr / kTN;
             const char* ga = reinterpret_cast<const char*>(a.adig);
             const char* gb = reinterpret_cast<const char*>(a.bdig);
             for (int st = 0; st < nstages; ++st) {
-                const int buf = st & 1;
-                if (st >= 2 && !wait_or_abort(smem_u32(&bars[buf ? kOpFree1 : kOpFree0]), (uint32_t)((st >> 1) - 1) & 1u,
-                                              a.spin_limit, &abort_flag)) {
-                    atomicExch(a.status, 1u);
+                const int buf = st % kStages;
+                if (st >= kStages && !wait_or_abort(smem_u32(&bars[kOpFree0 + buf]), (uint32_t)(st / kStages - 1) & 1u,
+                                                    a.spin_limit, &abort_flag)) {
+                    tc::raise_status(a.status);
                     break;
                 }
-                uint64_t* rb = &bars[buf ? kReady1 : kReady0];
+                uint64_t* rb = &bars[kReady0 + buf];
                 mbar_expect_tx(rb, kStageBytes);
 #pragma unroll 1
                 for (int i = 0; i < kD; ++i) {
@@ -405,19 +422,19 @@ struct Workspace {
     uint16_t* bdig;
     int* ea;
     int* fb;
-    uint32_t* status;
+    uint32_t* cmax;
 };
 
 Workspace workspace(qe_state* s, int64_t Mp, int64_t Nr, int64_t Kr) {
     const size_t abytes = (size_t)kD * Mp * Kr * 2, bbytes = (size_t)kD * Nr * Kr * 2;
-    const size_t need = abytes + bbytes + (size_t)(Mp + Nr) * 4 + 256;
+    const size_t need = abytes + bbytes + (size_t)(Mp + Nr + Nr / 2) * 4;
     char* p = (char*)ensure_oz_workspace(s, need);
     Workspace w;
-    w.adig = (uint16_t*)p;
-    w.bdig = (uint16_t*)(p + abytes);
-    w.ea = (int*)(p + abytes + bbytes);
-    w.fb = w.ea + Mp;
-    w.status = (uint32_t*)(p + ((abytes + bbytes + (size_t)(Mp + Nr) * 4 + 255) & ~(size_t)255));
+    w.bdig = (uint16_t*)p;       // B's part first: its place does not depend on A's size
+    w.fb = (int*)(p + bbytes);
+    w.cmax = (uint32_t*)(w.fb + Nr);
+    w.adig = (uint16_t*)(w.cmax + Nr / 2);
+    w.ea = (int*)((char*)w.adig + abytes);
     return w;
 }
 
@@ -429,10 +446,17 @@ bool oz_gemm_available(int64_t M, int64_t K, int64_t N) {
     return M >= 1 && K >= 32 && K % 32 == 0 && N >= 16 && N % 16 == 0;
 }
 
+void oz_zgemm_reserve(qe_state* s, int64_t M, int64_t K, int64_t N) {
+    workspace(s, (M + kTM - 1) / kTM * kTM, 2 * N, 2 * K);
+}
+
 // C (M x N complex, row-major, ldc) = A (M x K, rows through the optional
-// inserted row bit) B (K x N, row-major, ldb); enqueued on s's stream.
+// inserted row bit) B (K x N, row-major, ldb); enqueued on s's stream (the
+// caller ends with complete_pending).  same_b: s's last product had this very B,
+// unchanged since, in a workspace reserved for the larger of the two, so B's
+// digits are in place.
 void oz_zgemm(qe_state* s, double2* C, int64_t ldc, const double2* A, int64_t M, int64_t K, int64_t lda, int a_rowbit,
-              const double2* B, int64_t N, int64_t ldb) {
+              const double2* B, int64_t N, int64_t ldb, bool same_b) {
     if (!oz_gemm_available(M, K, N)) fail(QE_ERR_UNSUPPORTED, "matrix shape not supported by the tensor-core product");
     const int64_t Mp = (M + kTM - 1) / kTM * kTM, Kr = 2 * K, Nr = 2 * N;
     const Workspace w = workspace(s, Mp, Nr, Kr);
@@ -443,9 +467,12 @@ void oz_zgemm(qe_state* s, double2* C, int64_t ldc, const double2* A, int64_t M,
                                                        Mp);
         QE_CUDA(cudaGetLastError());
     }
-    {
+    if (!same_b) {
         Launch L(s, "oz_split_b", (double)K * N * 16.0, false);
-        k_split_b<<<(unsigned)(N / 16), 256, 0, s->stream>>>(B, K, ldb, reinterpret_cast<uint32_t*>(w.bdig), w.fb, Nr);
+        const dim3 grid((unsigned)(N / 16), (unsigned)((K + kSplitK - 1) / kSplitK));
+        QE_CUDA(cudaMemsetAsync(w.cmax, 0, (size_t)N * 4, s->stream));
+        k_colmax<<<grid, 256, 0, s->stream>>>(B, K, ldb, w.cmax);
+        k_split_b<<<grid, 256, 0, s->stream>>>(B, K, ldb, w.cmax, reinterpret_cast<uint32_t*>(w.bdig), w.fb, Nr);
         QE_CUDA(cudaGetLastError());
     }
     GemmOzArgs g;
@@ -459,19 +486,14 @@ void oz_zgemm(qe_state* s, double2* C, int64_t ldc, const double2* A, int64_t M,
     g.Nr = Nr;
     g.Kr = Kr;
     g.ldc = ldc;
-    g.status = w.status;
+    g.status = status_word(s);
     g.spin_limit = 1ll << 21;   // polls of up to 1 us each
-    QE_CUDA(cudaMemsetAsync(w.status, 0, sizeof(uint32_t), s->stream));
     QE_CUDA(cudaFuncSetAttribute(k_oz_zgemm, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmem));
     {
         Launch L(s, "oz_zgemm", (double)(M * K + K * N + M * N) * 16.0, false);
         k_oz_zgemm<<<dim3((unsigned)(Nr / kTN), (unsigned)(Mp / kTM)), kThreads, kSmem, s->stream>>>(g);
         QE_CUDA(cudaGetLastError());
     }
-    uint32_t st = 0;
-    QE_CUDA(cudaMemcpyAsync(&st, w.status, sizeof(uint32_t), cudaMemcpyDeviceToHost, s->stream));
-    QE_CUDA(cudaStreamSynchronize(s->stream));
-    if (st != 0) fail(QE_ERR_TIMEOUT, "a tensor-core matrix product wait ran out");
 }
 
 }  // namespace qe

@@ -64,6 +64,9 @@ struct qe_state {
     // digit planes of the tensor-core matrix product, grown on demand
     void* oz_ws = nullptr;
     size_t oz_ws_bytes = 0;
+    // the two matrix powers of phase estimation (at most 64 MB in all)
+    void* powers = nullptr;
+    size_t powers_bytes = 0;
     // pinned host mirror of small results
     double* host_result = nullptr;
     qe::Stats stats;
@@ -112,8 +115,9 @@ void* ensure_oz_workspace(qe_state* s, size_t bytes);
 // false from the first when the shape is not supported (K a multiple of 32, N
 // of 16) or QE_GEMM_F64=1 asks for the FP64 kernel
 bool oz_gemm_available(int64_t M, int64_t K, int64_t N);
+void oz_zgemm_reserve(qe_state* s, int64_t M, int64_t K, int64_t N);   // workspace for products up to this size
 void oz_zgemm(qe_state* s, double2* C, int64_t ldc, const double2* A, int64_t M, int64_t K, int64_t lda, int a_rowbit,
-              const double2* B, int64_t N, int64_t ldb);
+              const double2* B, int64_t N, int64_t ldb, bool same_b = false);
 
 // ---- kernels (each launcher enqueues on s->stream and updates s->stats)
 void launch_init_basis(qe_state* s, uint64_t index);
@@ -180,8 +184,9 @@ void reduce_probs_device(qe_state* s, int m, const int* qubits, double2* partial
 // column-major complex products (FP64), a dense matrix applied to the system
 // register [0, nsys) of the rows whose qubit ctrl is set
 void launch_init_identity(qe_state* s, int nsys);
-void launch_matmul(qe_state* acct, void* c, const void* a, const void* b, int k);
-void launch_dense_controlled(qe_state* s, const void* mat, int nsys, int ctrl);
+void launch_matmul(qe_state* acct, void* c, const void* a, const void* b, int k, bool same_b = false);
+// (whether that ran on the tensor cores: mat's digits are then in s's workspace)
+bool launch_dense_controlled(qe_state* s, const void* mat, int nsys, int ctrl);
 
 // measurement (Sec. II): inverse-CDF sampling with caller-given uniforms, and
 // the collapse onto an outcome

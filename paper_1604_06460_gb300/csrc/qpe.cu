@@ -124,12 +124,12 @@ void launch_init_identity(qe_state* s, int nsys) {
 // c = a b for 2^k x 2^k matrices stored column-major (entry (i, j) at
 // (j << k) | i): as row-major arrays they are the transposes, and
 // C^T = B^T A^T.  Enqueued on acct's stream, counted in its statistics.
-void launch_matmul(qe_state* acct, void* c, const void* a, const void* b, int k) {
+void launch_matmul(qe_state* acct, void* c, const void* a, const void* b, int k, bool same_b) {
     const int64_t D = 1ll << k;
     if (acct->tensor_cores && k >= 6 && oz_gemm_available(D, D, D)) {
         // on the tensor cores: exact digit products, 128-bit sums
         oz_zgemm(acct, reinterpret_cast<double2*>(c), D, reinterpret_cast<const double2*>(b), D, D, D, -1,
-                 reinterpret_cast<const double2*>(a), D, D);
+                 reinterpret_cast<const double2*>(a), D, D, same_b);
         return;
     }
     GemmArgs g{};
@@ -144,13 +144,15 @@ void launch_matmul(qe_state* acct, void* c, const void* a, const void* b, int k)
 
 // The rows of s (system register [0, nsys)) whose qubit ctrl is set times
 // M^T: psi_row <- M psi_row.  M is held column-major in mat (2 nsys qubits),
-// i.e. mat's amplitudes read row-major are M^T.  On the tensor cores from 128
-// rows and nsys >= 6, else FP64 fused multiply-adds.
-void launch_dense_controlled(qe_state* s, const void* mat, int nsys, int ctrl) {
+// i.e. mat's amplitudes read row-major are M^T.  On the tensor cores from
+// nsys = 6 on, else FP64 fused multiply-adds (few rows leave the FP64 kernel's
+// tiles and most SMs empty: 8 rows, nsys = 11, 8.3 ms against 0.1).
+bool launch_dense_controlled(qe_state* s, const void* mat, int nsys, int ctrl) {
     const int64_t D = 1ll << nsys;
     const uint64_t rows = 1ull << (s->n - nsys - 1);
     double2* scr = reinterpret_cast<double2*>(ensure_scratch(s, (size_t)(rows << nsys) * sizeof(double2)));
-    if (s->tensor_cores && nsys >= 6 && rows >= 128 && oz_gemm_available((int64_t)rows, D, D)) {
+    const bool tc = s->tensor_cores && nsys >= 6 && oz_gemm_available((int64_t)rows, D, D);
+    if (tc) {
         // on the tensor cores (rows padded to 128 inside the product)
         oz_zgemm(s, scr, D, reinterpret_cast<const double2*>(s->d), (int64_t)rows, D, D, ctrl - nsys,
                  reinterpret_cast<const double2*>(mat), D, D);
@@ -170,6 +172,7 @@ void launch_dense_controlled(qe_state* s, const void* mat, int nsys, int ctrl) {
     Launch L(s, "copy_rows", 2.0 * (double)total * 16.0, false);
     k_copy_rows<<<grid, 256, 0, s->stream>>>(reinterpret_cast<double2*>(s->d), scr, rows, nsys, ctrl - nsys);
     QE_CUDA(cudaGetLastError());
+    return tc;
 }
 
 }  // namespace qe
