@@ -458,7 +458,7 @@ void complete_pending(qe_state* s) {
     QE_CUDA(cudaStreamSynchronize(s->stream));
     const uint32_t st = *(volatile uint32_t*)s->status_host;
     *s->status_host = 0u;
-    if (st) fail(QE_ERR_TIMEOUT, "tensor-core gate: an mbarrier wait exceeded its limit");
+    if (st) fail(QE_ERR_TIMEOUT, "a kernel's bounded wait exceeded its limit");
 }
 
 

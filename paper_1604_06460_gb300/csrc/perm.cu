@@ -8,7 +8,7 @@
 // rotation by c of 2^m entries, which splits into g = gcd(c, 2^m) cycles of
 // length 2^m / g.  In-place strategies:
 //   bulk    - register [lo, lo+m), lo < 5, whose slice of 2^(lo+m) contiguous
-//             amplitudes fits one CTA's (or a cluster of eight CTAs')
+//             amplitudes fits one CTA's (or a cluster of 8 or 16 CTAs')
 //             shared memory, with 16-byte-aligned rotation runs: each CTA
 //             bulk-copies its contiguous part of the slice in, waits at the
 //             cluster barrier until every part is held, and bulk-copies it
@@ -18,6 +18,17 @@
 //   cluster - slices up to 8x larger in that case: eight CTAs of a
 //             thread-block cluster each stage 1/8 of the slice and read the
 //             rotated source from the owner's shared memory;
+//   split   - larger registers from a qubit lo with runs of 2^lo amplitudes
+//             below 64 bytes, states of at least 256 MB: with k
+//             slice bits and s = c 2^lo mod 2^k, first the rotation of every
+//             slice of 2^k by s, then the upper register bits plus the rest of
+//             c, plus the carry where the place in the slice is now below s:
+//             walks over columns that are contiguous runs.  20 qubits at n = 29,
+//             the walk below (whose warps read 2^lo neighbours at a time) against
+//             the split: complex128 lo = 0 35.2 -> 5.6 ms, lo = 1 13.4 -> 5.5, but
+//             lo = 2 6.0 (mean) and 5.8, lo = 3 3.1 and 5.7; complex64 lo = 0, 1, 2
+//             32.6, 14.8, 5.9 -> 3.1, lo = 3 2.9 and 3.3.  Smaller states sit in
+//             the cache: 64 MB, lo = 1, 0.050 and 0.072;
 //   walk    - otherwise every thread follows one cycle of one column,
 //             prefetching several positions ahead (coalesced when the
 //             lowest non-register qubits vary across the warp).
@@ -39,7 +50,9 @@ namespace {
 template <class S>
 struct WalkArgs {
     S* x;
-    uint64_t columns;     // 2^(n-m)
+    uint64_t columns;     // columns walked: all 2^(n-m), or those whose low kb bits lie in [off0, off0 + len)
+    uint64_t off0, len;
+    int kb;
     uint64_t g;           // cycles per column: gcd(c, 2^m)
     uint64_t nseg;        // segments per cycle
     uint64_t seg_len;     // cycle positions per segment
@@ -71,7 +84,8 @@ __device__ __forceinline__ uint64_t reg_deposit(const WalkArgs<S>& a, uint64_t r
 template <class S>
 __device__ __forceinline__ void walk_item(const WalkArgs<S>& a, uint64_t t, uint64_t& x0,
                                           uint64_t& start, uint64_t& seg) {
-    const uint64_t col = t % a.columns;
+    const uint64_t ci = t % a.columns;
+    const uint64_t col = ((ci / a.len) << a.kb) | (a.off0 + ci % a.len);
     const uint64_t rest = t / a.columns;
     start = rest % a.g;
     seg = rest / a.g;
@@ -166,15 +180,12 @@ __global__ void __launch_bounds__(512) k_add_cluster(S* __restrict__ x, int Sbit
     cl.sync();
 }
 
-// Status of the bulk path: set when a wait for a CTA's incoming copy ran out.
-__device__ uint32_t g_add_status;
-
 // One CTA (nblk = 1) or one cluster of nblk CTAs per slice of 2^S amplitudes;
 // CTA `rank` holds the contiguous part [rank E, rank E + E), E = 2^S / nblk,
 // and writes it back rotated by `shift` within the slice.
 template <class S>
 __global__ void __launch_bounds__(32) k_add_bulk(S* __restrict__ x, int Sbits, uint32_t shift, long long limit,
-                                                 int stall_test) {
+                                                 int stall_test, uint32_t* status) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ __align__(8) uint64_t bar;
     __shared__ uint32_t abort_flag;
@@ -213,9 +224,100 @@ __global__ void __launch_bounds__(32) k_add_bulk(S* __restrict__ x, int Sbits, u
         for (uint32_t off = 0; off < rest; off += kPiece)
             oz::bulk_s2g(dst1 + off, sm + rest0 + off, min(kPiece, rest - off));
         oz::bulk_commit();
-        oz::bulk_wait_all();
+        oz::bulk_wait_read();   // the shared memory may go; the writes are complete when the kernel is
     }
-    if (!ok && threadIdx.x == 0) atomicExch(&g_add_status, 1u);
+    if (!ok && threadIdx.x == 0) tc::raise_status(status);
+}
+
+// Cycles of a register of m qubits advanced by c != 0 mod 2^m.
+template <class S>
+WalkArgs<S> walk_args(qe_state* s, int m, const int* qubits, uint64_t c, bool contiguous) {
+    WalkArgs<S> a;
+    a.x = reinterpret_cast<S*>(s->d);
+    a.m = m;
+    a.c = c;
+    a.mmask = (m >= 64) ? ~0ull : ((1ull << m) - 1ull);
+    a.contiguous = contiguous;
+    a.lo = qubits[0];
+    a.g = 1ull << __builtin_ctzll(c);   // gcd(c, 2^m)
+    a.cycle_len = (a.mmask >> __builtin_ctzll(c)) + 1ull;
+    int tmp[64];
+    for (int j = 0; j < m; ++j) tmp[j] = a.reg[j] = (uint8_t)qubits[j];
+    std::sort(tmp, tmp + m);
+    for (int j = 0; j < m; ++j) a.reg_sorted[j] = (uint8_t)tmp[j];
+    return a;
+}
+
+// The columns whose low kb bits lie in [off, off + len) (kb = 0: all); sets the
+// split of the cycles: enough independent walks to fill the GPU, segments of
+// >= 64 steps.
+template <class S>
+void walk_columns(WalkArgs<S>& a, int n, int kb, uint64_t off, uint64_t len) {
+    a.kb = kb;
+    a.off0 = off;
+    a.len = len;
+    a.columns = len << (n - a.m - kb);
+    const uint64_t want = (uint64_t)num_sms() * 2048;
+    const uint64_t base_items = a.columns * a.g;
+    uint64_t nseg = (want + base_items - 1) / base_items;
+    nseg = std::max<uint64_t>(1, std::min<uint64_t>(nseg, a.cycle_len / 64));
+    a.seg_len = (a.cycle_len + nseg - 1) / nseg;
+    a.nseg = (a.cycle_len + a.seg_len - 1) / a.seg_len;
+    a.items = base_items * a.nseg;
+}
+
+template <class S>
+void walk_launch(qe_state* s, WalkArgs<S>& a) {
+    a.scratch = (S*)ensure_scratch(s, a.items * sizeof(S));
+    uint64_t grid = std::min<uint64_t>((a.items + 255) / 256, (uint64_t)num_sms() * 8);
+    grid = std::max<uint64_t>(grid, 1);
+    k_add_walk_save<S><<<(unsigned)grid, 256, 0, s->stream>>>(a);
+    QE_CUDA(cudaGetLastError());
+    k_add_walk<S, 8><<<(unsigned)grid, 256, 0, s->stream>>>(a);
+    QE_CUDA(cudaGetLastError());
+}
+
+// Split of a contiguous register at 2^k amplitudes (the file's comment).  The
+// walks go over at most 2^21 saved elements at a time; their scratch is had
+// before anything is moved, and without it the caller takes the plain walk.
+template <class S>
+bool add_split(qe_state* s, int lo, int m, uint64_t c, int k, void (*rotate)(qe_state*, int, const int*, uint64_t)) {
+    const int h = lo + m - k;
+    int low[64], high[64];
+    for (int j = 0; j < k - lo; ++j) low[j] = lo + j;
+    for (int j = 0; j < h; ++j) high[j] = k + j;
+    const uint64_t clow = c & ((1ull << (k - lo)) - 1ull), place = clow << lo, part = 1ull << k;
+    const uint64_t hmask = (1ull << h) - 1ull, chigh = (c >> (k - lo)) & hmask;
+    struct Run {
+        uint64_t c, off, len, step;
+    } run[2] = {{chigh, place, part - place, 0}, {(chigh + 1) & hmask, 0, place, 0}};
+    uint64_t most = 0;
+    for (Run& r : run) {
+        if (r.c == 0 || r.len == 0) continue;
+        WalkArgs<S> a = walk_args<S>(s, h, high, r.c, true);
+        r.step = std::max<uint64_t>(1, std::min<uint64_t>(r.len, (1ull << 21) / (a.g << (s->n - h - k))));
+        walk_columns(a, s->n, k, r.off, r.step);
+        most = std::max(most, a.items);
+        walk_columns(a, s->n, k, r.off, (r.len - 1) % r.step + 1);
+        most = std::max(most, a.items);
+    }
+    try {
+        ensure_scratch(s, most * sizeof(S));
+    } catch (const Error&) {
+        cudaGetLastError();   // the refused allocation's
+        return false;
+    }
+    if (clow) rotate(s, k - lo, low, clow);
+    Launch L(s, "add_walk", 2.0 * dim(s) * amp_bytes(s));
+    for (const Run& r : run) {
+        if (r.c == 0 || r.len == 0) continue;
+        WalkArgs<S> a = walk_args<S>(s, h, high, r.c, true);
+        for (uint64_t o = 0; o < r.len; o += r.step) {
+            walk_columns(a, s->n, k, r.off + o, std::min(r.step, r.len - o));
+            walk_launch(s, a);
+        }
+    }
+    return true;
 }
 
 template <class S>
@@ -237,17 +339,20 @@ void add_impl(qe_state* s, int m, const int* qubits, uint64_t c) {
     const int bulk_bits = (sizeof(S) >= 16) ? 13 : 14;
     const int bulk_min = (sizeof(S) >= 16) ? 11 : 12;
     const uint64_t shift = c << lo;
-    const int nblk = (contiguous && Sbits >= 3 && Sbits <= bulk_bits) ? 1 : 8;
-    const bool use_bulk = contiguous && lo < 5 && Sbits >= bulk_min && Sbits <= bulk_bits + 3 &&
+    // clusters of eight up to 64 KB a CTA; sixteen above that: several CTAs an
+    // SM where 128 KB leave room for one, and 16 of a GPC's 18 to 20 SMs for two
+    // clusters of eight (1 MB slices at n = 29: 3.31 against 2.98 ms, 512 KB 2.76
+    // against 2.96).  Slices of 2 MB: only where the walk's runs are at most 64
+    // bytes (complex128 lo = 2 5.6 -> 3.6 ms, lo = 3 3.2 and 3.6)
+    const int nblk = (contiguous && Sbits >= 3 && Sbits <= bulk_bits) ? 1 : Sbits <= bulk_bits + 2 ? 8 : 16;
+    const bool use_bulk = contiguous && lo < 5 && Sbits >= bulk_min && Sbits <= bulk_bits + ((sizeof(S) << lo) <= 64 ? 4 : 3) &&
                           ((shift * sizeof(S)) % 16 == 0) && ((((uint64_t)sizeof(S) << Sbits) / nblk) % 16 == 0);
     if (use_bulk) {
         Launch L(s, nblk == 1 ? "add_bulk" : "add_bulk_cluster", 2.0 * dim(s) * amp_bytes(s));
         const uint64_t nslices = 1ull << (n - Sbits);
         const size_t smem = (sizeof(S) << Sbits) / nblk;
         QE_CUDA(cudaFuncSetAttribute(k_add_bulk<S>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-        void* st_addr = nullptr;
-        QE_CUDA(cudaGetSymbolAddress(&st_addr, g_add_status));
-        QE_CUDA(cudaMemsetAsync(st_addr, 0, sizeof(uint32_t), s->stream));
+        QE_CUDA(cudaFuncSetAttribute(k_add_bulk<S>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
         cudaLaunchConfig_t cfg = {};
         if (nslices * nblk > 0x7FFFFFFFull) fail(QE_ERR_UNSUPPORTED, "too many slices for one launch");
         cfg.gridDim = dim3((unsigned)(nslices * nblk));
@@ -267,13 +372,13 @@ void add_impl(qe_state* s, int m, const int* qubits, uint64_t c) {
         const char* stall = std::getenv("QE_TEST_STALL_ADD");
         const int stall_test = (stall != nullptr && stall[0] == '1') ? 1 : 0;
         const long long limit = stall_test ? (1ll << 12) : (1ll << 20);   // polls of up to 1 us each
-        QE_CUDA(cudaLaunchKernelEx(&cfg, k_add_bulk<S>, x, Sbits, (uint32_t)shift, limit, stall_test));
+        QE_CUDA(cudaLaunchKernelEx(&cfg, k_add_bulk<S>, x, Sbits, (uint32_t)shift, limit, stall_test, status_word(s)));
         QE_CUDA(cudaGetLastError());
-        uint32_t st = 0;
-        QE_CUDA(cudaMemcpyAsync(&st, st_addr, sizeof(uint32_t), cudaMemcpyDeviceToHost, s->stream));
-        QE_CUDA(cudaStreamSynchronize(s->stream));
-        if (st != 0) fail(QE_ERR_TIMEOUT, "an add-constant copy wait ran out");
+        complete_pending(s);
         return;
+    }
+    if (contiguous && Sbits > bulk_bits + 3 && (sizeof(S) << lo) < 64 && dim(s) * sizeof(S) >= (1ull << 28)) {
+        if (add_split<S>(s, lo, m, c, cap_bits, add_impl<S>)) return;
     }
     const bool use_slice = contiguous && lo < 5 && Sbits <= cap_bits;
     const bool use_cluster = !use_slice && contiguous && lo < 5 && Sbits <= ccap_bits + 3 && Sbits >= 3;
@@ -308,35 +413,9 @@ void add_impl(qe_state* s, int m, const int* qubits, uint64_t c) {
         if (nslices * 8 > 0x7FFFFFFFull) fail(QE_ERR_UNSUPPORTED, "too many slices for one launch");
         QE_CUDA(cudaLaunchKernelEx(&cfg, k_add_cluster<S>, x, Sbits, (uint64_t)(c << lo)));
     } else {
-        static thread_local WalkArgs<S> a;
-        a.x = x;
-        a.m = m;
-        a.c = c;
-        a.mmask = mmask;
-        a.contiguous = contiguous;
-        a.lo = lo;
-        a.g = 1ull << __builtin_ctzll(c);   // gcd(c, 2^m), c != 0 mod 2^m
-        a.columns = 1ull << (n - m);
-        a.cycle_len = (mmask >> __builtin_ctzll(c)) + 1ull;
-        // enough independent walks to fill the GPU, segments of >= 64 steps
-        const uint64_t want = (uint64_t)num_sms() * 2048;
-        const uint64_t base_items = a.columns * a.g;
-        uint64_t nseg = (want + base_items - 1) / base_items;
-        nseg = std::max<uint64_t>(1, std::min<uint64_t>(nseg, a.cycle_len / 64));
-        a.seg_len = (a.cycle_len + nseg - 1) / nseg;
-        a.nseg = (a.cycle_len + a.seg_len - 1) / a.seg_len;
-        a.items = base_items * a.nseg;
-        a.scratch = (S*)ensure_scratch(s, a.items * sizeof(S));
-        for (int j = 0; j < m; ++j) a.reg[j] = (uint8_t)qubits[j];
-        int tmp[64];
-        for (int j = 0; j < m; ++j) tmp[j] = qubits[j];
-        std::sort(tmp, tmp + m);
-        for (int j = 0; j < m; ++j) a.reg_sorted[j] = (uint8_t)tmp[j];
-        uint64_t grid = std::min<uint64_t>((a.items + 255) / 256, (uint64_t)num_sms() * 8);
-        grid = std::max<uint64_t>(grid, 1);
-        k_add_walk_save<S><<<(unsigned)grid, 256, 0, s->stream>>>(a);
-        QE_CUDA(cudaGetLastError());
-        k_add_walk<S, 8><<<(unsigned)grid, 256, 0, s->stream>>>(a);
+        WalkArgs<S> a = walk_args<S>(s, m, qubits, c, contiguous);
+        walk_columns(a, n, 0, 0, 1);
+        walk_launch(s, a);
     }
     QE_CUDA(cudaGetLastError());
 }
