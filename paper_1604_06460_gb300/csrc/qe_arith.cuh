@@ -225,6 +225,92 @@ struct DF {
     }
 };
 
+// ------------------------------------------------ |alpha|^2 in fixed point
+// Sum of |alpha|^2 over a thread's N <= 8 amplitudes.  The FP64 pipe (two lanes a
+// clock and SM) would bound every pass that only sums probabilities: two
+// multiply-adds an amplitude take 0.91 ms for 2^28 complex128 amplitudes, whose
+// read takes 0.63, and complex64 adds two conversions.  With E the largest
+// biased exponent of the components, component v is the integer
+// q = |v| 2^(1076 - E) below 2^54, rounded to the nearest (complex64: below
+// 2^54, truncated more than 30 binary orders down), in two limbs
+// q = (h 2^29 + l) / 2, and the three limb products are summed exactly in 64
+// bits: one conversion and two multiplications in FP64 for the N amplitudes.
+// Components that the window cannot hold (E below 64, infinities, NaN) take the
+// FP64 sum.
+__device__ __forceinline__ double mass_f64(double re, double im, double s) {
+    return __fma_rn(re, re, __fma_rn(im, im, s));
+}
+struct MassAcc {
+    uint64_t hh = 0, hl = 0, ll = 0;
+    __device__ __forceinline__ void add(uint32_t h, uint32_t l) {
+        hh += (uint64_t)h * h;
+        hl += (uint64_t)h * l;
+        ll += (uint64_t)l * l;
+    }
+    // sum of q^2 = hh 2^56 + hl 2^28 + ll / 4 at unit 2^56, hl < 2^59, ll < 2^62
+    __device__ __forceinline__ double value(int e1, int e2) const {
+        const uint64_t m = hl + (ll >> 30);                         // unit 2^28
+        const uint64_t t = (hh << 4) + ((m + (1ull << 23)) >> 24);   // unit 2^52, hh < 2^56
+        return __dmul_rn(__dmul_rn((double)(long long)t, __hiloint2double(e1 << 20, 0)), __hiloint2double(e2 << 20, 0));
+    }
+};
+template <int N>
+__device__ __forceinline__ double mass_of(const double2 (&v)[N]) {
+    static_assert(N <= 8, "limb sums below 2^62");
+    uint32_t top = 0u;
+#pragma unroll
+    for (int j = 0; j < N; ++j)
+        top = max(top, max((uint32_t)__double2hiint(v[j].x) & 0x7FFFFFFFu, (uint32_t)__double2hiint(v[j].y) & 0x7FFFFFFFu));
+    const uint32_t E = top >> 20;
+    if (E < 64u || E == 0x7FFu) {
+        double s = 0.0;
+#pragma unroll
+        for (int j = 0; j < N; ++j) s = mass_f64(v[j].x, v[j].y, s);
+        return s;
+    }
+    MassAcc a;
+    auto take = [&](double c) {
+        const uint32_t hi = (uint32_t)__double2hiint(c), lo = (uint32_t)__double2loint(c);
+        const uint64_t m4 = ((((uint64_t)((hi & 0xFFFFFu) | 0x100000u)) << 32) | lo) << 2;
+        const uint64_t t = (m4 >> min(E - ((hi >> 20) & 0x7FFu), 63u)) + 1u;   // 2 q, its last bit to drop
+        a.add((uint32_t)(t >> 29), (uint32_t)t & 0x1FFFFFFEu);
+    };
+#pragma unroll
+    for (int j = 0; j < N; ++j) {
+        take(v[j].x);
+        take(v[j].y);
+    }
+    return a.value((int)E - 1, (int)E - 53);   // 2^(2 E - 2152 + 52)
+}
+template <int N>
+__device__ __forceinline__ double mass_of(const float2 (&v)[N]) {
+    static_assert(N <= 8, "limb sums below 2^62");
+    uint32_t top = 0u;
+#pragma unroll
+    for (int j = 0; j < N; ++j)
+        top = max(top, max(__float_as_uint(v[j].x) & 0x7FFFFFFFu, __float_as_uint(v[j].y) & 0x7FFFFFFFu));
+    const uint32_t E = top >> 23;
+    if (E < 64u || E == 0xFFu) {
+        double s = 0.0;
+#pragma unroll
+        for (int j = 0; j < N; ++j) s = mass_f64((double)v[j].x, (double)v[j].y, s);
+        return s;
+    }
+    MassAcc a;
+    auto take = [&](float c) {
+        const uint32_t b = __float_as_uint(c);
+        const uint64_t m = (uint64_t)((b & 0x7FFFFFu) | 0x800000u) << 31;
+        const uint64_t t = m >> min(E - ((b >> 23) & 0xFFu), 63u);
+        a.add((uint32_t)(t >> 29), (uint32_t)t & 0x1FFFFFFEu);
+    };
+#pragma unroll
+    for (int j = 0; j < N; ++j) {
+        take(v[j].x);
+        take(v[j].y);
+    }
+    return a.value((int)E + 896 - 1, (int)E + 896 - 53);   // the biases differ by 896
+}
+
 // ------------------------------------------------------------ bit helpers
 // Insert a zero bit at each position of sorted[0..cnt-1] (ascending).
 __host__ __device__ __forceinline__ uint64_t insert_zero_bits(uint64_t t, const uint8_t* sorted, int cnt) {

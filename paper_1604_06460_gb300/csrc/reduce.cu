@@ -170,40 +170,113 @@ __device__ __forceinline__ double block_reduce_d(double a, double* sh) {
 }
 
 // ---------------------------------------------------------------- probs
-// Block b handles bin r = b / chunks and the chunk b % chunks of the
-// 2^(n-m) amplitudes whose bits at the qubits spell r.
+// Marginal probabilities.  Thread t of a block reads amplitudes whose low
+// eight index bits are t (lines of 4 KB, 2 KB in complex64, whichever qubits
+// are asked for): the register's qubits below 8 are bits of t, those above
+// are fixed by the block (blockIdx / chunks), and the block walks a chunk of the
+// places of the other high bits, eight amplitudes at a time summed in fixed
+// point (mass_of), the eights in FP64.  The threads that differ only in bits
+// outside the register are then combined pairwise with Neumaier's
+// compensation.  Bound by HBM: n = 28, three qubits, complex128 0.74 ms (1.05
+// to 1.30 by FP64 products, two an amplitude), complex64 0.33 (0.44 to 0.92);
+// eight qubits on both sides of 8, read bin by bin with a stride before, 1.43 ->
+// 0.74 and 1.62 -> 0.32.
+constexpr int kLowBits = 8;
 template <class S>
 struct ProbArgs {
     const S* x;
-    uint64_t per_bin;     // 2^(n-m)
-    uint64_t chunks;      // blocks per bin
-    uint64_t chunk_len;
+    uint64_t places;      // 2^(high bits outside the register)
+    uint64_t chunks;      // blocks per value of the register's high bits
+    uint64_t chunk_len;   // places a block
+    uint32_t lowmask;     // the register's qubits below 8
+    uint64_t highmask;    // and above, as amplitude bits
+    int n, mh;
     int m;
-    uint8_t q[32];
-    uint8_t q_sorted[32];
-    double2* partial;     // [bins * chunks]
+    uint8_t q[64];        // bit j <-> qubit q[j]
+    uint8_t qh[64];       // the high ones ascending
+    double2* partial;     // [bins * chunks], chunks > 1
+    double* out;          // [bins], chunks == 1
 };
 
-template <class S>
-__global__ void __launch_bounds__(kRThreads) k_probs_partial(const __grid_constant__ ProbArgs<S> a) {
-    __shared__ Acc sh[32];
-    const uint64_t bin = blockIdx.x / a.chunks, ch = blockIdx.x % a.chunks;
-    uint64_t dep = 0;
-    for (int j = 0; j < a.m; ++j) dep |= ((bin >> j) & 1ull) << a.q[j];
-    const uint64_t t0 = ch * a.chunk_len;
-    const uint64_t t1 = min(a.per_bin, t0 + a.chunk_len);
+// Sum of |alpha|^2 of up to eight amplitudes: fixed point for complex128;
+// float pairs for complex64, as its expectations (products exact, about 44
+// bits), cheaper there than limbs.
+template <int N>
+__device__ __forceinline__ double group_mass(const double2 (&v)[N]) {
+    return mass_of(v);
+}
+template <int N>
+__device__ __forceinline__ double group_mass(const float2 (&v)[N]) {
     Acc acc{0.f, 0.f};
-    for (uint64_t t = t0 + threadIdx.x; t < t1; t += blockDim.x) {
-        const uint64_t x = insert_zero_bits(t, a.q_sorted, a.m) | dep;
+#pragma unroll
+    for (int j = 0; j < N; ++j) {
         float h, l;
-        abs2(rview(a.x[x]), h, l);
+        abs2(rview(v[j]), h, l);
         acc_add(acc, h, l);
     }
-    acc = block_reduce(acc, sh);
-    if (threadIdx.x == 0) {
-        df r = df_norm(acc.s, acc.e);
-        a.partial[blockIdx.x] = make_double2(df2d(r.h, r.l), 0.0);
+    const df r = df_norm(acc.s, acc.e);
+    return df2d(r.h, r.l);
+}
+
+template <class S>
+__global__ void __launch_bounds__(1 << kLowBits) k_probs(const __grid_constant__ ProbArgs<S> a) {
+    constexpr uint32_t T = 1u << kLowBits;
+    __shared__ double ss[T], sc[T];
+    const uint32_t t = threadIdx.x;
+    const uint64_t hv = blockIdx.x / a.chunks, ch = blockIdx.x % a.chunks;
+    uint64_t dep = 0;   // hv's bits at the register's high qubits
+    for (int j = 0; j < a.mh; ++j) dep |= ((hv >> j) & 1ull) << a.qh[j];
+    double s = 0.0, c = 0.0;
+    const bool in = a.n >= kLowBits || t < (1u << a.n);
+    const uint64_t p0 = ch * a.chunk_len, p1 = min(a.places, p0 + a.chunk_len);
+    if (in && p0 < p1) {
+        const uint64_t fixed = a.highmask | (T - 1u);
+        const S* const x = a.x + (dep | t);
+        // place p0: its bits put into the free positions
+        uint64_t at = p0 << kLowBits;
+        for (int j = 0; j < a.mh; ++j) {
+            const uint64_t lowb = at & ((1ull << a.qh[j]) - 1ull);
+            at = ((at >> a.qh[j]) << (a.qh[j] + 1)) | lowb;
+        }
+        uint64_t p = p0;
+        for (; p + 8 <= p1; p += 8) {
+            S v[8];
+#pragma unroll
+            for (int j = 0; j < 8; ++j) {
+                v[j] = x[at];
+                at = ((at | fixed) + 1ull) & ~fixed;
+            }
+            s += group_mass(v);
+        }
+        for (; p < p1; ++p) {
+            const S v[1] = {x[at]};
+            s += group_mass(v);
+            at = ((at | fixed) + 1ull) & ~fixed;
+        }
     }
+    // pairwise over the thread bits outside the register
+    for (int b = 0; b < 5; ++b) {
+        if ((a.lowmask >> b) & 1u) continue;
+        const double os = __shfl_down_sync(0xffffffffu, s, 1u << b), oc = __shfl_down_sync(0xffffffffu, c, 1u << b);
+        neumaier(s, c, os);
+        c += oc;
+    }
+    for (int b = 5; b < kLowBits; ++b) {
+        if ((a.lowmask >> b) & 1u) continue;
+        ss[t] = s;
+        sc[t] = c;
+        __syncthreads();
+        if (((t >> b) & 1u) == 0u) {
+            neumaier(s, c, ss[t + (1u << b)]);
+            c += sc[t + (1u << b)];
+        }
+        __syncthreads();
+    }
+    if (!in || (t & ~a.lowmask) != 0u) return;
+    uint64_t bin = 0;
+    for (int j = 0; j < a.m; ++j) bin |= (((dep | t) >> a.q[j]) & 1ull) << j;
+    if (a.chunks == 1) a.out[bin] = s + c;
+    else a.partial[bin * a.chunks + ch] = make_double2(s, c);
 }
 
 // One block per output (grid-stride over outputs): Neumaier sums of the
@@ -236,6 +309,22 @@ __global__ void __launch_bounds__(kSumThreads) k_sum_partials(const double2* __r
         }
         if (threadIdx.x == 0) out[o] = (ss[0] + cs[0]) * (weight ? weight[o] : 1.0);
         __syncthreads();
+    }
+}
+
+// The same for few partials an output (many bins): a thread an output.  2^16
+// bins of four partials each: 485 us by blocks, 14 us.
+constexpr uint64_t kFewPartials = 16;
+__global__ void __launch_bounds__(kSumThreads) k_sum_few(const double2* __restrict__ partial, uint64_t nout,
+                                                         uint32_t count, double* __restrict__ out) {
+    for (uint64_t o = blockIdx.x * (uint64_t)kSumThreads + threadIdx.x; o < nout; o += (uint64_t)gridDim.x * kSumThreads) {
+        double s = 0.0, c = 0.0;
+        for (uint32_t i = 0; i < count; ++i) {
+            const double2 p = partial[o * count + i];
+            neumaier(s, c, p.x);
+            neumaier(s, c, p.y);
+        }
+        out[o] = s + c;
     }
 }
 
@@ -1120,124 +1209,29 @@ __global__ void __launch_bounds__(kThr2, 1) k_expect_fx(const __grid_constant__ 
     if (tid == 0) a.partial[blockIdx.x] = make_double2(s, c);
 }
 
-// Native FP64 variants (baseline policy).
-__global__ void __launch_bounds__(kRThreads) k_probs_partial_f64(const __grid_constant__ ProbArgs<double2> a) {
-    __shared__ double shs[32];
-    const uint64_t bin = blockIdx.x / a.chunks, ch = blockIdx.x % a.chunks;
-    uint64_t dep = 0;
-    for (int j = 0; j < a.m; ++j) dep |= ((bin >> j) & 1ull) << a.q[j];
-    const uint64_t t0 = ch * a.chunk_len;
-    const uint64_t t1 = min(a.per_bin, t0 + a.chunk_len);
-    // two FP64 accumulators a thread (products by fused multiply-add); the
-    // block's warp sums are combined with Neumaier's compensation
-    double s = 0.0, c = 0.0;
-    uint64_t t = t0 + threadIdx.x;
-    for (; t + blockDim.x < t1; t += 2 * (uint64_t)blockDim.x) {
-        const double2 v = a.x[insert_zero_bits(t, a.q_sorted, a.m) | dep];
-        const double2 u = a.x[insert_zero_bits(t + blockDim.x, a.q_sorted, a.m) | dep];
-        s = __fma_rn(v.x, v.x, __fma_rn(v.y, v.y, s));
-        c = __fma_rn(u.x, u.x, __fma_rn(u.y, u.y, c));
-    }
-    if (t < t1) {
-        const double2 v = a.x[insert_zero_bits(t, a.q_sorted, a.m) | dep];
-        s = __fma_rn(v.x, v.x, __fma_rn(v.y, v.y, s));
-    }
-    s += c;
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
-    if ((threadIdx.x & 31) == 0) shs[threadIdx.x >> 5] = s;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double ts = 0.0, tc = 0.0;
-        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) neumaier(ts, tc, shs[w]);
-        a.partial[blockIdx.x] = make_double2(ts, tc);
-    }
+// The split of a marginal's reduction: places of the high bits outside the
+// register, in chunks of a multiple of eight, about eight blocks an SM in all.
+void probs_split(const qe_state* s, int mh, uint64_t& places, uint64_t& chunks, uint64_t& len) {
+    const int hb = std::max(0, s->n - kLowBits);
+    places = 1ull << (hb - mh);
+    const uint64_t want = std::max<uint64_t>(1, ((uint64_t)num_sms() * 8) >> mh);
+    len = std::max<uint64_t>(8, (((places + want - 1) / want) + 7) & ~7ull);
+    chunks = (places + len - 1) / len;
 }
 
-// Marginals of qubits that all lie below qubit 8: thread t of a 256-thread
-// block reads the amplitudes whose low 8 bits are t, so its bin is fixed and
-// the block reads a contiguous range (the bin-major kernels read each bin
-// with a stride); the block then sums its threads per bin.  Partials at
-// [bin * nblocks + block].  FP64 mode: FP64 products and sums (two
-// accumulators a thread); otherwise float-pair sums as in k_probs_partial.
-constexpr int kLowBits = 8;
-template <class S, bool NAT>
-__global__ void __launch_bounds__(1 << kLowBits) k_probs_low(const __grid_constant__ ProbArgs<S> a) {
-    constexpr uint32_t T = 1u << kLowBits;
-    __shared__ double ss[T], sc[T];
-    const uint32_t t = threadIdx.x;
-    uint32_t bin = 0;
-    for (int j = 0; j < a.m; ++j) bin |= ((t >> a.q[j]) & 1u) << j;
-    const uint64_t base = blockIdx.x * a.chunk_len + t;   // chunk_len: amplitudes a block, a multiple of 4 T
-    double s = 0.0, c = 0.0;
-    if constexpr (NAT) {
-        double s2 = 0.0, s3 = 0.0, s4 = 0.0;
-        for (uint64_t k = 0; k < a.chunk_len; k += 4 * T) {
-            const double2 v0 = reinterpret_cast<const double2*>(a.x)[base + k];
-            const double2 v1 = reinterpret_cast<const double2*>(a.x)[base + k + T];
-            const double2 v2 = reinterpret_cast<const double2*>(a.x)[base + k + 2 * T];
-            const double2 v3 = reinterpret_cast<const double2*>(a.x)[base + k + 3 * T];
-            s = __fma_rn(v0.x, v0.x, __fma_rn(v0.y, v0.y, s));
-            s2 = __fma_rn(v1.x, v1.x, __fma_rn(v1.y, v1.y, s2));
-            s3 = __fma_rn(v2.x, v2.x, __fma_rn(v2.y, v2.y, s3));
-            s4 = __fma_rn(v3.x, v3.x, __fma_rn(v3.y, v3.y, s4));
-        }
-        neumaier(s, c, s2);
-        neumaier(s, c, s3);
-        neumaier(s, c, s4);
-    } else {
-        Acc acc{0.f, 0.f};
-        for (uint64_t k = 0; k < a.chunk_len; k += 4 * T) {
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                float h, l;
-                abs2(rview(a.x[base + k + (uint64_t)u * T]), h, l);
-                acc_add(acc, h, l);
-            }
-        }
-        const df r = df_norm(acc.s, acc.e);
-        s = df2d(r.h, r.l);
+// Block partials for any register of m qubits (its high ones unknown here).
+uint64_t probs_partials(const qe_state* s, int m) {
+    uint64_t most = 0;
+    for (int mh = std::max(0, m - kLowBits); mh <= std::min(m, std::max(0, s->n - kLowBits)); ++mh) {
+        uint64_t places, chunks, len;
+        probs_split(s, mh, places, chunks, len);
+        if (chunks > 1) most = std::max(most, chunks << m);
     }
-    ss[t] = s;
-    sc[t] = c;
-    __syncthreads();
-    if (t < (1u << a.m)) {
-        // the threads of bin t, in index order
-        double bs = 0.0, bc = 0.0;
-        for (uint32_t u = 0; u < T; ++u) {
-            uint32_t b = 0;
-            for (int j = 0; j < a.m; ++j) b |= ((u >> a.q[j]) & 1u) << j;
-            if (b != t) continue;
-            neumaier(bs, bc, ss[u]);
-            bc += sc[u];
-        }
-        a.partial[(uint64_t)t * gridDim.x + blockIdx.x] = make_double2(bs, bc);
-    }
-}
-
-// Blocks of the low-qubit marginal kernel: about 8 per SM, at least 2^14
-// amplitudes each (a power of two).
-uint64_t probs_low_blocks(const qe_state* s) {
-    if (s->n < 14) return 0;
-    uint64_t per = 1ull << 14;
-    while (((1ull << s->n) / per) > (uint64_t)num_sms() * 8) per <<= 1;
-    return (1ull << s->n) / per;
-}
-
-// Blocks of the probability reduction for m register qubits: about 8 blocks
-// per SM in total, at least 2^14 amplitudes per block.
-uint64_t probs_chunks(const qe_state* s, int m) {
-    const uint64_t bins = 1ull << m;
-    const uint64_t want_blocks = (uint64_t)num_sms() * 8;
-    uint64_t chunks = std::max<uint64_t>(1, want_blocks / bins);
-    return std::min<uint64_t>(chunks, std::max<uint64_t>(1, (1ull << (s->n - m)) >> 14));
+    return most;
 }
 
 template <class S>
 void probs_device(qe_state* s, int m, const int* qubits, double2* partial, double* dout);
-
-uint64_t probs_partials(const qe_state* s, int m) {
-    return (1ull << m) * std::max(probs_chunks(s, m), probs_low_blocks(s));
-}
 
 template <class S>
 void probs_impl(qe_state* s, int m, const int* qubits, double* host_out) {
@@ -1251,62 +1245,45 @@ void probs_impl(qe_state* s, int m, const int* qubits, double* host_out) {
 }
 
 // The 2^m marginal probabilities into device memory dout (partial: room for
-// 2^m * probs_chunks(s, m) block partials); enqueued only.
+// probs_partials(s, m) block partials); enqueued only.
 template <class S>
 void probs_device(qe_state* s, int m, const int* qubits, double2* partial, double* dout) {
     static thread_local ProbArgs<S> a;
     a.x = reinterpret_cast<const S*>(s->d);
+    a.n = s->n;
     a.m = m;
-    int tmp[32];
+    a.mh = 0;
+    a.lowmask = 0;
+    a.highmask = 0;
     for (int j = 0; j < m; ++j) {
         a.q[j] = (uint8_t)qubits[j];
-        tmp[j] = qubits[j];
-    }
-    std::sort(tmp, tmp + m);
-    for (int j = 0; j < m; ++j) a.q_sorted[j] = (uint8_t)tmp[j];
-    const uint64_t bins = 1ull << m;
-    bool low = m >= 1 && probs_low_blocks(s) > 0;
-    for (int j = 0; j < m; ++j) low &= qubits[j] < kLowBits;
-    if (low) {
-        const uint64_t nb = probs_low_blocks(s);
-        a.chunk_len = (1ull << s->n) / nb;
-        a.partial = partial;
-        {
-            Launch L(s, "probs_low", (double)dim(s) * amp_bytes(s));
-            if (std::is_same<S, double2>::value && c128_f64(s))
-                k_probs_low<S, true><<<(unsigned)nb, 1 << kLowBits, 0, s->stream>>>(a);
-            else
-                k_probs_low<S, false><<<(unsigned)nb, 1 << kLowBits, 0, s->stream>>>(a);
-            QE_CUDA(cudaGetLastError());
+        if (qubits[j] < kLowBits) {
+            a.lowmask |= 1u << qubits[j];
+        } else {
+            a.highmask |= 1ull << qubits[j];
+            a.qh[a.mh++] = (uint8_t)qubits[j];
         }
-        Launch L(s, "sum_partials", 0.0, false);
-        const unsigned g2 = (unsigned)std::min<uint64_t>(bins, 4096);
-        k_sum_partials<<<g2, kSumThreads, 0, s->stream>>>(a.partial, bins, nb, nullptr, dout);
-        QE_CUDA(cudaGetLastError());
-        return;
     }
-    a.per_bin = 1ull << (s->n - m);
-    const uint64_t chunks = probs_chunks(s, m);
-    a.chunks = chunks;
-    a.chunk_len = (a.per_bin + chunks - 1) / chunks;
-    const uint64_t nblocks = bins * chunks;
+    std::sort(a.qh, a.qh + a.mh);
+    probs_split(s, a.mh, a.places, a.chunks, a.chunk_len);
     a.partial = partial;
+    a.out = dout;
+    const uint64_t bins = 1ull << m, nblocks = a.chunks << a.mh;
     if (nblocks > 0x7FFFFFFFull) fail(QE_ERR_UNSUPPORTED, "too many probability blocks");
     {
-        Launch L(s, "probs_partial", (double)dim(s) * amp_bytes(s));
-        if (std::is_same<S, double2>::value && c128_f64(s))
-            k_probs_partial_f64<<<(unsigned)nblocks, kRThreads, 0, s->stream>>>(
-                *reinterpret_cast<ProbArgs<double2>*>(&a));
-        else
-            k_probs_partial<S><<<(unsigned)nblocks, kRThreads, 0, s->stream>>>(a);
+        Launch L(s, m >= 1 && a.mh == 0 ? "probs_low" : "probs_partial", (double)dim(s) * amp_bytes(s));
+        k_probs<S><<<(unsigned)nblocks, 1 << kLowBits, 0, s->stream>>>(a);
         QE_CUDA(cudaGetLastError());
     }
-    {
-        Launch L(s, "sum_partials", 0.0, false);
-        const unsigned g2 = (unsigned)std::min<uint64_t>(bins, 4096);
-        k_sum_partials<<<g2, kSumThreads, 0, s->stream>>>(a.partial, bins, chunks, nullptr, dout);
-        QE_CUDA(cudaGetLastError());
-    }
+    if (a.chunks == 1) return;
+    Launch L(s, "sum_partials", 0.0, false);
+    const unsigned g2 = (unsigned)std::min<uint64_t>(bins, 4096);
+    if (a.chunks <= kFewPartials)
+        k_sum_few<<<(unsigned)std::min<uint64_t>((bins + kSumThreads - 1) / kSumThreads, 4096), kSumThreads, 0,
+                    s->stream>>>(a.partial, bins, (uint32_t)a.chunks, dout);
+    else
+        k_sum_partials<<<g2, kSumThreads, 0, s->stream>>>(a.partial, bins, a.chunks, nullptr, dout);
+    QE_CUDA(cudaGetLastError());
 }
 
 // Terms whose X/Y qubits do not fit one tile layout: grid-stride over x with

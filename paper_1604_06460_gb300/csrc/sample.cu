@@ -9,13 +9,13 @@
 // r whose cumulative probability exceeds u_s times the total, or, when
 // rounding leaves none, the largest r with P(r) > 0.
 //   - all qubits: the state is cut into blocks of 2^12 amplitudes; one pass
-//     sums |alpha|^2 per block (FP64), one CTA scans the block sums, and a
-//     warp per shot finds the block by binary search and the amplitude
-//     inside it by a warp scan of lane sums and a scan of one lane's run;
+//     sums |alpha|^2 per block, the block sums are scanned, and a warp per
+//     shot finds the block by binary search and the amplitude inside it by
+//     scans of segment sums, lane sums and one lane's run;
 //   - m <= 16 qubits: the 2^m marginal probabilities (the probability
 //     reduction), the same scan, and a binary search per shot.
-// All sums are FP64 in a fixed order, so a sample depends only on the state
-// and the uniforms.
+// All sums are FP64 (their first eight terms exact, in fixed point) in a fixed
+// order, so a sample depends only on the state and the uniforms.
 //
 // Collapse: one reduction of the outcome's probability p (FP64), then one
 // pass that zeroes the other amplitudes and scales the outcome's by 1/sqrt(p).
@@ -32,7 +32,7 @@ namespace {
 
 constexpr int kBlockBits = 12;   // amplitudes per block of the full distribution
 constexpr int kMassThreads = 256;
-constexpr int kScanThreads = 1024;
+constexpr int kScanThreads = 256;
 
 __device__ __forceinline__ double prob_of(double2 v) { return __fma_rn(v.x, v.x, __dmul_rn(v.y, v.y)); }
 __device__ __forceinline__ double prob_of(float2 v) {
@@ -40,17 +40,25 @@ __device__ __forceinline__ double prob_of(float2 v) {
     return __fma_rn(re, re, __dmul_rn(im, im));
 }
 
-// mass[k] = sum of |alpha|^2 over block k: thread t takes elements t, t + 256,
-// ... of the block, then a fixed reduction tree.
+// mass[k] = sum of |alpha|^2 over block k of 2^12: thread t takes elements t,
+// t + 256, ... of the block, then a fixed reduction tree.  Bound by HBM: the
+// squares are summed in fixed point (2^28 amplitudes, complex128: 1.74 ms with
+// three FP64 operations an amplitude, 0.74 now; complex64 2.71 -> 0.65).
 template <class S>
-__global__ void __launch_bounds__(kMassThreads) k_block_mass(const S* __restrict__ x, uint64_t nblocks, int B,
+__global__ void __launch_bounds__(kMassThreads) k_block_mass(const S* __restrict__ x, uint64_t nblocks,
                                                              double* __restrict__ mass) {
     __shared__ double sh[kMassThreads / 32];
-    const uint32_t E = 1u << B;
+    constexpr int kBatches = (1 << kBlockBits) / (8 * kMassThreads);
     for (uint64_t k = blockIdx.x; k < nblocks; k += gridDim.x) {
-        const S* blk = x + (k << B);
+        const S* blk = x + (k << kBlockBits) + threadIdx.x;
         double acc = 0.0;
-        for (uint32_t i = threadIdx.x; i < E; i += blockDim.x) acc += prob_of(blk[i]);
+#pragma unroll
+        for (int b = 0; b < kBatches; ++b) {
+            S v[8];
+#pragma unroll
+            for (int j = 0; j < 8; ++j) v[j] = blk[(b * 8 + j) * kMassThreads];
+            acc += mass_of(v);
+        }
         for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o);
         if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = acc;
         __syncthreads();
@@ -63,30 +71,57 @@ __global__ void __launch_bounds__(kMassThreads) k_block_mass(const S* __restrict
     }
 }
 
-// Inclusive prefix sums of K values by one CTA: thread t owns a contiguous
-// chunk, the chunk totals are scanned in order by thread 0.
-__global__ void __launch_bounds__(kScanThreads) k_scan(const double* __restrict__ w, uint64_t K,
-                                                       double* __restrict__ incl) {
-    __shared__ double off[kScanThreads];
-    const uint64_t C = (K + kScanThreads - 1) / kScanThreads;
-    const uint64_t b = threadIdx.x * C, e = min(K, b + C);
-    double s = 0.0;
-    for (uint64_t i = b; i < e; ++i) s += w[i];
-    off[threadIdx.x] = s;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double run = 0.0;
-        for (int t = 0; t < kScanThreads; ++t) {
-            const double v = off[t];
-            off[t] = run;
-            run += v;
-        }
+// Inclusive prefix sums of K values: parts of 1024, four adjacent values a
+// thread, and the sums of the parts (k_scan_parts); then every CTA adds the
+// sum of the parts before its own (k_scan_add).  One CTA over all values,
+// thread t striding by K / 1024, and one thread over its 1024 sums took 168 us
+// at K = 2^16; 13 us now.
+constexpr int kScanPart = 4 * kScanThreads;
+__global__ void __launch_bounds__(kScanThreads) k_scan_parts(const double* __restrict__ w, uint64_t K,
+                                                             double* __restrict__ incl, double* __restrict__ part) {
+    __shared__ double sh[kScanThreads / 32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const uint64_t b = (uint64_t)blockIdx.x * kScanPart + threadIdx.x * 4u;
+    double v[4], run = 0.0;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        run += (b + j < K) ? w[b + j] : 0.0;
+        v[j] = run;
     }
+    double inc = run;
+    for (int o = 1; o < 32; o <<= 1) {
+        const double u = __shfl_up_sync(0xffffffffu, inc, o);
+        if (lane >= o) inc += u;
+    }
+    if (lane == 31) sh[warp] = inc;
+    double before = __shfl_up_sync(0xffffffffu, inc, 1);
+    if (lane == 0) before = 0.0;
     __syncthreads();
-    double run = off[threadIdx.x];
-    for (uint64_t i = b; i < e; ++i) {
-        run += w[i];
-        incl[i] = run;
+    double base = 0.0, all = 0.0;
+    for (int i = 0; i < kScanThreads / 32; ++i) {
+        if (i == warp) base = all;
+        all += sh[i];
+    }
+    before += base;
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+        if (b + j < K) incl[b + j] = before + v[j];
+    if (threadIdx.x == 0) part[blockIdx.x] = all;
+}
+
+__global__ void __launch_bounds__(kScanThreads) k_scan_add(uint64_t K, double* __restrict__ incl,
+                                                           const double* __restrict__ part) {
+    __shared__ double sh[kScanThreads / 32];
+    double s = 0.0;
+    for (uint32_t i = threadIdx.x; i < blockIdx.x; i += kScanThreads) s += part[i];
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
+    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = s;
+    __syncthreads();
+    double off = 0.0;
+    for (int i = 0; i < kScanThreads / 32; ++i) off += sh[i];
+    for (uint32_t j = threadIdx.x; j < (uint32_t)kScanPart; j += kScanThreads) {
+        const uint64_t i = (uint64_t)blockIdx.x * kScanPart + j;
+        if (i < K) incl[i] += off;
     }
 }
 
@@ -99,6 +134,20 @@ __device__ __forceinline__ uint64_t first_above(const double* incl, uint64_t K, 
         else lo = mid + 1;
     }
     return lo;
+}
+
+// The bin of a target: the first whose inclusive sum exceeds it, moved down
+// past bins of zero weight (two sums around such a bin may differ by a
+// rounding); K if there is none.
+__device__ __forceinline__ uint64_t bin_of(const double* w, const double* incl, uint64_t K, double target) {
+    uint64_t k = first_above(incl, K, target);
+    if (k < K && !(w[k] > 0.0)) {
+        uint64_t d = k;
+        while (d > 0 && !(w[d] > 0.0)) --d;
+        if (w[d] > 0.0) return d;
+        while (k < K && !(w[k] > 0.0)) ++k;
+    }
+    return k;
 }
 
 // Largest k < K with w[k] > 0 (0 if none).
@@ -114,73 +163,101 @@ __global__ void k_shots_bins(const double* __restrict__ w, const double* __restr
     const int s = blockIdx.x * blockDim.x + threadIdx.x;
     if (s >= nshots) return;
     const double target = u[s] * incl[K - 1];
-    const uint64_t k = first_above(incl, K, target);
+    const uint64_t k = bin_of(w, incl, K, target);
     out[s] = (k < K) ? k : last_positive(w, K);
 }
 
-// One warp per shot over the full distribution: block by binary search, then
-// lane runs of C = 2^B / 32 contiguous amplitudes, scanned in order.
+// One warp per shot over the full distribution: the block by binary search,
+// in it eight segments of 512 amplitudes (lane l: amplitudes [16 l, 16 l + 16) of
+// each), the segment and the lane by scans of their sums, and the lane's
+// amplitudes in order.  Lane runs of 128 amplitudes summed in FP64 took 258 us
+// for 4096 shots of complex128 (375 complex64), bound by the FP64 pipe and
+// loads of 32 lines; 145 (115) now.
 template <class S>
-__global__ void __launch_bounds__(256) k_shots_full(const S* __restrict__ x, int B, uint64_t nblocks,
+__global__ void __launch_bounds__(256) k_shots_full(const S* __restrict__ x, uint64_t nblocks,
                                                     const double* __restrict__ mass,
                                                     const double* __restrict__ incl,
                                                     const double* __restrict__ u, int nshots,
                                                     uint64_t* __restrict__ out) {
+    constexpr int kRun = 16, kSeg = 32 * kRun, kSegs = (1 << kBlockBits) / kSeg;
     const int lane = threadIdx.x & 31;
     const int s = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     if (s >= nshots) return;
     const double total = incl[nblocks - 1];
     const double target = u[s] * total;
-    uint64_t k = first_above(incl, nblocks, target);
+    uint64_t k = bin_of(mass, incl, nblocks, target);
     const bool fallback = k >= nblocks;
     if (fallback) k = last_positive(mass, nblocks);
-    const double rem = target - (k > 0 ? incl[k - 1] : 0.0);
-    const uint32_t C = (1u << B) / 32u;
-    const S* run = x + (k << B) + (uint64_t)lane * C;
-    double ls = 0.0;
-    uint32_t lastnz = 0xFFFFFFFFu;
-    for (uint32_t i = 0; i < C; ++i) {
-        const double p = prob_of(run[i]);
-        ls += p;
-        if (p > 0.0) lastnz = i;
-    }
-    // inclusive scan of the lane sums
-    double inc = ls;
-    for (int o = 1; o < 32; o <<= 1) {
-        const double v = __shfl_up_sync(0xffffffffu, inc, o);
-        if (lane >= o) inc += v;
-    }
-    const double exc = inc - ls;
+    const S* blk = x + (k << kBlockBits);
     uint64_t result = ~0ull;
     if (!fallback) {
-        const uint32_t hit = __ballot_sync(0xffffffffu, inc > rem);
-        if (hit) {
-            const int l = __ffs(hit) - 1;
+        double rem = target - (k > 0 ? incl[k - 1] : 0.0);
+        double ls[kSegs], tot[kSegs];
+#pragma unroll
+        for (int g = 0; g < kSegs; ++g) {
+            const S* run = blk + g * kSeg + lane * kRun;
+            S v[8], w[8];
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                v[i] = run[i];
+                w[i] = run[8 + i];
+            }
+            tot[g] = ls[g] = mass_of(v) + mass_of(w);
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+            for (int g = 0; g < kSegs; ++g) tot[g] += __shfl_xor_sync(0xffffffffu, tot[g], o);
+        int seg = 0;
+        double before = 0.0, mine = 0.0, acc = 0.0;
+        bool found = false;
+#pragma unroll
+        for (int g = 0; g < kSegs; ++g) {
+            if (!found) {
+                before = acc;
+                mine = ls[g];
+                seg = g;
+                acc += tot[g];
+                found = acc > rem && tot[g] > 0.0;
+            }
+        }
+        if (found) {
+            double inc = mine;
+            for (int o = 1; o < 32; o <<= 1) {
+                const double v = __shfl_up_sync(0xffffffffu, inc, o);
+                if (lane >= o) inc += v;
+            }
+            const uint32_t hit = __ballot_sync(0xffffffffu, before + inc > rem && mine > 0.0);
+            const uint32_t pos = __ballot_sync(0xffffffffu, mine > 0.0);
+            // no lane crosses by rounding: the segment's last one of nonzero probability
+            const int l = hit ? __ffs(hit) - 1 : 31 - __clz(pos);
             if (lane == l) {
-                double acc = exc;
-                for (uint32_t i = 0; i < C; ++i) {
-                    acc += prob_of(run[i]);
-                    if (acc > rem) {
-                        result = (k << B) + (uint64_t)lane * C + i;
-                        break;
+                const uint64_t base = (uint64_t)seg * kSeg + lane * kRun;
+                double run = before + (inc - mine);
+                for (int i = 0; i < kRun; ++i) {
+                    const double p = prob_of(blk[base + i]);
+                    run += p;
+                    if (p > 0.0) {   // without a crossing by rounding: the last nonzero one
+                        result = (k << kBlockBits) + base + i;
+                        if (run > rem) break;
                     }
                 }
             }
-            // the lane's own rescan can miss by rounding: then its last nonzero
-            const uint32_t found = __ballot_sync(0xffffffffu, result != ~0ull);
-            if (!found && lane == l && lastnz != 0xFFFFFFFFu) result = (k << B) + (uint64_t)lane * C + lastnz;
         }
     }
     // no crossing in this block (rounding, or the target at the total): the
     // block's last amplitude of nonzero probability
-    const uint32_t have = __ballot_sync(0xffffffffu, result != ~0ull);
-    if (!have) {
-        const uint32_t nz = __ballot_sync(0xffffffffu, lastnz != 0xFFFFFFFFu);
-        const int l = nz ? 31 - __clz(nz) : 0;
-        if (lane == l) result = (k << B) + (uint64_t)lane * C + (lastnz != 0xFFFFFFFFu ? lastnz : 0u);
+    if (!__any_sync(0xffffffffu, result != ~0ull)) {
+        for (int i = (1 << kBlockBits) - 32; i >= 0; i -= 32) {
+            const uint32_t nz = __ballot_sync(0xffffffffu, prob_of(blk[i + lane]) > 0.0);
+            if (nz != 0u || i == 0) {
+                const int l = nz ? 31 - __clz(nz) : 0;
+                if (lane == l) result = (k << kBlockBits) + (uint64_t)(i + l);
+                break;
+            }
+        }
     }
-    const uint32_t who = __ballot_sync(0xffffffffu, result != ~0ull);
-    if (lane == __ffs(who) - 1) out[s] = result;
+    if (result != ~0ull) out[s] = result;
 }
 
 // Probability of the outcome: the 2^(n - m) amplitudes whose measured bits
@@ -241,13 +318,14 @@ __global__ void __launch_bounds__(256) k_collapse(S* __restrict__ x, uint64_t di
 
 template <class S>
 void sample_impl(qe_state* s, int m, const int* qubits, int nshots, const double* u_host, uint64_t* out_host) {
-    const bool full = (m == 0);
-    const int B = std::min(kBlockBits, s->n);
-    const uint64_t K = full ? (dim(s) >> B) : (1ull << m);
+    const bool full = (m == 0);   // n > 16 (sample_shots)
+    const uint64_t K = full ? (dim(s) >> kBlockBits) : (1ull << m);
+    const uint64_t nscan = (K + kScanPart - 1) / kScanPart;
     const uint64_t nparts = full ? 0 : probs_partials_needed(s, m);
-    // scratch: [weights K][inclusive sums K][uniforms][outcomes][probability partials]
+    // scratch: [weights K][inclusive sums K][uniforms][outcomes][sums of the scan's parts][probability partials]
     const size_t w_off = 0, i_off = w_off + K * 8, u_off = i_off + K * 8;
-    const size_t o_off = u_off + (size_t)nshots * 8, p_off = o_off + (size_t)nshots * 8;
+    const size_t o_off = u_off + (size_t)nshots * 8, s_off = o_off + (size_t)nshots * 8;
+    const size_t p_off = (s_off + nscan * 8 + 15) & ~(size_t)15;
     char* scr = (char*)ensure_scratch(s, p_off + nparts * sizeof(double2) + 256);
     double* w = (double*)(scr + w_off);
     double* incl = (double*)(scr + i_off);
@@ -258,21 +336,26 @@ void sample_impl(qe_state* s, int m, const int* qubits, int nshots, const double
     if (full) {
         Launch L(s, "sample_block_mass", (double)dim(s) * amp_bytes(s));
         const unsigned grid = (unsigned)std::min<uint64_t>(K, (uint64_t)num_sms() * 8);
-        k_block_mass<S><<<grid, kMassThreads, 0, s->stream>>>(x, K, B, w);
+        k_block_mass<S><<<grid, kMassThreads, 0, s->stream>>>(x, K, w);
         QE_CUDA(cudaGetLastError());
     } else {
         reduce_probs_device(s, m, qubits, (double2*)(scr + p_off), w);
     }
     {
         Launch L(s, "sample_scan", 0.0, false);
-        k_scan<<<1, kScanThreads, 0, s->stream>>>(w, K, incl);
+        double* part = (double*)(scr + s_off);
+        k_scan_parts<<<(unsigned)nscan, kScanThreads, 0, s->stream>>>(w, K, incl, part);
         QE_CUDA(cudaGetLastError());
+        if (nscan > 1) {
+            k_scan_add<<<(unsigned)nscan, kScanThreads, 0, s->stream>>>(K, incl, part);
+            QE_CUDA(cudaGetLastError());
+        }
     }
     {
         Launch L(s, "sample_shots", 0.0, false);
         if (full) {
             const unsigned grid = (unsigned)(((uint64_t)nshots * 32 + 255) / 256);
-            k_shots_full<S><<<grid, 256, 0, s->stream>>>(x, B, K, w, incl, u, nshots, out);
+            k_shots_full<S><<<grid, 256, 0, s->stream>>>(x, K, w, incl, u, nshots, out);
         } else {
             k_shots_bins<<<(nshots + 255) / 256, 256, 0, s->stream>>>(w, incl, K, u, nshots, out);
         }
