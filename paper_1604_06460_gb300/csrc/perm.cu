@@ -53,6 +53,7 @@ struct WalkArgs {
     uint64_t columns;     // columns walked: all 2^(n-m), or those whose low kb bits lie in [off0, off0 + len)
     uint64_t off0, len;
     int kb;
+    int columns_log2, g_log2;   // columns_log2: kb = 0
     uint64_t g;           // cycles per column: gcd(c, 2^m)
     uint64_t nseg;        // segments per cycle
     uint64_t seg_len;     // cycle positions per segment
@@ -84,11 +85,17 @@ __device__ __forceinline__ uint64_t reg_deposit(const WalkArgs<S>& a, uint64_t r
 template <class S>
 __device__ __forceinline__ void walk_item(const WalkArgs<S>& a, uint64_t t, uint64_t& x0,
                                           uint64_t& start, uint64_t& seg) {
-    const uint64_t ci = t % a.columns;
-    const uint64_t col = ((ci / a.len) << a.kb) | (a.off0 + ci % a.len);
-    const uint64_t rest = t / a.columns;
-    start = rest % a.g;
-    seg = rest / a.g;
+    uint64_t col, rest;
+    if (a.kb == 0) {   // all columns, a power of two: no divisions
+        col = t & (a.columns - 1ull);
+        rest = t >> a.columns_log2;
+    } else {
+        const uint64_t ci = t % a.columns;
+        col = ((ci / a.len) << a.kb) | (a.off0 + ci % a.len);
+        rest = t / a.columns;
+    }
+    start = rest & (a.g - 1ull);
+    seg = rest >> a.g_log2;
     x0 = insert_zero_bits(col, a.reg_sorted, a.m);
 }
 
@@ -239,7 +246,8 @@ WalkArgs<S> walk_args(qe_state* s, int m, const int* qubits, uint64_t c, bool co
     a.mmask = (m >= 64) ? ~0ull : ((1ull << m) - 1ull);
     a.contiguous = contiguous;
     a.lo = qubits[0];
-    a.g = 1ull << __builtin_ctzll(c);   // gcd(c, 2^m)
+    a.g_log2 = __builtin_ctzll(c);
+    a.g = 1ull << a.g_log2;   // gcd(c, 2^m)
     a.cycle_len = (a.mmask >> __builtin_ctzll(c)) + 1ull;
     int tmp[64];
     for (int j = 0; j < m; ++j) tmp[j] = a.reg[j] = (uint8_t)qubits[j];
@@ -257,6 +265,7 @@ void walk_columns(WalkArgs<S>& a, int n, int kb, uint64_t off, uint64_t len) {
     a.off0 = off;
     a.len = len;
     a.columns = len << (n - a.m - kb);
+    a.columns_log2 = n - a.m;
     const uint64_t want = (uint64_t)num_sms() * 2048;
     const uint64_t base_items = a.columns * a.g;
     uint64_t nseg = (want + base_items - 1) / base_items;
