@@ -16,8 +16,15 @@
 //     bit = logical bit ^ flip") instead of being moved.  |kappa| <= 1, and
 //     two real multiply-adds an amplitude and gate replace the eight of the
 //     complex 2 x 2 matrix RZ RY.
+//   - The scales of all rotations (and the deviation of the rounded RZ phases
+//     from modulus one, the same for both slot bits) are one number of the
+//     circuit: the host keeps the squared norm of the unscaled state as a pair
+//     of FP64 numbers and the energy is divided by it; only its power of two
+//     is taken out of the amplitudes, exactly, layer by layer.  Scales folded
+//     into rounded factors put the energies off by 2e-14 (double-float) and
+//     3e-15 (FP64) relative; 0.5 to 1.5e-14 and 1.5e-15 without.
 //   - The diagonal of the layer is the product over the qubits of a factor for
-//     each slot bit (the scale, the sign of the flip and the RZ phase) times
+//     each slot bit (the sign of the flip and the RZ phase) times
 //     (-1)^popcount(x & x >> 1) for logical x.  Two tables of at most 64 and
 //     128 partial products (and one scalar for the bits outside a tile) give
 //     an amplitude's factor with one complex product.
@@ -26,7 +33,7 @@
 // Double-float values keep (re, im) of the high and of the low words in packed
 // pairs, so that one f32x2 instruction serves both components.
 // 512 circuits of 10..22 qubits, 8 layers: complex128 double-float 242 ms with
-// the complex matrices, 72 ms so; FP64 1030 and 215 ms (its pipe's rate);
+// the complex matrices, 74 ms so; FP64 1030 and 215 ms (its pipe's rate);
 // complex64 66 and 25 ms.
 //
 // Work decomposition (one work queue, claimed in order with an atomic head):
@@ -81,6 +88,7 @@ struct Circ {
     uint64_t state_off; // amplitude offset of its HBM state (large circuits)
     uint64_t u_off;     // offset of its rotations (layers * n entries)
     uint64_t f_off;     // offset of its flip masks (layers entries)
+    double scale2;      // its energy / the energy of the kept amplitudes
 };
 
 // ------------------------------------------------- packed pairs of floats
@@ -128,6 +136,11 @@ __device__ __forceinline__ f2 fma2(f2 a, f2 b, f2 c) {
 struct BF32 {
     using V = f2;
     using K = float;
+    using F = V;                             // a diagonal's factor
+    static F make_f(double re, double im) { return make_v(re, im); }
+    static double kept(double x) { return (double)(float)x; }
+    __device__ __forceinline__ static F fmul(const F& a, const F& b) { return cmul(a, b); }
+    __device__ __forceinline__ static V to_v(const F& f) { return f; }
     static constexpr int kGroup = 4;         // bits per register group
     static constexpr int kSw = 4;            // swizzle: 16 8-byte slots a row
     struct R { f2 k, nk; };
@@ -140,7 +153,7 @@ struct BF32 {
         return r;
     }
     __device__ __forceinline__ static R expand(K k) { return R{dup2(k), dup2(-k)}; }
-    __device__ __forceinline__ static V one() { return pack2(1.f, 0.f); }
+    __device__ __forceinline__ static F one() { return pack2(1.f, 0.f); }
     __device__ __forceinline__ static void rot(V& a, V& b, const R& r) {
         const V p = fma2(r.k, b, a);
         b = fma2(r.nk, a, b);
@@ -168,6 +181,19 @@ __device__ __forceinline__ void two_sum(f2 a, f2 b, f2& s, f2& e) {
 struct BDF {
     struct alignas(16) V { f2 h, l; };
     using K = float2;                        // (high, low)
+    // The diagonal's factors, few and shared by many amplitudes, are multiplied
+    // in FP64 (idle otherwise) and split once: a pair product's error of about
+    // 2^-47 in a table entry would not average out over the amplitudes.
+    using F = double2;
+    static F make_f(double re, double im) { return make_double2(re, im); }
+    static double kept(double x) { return x; }
+    __device__ __forceinline__ static F fmul(const F& a, const F& b) {
+        return make_double2(__fma_rn(a.x, b.x, -__dmul_rn(a.y, b.y)), __fma_rn(a.x, b.y, __dmul_rn(a.y, b.x)));
+    }
+    __device__ __forceinline__ static V to_v(const F& f) {
+        const float x = (float)f.x, y = (float)f.y;
+        return V{pack2(x, y), pack2((float)__dsub_rn(f.x, (double)x), (float)__dsub_rn(f.y, (double)y))};
+    }
     static constexpr int kGroup = 3;
     static constexpr int kSw = 3;            // 8 16-byte slots a row
     struct R { f2 h, l; };
@@ -185,7 +211,7 @@ struct BDF {
         return r;
     }
     __device__ __forceinline__ static R expand(K k) { return R{dup2(k.x), dup2(k.y)}; }
-    __device__ __forceinline__ static V one() { return V{pack2(1.f, 0.f), 0ull}; }
+    __device__ __forceinline__ static F one() { return make_double2(1.0, 0.0); }
     // v + k u: the product's high part exactly (its negative n, so that the
     // residual is one fused multiply-add), the cross terms in FP32, TwoSum
     __device__ __forceinline__ static V madd(const V& v, f2 kh, f2 kl, f2 nkh, const V& u) {
@@ -243,8 +269,13 @@ struct BF64 {
     static K make_k(double k) { return k; }
     static double value(K k) { return k; }
     static V make_v(double re, double im) { return make_double2(re, im); }
+    using F = V;
+    static F make_f(double re, double im) { return make_double2(re, im); }
+    static double kept(double x) { return x; }
+    __device__ __forceinline__ static F fmul(const F& a, const F& b) { return cmul(a, b); }
+    __device__ __forceinline__ static V to_v(const F& f) { return f; }
     __device__ __forceinline__ static R expand(K k) { return k; }
-    __device__ __forceinline__ static V one() { return make_double2(1.0, 0.0); }
+    __device__ __forceinline__ static F one() { return make_double2(1.0, 0.0); }
     __device__ __forceinline__ static void rot(V& a, V& b, R k) {
         const V p = make_double2(__fma_rn(k, b.x, a.x), __fma_rn(k, b.y, a.y));
         b = make_double2(__fma_rn(-k, a.x, b.x), __fma_rn(-k, a.y, b.y));
@@ -322,7 +353,7 @@ template <class P>
 struct BatchArgs {
     typename P::V* states;
     const typename P::K* kap;      // kappa per (circuit, layer, qubit)
-    const typename P::V* fac;      // factors per (circuit, layer, qubit, slot bit)
+    const typename P::F* fac;      // factors per (circuit, layer, qubit, slot bit)
     const uint32_t* flips;         // per (circuit, layer): slot ^ logical
     const Item* items;
     const Circ* circ;
@@ -540,37 +571,37 @@ __device__ void run_energy(Group<P> g, int b0, int cnt, bool z, int n, EAcc<P>& 
 // Partial products of the factors (2 per qubit) over the local bits 0..5 and
 // 6..nb-1, and (by the last warp) the product over the tile's bits into *tf.
 template <class P>
-__device__ void build_tables(const Layout& lay, const typename P::V* fac, typename P::V* tabA, typename P::V* tabB) {
+__device__ void build_tables(const Layout& lay, const typename P::F* fac, typename P::V* tabA, typename P::V* tabB) {
     const int na = lay.nb < 6 ? lay.nb : 6;
     const int ta = 1 << na, tb = 1 << (lay.nb - na);
     for (int i = threadIdx.x; i < ta + tb; i += blockDim.x) {
         const bool low = i < ta;
         const uint32_t e = low ? i : i - ta;
         const int j0 = low ? 0 : na, cnt = low ? na : lay.nb - na;
-        typename P::V w = P::one();
+        typename P::F w = P::one();
         for (int j = 0; j < cnt; ++j) {
-            const typename P::V f = fac[2 * lay.qubit(j0 + j) + ((e >> j) & 1u)];
-            w = j == 0 ? f : P::cmul(f, w);
+            const typename P::F f = fac[2 * lay.qubit(j0 + j) + ((e >> j) & 1u)];
+            w = j == 0 ? f : P::fmul(f, w);
         }
-        if (low) tabA[e] = w;
-        else tabB[e] = w;
+        if (low) tabA[e] = P::to_v(w);
+        else tabB[e] = P::to_v(w);
     }
 }
 template <class P>
-__device__ void build_tile_factor(const Layout& lay, const typename P::V* fac, uint32_t t, typename P::V* tf) {
+__device__ void build_tile_factor(const Layout& lay, const typename P::F* fac, uint32_t t, typename P::V* tf) {
     const int last = (blockDim.x >> 5) - 1;
     if ((int)(threadIdx.x >> 5) != last) return;
     const int lane = threadIdx.x & 31;
-    typename P::V w = lane < lay.nt ? fac[2 * (lay.tq + lane) + ((t >> lane) & 1u)] : P::one();
+    typename P::F w = lane < lay.nt ? fac[2 * (lay.tq + lane) + ((t >> lane) & 1u)] : P::one();
     for (int o = 1; o < lay.nt; o <<= 1) {
-        typename P::V u;
+        typename P::F u;
         const uint32_t* s = reinterpret_cast<const uint32_t*>(&w);
         uint32_t* d = reinterpret_cast<uint32_t*>(&u);
 #pragma unroll
         for (int k = 0; k < (int)(sizeof(w) / 4); ++k) d[k] = __shfl_xor_sync(0xffffffffu, s[k], o);
-        w = P::cmul(u, w);
+        w = P::fmul(u, w);
     }
-    if (lane == 0) *tf = w;
+    if (lane == 0) *tf = P::to_v(w);
 }
 
 // Block-wide sum; result valid in thread 0.
@@ -627,7 +658,7 @@ __global__ void __maxnreg__(128) k_batch(const __grid_constant__ BatchArgs<P> a)
         __syncthreads();
         if (!s_ok) continue;
         const typename P::K* kap = a.kap + cc.u_off;
-        const V* fac = a.fac + 2 * cc.u_off;
+        const typename P::F* fac = a.fac + 2 * cc.u_off;
         const uint32_t* flips = a.flips + cc.f_off;
         EAcc<P> acc;
         Group<P> g;
@@ -659,7 +690,7 @@ __global__ void __maxnreg__(128) k_batch(const __grid_constant__ BatchArgs<P> a)
             run_energy<P>(g, 0, n, true, n, acc);
             const double z = block_sum(acc.z(), shred);
             const double x = block_sum(acc.x(), shred);
-            if (threadIdx.x == 0) a.energies[it.circuit] = z + 2.0 * a.hx * x;
+            if (threadIdx.x == 0) a.energies[it.circuit] = (z + 2.0 * a.hx * x) * cc.scale2;
             __syncthreads();
             continue;
         }
@@ -721,7 +752,7 @@ __global__ void __maxnreg__(128) k_batch(const __grid_constant__ BatchArgs<P> a)
                     zsum += p.x;
                     xsum += p.y;
                 }
-                a.energies[it.circuit] = zsum + 2.0 * a.hx * xsum;
+                a.energies[it.circuit] = (zsum + 2.0 * a.hx * xsum) * cc.scale2;
             }
         }
         __syncthreads();
@@ -736,20 +767,35 @@ namespace qe {
 
 namespace {
 
+// A product of sums of two squares in twice FP64's precision (hundreds of
+// factors: FP64 roundings alone would add 5e-15).
+struct Pair {
+    double h = 1.0, l = 0.0;
+    void times_squares(double a, double b) {
+        const double aa = a * a, bb = b * b, s = aa + bb, t = s - aa;
+        const double e = ((aa - (s - t)) + (bb - t)) + (std::fma(a, a, -aa) + std::fma(b, b, -bb));
+        const double p = h * s, q = std::fma(h, s, -p) + (h * e + l * s);
+        h = p + q;
+        l = q - (h - p);
+    }
+};
+
 // Host side of a layer: kappa, the slot factors and the flips of every
 // rotation (see the top of the file), angles in qe_batch_create's order.
 template <class P>
-void upload_rotations(qe_batch* b, std::vector<uint64_t>& u_off) {
+void upload_rotations(qe_batch* b, std::vector<uint64_t>& u_off, std::vector<double>& scale2) {
     u_off.resize(b->count);
+    scale2.assign(b->count, 1.0);
     const size_t total = b->angles.size() / 2;
     std::vector<typename P::K> kap(total);
-    std::vector<typename P::V> fac(2 * total);
+    std::vector<typename P::F> fac(2 * total);
     std::vector<uint32_t> flips((size_t)b->count * b->layers);
     size_t i = 0;
     for (int c = 0; c < b->count; ++c) {
         const int n = b->n[c];
         u_off[c] = i;
         uint32_t flip = 0;
+        Pair norm;   // squared norm of the kept state, true state = kept / sqrt(norm)
         for (int l = 0; l < b->layers; ++l) {
             for (int q = 0; q < n; ++q, ++i) {
                 const double th = b->angles[2 * i], ph = b->angles[2 * i + 1];
@@ -759,18 +805,28 @@ void upload_rotations(qe_batch* b, std::vector<uint64_t>& u_off) {
                 const bool trade = std::fabs(sn) > std::fabs(cs);
                 kap[i] = P::make_k(trade ? cs / sn : -sn / cs);
                 const double k = P::value(kap[i]);
-                const double mag = 1.0 / std::sqrt(1.0 + k * k);
                 if (trade) flip ^= 1u << q;
-                // scales of slots 0 and 1: (c, c), or (s, -s) when traded
-                double f0 = std::copysign(mag, trade ? sn : cs), f1 = trade ? -f0 : f0;
+                // signs of slots 0 and 1: those of (c, c), or of (s, -s) when traded
+                double f0 = std::copysign(1.0, trade ? sn : cs), f1 = trade ? -f0 : f0;
                 if (l == 0) f1 *= -k;            // the product state: (p, q) of (1, 0)
                 const double pc = std::cos(0.5 * ph), ps = std::sin(0.5 * ph);
                 const double s0 = ((flip >> q) & 1u) ? ps : -ps;   // slot 0's logical bit is the flip
-                fac[2 * i] = P::make_v(f0 * pc, f0 * s0);
-                fac[2 * i + 1] = P::make_v(f1 * pc, -f1 * s0);
+                // the squared norm's power of two, out of the layer's first factors
+                double two = 1.0;
+                if (q == 0 && std::isfinite(norm.h)) {
+                    const int e = std::ilogb(norm.h) / 2;
+                    two = std::ldexp(1.0, -e);
+                    norm.h = std::ldexp(norm.h, -2 * e);
+                    norm.l = std::ldexp(norm.l, -2 * e);
+                }
+                fac[2 * i] = P::make_f(two * f0 * pc, two * f0 * s0);
+                fac[2 * i + 1] = P::make_f(two * f1 * pc, -two * f1 * s0);
+                norm.times_squares(1.0, k);
+                norm.times_squares(P::kept(pc), P::kept(ps));   // both slots' modulus
             }
             flips[(size_t)c * b->layers + l] = flip;
         }
+        scale2[c] = 1.0 / norm.h;
     }
     const size_t fb = fac.size() * sizeof(fac[0]), kb = kap.size() * sizeof(kap[0]);
     if (b->fac) cudaFree(b->fac);
@@ -796,7 +852,8 @@ template <class P>
 void build_plan(qe_batch* b) {
     const int T = b->plan.T;
     std::vector<uint64_t> u_off;
-    upload_rotations<P>(b, u_off);
+    std::vector<double> scale2;
+    upload_rotations<P>(b, u_off, scale2);
     std::vector<Circ> circ(b->count);
     std::vector<Item> items;
     uint64_t state_off = 0;
@@ -806,6 +863,7 @@ void build_plan(qe_batch* b) {
         Circ& cc = circ[c];
         cc.n = b->n[c];
         cc.u_off = u_off[c];
+        cc.scale2 = scale2[c];
         cc.f_off = (uint64_t)c * b->layers;
         cc.state_off = 0;
         if (cc.n <= T) {
@@ -930,7 +988,7 @@ void capture(qe_batch* b) {
     static thread_local BatchArgs<P> a;
     a.states = reinterpret_cast<typename P::V*>(b->states);
     a.kap = reinterpret_cast<const typename P::K*>(b->kap);
-    a.fac = reinterpret_cast<const typename P::V*>(b->fac);
+    a.fac = reinterpret_cast<const typename P::F*>(b->fac);
     a.flips = b->flips;
     a.items = reinterpret_cast<const Item*>(b->items);
     a.circ = reinterpret_cast<const Circ*>(b->circ);
