@@ -351,7 +351,7 @@ KERNEL_SOURCES = {
     "digitrev": ["fft.cu", "qe_arith.cuh"],
     "gate_tc_k5": ["tcgen05.cu", "qe_tc.cuh", "qe_arith.cuh"],
     "gate_direct": ["gates.cu", "qe_arith.cuh"],
-    "expect_fx": ["reduce.cu", "qe_oz.cuh", "qe_tc.cuh", "qe_arith.cuh"],
+    "expect_fx": ["reduce.cu", "expect.cu", "qe_oz.cuh", "qe_tc.cuh", "qe_arith.cuh"],
     "fft": ["fft.cu", "qe_arith.cuh"],
 }
 

@@ -237,6 +237,17 @@ struct DF {
 // bits: one conversion and two multiplications in FP64 for the N amplitudes.
 // Components that the window cannot hold (E below 64, infinities, NaN) take the
 // FP64 sum.
+// (C shifts by 64 or 32 and more are undefined, PTX's give 0)
+__device__ __forceinline__ uint64_t shift_down(uint64_t v, uint32_t d) {
+    uint64_t r;
+    asm("shr.u64 %0, %1, %2;" : "=l"(r) : "l"(v), "r"(d));
+    return r;
+}
+__device__ __forceinline__ uint32_t shift_down(uint32_t v, uint32_t d) {
+    uint32_t r;
+    asm("shr.u32 %0, %1, %2;" : "=r"(r) : "r"(v), "r"(d));
+    return r;
+}
 __device__ __forceinline__ double mass_f64(double re, double im, double s) {
     return __fma_rn(re, re, __fma_rn(im, im, s));
 }
@@ -272,7 +283,7 @@ __device__ __forceinline__ double mass_of(const double2 (&v)[N]) {
     auto take = [&](double c) {
         const uint32_t hi = (uint32_t)__double2hiint(c), lo = (uint32_t)__double2loint(c);
         const uint64_t m4 = ((((uint64_t)((hi & 0xFFFFFu) | 0x100000u)) << 32) | lo) << 2;
-        const uint64_t t = (m4 >> min(E - ((hi >> 20) & 0x7FFu), 63u)) + 1u;   // 2 q, its last bit to drop
+        const uint64_t t = shift_down(m4, E - ((hi & 0x7FFFFFFFu) >> 20)) + 1u;   // 2 q, its last bit to drop
         a.add((uint32_t)(t >> 29), (uint32_t)t & 0x1FFFFFFEu);
     };
 #pragma unroll
@@ -300,7 +311,7 @@ __device__ __forceinline__ double mass_of(const float2 (&v)[N]) {
     auto take = [&](float c) {
         const uint32_t b = __float_as_uint(c);
         const uint64_t m = (uint64_t)((b & 0x7FFFFFu) | 0x800000u) << 31;
-        const uint64_t t = m >> min(E - ((b >> 23) & 0xFFu), 63u);
+        const uint64_t t = shift_down(m, E - ((b & 0x7FFFFFFFu) >> 23));
         a.add((uint32_t)(t >> 29), (uint32_t)t & 0x1FFFFFFEu);
     };
 #pragma unroll

@@ -172,6 +172,11 @@ int choose_fusion_width(qe_state* s, const std::vector<PendingGate>& queue);
 
 // reductions (synchronise the stream)
 double reduce_norm2(qe_state* s);
+// expectation by passes over register sets of four qubits (large states, terms
+// of at most four X/Y qubits); false where another path has to take it.
+// `other`: the launches of that path
+bool expect_sets(qe_state* s, int nterms, const uint64_t* xm, const uint64_t* zm, const double* cf, size_t other,
+                 double* out);
 double reduce_expectation(qe_state* s, int nterms, const uint64_t* xm, const uint64_t* zm,
                           const double* cf);
 void reduce_probs(qe_state* s, int m, const int* qubits, double* out);

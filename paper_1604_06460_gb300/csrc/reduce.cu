@@ -16,6 +16,7 @@
 // the register rounds are computed in exact fixed point instead, in either
 // mode (k_expect_fx).
 #include <algorithm>
+#include <cstdint>
 #include <cstdlib>
 #include <type_traits>
 #include <vector>
@@ -32,11 +33,11 @@ constexpr int kRThreads = 256;
 
 // Expectation kernel choice (a test and measurement switch, read per call):
 // QE_EXPECT_TILE=1 keeps every expectation on the pair-indexed tile kernel,
-// =2 takes the register-round kernel whenever the terms fit it; otherwise it
-// is taken when it needs no more launches.
+// =2 takes the register-round kernel whenever the terms fit it, =3 the register
+// sets (expect.cu) whenever they do; otherwise the cheaper one is taken.
 int expect_kernel_switch() {
     const char* e = std::getenv("QE_EXPECT_TILE");
-    return (e && (e[0] == '1' || e[0] == '2')) ? e[0] - '0' : 0;
+    return (e && e[0] >= '1' && e[0] <= '3') ? e[0] - '0' : 0;
 }
 
 // ------------------------------------------------ compensated accumulators
@@ -1705,9 +1706,13 @@ double expect_impl(qe_state* s, int nterms, const uint64_t* xm, const uint64_t* 
     if (const int sw = expect_kernel_switch(); sw != 1) {
         constexpr bool kFx = sizeof(S) == 16;
         std::vector<RoundLaunch> rl;
-        if (plan_rounds(n, nterms, xm, cf, zchunks, rl) && !rl.empty() &&
-            (sw == 2 || kFx || rl.size() <= plans.size() + (size_t)nwide))
-            return expect_rounds<S, NAT>(s, rl, xm, zm, wv);
+        const bool rounds = plan_rounds(n, nterms, xm, cf, zchunks, rl) && !rl.empty() &&
+                            (sw == 2 || kFx || rl.size() <= plans.size() + (size_t)nwide);
+        // large states by register sets, where that is cheaper
+        double e = 0.0;
+        const size_t other = sw == 3 ? SIZE_MAX : rounds ? rl.size() : plans.size() + (size_t)nwide;
+        if (sw != 2 && expect_sets(s, nterms, xm, zm, cf, other, &e)) return e;
+        if (rounds) return expect_rounds<S, NAT>(s, rl, xm, zm, wv);
     }
     uint64_t max_grid = (uint64_t)num_sms() * 8;
     std::vector<unsigned> grids(plans.size());
