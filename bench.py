@@ -72,14 +72,14 @@ KERNEL_CASES = {
                "3 passes",
     "tc64": "complex64 5-qubit block on qubits (3,7,11,15,19) of a 26-qubit state, 3 passes",
     "direct2": "complex128 2-qubit block on qubits (5,17) of a 26-qubit state (fusion width 2), 3 passes",
-    "expect": "TFIM energy of a 26-qubit complex128 state (fixed-point register rounds), 2 evaluations",
+    "expect": "TFIM energy of a 26-qubit complex128 state (fixed point, register sets), 2 evaluations",
     "fft": "emulated 25-qubit QFT of a complex128 state, FP64 mode (5-qubit digit passes), 2 transforms",
-    "fftdf": "emulated 26-qubit QFT of a complex128 state, double-float mode (radix-2 shared-memory passes), "
+    "fftdf": "emulated 26-qubit QFT of a complex128 state, double-float mode (digit passes), "
              "2 transforms",
     "qpegemm": "one squaring of a 2^10 x 2^10 complex128 matrix on the tensor cores (digit splitting + product), "
                "2 products",
-    "addc": "emulated add-constant on qubits [0,16) of a 26-qubit complex128 state (1 MiB slices, eight CTAs "
-            "each, bulk copies), 2 additions",
+    "addc": "emulated add-constant on qubits [0,16) of a 26-qubit complex128 state (1 MiB slices, sixteen "
+            "CTAs each, bulk copies), 2 additions",
     "mul": "emulated multiplication c += a b of 8-qubit registers (index = a b c) of a 26-qubit complex128 "
            "state (planes in shared memory), 2 multiplications",
     "batch": "512 ansatz circuits, n ~ U{10..20}, 8 layers, TFIM energy each, complex128 double-float, "

@@ -148,7 +148,7 @@ int qe_apply_add_const(qe_state* s, int m, const int* qubits, uint64_t c);
  *     QE_POLICY_SIMULATE.
  * Both are permutations of the amplitudes, bit-exact.  A permutation whose
  * plane (the 2^N values of c, or the 2^(2N) of (a, c)) exceeds 64 KB goes
- * through a device scratch buffer of at most 1 GiB owned by the state.
+ * through a device scratch buffer owned by the state, 32 MiB or two planes.
  * QE_ERR_ARG for N out of range, a qubit >= n, a repeated qubit or
  * overlapping registers. */
 int qe_apply_mul(qe_state* s, int N, const int* qa, const int* qb, const int* qc);
@@ -157,15 +157,16 @@ int qe_apply_div(qe_state* s, int N, const int* qa, const int* qb, const int* qc
 /* <psi| sum_t coeff[t] P_t |psi> for Pauli strings P_t given by bit masks
  * over the qubits: (x,z) = (0,0) I, (1,0) X, (0,1) Z, (1,1) Y (Sec. III-D:
  * the expectation computed in one step instead of by repeated sampling).
- * complex128 states, terms whose X/Y bits below qubit 12 lie in one of the
- * triples {0,1,2} .. {9,10,11} and whose X/Y bits above it number at most
- * three (every term of a nearest-neighbour Ising or Heisenberg model): in
- * fixed point: every component rounded once to the nearest multiple of
- * 2^(e - 54), 2^e the power of two just above the largest component among
- * the 4096 amplitudes read with it (tiles below 2^-959 flush to zero),
- * products and tile sums exact in integers, tile results combined in FP64
- * with compensation.  Other terms and complex64 states: FP64 (FP64 mode) or
- * double-float products, compensated sums.  *out receives the real
+ * States of at least 17 qubits, terms of at most four X/Y qubits, where an
+ * estimate finds that path the cheaper one; smaller complex128 states, terms
+ * whose X/Y bits below qubit 12 lie in one of the triples {0,1,2} ..
+ * {9,10,11} and whose X/Y bits above it number at most three: in fixed point:
+ * every component rounded once to the nearest multiple of 2^(e - 54), 2^e the
+ * power of two just above the largest component among the 4096 amplitudes
+ * read with it (tiles below 2^-959 flush to zero), products (on smaller
+ * states to 2^-52 of the largest) and tile sums exact in integers, tile
+ * results combined in FP64.  Other terms and complex64 states: FP64 (FP64
+ * mode) or double-float products, compensated sums.  *out receives the real
  * value (0 for nterms = 0).  QE_ERR_ARG for nterms < 0, a mask naming a
  * qubit >= n or a non-finite coefficient; QE_ERR_TIMEOUT if a copy wait of
  * the fixed-point kernel ran out (bounded waits). */
@@ -263,8 +264,10 @@ int qe_set_policy(qe_state* s, int policy, int max_k);
  *     rounded once to a double, so an output is within 2^-50 of the product
  *     of the two scales -- inside the worst-case rounding error of an FP64
  *     dot product of the same 64 real terms.  1-2-qubit, diagonal,
- *     controlled and smaller-state gates, the FFT, expectation values and
- *     probabilities run in native FP64 (53-bit significands).
+ *     controlled and smaller-state gates and the FFT's twiddles run in native
+ *     FP64 (53-bit significands), expectation values as qe_expectation says;
+ *     probabilities are sums of squares rounded to 2^-54 of the largest of
+ *     eight, exact in integers, then FP64.
  *   QE_ARITH_DF64: the fast mode.  Values are split into pairs of floats
  *     (double-float, 47 significant bits; magnitudes below 2^-80 keep only
  *     the leading float, below 2^-126 become zero, and magnitudes of 2^127

@@ -3,8 +3,13 @@
 // transform with kernel exp(+2 pi i k l / 2^m) and scale 2^{-m/2}.  The
 // emulator computes it as an in-place FFT instead of m(m+1)/2 gates.
 //
-// Decomposition: radix-2^r passes from the top register bits down
-// (decimation in frequency).  A pass loads tiles that hold whole groups of
+// Three decompositions, all from the top register bits down (decimation in
+// frequency) with one reversal at the end: digits of 3 to 5 qubits on the tensor
+// cores (complex128, qft_tc; qft_on_tensor_cores says where), passes of up to 12
+// radix-2 stages in registers four at a time (complex64 registers of several
+// passes, k_fft4), and radix-2 passes in shared memory:
+//
+// Radix-2^r passes.  A pass loads tiles that hold whole groups of
 // 2^r elements strided along its r bits into shared memory, runs r radix-2
 // DIF stages there, multiplies every element by the inter-pass twiddle
 // exp(s 2 pi i j2 k1 / 2^(b0+r)) (j2: the register bits below the pass, k1:
