@@ -562,8 +562,8 @@ ARITH_DESC = {
              "scale, one rounding per output), everything else (FFT, reductions, smaller gates) in native "
              "FP64"),
     "df64": ("complex128 in the fast mode: 3-5-qubit blocks as exact fp16-digit products of 48-bit "
-             "splittings on the tensor cores, smaller blocks, the FFT and the reductions in double-float "
-             "(f32 pair, 47-bit) arithmetic"),
+             "splittings on the tensor cores, smaller blocks and short FFTs in double-float (f32 pair, 47-bit) "
+             "arithmetic, QFTs of several passes and sums as in the FP64 mode"),
 }
 
 
@@ -789,9 +789,9 @@ def compare(st, qe, n, reg, cconst):
     st.set_policy(qe.POLICY_EMULATE, 1)
     st.init_random(8)
     t_div = timed(lambda: st.div(qa, qb, qc))
-    out["div"] = {"N": N, "emulated_ms": t_div, "emulated_GB_per_s": 4 * (16 << n) / t_div / 1e6,
-                  "note": "planes of 2^(2N) amplitudes through the scratch buffer (gather + copy back: "
-                          "4 x state bytes); no simulated division (its circuit needs work qubits)"}
+    out["div"] = {"N": N, "emulated_ms": t_div, "emulated_GB_per_s": 2 * (16 << n) / t_div / 1e6,
+                  "note": "planes of 2^(2N) amplitudes scattered into a buffer that stays in L2 and copied "
+                          "back; no simulated division (its circuit needs work qubits)"}
     st.set_policy(qe.POLICY_AUTO, 2)
     return out
 
@@ -866,7 +866,7 @@ def bench_config0(qe, I, n=20, layers=10, seed=0):
             "max_abs_vs_oracle": float(np.max(np.abs(got - ref))),
             "fidelity_vs_oracle": float(abs(np.vdot(ref, got)) ** 2 / (np.vdot(ref, ref).real * np.vdot(got, got).real)),
             "note": "host-timed through the public API (enqueue + kernels + sync); 32 MB state is L2-resident; "
-                    "device_ms: the kernels' own time (CUDA events per launch, one run)"}
+                    "device_ms: each kernel by itself (CUDA events per launch, one run; unprofiled launches overlap)"}
 
 
 def bench_batch(qe, I, count=4096, layers=8, seed=3):
@@ -918,7 +918,7 @@ def bench_batch(qe, I, count=4096, layers=8, seed=3):
                       "time_to_solution_ms": dt * 1e3, "circuits_per_s": count / dt,
                       "pass_bytes_GB_per_s": info["hbm_bytes"] / dt / 1e9, "items": info["items"],
                       "pass_bytes_note": "state bytes the passes of the large circuits read and write; waves of "
-                                         "<= 64 MiB keep them largely in L2, so DRAM moves less",
+                                         "<= 64 MiB (complex128 256 MiB) keep them partly in L2, so DRAM moves less",
                       "plan": plan, "tune_s": tune_s, "max_abs_dE_vs_oracle_sampled": err,
                       **({"fp64_mode": {"arith": "native FP64 gates and FP64 energy sums (same plan)",
                                         "time_to_solution_ms": dt64 * 1e3, "circuits_per_s": count / dt64,
