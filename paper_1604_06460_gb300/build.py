@@ -18,7 +18,7 @@ INCLUDE = HERE.parent / "include"
 NVCC = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-std=c++17", "-lineinfo", "--expt-relaxed-constexpr",
-         "-Xcompiler", "-fPIC", "-Xcompiler", "-Wall", "-Xcompiler", "-ffp-contract=off", f"-I{INCLUDE}"]
+         "-Xcompiler", "-fPIC", "-Xcompiler", "-Wall", f"-I{INCLUDE}"]
 SOURCES = ["api.cu", "plan.cu", "state.cu", "gates.cu", "fft.cu", "perm.cu", "reduce.cu", "expect.cu", "batch.cu", "mlp.cu", "tcgen05.cu",
            "tc_c128.cu", "oz_gemm.cu", "arith.cu", "sample.cu", "qpe.cu",
            "noalloc.cu"]

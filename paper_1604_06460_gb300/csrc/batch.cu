@@ -767,14 +767,18 @@ namespace qe {
 
 namespace {
 
+// Not inlined: compilers that contract a product and a sum into one rounding
+// would break the error terms below.
+__attribute__((noinline)) double rounded_product(double a, double b) { return a * b; }
+
 // A product of sums of two squares in twice FP64's precision (hundreds of
 // factors: FP64 roundings alone would add 5e-15).
 struct Pair {
     double h = 1.0, l = 0.0;
     void times_squares(double a, double b) {
-        const double aa = a * a, bb = b * b, s = aa + bb, t = s - aa;
+        const double aa = rounded_product(a, a), bb = rounded_product(b, b), s = aa + bb, t = s - aa;
         const double e = ((aa - (s - t)) + (bb - t)) + (std::fma(a, a, -aa) + std::fma(b, b, -bb));
-        const double p = h * s, q = std::fma(h, s, -p) + (h * e + l * s);
+        const double p = rounded_product(h, s), q = std::fma(h, s, -p) + (h * e + l * s);
         h = p + q;
         l = q - (h - p);
     }
