@@ -178,10 +178,11 @@ __device__ __forceinline__ double block_reduce_d(double a, double* sh) {
 // places of the other high bits, eight amplitudes at a time summed in fixed
 // point (mass_of), the eights in FP64.  The threads that differ only in bits
 // outside the register are then combined pairwise with Neumaier's
-// compensation.  Bound by HBM: n = 28, three qubits, complex128 0.74 ms (1.05
-// to 1.30 by FP64 products, two an amplitude), complex64 0.33 (0.44 to 0.92);
+// compensation.  Bound by HBM: n = 28, three qubits, complex128 0.67 ms (1.05
+// to 1.30 by FP64 products, two an amplitude; 0.71 at four blocks an SM, 0.80 at
+// six, whose registers spill), complex64 0.33 (0.44 to 0.92; 0.35 with five);
 // eight qubits on both sides of 8, read bin by bin with a stride before, 1.43 ->
-// 0.74 and 1.62 -> 0.32.
+// 0.67 and 1.62 -> 0.32.
 constexpr int kLowBits = 8;
 template <class S>
 struct ProbArgs {
@@ -220,7 +221,7 @@ __device__ __forceinline__ double group_mass(const float2 (&v)[N]) {
 }
 
 template <class S>
-__global__ void __launch_bounds__(1 << kLowBits) k_probs(const __grid_constant__ ProbArgs<S> a) {
+__global__ void __launch_bounds__(1 << kLowBits, sizeof(S) == 16 ? 5 : 8) k_probs(const __grid_constant__ ProbArgs<S> a) {
     constexpr uint32_t T = 1u << kLowBits;
     __shared__ double ss[T], sc[T];
     const uint32_t t = threadIdx.x;

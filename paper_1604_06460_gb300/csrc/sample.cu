@@ -43,7 +43,7 @@ __device__ __forceinline__ double prob_of(float2 v) {
 // mass[k] = sum of |alpha|^2 over block k of 2^12: thread t takes elements t,
 // t + 256, ... of the block, then a fixed reduction tree.  Bound by HBM: the
 // squares are summed in fixed point (2^28 amplitudes, complex128: 1.74 ms with
-// three FP64 operations an amplitude, 0.74 now; complex64 2.71 -> 0.65).
+// three FP64 operations an amplitude, 0.69 now; complex64 2.71 -> 0.59).
 template <class S>
 __global__ void __launch_bounds__(kMassThreads) k_block_mass(const S* __restrict__ x, uint64_t nblocks,
                                                              double* __restrict__ mass) {
