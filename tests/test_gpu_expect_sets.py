@@ -39,6 +39,15 @@ def _chain(n):
     return xm, zm, cf
 
 
+def _fields(n):
+    # single X on two, three and four qubits of a set, of several weights and signs, some twice
+    xm, zm, cf = [], [], []
+    for i in range(n):
+        for w in ([0.7], [0.7, -0.4], [-0.4], [0.7, 0.7, 1.3])[(i * 7 // 4) % 4]:
+            xm.append(1 << i); zm.append(0); cf.append(w)
+    return xm, zm, cf
+
+
 def _mixed(n, seed, count=90):
     rng = np.random.default_rng(seed)
     xm, zm, cf = [], [], []
@@ -56,13 +65,13 @@ def _mixed(n, seed, count=90):
     return xm, zm, cf
 
 
-CASES = [(17, "chain"), (18, "mixed"), (20, "chain"), (21, "mixed"), (20, "mixed"), (22, "chain")]
+CASES = [(17, "chain"), (18, "fields"), (19, "fields"), (18, "mixed"), (20, "chain"), (21, "mixed"), (20, "mixed"), (22, "chain")]
 
 
 @pytest.mark.parametrize("dtype,arith", [("c128", "fp64"), ("c128", "df64"), ("c64", "fp64")])
 @pytest.mark.parametrize("n,kind", CASES)
 def test_expectation_register_sets(n, kind, dtype, arith):
-    xm, zm, cf = _chain(n) if kind == "chain" else _mixed(n, n)
+    xm, zm, cf = _chain(n) if kind == "chain" else _fields(n) if kind == "fields" else _mixed(n, n)
     rng = np.random.default_rng(n)
     psi = I.random_state(n, n)
     psi = (psi.reshape(-1, 128) * 2.0 ** rng.integers(-40 if dtype == "c128" else -20, 1, (1 << n) // 128)[:, None]).reshape(-1)
