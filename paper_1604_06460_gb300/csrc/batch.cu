@@ -907,7 +907,7 @@ void build_plan(qe_batch* b) {
             Item it{};
             it.circuit = c;
             it.kind = (p == P_ - 1) ? 3 : (b->layers > 1 && p % 2 == 0) ? 1 : 2;
-            it.layer = b->layers > 1 ? 1 + p / 2 : 0;
+            it.layer = std::min(1 + p / 2, b->layers - 1);   // of the energy pass too: its flips are loaded
             it.first = p == 0;
             it.tile0 = j * per;
             it.tile1 = std::min(tiles, (uint32_t)(j + 1) * per);
@@ -956,6 +956,9 @@ void build_plan(qe_batch* b) {
             for (; si < upto; ++si) push_small(small[si]);
         }
     for (; si < small.size(); ++si) push_small(small[si]);
+    // a layer indexes the flips, factors and kappas of the item's circuit
+    for (const Item& it : items)
+        if ((int)it.layer >= b->layers) fail(QE_ERR_STATE, "a batch work item names a layer beyond its circuit's last");
     b->nitems = (int)items.size();
     // device buffers
     const size_t need_states = state_off * sizeof(typename P::V);
