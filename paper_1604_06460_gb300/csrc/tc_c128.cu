@@ -419,7 +419,7 @@ __global__ void __maxnreg__(96) k_gate_tc5_c128(const __grid_constant__ Args arg
     // hold any tile index).  With kDft they live in shared memory, where they
     // cost the roles no registers (the digit kernel spilled with them in
     // registers: 12.3 against 11.3 ms a pass at n = 30).
-    __shared__ uint32_t s_begin, s_end, s_step;
+    __shared__ uint32_t s_begin, s_end, s_step, s_matrix;
     auto seg_begin = [&]() -> uint32_t { return kDft ? s_begin : blockIdx.x; };
     auto seg_end = [&]() -> uint32_t { return kDft ? s_end : (uint32_t)a.ntiles; };
     auto seg_step = [&]() -> uint32_t { return kDft ? s_step : gridDim.x; };
@@ -435,11 +435,12 @@ __global__ void __maxnreg__(96) k_gate_tc5_c128(const __grid_constant__ Args arg
             if (!begin) {
                 __syncthreads();
                 if (*reinterpret_cast<volatile uint32_t*>(&abort_flag)) return false;
-                v = (s_begin >> arg.lt) + arg.teams;
+                v = s_matrix + arg.teams;   // (not from s_begin: a CTA's place in its team may reach 2^lt)
                 __syncthreads();
             }
             if (v >> arg.P) return false;
             if (tid == 0) {
+                s_matrix = v;
                 s_begin = (v << arg.lt) + blockIdx.x / arg.teams;
                 s_end = (v + 1) << arg.lt;
                 s_step = (gridDim.x - team + arg.teams - 1) / arg.teams;    // CTAs of the team
