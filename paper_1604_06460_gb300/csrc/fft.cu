@@ -755,7 +755,7 @@ void fft4(qe_state* s, int lo, int m, int inverse) {
 // A digit joins the group while a matrix still serves at least 16 tiles
 // (P <= n - 16: rebuilding it costs a segment of the pipeline, about two tiles)
 // and its roots fit a direct table (P + d <= 20); the digits are then spread
-// evenly over that number of groups.  Measured on complex128 in the FP64 mode,
+// evenly over that number of groups where that keeps both limits.  Measured on complex128 in the FP64 mode,
 // against dense blocks with a twiddle pass after each (m a multiple of its
 // digit) or the shared-memory transform: the 30-qubit QFT 121 -> 79 ms (six
 // digits 54, one twiddle pass 15.4, reversal 9), 29 qubits 161 -> 39.5 ms, 17
@@ -827,16 +827,34 @@ const typename P::M* get_direct(qe_state* s, int k, int sign, int pol) {
     return (const typename P::M*)t;
 }
 
-void qft_tc(qe_state* s, int lo, int m, int inverse) {
-    const int sign = inverse ? -1 : 1;
+}  // namespace
+
+int qft_digits(int n, int m, int* digit, int* group) {
     const int G = (m + 4) / 5;
-    int digit[7];
     for (int j = 0; j < G; ++j) digit[j] = m / G + (j >= G - m % G ? 1 : 0);   // wider ones lowest: longer runs
-    // the fewest groups, then as even as possible
-    auto fits = [&](int P, int d) { return P == 0 || (P <= s->n - 16 && P + d <= 20); };
+    auto fits = [&](int P, int d) { return P == 0 || (P <= n - 16 && P + d <= 20); };
+    // the fewest groups, each as long as it can be ...
     int groups = 0;
     for (int j = 0; j < G; ++groups)
-        for (int P = 0; j < G && fits(P, digit[j]); P += digit[j++]) {}
+        for (int P = 0; j < G && fits(P, digit[j]); P += digit[j++]) group[j] = groups;
+    // ... then as even as possible, where every digit still fits
+    int even[7];
+    bool ok = true;
+    for (int g = 0, j = 0; g < groups; ++g)
+        for (int P = 0; j < G * (g + 1) / groups; P += digit[j++]) {
+            ok &= fits(P, digit[j]);
+            even[j] = g;
+        }
+    if (ok) std::copy(even, even + G, group);
+    return G;
+}
+
+namespace {
+
+void qft_tc(qe_state* s, int lo, int m, int inverse) {
+    const int sign = inverse ? -1 : 1;
+    int digit[7], group[7];
+    const int G = qft_digits(s->n, m, digit, group), groups = group[G - 1] + 1;
     static thread_local TwArgs a;
     a.x = reinterpret_cast<double2*>(s->d);
     a.count = dim(s);
@@ -844,9 +862,8 @@ void qft_tc(qe_state* s, int lo, int m, int inverse) {
     a.h = (m + 1) / 2;
     int top = m, j = 0;
     for (int g = 0; g < groups; ++g) {
-        const int last = G * (g + 1) / groups;
         int P = 0;
-        for (; j < last; ++j) {
+        for (; j < G && group[j] == g; ++j) {
             const int d = digit[j];
             top -= d;
             launch_dft_digit_c128(s, lo + top, d, P, G > 1, get_direct<F64>(s, P + d, sign, 1));

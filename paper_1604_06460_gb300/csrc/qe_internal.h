@@ -139,6 +139,9 @@ void launch_gate_tc5_c128(qe_state* s, const int* qubits, const cd* U);
 // one digit [q0, q0 + d) of a Fourier transform on a complex128 state, its
 // matrix chosen by the P qubits above it (tc_c128.cu)
 void launch_dft_digit_c128(qe_state* s, int q0, int d, int P, bool reversed, const double2* roots);
+// the digits of an m-qubit register from the top, the group of each (at most
+// seven of both); their number (fft.cu)
+int qft_digits(int n, int m, int* digit, int* group);
 // diagonal gate: amplitude x *= d[row(x)] for all x
 void launch_gate_diag(qe_state* s, int k, const int* qubits, const cd* d);
 // amplitudes with (x & mask) == value are multiplied by phase
