@@ -121,8 +121,12 @@ int qe_apply_controlled(qe_state* s, int nc, const int* controls, int k,
  *     alpha_l -> 2^{-m/2} sum_k alpha_k exp(+2 pi i k l / 2^m),
  * natural output order; inverse != 0 uses the opposite sign.  Emulated as an
  * in-place FFT, or simulated as m Hadamards, m(m-1)/2 CR gates and the
- * qubit reversal, as the policy decides.  QE_ERR_ARG unless m >= 1, lo >= 0
- * and lo + m <= n. */
+ * qubit reversal, as the policy decides.  Emulated on larger complex128 states,
+ * the FFT runs as dense blocks on the tensor cores, rounded as QE_ARITH_FP64
+ * says of them in both modes; the 32 amplitudes that share a scale belong to
+ * one assignment of the other qubits, except in registers of three and four
+ * qubits (FP64 mode only).  Groups whose largest component is below 2^-920
+ * become zero there.  QE_ERR_ARG unless m >= 1, lo >= 0 and lo + m <= n. */
 int qe_apply_qft(qe_state* s, int lo, int m, int inverse);
 
 /* Add the classical constant c to the m-qubit register qubits[] (bit j of

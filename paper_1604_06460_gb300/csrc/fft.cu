@@ -4,7 +4,7 @@
 // emulator computes it as an in-place FFT instead of m(m+1)/2 gates.
 //
 // Three decompositions, all from the top register bits down (decimation in
-// frequency) with one reversal at the end: digits of 3 to 5 qubits on the tensor
+// frequency) with one reversal at the end: digits of up to five qubits on the tensor
 // cores (complex128, qft_tc; qft_on_tensor_cores says where), passes of up to 12
 // radix-2 stages in registers four at a time (complex64 registers of several
 // passes, k_fft4), and radix-2 passes in shared memory:
@@ -738,7 +738,7 @@ void fft4(qe_state* s, int lo, int m, int inverse) {
 }
 
 // ------------------------------------------------ tensor-core digit passes
-// The QFT of a register of m qubits as G = ceil(m / 5) dense blocks of 3..5
+// The QFT of a register of m qubits as G = ceil(m / 5) dense blocks of up to five
 // qubits on the tensor cores (Cooley-Tukey, digits from the top).  With the
 // digits of the register value from the top k_0, k_1, ... (k = k_0 2^(m-d_0) + k')
 // and the outputs so far l = l_0 + 2^(d_0) l_1 + ..., digit j is
@@ -831,7 +831,14 @@ const typename P::M* get_direct(qe_state* s, int k, int sign, int pol) {
 
 int qft_digits(int n, int m, int* digit, int* group) {
     const int G = (m + 4) / 5;
-    for (int j = 0; j < G; ++j) digit[j] = m / G + (j >= G - m % G ? 1 : 0);   // wider ones lowest: longer runs
+    // The lowest of five qubits, the others even (wider ones lowest: longer runs):
+    // blocks are then filled up with register qubits only, and amplitudes that
+    // differ outside a register of five qubits or more, however different in size,
+    // share no scale.  (A lowest digit of three or four, with all of the
+    // register above it choosing its matrix, took in qubits outside: a branch
+    // 2^-30 of its neighbour kept 26 bits.)
+    if (G > 1) digit[G - 1] = 5;
+    for (int j = 0, r = G > 1 ? m - 5 : m, k = std::max(1, G - 1); j < k; ++j) digit[j] = r / k + (j >= k - r % k ? 1 : 0);
     auto fits = [&](int P, int d) { return P == 0 || (P <= n - 16 && P + d <= 20); };
     // the fewest groups, each as long as it can be ...
     int groups = 0;
@@ -866,7 +873,7 @@ void qft_tc(qe_state* s, int lo, int m, int inverse) {
         for (; j < G && group[j] == g; ++j) {
             const int d = digit[j];
             top -= d;
-            launch_dft_digit_c128(s, lo + top, d, P, G > 1, get_direct<F64>(s, P + d, sign, 1));
+            launch_dft_digit_c128(s, lo, lo + top, d, P, G > 1, get_direct<F64>(s, P + d, sign, 1));
             P += d;
         }
         if (top == 0) break;
@@ -902,11 +909,14 @@ void qft_tc(qe_state* s, int lo, int m, int inverse) {
 //   double-float mode: n = 24, m = 5 0.294 / 0.195 (n = 20 0.031 / 0.038),
 //   m = 10 0.439 / 0.483, m = 24 1.48 / 1.34, n = 20, m = 20 0.120 / 0.160,
 //   n = 30, m = 30 118 / 79.
+// Registers of three and four qubits share their blocks' scale with amplitudes
+// outside the register; the double-float mode leaves them to the elementwise
+// transform.
 static bool qft_on_tensor_cores(const qe_state* s, int lo, int m) {
     if (s->dtype != QE_C128 || !s->c128_tc || !s->tensor_cores || s->force_tile || s->n < 12 || m < 3) return false;
     const bool one_pass = m <= 11 - std::min(lo, 3);
     if (s->arith == QE_ARITH_FP64) return one_pass ? s->n >= 20 : s->n >= 19 || m % 5 == 0;
-    return m <= 5 ? s->n >= 22 : !one_pass && s->n >= 23;
+    return m <= 5 ? m == 5 && s->n >= 22 : !one_pass && s->n >= 23;
 }
 
 void launch_qft_fft(qe_state* s, int lo, int m, int inverse) {

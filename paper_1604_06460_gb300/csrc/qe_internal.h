@@ -136,9 +136,9 @@ void complete_pending(qe_state* s);
 // (n >= 12, qubits ascending)
 void launch_gate_tc5(qe_state* s, const int* qubits, const cd* U);
 void launch_gate_tc5_c128(qe_state* s, const int* qubits, const cd* U);
-// one digit [q0, q0 + d) of a Fourier transform on a complex128 state, its
-// matrix chosen by the P qubits above it (tc_c128.cu)
-void launch_dft_digit_c128(qe_state* s, int q0, int d, int P, bool reversed, const double2* roots);
+// one digit [q0, q0 + d) of a Fourier transform of a register from qubit lo on
+// (complex128), its matrix chosen by the P qubits above it (tc_c128.cu)
+void launch_dft_digit_c128(qe_state* s, int lo, int q0, int d, int P, bool reversed, const double2* roots);
 // the digits of an m-qubit register from the top, the group of each (at most
 // seven of both); their number (fft.cu)
 int qft_digits(int n, int m, int* digit, int* group);

@@ -784,13 +784,18 @@ void launch_gate_tc5_c128(qe_state* s, const int* qubits, const cd* U) {
 }
 
 // One digit of a Fourier transform on a complex128 state (n >= 12): the qubits
-// [q0, q0 + d), 3 <= d <= 5, whose matrix depends on the P qubits above them
-// (P + d <= 20, n - 12 - P >= 0).  `roots` holds the 2^(P + d) roots of unity
+// [q0, q0 + d), 1 <= d <= 5, whose matrix depends on the P qubits above them
+// (P + d <= 20, n - 12 - P >= 0), of a register from qubit lo on.  With d < 5 the
+// block is filled up with qubits of the register below the digit, so that its
+// 32 amplitudes, which share a scale, stay within the register: with those that
+// the tile has anyway if there are such (17 qubits from 5 on at n = 27 5.84 ms,
+// 5.96 with the ones next to the digit), and not with qubit 0, whose blocks are
+// the slower ones.  A register of fewer than five qubits takes in others.  `roots` holds the 2^(P + d) roots of unity
 // of the transform's sign; `reversed`: leave the output bit-reversed.  56-bit
 // splitting in both arithmetic modes (the seventh digit costs 3 %).
-void launch_dft_digit_c128(qe_state* s, int q0, int d, int P, bool reversed, const double2* roots) {
+void launch_dft_digit_c128(qe_state* s, int lo, int q0, int d, int P, bool reversed, const double2* roots) {
     constexpr int D = 7;
-    if (s->n < 12 + P) fail(QE_ERR_UNSUPPORTED, "transform digits need n >= 12 + P");
+    if (d < 1 || d > 5 || s->n < 12 + P) fail(QE_ERR_UNSUPPORTED, "transform digits need 1 to 5 qubits and n >= 12 + P");
     static thread_local DftArgs f;
     std::memset(&f, 0, sizeof(f));
     OzArgs& a = f.z;
@@ -803,32 +808,37 @@ void launch_dft_digit_c128(qe_state* s, int q0, int d, int P, bool reversed, con
     f.scale = std::pow(2.0, -0.5 * d);
     f.roots = roots;
     f.lt = s->n - 12 - P;
-    // The tile: the digit, the lowest qubits outside it and the matrix bits.
-    // Gate bits are the digit and, for d < 5, the lowest other tile qubits.
+    // The block: the digit and, for d < 5, idle qubits; the tile: the block and
+    // the lowest qubits outside it and the matrix bits.
     bool matrix[64] = {}, local[64] = {};
     for (int j = 0; j < P; ++j) matrix[f.vlo + j] = true;
-    for (int j = 0; j < d; ++j) local[q0 + j] = true;
-    int nlocal = d;
+    int gate[5], ng = 0;
+    auto take = [&](int q) {
+        gate[ng++] = q;
+        local[q] = true;
+        f.below += q < q0;
+    };
+    for (int j = 0; j < d; ++j) take(q0 + j);
+    for (int q = std::min(q0 - 1, 11 - d); q >= std::max(lo, 1) && ng < 5; --q) take(q);
+    for (int q = q0 - 1; q >= std::max(lo, 1) && ng < 5; --q)
+        if (!local[q]) take(q);
+    for (int q = q0 + d; q < 12 && ng < 5; ++q)
+        if (!matrix[q]) take(q);
+    for (int q = std::min(q0 - 1, 11 - d); q >= 0 && ng < 5; --q)
+        if (!local[q]) take(q);
+    for (int q = q0 + d; ng < 5; ++q)
+        if (!matrix[q] && !local[q]) take(q);
+    int nlocal = 5;
     for (int q = 0; nlocal < 12; ++q)
         if (!local[q] && !matrix[q]) {
             local[q] = true;
             ++nlocal;
         }
-    // idle matrix bits (d < 5): tile bits next to the digit, so that qubit 0
-    // stays a row bit where it can
-    int gate[5], ng = 0;
-    for (int j = 0; j < d; ++j) gate[ng++] = q0 + j;
-    for (int q = q0 + d; q < s->n && ng < 5; ++q)
-        if (local[q]) gate[ng++] = q;
-    for (int q = q0 - 1; q >= 0 && ng < 5; --q)
-        if (local[q]) {
-            gate[ng++] = q;
-            ++f.below;
-        }
     std::sort(gate, gate + 5);
     const bool pair = gate[0] == 0;
     while (local[a.L]) ++a.L;
     if (a.L > 12) a.L = 12;
+    if (a.L < 3) fail(QE_ERR_UNSUPPORTED, "transform digits need runs of eight amplitudes");
     int pos[64];
     for (int q = 0; q < s->n; ++q) {
         pos[q] = q < a.L ? q : a.L + a.kh;

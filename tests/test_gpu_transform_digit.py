@@ -17,7 +17,8 @@ def _reversed(v, bits):
     return sum(((v >> j) & 1) << (bits - 1 - j) for j in range(bits))
 
 
-@pytest.mark.parametrize("n,q0,d,P", [(20, 0, 5, 8), (20, 3, 4, 8), (22, 2, 5, 10), (21, 0, 5, 8), (20, 1, 3, 5), (16, 4, 5, 0)])
+@pytest.mark.parametrize("n,q0,d,P", [(20, 0, 5, 8), (20, 3, 4, 8), (22, 2, 5, 10), (21, 0, 5, 8), (20, 1, 3, 5), (20, 0, 3, 8), (20, 12, 1, 0),
+                                      (20, 18, 2, 0), (16, 4, 5, 0)])
 def test_every_matrix_is_applied(n, q0, d, P):
     import torch
     from paper_1604_06460_gb300 import qe
@@ -26,9 +27,9 @@ def test_every_matrix_is_applied(n, q0, d, P):
     roots = torch.tensor(np.exp(2j * np.pi * k / (1 << (P + d)))).cuda()
     with qe.State(n) as st:
         st.set(psi)
-        digit = qe.load()["_ZN2qe21launch_dft_digit_c128EP8qe_stateiiibPK7double2"]
-        digit.argtypes, digit.restype = [C.c_void_p, C.c_int, C.c_int, C.c_int, C.c_bool, C.c_void_p], None
-        digit(st._h, q0, d, P, True, roots.data_ptr())
+        digit = qe.load()["_ZN2qe21launch_dft_digit_c128EP8qe_stateiiiibPK7double2"]
+        digit.argtypes, digit.restype = [C.c_void_p, C.c_int, C.c_int, C.c_int, C.c_int, C.c_bool, C.c_void_p], None
+        digit(st._h, 0, q0, d, P, True, roots.data_ptr())
         got = st.get()
         torch.cuda.synchronize()
     v = np.moveaxis(psi.reshape(-1, 1 << P, 1 << d, 1 << q0), 1, 0)
