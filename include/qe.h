@@ -126,7 +126,7 @@ int qe_apply_controlled(qe_state* s, int nc, const int* controls, int k,
  * says of them in both modes; the 32 amplitudes that share a scale belong to
  * one assignment of the other qubits, except in registers of three and four
  * qubits (FP64 mode only).  Groups whose largest component is below 2^-920
- * become zero there.  QE_ERR_ARG unless m >= 1, lo >= 0 and lo + m <= n. */
+ * become zero there, groups with an infinity or NaN become NaN.  QE_ERR_ARG unless m >= 1, lo >= 0 and lo + m <= n. */
 int qe_apply_qft(qe_state* s, int lo, int m, int inverse);
 
 /* Add the classical constant c to the m-qubit register qubits[] (bit j of

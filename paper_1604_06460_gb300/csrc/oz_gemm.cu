@@ -405,7 +405,10 @@ __global__ void __launch_bounds__(kThreads, 1) k_oz_zgemm(const __grid_constant_
                 const int b = 8 * u + j;                       // Bt row of the tile
                 const int64_t cc = (int64_t)blockIdx.x * 16 + (b & 15);
                 const double y = i128_to_double(hi[j], lo[j]);
-                out[2 * (r * a.ldc + cc) + (b >> 4)] = scalbn(y, er + a.fb[brow0 + b] - 56);
+                const int f = a.fb[brow0 + b];
+                // an infinity or NaN in the row of A or the column of B (scale 2^1026)
+                const double z = max(er, f) > 1025 ? __hiloint2double(0x7FF80000, 0) : scalbn(y, er + f - 56);
+                out[2 * (r * a.ldc + cc) + (b >> 4)] = z;
             }
         }
     }

@@ -309,6 +309,10 @@ __device__ __forceinline__ uint32_t stage_off(uint32_t row, uint32_t c) {
 __device__ __forceinline__ const OzArgs& oz_args(const GateArgs& a) { return a.z; }
 __device__ __forceinline__ const OzArgs& oz_args(const DftArgs& a) { return a.z; }
 
+// The exponent term of a row whose largest biased exponent is em.
+__host__ __device__ constexpr int eterm_of(int em) { return (em - 1021 - 56) * (1 << 20); }
+constexpr int kEtermBad = eterm_of(0x7FF);
+
 // 19 warps of 96 registers a thread: a sub-partition holding five of the warps
 // uses 15,360 of its 16,384 registers (104 would exceed them).
 //
@@ -602,7 +606,7 @@ __global__ void __maxnreg__(96) k_gate_tc5_c128(const __grid_constant__ Args arg
                         // the row scale, for the recombination of this tile
                         // (the slot's previous tile was read before set X
                         // was released for the previous tile's MMAs)
-                        s_eterm[it & 1][r] = ((int)em - 1021 - 56) * (1 << 20);
+                        s_eterm[it & 1][r] = eterm_of((int)em);
                         mbar_arrive(&bars[(it & 1) ? kEt1 : kEt0]);
                     }
                     if (h == 1) {
@@ -726,6 +730,12 @@ __global__ void __maxnreg__(96) k_gate_tc5_c128(const __grid_constant__ Args arg
                 store(gb, 16 * hh + 8 * eh + 4, yb, eterm);
             }
             if (!ok) break;
+            if (kDft && eterm == kEtermBad) {   // an infinity or NaN among the row's inputs
+                const double nan = __hiloint2double(0x7FF80000, 0);
+#pragma unroll 1
+                for (int c = 8 * eh; c < 32; c = (c & 7) == 7 ? c + 9 : c + 1)
+                    *reinterpret_cast<double2*>(gb + coloff[c]) = make_double2(nan, nan);
+            }
         }
     }
     asm volatile("tcgen05.fence::before_thread_sync;");
