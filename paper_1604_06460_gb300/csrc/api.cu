@@ -775,9 +775,6 @@ int qe_apply_gate(qe_state* s, int k, const int* qubits, const double* matrix) {
         g.U[i] = cd(matrix[2 * i], matrix[2 * i + 1]);
     }
     s->queue.push_back(std::move(g));
-    // without fusion there is nothing to wait for: hand the gates over in small
-    // lots, so that the device works while the caller queues the next ones
-    if (s->max_k == 1 && s->queue.size() >= 16) launch_queue(s);
     QE_API_END
 }
 
