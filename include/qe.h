@@ -150,9 +150,11 @@ int qe_apply_add_const(qe_state* s, int m, const int* qubits, uint64_t c);
  *     on c = 0 this is the paper's (a, b, 0) -> (a mod b, b, a div b) (b = 0
  *     leaves the state unchanged).  Emulated only: QE_ERR_UNSUPPORTED under
  *     QE_POLICY_SIMULATE.
- * Both are permutations of the amplitudes, bit-exact.  A permutation whose
- * plane (the 2^N values of c, or the 2^(2N) of (a, c)) exceeds 64 KB goes
- * through a device scratch buffer owned by the state, 32 MiB or two planes.
+ * Both are permutations of the amplitudes, bit-exact.  A division whose planes
+ * (the 2^(2N) values of (a, c)) exceed 64 KB goes through a device scratch
+ * buffer owned by the state, of 32 MiB or two blocks if that is more; a block is
+ * up to eight planes (2^w with w <= 3 the qubits below those of a and c): 64 MiB
+ * for nine-qubit complex128 registers from qubit 3 on, 1 GiB at most.
  * QE_ERR_ARG for N out of range, a qubit >= n, a repeated qubit or
  * overlapping registers. */
 int qe_apply_mul(qe_state* s, int N, const int* qa, const int* qb, const int* qc);

@@ -77,14 +77,9 @@ __device__ __forceinline__ void preimage(int N, uint32_t& a, uint32_t b, uint32_
     }
 }
 
-// The map itself: the image of (a, b, c) in a, c.
-template <int OP>
+// The division itself: the image of (a, b, c) in a, c.
 __device__ __forceinline__ void image(int N, uint32_t& a, uint32_t b, uint32_t& c) {
     const uint32_t mask = (1u << N) - 1u;
-    if (OP == kMul) {
-        c = (c + a * b) & mask;
-        return;
-    }
     if (b == 0u) {       // c_i set subtracts nothing
         return;
     }
@@ -145,7 +140,8 @@ __global__ void __launch_bounds__(kArithThreads) k_arith_plane(const __grid_cons
     }
 }
 
-// Larger planes.  A block is 2^w planes that differ in the lowest w <= 3 qubits
+// Larger planes: of divisions only (registers have at most 11 qubits, and 2^11
+// values of c are 32 KB).  A block is 2^w planes that differ in the lowest w <= 3 qubits
 // (those below every plane qubit), its value e = (plane value y) 2^w + (low
 // bits l), so that a warp touches whole lines of the state wherever the
 // registers lie.
@@ -155,7 +151,7 @@ struct ArithArgs {
     S* scratch;                 // blocks [blk0, blk0 + nblk) are scattered into scratch,
     const S* back;              // [back0, back0 + nback) copied back from `back`
     uint64_t blk0, nblk, back0, nback;
-    int N, P, w;                // register width, plane bits (N or 2N), low bits
+    int N, P, w;                // register width, plane bits (2N), low bits
     RegArg a, b, c;
     int nruns;                  // the block's qubits as runs of consecutive ones, ascending
     uint8_t run_lo[34], run_len[34];
@@ -172,17 +168,20 @@ __device__ __forceinline__ uint64_t block_base(const ArithArgs<S>& a, uint64_t p
 }
 
 // Offset of block value e in the state: the c register holds y's low N bits,
-// and for the division the a register its high N bits.
-template <class S, int OP>
+// the a register its high N bits.
+template <class S>
 __device__ __forceinline__ uint64_t block_offset(const ArithArgs<S>& a, uint32_t e) {
     const uint32_t mask = (1u << a.N) - 1u, l = e & ((1u << a.w) - 1u), y = e >> a.w;
-    if (OP == kMul) return l | reg_put(a.c, a.N, y);
     return l | reg_put(a.c, a.N, y & mask) | reg_put(a.a, a.N, y >> a.N);
 }
 
 // Bytes of a batch of blocks, and block values of one CTA pass.  Two batches of
 // 16 MB (one scattered, one copied back) stay in L2: nine-qubit registers at
-// n = 28 with batches of 8, 16, 32, 64 MB: 4.4, 3.7, 4.3, 5.4 ms.
+// n = 28 with batches of 8, 16, 32, 64 MB: 4.4, 3.7, 4.3, 5.4 ms.  A block above
+// that is a batch of its own: whole lines count for more than L2 (complex128 at
+// n = 30, a and c from qubit 10 on: ten-qubit registers, blocks of eight planes,
+// 128 MB, 38.7 ms, of one plane 78.0; nine-qubit ones from qubit 3 on, 32 MB,
+// 12.8 and, of four planes, 16.5 ms).
 constexpr uint64_t kBatch = 1ull << 24;
 constexpr int kChunk = 1024;
 
@@ -192,7 +191,7 @@ constexpr int kChunk = 1024;
 // (The reverse, a gather of the preimages, scatters its reads over the block's
 // places in the state, 512 runs 4 MB apart for nine-qubit registers a b c, and
 // read DRAM four times over: 6.6 ms for the gather alone.)
-template <class S, int OP>
+template <class S>
 __device__ __forceinline__ void scatter_chunk(const ArithArgs<S>& a, uint64_t k) {
     constexpr int kAtOnce = kChunk / 256;   // independent loads in flight a thread
     const int bits = a.P + a.w;
@@ -203,19 +202,19 @@ __device__ __forceinline__ void scatter_chunk(const ArithArgs<S>& a, uint64_t k)
     S v[kAtOnce];
 #pragma unroll
     for (int j = 0; j < kAtOnce; ++j)
-        v[j] = a.x[base | block_offset<S, OP>(a, (uint32_t)(e0 + 256 * j + threadIdx.x) & emask)];
+        v[j] = a.x[base | block_offset(a, (uint32_t)(e0 + 256 * j + threadIdx.x) & emask)];
 #pragma unroll
     for (int j = 0; j < kAtOnce; ++j) {
         const uint32_t e = (uint32_t)(e0 + 256 * j + threadIdx.x) & emask, l = e & wmask, y = e >> a.w;
         const uint32_t bv = reg_get(a.b, a.N, base | l);
-        uint32_t av = OP == kMul ? reg_get(a.a, a.N, base | l) : y >> a.N, cv = y & mask;
-        image<OP>(a.N, av, bv, cv);
-        out[((OP == kMul ? cv : cv | (av << a.N)) << a.w) | l] = v[j];
+        uint32_t av = y >> a.N, cv = y & mask;
+        image(a.N, av, bv, cv);
+        out[((cv | (av << a.N)) << a.w) | l] = v[j];
     }
 }
 
 // ... and a chunk copied back to its places in the state.
-template <class S, int OP>
+template <class S>
 __device__ __forceinline__ void copy_back_chunk(const ArithArgs<S>& a, uint64_t k) {
     const int bits = a.P + a.w;
     const uint32_t emask = (1u << bits) - 1u;
@@ -226,12 +225,12 @@ __device__ __forceinline__ void copy_back_chunk(const ArithArgs<S>& a, uint64_t 
     for (int j = 0; j < kChunk / 256; ++j) v[j] = a.back[e0 + 256 * j + threadIdx.x];
 #pragma unroll
     for (int j = 0; j < kChunk / 256; ++j)
-        a.x[base | block_offset<S, OP>(a, (uint32_t)(e0 + 256 * j + threadIdx.x) & emask)] = v[j];
+        a.x[base | block_offset(a, (uint32_t)(e0 + 256 * j + threadIdx.x) & emask)] = v[j];
 }
 
 // One launch copies a batch back and scatters the next one (other blocks, the
 // other half of the buffer): half as many launches, reads and writes mixed.
-template <class S, int OP>
+template <class S>
 __global__ void __launch_bounds__(256) k_arith_batch(const __grid_constant__ ArithArgs<S> a) {
     const uint64_t backs = (a.nback << (a.P + a.w)) / kChunk, scatters = (a.nblk << (a.P + a.w)) / kChunk;
     const uint64_t both = backs < scatters ? backs : scatters, all = backs + scatters;
@@ -239,8 +238,8 @@ __global__ void __launch_bounds__(256) k_arith_batch(const __grid_constant__ Ari
         // alternately while both last, then what is left of either
         const bool back = k < 2 * both ? (k & 1) : backs > scatters;
         const uint64_t i = k < 2 * both ? k >> 1 : k - both;
-        if (back) copy_back_chunk<S, OP>(a, i);
-        else scatter_chunk<S, OP>(a, i);
+        if (back) copy_back_chunk(a, i);
+        else scatter_chunk(a, i);
     }
 }
 
@@ -301,15 +300,10 @@ void arith_tiles(qe_state* s, int N, const int* qa, const int* qb, const int* qc
     QE_CUDA(cudaGetLastError());
 }
 
-template <class S, int OP>
-void arith_impl(qe_state* s, int N, const int* qa, const int* qb, const int* qc) {
-    const int P = OP == kMul ? N : 2 * N;
-    const char* tag = OP == kMul ? "mul_emulated" : "div_emulated";
+template <class S>
+void div_batches(qe_state* s, int N, const int* qa, const int* qb, const int* qc) {
+    const int P = 2 * N;
     const size_t plane_bytes = sizeof(S) << P;
-    if (plane_bytes <= 64 * 1024) {
-        arith_tiles<S, OP>(s, N, qa, qb, qc, P, tag);
-        return;
-    }
     static thread_local ArithArgs<S> a;
     std::memset(&a, 0, sizeof(a));
     a.x = reinterpret_cast<S*>(s->d);
@@ -320,8 +314,7 @@ void arith_impl(qe_state* s, int N, const int* qa, const int* qb, const int* qc)
     a.c = make_reg(N, qc);
     int bq[35], nq = 0;
     for (int j = 0; j < N; ++j) bq[nq++] = qc[j];
-    if (OP == kDiv)
-        for (int j = 0; j < N; ++j) bq[nq++] = qa[j];
+    for (int j = 0; j < N; ++j) bq[nq++] = qa[j];
     a.w = std::min(3, *std::min_element(bq, bq + nq));
     for (int q = 0; q < a.w; ++q) bq[nq++] = q;
     std::sort(bq, bq + nq);
@@ -348,8 +341,8 @@ void arith_impl(qe_state* s, int N, const int* qa, const int* qb, const int* qc)
         a.nblk = p0 < blocks ? std::min<uint64_t>(per_batch, blocks - p0) : 0;
         const uint64_t total = (a.nblk + a.nback) << (P + a.w);
         const unsigned grid = (unsigned)std::min<uint64_t>(total / kChunk, (uint64_t)num_sms() * 8);
-        Launch L(s, tag, 1.0 * (double)total * amp_bytes(s), false);
-        k_arith_batch<S, OP><<<grid, 256, 0, s->stream>>>(a);
+        Launch L(s, "div_emulated", 1.0 * (double)total * amp_bytes(s), false);
+        k_arith_batch<S><<<grid, 256, 0, s->stream>>>(a);
         QE_CUDA(cudaGetLastError());
     }
     s->stats.passes += 2;   // two full passes in total over the batches
@@ -358,13 +351,19 @@ void arith_impl(qe_state* s, int N, const int* qa, const int* qb, const int* qc)
 }  // namespace
 
 void launch_mul(qe_state* s, int N, const int* qa, const int* qb, const int* qc) {
-    if (s->dtype == QE_C128) arith_impl<double2, kMul>(s, N, qa, qb, qc);
-    else arith_impl<float2, kMul>(s, N, qa, qb, qc);
+    if (s->dtype == QE_C128) arith_tiles<double2, kMul>(s, N, qa, qb, qc, N, "mul_emulated");
+    else arith_tiles<float2, kMul>(s, N, qa, qb, qc, N, "mul_emulated");
 }
 
 void launch_div(qe_state* s, int N, const int* qa, const int* qb, const int* qc) {
-    if (s->dtype == QE_C128) arith_impl<double2, kDiv>(s, N, qa, qb, qc);
-    else arith_impl<float2, kDiv>(s, N, qa, qb, qc);
+    if (((size_t)amp_bytes(s) << 2 * N) <= 64 * 1024) {
+        if (s->dtype == QE_C128) arith_tiles<double2, kDiv>(s, N, qa, qb, qc, 2 * N, "div_emulated");
+        else arith_tiles<float2, kDiv>(s, N, qa, qb, qc, 2 * N, "div_emulated");
+    } else if (s->dtype == QE_C128) {
+        div_batches<double2>(s, N, qa, qb, qc);
+    } else {
+        div_batches<float2>(s, N, qa, qb, qc);
+    }
 }
 
 }  // namespace qe
