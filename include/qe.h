@@ -126,7 +126,8 @@ int qe_apply_controlled(qe_state* s, int nc, const int* controls, int k,
  * says of them in both modes; the 32 amplitudes that share a scale belong to
  * one assignment of the other qubits, except in registers of three and four
  * qubits (FP64 mode only).  Groups whose largest component is below 2^-920
- * become zero there, groups with an infinity or NaN become NaN.  QE_ERR_ARG unless m >= 1, lo >= 0 and lo + m <= n. */
+ * become zero there, groups with an infinity or NaN become NaN.  QE_ERR_ARG
+ * unless m >= 1, lo >= 0 and lo + m <= n. */
 int qe_apply_qft(qe_state* s, int lo, int m, int inverse);
 
 /* Add the classical constant c to the m-qubit register qubits[] (bit j of
@@ -163,16 +164,15 @@ int qe_apply_div(qe_state* s, int N, const int* qa, const int* qb, const int* qc
 /* <psi| sum_t coeff[t] P_t |psi> for Pauli strings P_t given by bit masks
  * over the qubits: (x,z) = (0,0) I, (1,0) X, (0,1) Z, (1,1) Y (Sec. III-D:
  * the expectation computed in one step instead of by repeated sampling).
- * States of at least 17 qubits, terms of at most four X/Y qubits, where an
- * estimate finds that path the cheaper one; smaller complex128 states, terms
- * whose X/Y bits below qubit 12 lie in one of the triples {0,1,2} ..
- * {9,10,11} and whose X/Y bits above it number at most three: in fixed point:
- * every component rounded once to the nearest multiple of 2^(e - 54), 2^e the
- * power of two just above the largest component among the 4096 amplitudes
- * read with it (tiles below 2^-959 flush to zero), products (on smaller
- * states to 2^-52 of the largest) and tile sums exact in integers, tile
- * results combined in FP64.  Other terms and complex64 states: FP64 (FP64
- * mode) or double-float products, compensated sums.  *out receives the real
+ * complex128 sums whose terms all have their X/Y bits below qubit 12 in one of
+ * the triples {0,1,2} .. {9,10,11} and at most three above it (a
+ * transverse-field Ising model, Z-only sums): in fixed point: every component
+ * rounded once to the nearest multiple of 2^(e - 54), 2^e the power of two just
+ * above the largest component among the 4096 amplitudes read with it (tiles
+ * below 2^-959 flush to zero), products (on states below 17 qubits to 2^-52 of
+ * the largest) and tile sums exact in integers, tile results combined in FP64.
+ * Other complex128 sums: FP64 products, or double-float ones in that mode;
+ * complex64 states: pairs of floats, products exact, sums compensated.  *out receives the real
  * value (0 for nterms = 0).  QE_ERR_ARG for nterms < 0, a mask naming a
  * qubit >= n or a non-finite coefficient; QE_ERR_TIMEOUT if a copy wait of
  * the fixed-point kernel ran out (bounded waits). */

@@ -64,6 +64,7 @@
 #include <vector>
 
 #include "qe_batch.h"
+#include "qe_f32x2.cuh"
 #include "qe_internal.h"
 
 namespace qe {
@@ -90,45 +91,6 @@ struct Circ {
     uint64_t f_off;     // offset of its flip masks (layers entries)
     double scale2;      // its energy / the energy of the kept amplitudes
 };
-
-// ------------------------------------------------- packed pairs of floats
-using f2 = unsigned long long;   // (x, y) in the low, high word
-__device__ __forceinline__ f2 pack2(float x, float y) {
-    f2 r;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(x), "f"(y));
-    return r;
-}
-__device__ __forceinline__ float2 unpack2(f2 a) {
-    float2 r;
-    asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(a));
-    return r;
-}
-__device__ __forceinline__ f2 dup2(float x) { return pack2(x, x); }
-__device__ __forceinline__ f2 swap2(f2 a) {
-    const float2 v = unpack2(a);
-    return pack2(v.y, v.x);
-}
-__device__ __forceinline__ f2 neg2(f2 a) { return a ^ 0x8000000080000000ull; }
-__device__ __forceinline__ f2 add2(f2 a, f2 b) {
-    f2 r;
-    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-    return r;
-}
-__device__ __forceinline__ f2 sub2(f2 a, f2 b) {
-    f2 r;
-    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-    return r;
-}
-__device__ __forceinline__ f2 mul2(f2 a, f2 b) {
-    f2 r;
-    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-    return r;
-}
-__device__ __forceinline__ f2 fma2(f2 a, f2 b, f2 c) {
-    f2 r;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
-    return r;
-}
 
 // Each policy: V one amplitude (also its memory form), K a rotation's kappa,
 // R kappa expanded for the device, rot the unscaled rotation, norm the
@@ -171,13 +133,7 @@ struct BF32 {
     __device__ __forceinline__ static void ld(V& v, const V* p) { v = __ldcg(p); }
 };
 
-// unnormalised double-float pairs (h + l), |l| a few units of h's last place
-__device__ __forceinline__ void two_sum(f2 a, f2 b, f2& s, f2& e) {
-    s = add2(a, b);
-    const f2 bb = sub2(s, a);
-    e = add2(sub2(a, sub2(s, bb)), sub2(b, bb));
-}
-
+// double-float pairs h + l, unnormalised: |l| a few units of h's last place
 struct BDF {
     struct alignas(16) V { f2 h, l; };
     using K = float2;                        // (high, low)

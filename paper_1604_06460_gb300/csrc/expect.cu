@@ -3,37 +3,46 @@
 //
 // A pass works on tiles of 2^12 amplitudes: two sets A and B of four qubits and
 // the four lowest others, the row.  A thread first holds the 16 amplitudes that
-// differ in A, as loaded (rows of 256 bytes, 128 complex64); their fixed-point
-// limbs go to shared memory and come back as the 16 that differ in B, and in
-// one pass as those that differ in the row (qubits 0 to 3).  Every term whose
-// X/Y qubits lie in the set held pairs two of the thread's registers.  One pass
-// also sums the Z-only terms.
+// differ in A, as loaded (rows of 256 bytes, 128 complex64); they go to shared
+// memory and come back as the 16 that differ in B, and in one pass as those
+// that differ in the row (qubits 0 to 3).  Every term whose X/Y qubits lie in the
+// set held pairs two of the thread's registers.  One pass also sums the Z-only
+// terms.  Terms of one pattern (X X and Y Y) share their products.
 //
-// Fixed point: with E the largest biased exponent of the tile's components,
-// q = v 2^(1076 - E) rounded to the nearest, |q| < 2^54 (complex64: exact down to
-// 30 binary orders below the largest), in the limbs q = h 2^28 + l.  The products
-// h h' at unit 2^56, h l' + l h' at unit 2^28 and l l' are summed exactly in 64 bits.
-// (Without l l' the sums of states that span many binary orders came out 2 to
-// 4 10^-15 short, as in the register rounds; with it they are off by a few 10^-17.)
-// A weight's sum goes to FP64 once a tile: three instructions on the FP64 pipe
-// (two lanes a clock and SM) for 16 amplitudes a thread.  The four single X of a
-// set are eight products of an amplitude of even parity with the sum of its
-// four odd neighbours instead of 32 products; terms of one pattern (X X and Y Y)
-// share theirs.
+// Three arithmetics, each with the precision of the path it stands in for:
+//   complex128 sums whose terms all fit the register rounds: fixed point.  With E
+//     the largest biased exponent of the tile's components, q = v 2^(1076 - E)
+//     rounded to the nearest, |q| < 2^54, in the limbs q = h 2^28 + l.  The products
+//     h h' at unit 2^56, h l' + l h' at unit 2^28 and l l' are summed exactly in 64
+//     bits.  (Without l l' the sums of states that span many binary orders came out
+//     2 to 4 10^-15 short, as in the register rounds; with it they are off by a few
+//     10^-17.)  A weight's sum goes to FP64 once a tile: three instructions on the
+//     FP64 pipe (two lanes a clock and SM) for 16 amplitudes a thread.  The four
+//     single X of a set are eight products of an amplitude of even parity with the
+//     sum of its four odd neighbours instead of 32 products.
+//   other complex128 sums: FP64 products, two multiply-adds a pair (in fixed point
+//     a term that pairs one large with one small amplitude of a tile would lose
+//     the small one's digits).
+//   complex64: exact products as pairs of floats, summed with their errors.
 //
-// Bound by instruction issue at 16 warps an SM (registers), the ALU pipe first:
-// about 100 instructions an amplitude and pass, 36 of them the limbs.  n = 28:
-// transverse-field Ising complex128 9.42 -> 4.31 ms (four passes of register
-// rounds with a third of the tile's terms each before, three now), complex64
-// 8.31 -> 3.92; Heisenberg chain (terms across the triples of those rounds, so
-// the FP64 or float-pair tile kernel before) 33.2 -> 12.2 and 19.6 -> 11.7.  Sets
-// of four qubits by warps alone, without the shared tile, took 7.0 ms: limbs made
-// anew for every set.
+// Fixed point is bound by instruction issue at 16 warps an SM (registers), the
+// ALU pipe first: about 100 instructions an amplitude and pass, 36 of them the
+// limbs; FP64 products by their pipe; the pairs of floats by the FMA pipe (ten
+// packed instructions a pair, 60 % of its rate).  n = 28, against the other path
+// (register rounds in fixed point, or tiles with FP64 or float-pair products):
+// transverse-field Ising complex128 9.42 -> 4.31 ms, complex64 8.31 -> 4.7;
+// Heisenberg chain with unequal couplings 33.3 -> 20.0 and 19.7 -> 6.4, with equal
+// ones (X X + Y Y is then half the pairs) 32.2 -> 10.5 and 18.9 -> 4.0.  In fixed
+// point the Heisenberg chain took 12.2 ms.  Sets of four qubits by warps alone,
+// without the shared tile, took 7.0 ms for Ising: limbs made anew for every set.
 #include <algorithm>
 #include <cmath>
+#include <cstring>
+#include <type_traits>
 #include <vector>
 
 #include "qe_arith.cuh"
+#include "qe_f32x2.cuh"
 #include "qe_internal.h"
 
 namespace qe {
@@ -42,8 +51,8 @@ namespace {
 
 constexpr int kTile = 12, kThreads = 256, kPerSm = 2;   // bits of a tile; threads; blocks an SM
 constexpr int kTerms = 96, kMasks = 64, kGroups = 16;   // a pass: sums of pairs, Z masks, their weights
-// states of at least 17 qubits: 32 tiles.  There Ising 0.033 ms against 0.040 by
-// register rounds, Heisenberg 0.059 against 0.113 by tiles; with fewer tiles
+// states of at least 17 qubits: 32 tiles.  There Ising 0.062 ms a call against 0.065 by
+// register rounds, Heisenberg 0.097 against 0.142 by tiles; with fewer tiles
 // the launches decide and the other paths take as few
 constexpr int kExpectSetsMin = 17;
 constexpr uint32_t kZero = 64;   // biased FP64 exponent below which a tile's amplitudes count as zero
@@ -52,7 +61,7 @@ constexpr uint32_t kZero = 64;   // biased FP64 exponent below which a tile's am
 // pattern and of the same Z bits outside the set share their products, each
 // pair weighed by the sum of the terms' signed coefficients
 struct Term {
-    double w;             // > 0, twice the sum of the coefficients; pairs of weight 0 are left out
+    double w;             // > 0, twice the sum of the coefficients (its arithmetic's form); pairs of weight 0 are left out
     uint64_t zm;          // Z bits outside the set
     uint32_t sel : 16;    // the pairs, by the j without xt's lowest bit
     uint32_t xt : 4;      // X/Y bits in the set; 0: the sum of its four single X
@@ -67,7 +76,7 @@ struct ZPattern {
     uint32_t n, pat[4];
 };
 struct ZGroup {
-    double w;             // twice the weight
+    double w;             // the weight (its arithmetic's form; twice it in fixed point)
     int c0, c1, masks;    // patterns [c0, c1), at most 64 masks
 };
 template <class S>
@@ -85,18 +94,8 @@ struct Args {
     double* partial;
 };
 
-struct Fx {
-    int xh, xl, yh, yl;
-};
-struct Acc4 {
-    long long h0 = 0, h1 = 0, m0 = 0, m1 = 0, ll = 0;   // ll: one term's, then into m0
-};
-
 __device__ __forceinline__ uint32_t top_bits(double2 v) {
     return max((uint32_t)__double2hiint(v.x) & 0x7FFFFFFFu, (uint32_t)__double2hiint(v.y) & 0x7FFFFFFFu);
-}
-__device__ __forceinline__ uint32_t top_bits(float2 v) {
-    return max(__float_as_uint(v.x) & 0x7FFFFFFFu, __float_as_uint(v.y) & 0x7FFFFFFFu);
 }
 // Limbs of a component d binary orders below the largest, its mantissa with the
 // leading bit at bit 63 of (hi, lo): h the top 26 bits of the window, l the rest,
@@ -114,63 +113,210 @@ __device__ __forceinline__ void limbs_of(double v, uint32_t E, int& h, int& l) {
     const uint32_t d = E - ((hi & 0x7FFFFFFFu) >> 20);
     limbs(__funnelshift_l(lo, (hi & 0xFFFFFu) | 0x100000u, 11), lo << 11, d, (int)hi >> 31, h, l);
 }
-__device__ __forceinline__ void limbs_of(float v, uint32_t E, int& h, int& l) {
-    const uint32_t b = __float_as_uint(v);
-    limbs((b << 8) | 0x80000000u, 0u, E - ((b & 0x7FFFFFFFu) >> 23), (int)b >> 31, h, l);
-}
 
-// a += Re (IM: Im) of conj(w) v
-template <bool IM>
-__device__ __forceinline__ void pair_add(Acc4& a, const Fx& w, const Fx& v) {
-    if constexpr (!IM) {
-        a.h0 += (long long)w.xh * v.xh;
-        a.h1 += (long long)w.yh * v.yh;
-        a.m0 += (long long)w.xh * v.xl;
-        a.m0 += (long long)w.xl * v.xh;
-        a.m1 += (long long)w.yh * v.yl;
-        a.m1 += (long long)w.yl * v.yh;
-        a.ll += (long long)w.xl * v.xl;
-        a.ll += (long long)w.yl * v.yl;
-    } else {
-        a.h0 += (long long)w.xh * v.yh;
-        a.h1 -= (long long)w.yh * v.xh;
-        a.m0 += (long long)w.xh * v.yl;
-        a.m0 += (long long)w.xl * v.yh;
-        a.m1 -= (long long)w.yh * v.xl;
-        a.m1 -= (long long)w.yl * v.xh;
-        a.ll += (long long)w.xl * v.yl;
-        a.ll -= (long long)w.yl * v.xl;
+__device__ __forceinline__ double pow2(int x) { return __hiloint2double(min(x, 2047) << 20, 0); }   // 2^(x - 1023), x >= 1
+
+// Times in ms at n = 26: a pass; the Z masks of a weight (the other path: a mask);
+// a term; eight of its pairs.
+// launch: what a pass takes at any size
+struct Cost {
+    double pass, masks, term, pairs, launch;
+};
+
+// The three arithmetics: S an amplitude in memory, V one as held, Acc a sum of
+// products, Sum a thread's sum of weighted Accs.  pair_add: a += Re (IM: Im) of
+// conj(w) v; add: a += t or -= t.
+struct Fixed {
+    using S = double2;
+    struct alignas(16) V {
+        int xh, xl, yh, yl;
+    };
+    struct Acc {
+        long long h0 = 0, h1 = 0, m0 = 0, m1 = 0, ll = 0;   // ll: one term's, then into m0
+    };
+    using Sum = double;
+    static constexpr bool kFixed = true;
+    static constexpr Cost kCost = {0.25, 0.06, 0.034, 0.0, 0.005}, kOther = {0.35, 0.01, 0.045, 0.0, 0.005};
+    static double weight(double w) { return w; }
+    template <bool IM>
+    __device__ __forceinline__ static void pair_add(Acc& a, const V& w, const V& v) {
+        if constexpr (!IM) {
+            a.h0 += (long long)w.xh * v.xh;
+            a.h1 += (long long)w.yh * v.yh;
+            a.m0 += (long long)w.xh * v.xl;
+            a.m0 += (long long)w.xl * v.xh;
+            a.m1 += (long long)w.yh * v.yl;
+            a.m1 += (long long)w.yl * v.yh;
+            a.ll += (long long)w.xl * v.xl;
+            a.ll += (long long)w.yl * v.yl;
+        } else {
+            a.h0 += (long long)w.xh * v.yh;
+            a.h1 -= (long long)w.yh * v.xh;
+            a.m0 += (long long)w.xh * v.yl;
+            a.m0 += (long long)w.xl * v.yh;
+            a.m1 -= (long long)w.yh * v.xl;
+            a.m1 -= (long long)w.yl * v.xh;
+            a.ll += (long long)w.xl * v.yl;
+            a.ll -= (long long)w.yl * v.xl;
+        }
     }
-}
-template <int XT, bool IM>
-__device__ __forceinline__ void pairs(const Fx (&v)[16], uint32_t sel, Acc4& a) {
-#pragma unroll
+    __device__ __forceinline__ static void term_end(Acc& a) {
+        a.m0 += a.ll >> 28;   // at most 2^62
+        a.ll = 0;
+    }
+    __device__ __forceinline__ static void add(Acc& a, const Acc& t, uint32_t neg) {
+        const long long f = -(long long)neg;
+        a.h0 += (t.h0 ^ f) - f;
+        a.h1 += (t.h1 ^ f) - f;
+        a.m0 += (t.m0 ^ f) - f;
+        a.m1 += (t.m1 ^ f) - f;
+    }
+    // s += z w 2^(2 E - 2096)
+    __device__ __forceinline__ static void fold(Sum& s, long long z, double w, int E) {
+        if (E > 800 && E < 1250) s = __fma_rn((double)z, __dmul_rn(w, pow2(2 * E - 1073)), s);
+        else s = __fma_rn(__dmul_rn(__dmul_rn((double)z, pow2(E + 3)), w), pow2(E - 53), s);
+    }
+    __device__ __forceinline__ static void fold(Sum& s, const Acc& a, double w, int E) {
+        fold(s, a.h0 + a.h1 + ((a.m0 + a.m1 + (1ll << 27)) >> 28), w, E);
+    }
+    __device__ __forceinline__ static double total(Sum s) { return s; }
+};
+struct Native {
+    using S = double2;
+    using V = double2;
+    struct Acc {
+        double a = 0.0, b = 0.0;
+    };
+    using Sum = double;
+    static constexpr bool kFixed = false;
+    static constexpr Cost kCost = {0.11, 0.5, 0.02, 0.1, 0.012}, kOther = {0.2, 0.015, 0.102, 0.0, 0.022},
+                          kOtherDf = {0.35, 0.0095, 0.061, 0.0, 0.022};
+    static double weight(double w) { return w; }
+    __device__ __forceinline__ static V held(double2 v) { return v; }
+    template <bool IM>
+    __device__ __forceinline__ static void pair_add(Acc& a, const V& w, const V& v) {
+        a.a = __fma_rn(w.x, IM ? v.y : v.x, a.a);
+        a.b = __fma_rn(w.y, IM ? -v.x : v.y, a.b);
+    }
+    __device__ __forceinline__ static void term_end(Acc&) {}
+    __device__ __forceinline__ static void add(Acc& a, const Acc& t, uint32_t neg) {
+        const int sg = (int)(neg << 31);
+        a.a += __hiloint2double(__double2hiint(t.a) ^ sg, __double2loint(t.a));
+        a.b += __hiloint2double(__double2hiint(t.b) ^ sg, __double2loint(t.b));
+    }
+    // a += n |v|^2 (n as a double by an addition: the conversion instruction takes
+    // as long as a dozen)
+    __device__ __forceinline__ static void count_add(Acc& a, const V& v, int n) {
+        const double c = __dadd_rn(__hiloint2double(0x43380000 + (n >> 31), n), -6755399441055744.0);   // 1.5 2^52
+        a.a = __fma_rn(__fma_rn(v.x, v.x, __dmul_rn(v.y, v.y)), c, a.a);
+    }
+    __device__ __forceinline__ static void fold(Sum& s, const Acc& a, double w, int) { s = __fma_rn(a.a + a.b, w, s); }
+    __device__ __forceinline__ static double total(Sum s) { return s; }
+};
+// Pairs of floats, a component a lane: products exact (product and residual),
+// sums by TwoSum with the errors summed beside them
+struct Pairs {
+    using S = float2;
+    using V = f2;
+    struct Acc {
+        f2 s = 0, e = 0;
+    };
+    using Sum = Acc;
+    static constexpr bool kFixed = false;
+    static constexpr Cost kCost = {0.19, 0.085, 0.011, 0.0065, 0.012}, kOther = {0.19, 0.0045, 0.04, 0.0, 0.022};
+    static double weight(double w) {   // as a pair of floats in a double's bits
+        const float h = (float)w, l = (float)(w - (double)h);
+        double r;
+        std::memcpy(&r, &h, 4);
+        std::memcpy(reinterpret_cast<char*>(&r) + 4, &l, 4);
+        return r;
+    }
+    __device__ __forceinline__ static V held(float2 v) { return pack2(v.x, v.y); }
+    // a += -n + l
+    __device__ __forceinline__ static void take(Acc& a, f2 n, f2 l) {
+        const f2 s = sub2(a.s, n), bb = sub2(s, a.s);
+        const f2 err = sub2(sub2(a.s, sub2(s, bb)), add2(n, bb));
+        a.s = s;
+        a.e = add2(a.e, add2(err, l));
+    }
+    template <bool IM>
+    __device__ __forceinline__ static void pair_add(Acc& a, const V& w, const V& v) {
+        f2 x = w, y = v;
+        if constexpr (IM) {
+            x ^= 0x8000000000000000ull;   // (w.x, -w.y)
+            y = swap2(v);
+        }
+        const f2 n = mul2(neg2(x), y);
+        take(a, n, fma2(x, y, n));
+    }
+    __device__ __forceinline__ static void term_end(Acc&) {}
+    __device__ __forceinline__ static void add(Acc& a, const Acc& t, uint32_t neg) {
+        const f2 m = neg ? 0ull : 0x8000000080000000ull;
+        take(a, t.s ^ m, neg2(t.e ^ m));
+    }
+    __device__ __forceinline__ static void count_add(Acc& a, const V& v, int n) {
+        const f2 f = dup2((float)n);
+        const f2 h = mul2(v, v), l = fma2(v, v, neg2(h)), p = mul2(neg2(h), f);
+        take(a, p, fma2(l, f, fma2(h, f, p)));
+    }
+    __device__ __forceinline__ static void fold(Sum& s, const Acc& a, double w, int) {
+        const f2 wh = dup2(__int_as_float(__double2loint(w))), wl = dup2(__int_as_float(__double2hiint(w)));
+        const f2 n = mul2(neg2(wh), a.s);
+        take(s, n, fma2(wl, a.s, fma2(wh, a.e, fma2(wh, a.s, n))));
+    }
+    __device__ __forceinline__ static double total(Sum s) {
+        const float2 a = unpack2(s.s), b = unpack2(s.e);
+        return ((double)a.x + (double)b.x) + ((double)a.y + (double)b.y);
+    }
+};
+
+// The pairs of a pattern fall in two halves by the parity of j's bits in it: X X
+// and Y Y of different weights weigh them differently, of equal weights cancel in
+// one.  A half that a term leaves out whole is jumped over (an FP64
+// instruction that is only predicated off takes the pipe's time all the same).
+template <int XT, bool ODD>
+__host__ __device__ constexpr uint32_t half_of() {
+    uint32_t m = 0;
     for (int j = 0; j < 16; ++j) {
-        if (j & (XT & -XT)) continue;
-        if ((sel >> j) & 1u) pair_add<IM>(a, v[j ^ XT], v[j]);
+        const int b = j & XT, odd = (b ^ (b >> 1) ^ (b >> 2) ^ (b >> 3)) & 1;
+        if (!(j & (XT & -XT)) && (odd != 0) == ODD) m |= 1u << j;
+    }
+    return m;
+}
+template <class P, int XT, bool IM, uint32_t HALF>
+__device__ __forceinline__ void half_pairs(const typename P::V (&v)[16], uint32_t sel, typename P::Acc& a) {
+    if constexpr (HALF != 0) {
+        if (sel & HALF) {
+#pragma unroll
+            for (int j = 0; j < 16; ++j)
+                if (((HALF >> j) & 1u) && ((sel >> j) & 1u)) P::template pair_add<IM>(a, v[j ^ XT], v[j]);
+        }
     }
 }
-template <int XT>
-__device__ __forceinline__ void term(const Fx (&v)[16], uint32_t sel, bool im, Acc4& a) {
-    if (im) pairs<XT, true>(v, sel, a);
-    else pairs<XT, false>(v, sel, a);
+template <class P, int XT, bool IM>
+__device__ __forceinline__ void pairs(const typename P::V (&v)[16], uint32_t sel, typename P::Acc& a) {
+    if constexpr (P::kFixed) {   // no slower for the few pairs that are predicated off
+        half_pairs<P, XT, IM, half_of<XT, false>() | half_of<XT, true>()>(v, sel, a);
+    } else {
+        half_pairs<P, XT, IM, half_of<XT, false>()>(v, sel, a);
+        half_pairs<P, XT, IM, half_of<XT, true>()>(v, sel, a);
+    }
 }
-__device__ __forceinline__ void chain(const Fx (&v)[16], Acc4& a) {
+template <class P, int XT>
+__device__ __forceinline__ void term(const typename P::V (&v)[16], uint32_t sel, bool im, typename P::Acc& a) {
+    if (im) pairs<P, XT, true>(v, sel, a);
+    else pairs<P, XT, false>(v, sel, a);
+}
+// the four single X of a set (fixed point, whose sums of four are exact)
+__device__ __forceinline__ void chain(const Fixed::V (&v)[16], Fixed::Acc& a) {
 #pragma unroll
     for (int j = 0; j < 16; ++j) {
         if (((j >> 3) ^ (j >> 2) ^ (j >> 1) ^ j) & 1) continue;
-        const Fx &b = v[j ^ 1], &c = v[j ^ 2], &d = v[j ^ 4], &e = v[j ^ 8];
-        const Fx w{(b.xh + c.xh) + (d.xh + e.xh), (b.xl + c.xl) + (d.xl + e.xl), (b.yh + c.yh) + (d.yh + e.yh),
-                   (b.yl + c.yl) + (d.yl + e.yl)};
-        pair_add<false>(a, w, v[j]);
+        const Fixed::V &b = v[j ^ 1], &c = v[j ^ 2], &d = v[j ^ 4], &e = v[j ^ 8];
+        const Fixed::V w{(b.xh + c.xh) + (d.xh + e.xh), (b.xl + c.xl) + (d.xl + e.xl), (b.yh + c.yh) + (d.yh + e.yh),
+                         (b.yl + c.yl) + (d.yl + e.yl)};
+        Fixed::pair_add<false>(a, w, v[j]);
     }
-}
-
-__device__ __forceinline__ double pow2(int x) { return __hiloint2double(min(x, 2047) << 20, 0); }   // 2^(x - 1023), x >= 1
-// s += z w 2^(2 E - 2096)
-__device__ __forceinline__ void fold(double& s, long long z, double w, int E) {
-    if (E > 800 && E < 1250) s = __fma_rn((double)z, __dmul_rn(w, pow2(2 * E - 1073)), s);
-    else s = __fma_rn(__dmul_rn(__dmul_rn((double)z, pow2(E + 3)), w), pow2(E - 53), s);
 }
 
 // bits of v at the set bits of m, lowest first
@@ -182,20 +328,22 @@ __device__ __forceinline__ uint64_t deposit(uint64_t v, uint64_t m) {
 }
 
 // Tile index bits: A (a lane's 16 registers), B (warp and top lane bit), row (low
-// lane bits).  Limbs lie at slot (A, B, row ^ B) of the shared tile, so that each
-// of the three ways a thread's 16 amplitudes are read or written is free of
-// bank conflicts.
-template <class S>
-__global__ void __launch_bounds__(kThreads, kPerSm) k_expect_sets(const __grid_constant__ Args<S> a) {
+// lane bits).  Held amplitudes lie at slot (A, B, row ^ B) of the shared tile, so
+// that each of the three ways a thread's 16 amplitudes are read or written is
+// free of bank conflicts (phases of 8 lanes of 16 bytes, 16 of 8).
+template <class P>
+__global__ void __launch_bounds__(kThreads, kPerSm) k_expect_sets(const __grid_constant__ Args<typename P::S> a) {
+    using S = typename P::S;
+    using V = typename P::V;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    int4* const tile = reinterpret_cast<int4*>(smem_raw);
+    constexpr uint32_t kSwz = sizeof(V) == 16 ? 7u : 15u;
+    V* const tile = reinterpret_cast<V*>(smem_raw);
     __shared__ __align__(16) uint32_t s_top[kThreads / 32];
     __shared__ uint32_t s_odd[2];
     __shared__ double sh[kThreads / 32];
     const uint32_t tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5;
     const uint32_t lo4 = tid & 15u, hi4 = tid >> 4;
-    constexpr int kBias = sizeof(S) == 16 ? 0 : 896;
-    double s = 0.0;
+    typename P::Sum s{};
     auto spread = [&](uint32_t v, const uint8_t (&q)[4]) {
         uint64_t x = 0;
 #pragma unroll
@@ -228,36 +376,44 @@ __global__ void __launch_bounds__(kThreads, kPerSm) k_expect_sets(const __grid_c
                 }
             }
             uint32_t top = 0u;
+            if constexpr (P::kFixed) {
 #pragma unroll
-            for (int j = 0; j < 16; ++j) top = max(top, top_bits(raw[j]));
-            top = __reduce_max_sync(0xffffffffu, top);
-            if (lane == 0) s_top[warp] = top;
+                for (int j = 0; j < 16; ++j) top = max(top, top_bits(raw[j]));
+                top = __reduce_max_sync(0xffffffffu, top);
+                if (lane == 0) s_top[warp] = top;
+            }
             if (a.nz > 0 && warp < 2) {   // parities of the masks at the tile's place
                 const uint64_t m = warp * 32 + lane < (uint32_t)a.nz ? a.z[warp * 32 + lane] : 0ull;
                 const uint32_t odd = __ballot_sync(0xffffffffu, __popcll(here & m) & 1);
                 if (lane == 0) s_odd[warp] = odd;
             }
             __syncthreads();   // also: the previous tile has been read
-            {
+            int E = 0;
+            V v[16];
+            if constexpr (P::kFixed) {
                 const uint4 u = *reinterpret_cast<const uint4*>(&s_top[0]), w = *reinterpret_cast<const uint4*>(&s_top[4]);
                 top = max(max(max(u.x, u.y), max(u.z, u.w)), max(max(w.x, w.y), max(w.z, w.w)));
-            }
-            const uint32_t El = sizeof(S) == 16 ? top >> 20 : top >> 23;
-            // the same for all threads: infinities, NaN; zero
-            const bool bad = El == (sizeof(S) == 16 ? 0x7FFu : 0xFFu);
-            if (bad) s = __hiloint2double(0x7FF80000, 0);
-            if (bad || El < (sizeof(S) == 16 ? kZero : 1u)) {
-                __syncthreads();   // s_top is written again
-                continue;
-            }
-            const int E = (int)El + kBias;
-            Fx v[16];
+                E = (int)(top >> 20);
+                // the same for all threads: infinities, NaN; zero
+                const bool bad = E == 0x7FF;
+                if (bad) s = __hiloint2double(0x7FF80000, 0);
+                if (bad || E < (int)kZero) {
+                    __syncthreads();   // s_top is written again
+                    continue;
+                }
 #pragma unroll
-            for (int j = 0; j < 16; ++j) {
-                limbs_of(raw[j].x, El, v[j].xh, v[j].xl);
-                limbs_of(raw[j].y, El, v[j].yh, v[j].yl);
-                if (a.t[3] > a.t[1]) tile[((uint32_t)j * 16u + hi4) * 16u + (lo4 ^ (hi4 & 7u))] =
-                    make_int4(v[j].xh, v[j].xl, v[j].yh, v[j].yl);
+                for (int j = 0; j < 16; ++j) {
+                    limbs_of(raw[j].x, (uint32_t)E, v[j].xh, v[j].xl);
+                    limbs_of(raw[j].y, (uint32_t)E, v[j].yh, v[j].yl);
+                }
+            } else {
+#pragma unroll
+                for (int j = 0; j < 16; ++j) v[j] = P::held(raw[j]);
+            }
+            if (a.t[3] > a.t[1]) {
+#pragma unroll
+                for (int j = 0; j < 16; ++j)
+                    tile[((uint32_t)j * 16u + hi4) * 16u + (lo4 ^ (hi4 & kSwz))] = v[j];
             }
             const uint64_t zbits = zown ^ ((uint64_t)s_odd[1] << 32 | s_odd[0]);
 #pragma unroll 1
@@ -274,24 +430,32 @@ __global__ void __launch_bounds__(kThreads, kPerSm) k_expect_sets(const __grid_c
                 }
 #pragma unroll
                 for (int w = 0; w < 4; ++w) odd[w] += even * 0x01010101u;
-                long long z[2] = {0, 0};   // each at most 2^62
+                if constexpr (P::kFixed) {
+                    long long z[2] = {0, 0};   // each at most 2^62
 #pragma unroll
-                for (int j = 0; j < 16; ++j) {
-                    // |q|^2 at unit 2^56
-                    const long long hh = (long long)v[j].xh * v[j].xh + (long long)v[j].yh * v[j].yh;
-                    const long long hl = (long long)v[j].xh * v[j].xl + (long long)v[j].yh * v[j].yl;
-                    const long long ll = (long long)v[j].xl * v[j].xl + (long long)v[j].yl * v[j].yl;
-                    const long long q2 = hh + ((hl + (ll >> 29) + (1ll << 26)) >> 27);
-                    const int cnt = masks - 2 * (int)((odd[j >> 2] >> (8 * (j & 3))) & 0xFFu);
-                    z[j & 1] += (long long)cnt * q2;
+                    for (int j = 0; j < 16; ++j) {
+                        // |q|^2 at unit 2^56
+                        const long long hh = (long long)v[j].xh * v[j].xh + (long long)v[j].yh * v[j].yh;
+                        const long long hl = (long long)v[j].xh * v[j].xl + (long long)v[j].yh * v[j].yl;
+                        const long long ll = (long long)v[j].xl * v[j].xl + (long long)v[j].yl * v[j].yl;
+                        const long long q2 = hh + ((hl + (ll >> 29) + (1ll << 26)) >> 27);
+                        const int cnt = masks - 2 * (int)((odd[j >> 2] >> (8 * (j & 3))) & 0xFFu);
+                        z[j & 1] += (long long)cnt * q2;
+                    }
+                    // half the sum, to even: cut off, every thread's tile loses a quarter unit, 10^-16 at n = 24
+                    long long half = (z[0] >> 1) + (z[1] >> 1) + (z[0] & z[1] & 1);
+                    half += (z[0] ^ z[1]) & half & 1;
+                    P::fold(s, half, a.g[g].w, E);
+                } else {
+                    typename P::Acc z;
+#pragma unroll
+                    for (int j = 0; j < 16; ++j)
+                        P::count_add(z, v[j], masks - 2 * (int)((odd[j >> 2] >> (8 * (j & 3))) & 0xFFu));
+                    P::fold(s, z, a.g[g].w, 0);
                 }
-                // half the sum, to even: cut off, every thread's tile loses a quarter unit, 10^-16 at n = 24
-                long long half = (z[0] >> 1) + (z[1] >> 1) + (z[0] & z[1] & 1);
-                half += (z[0] ^ z[1]) & half & 1;
-                fold(s, half, a.g[g].w, E);
             }
             __syncthreads();
-            Acc4 acc;
+            typename P::Acc acc;
 #pragma unroll 1
             for (int round = 0; round < 3; ++round) {
                 const int k0 = a.t[round], k1 = a.t[round + 1];
@@ -300,65 +464,57 @@ __global__ void __launch_bounds__(kThreads, kPerSm) k_expect_sets(const __grid_c
                 if (round == 1) {          // registers: B; thread: (A, row)
                     mine = here | spread(hi4, a.q[0]) | spread(lo4, a.q[2]);
 #pragma unroll
-                    for (int j = 0; j < 16; ++j) {
-                        const int4 q = tile[(hi4 * 16u + (uint32_t)j) * 16u + (lo4 ^ ((uint32_t)j & 7u))];
-                        v[j] = Fx{q.x, q.y, q.z, q.w};
-                    }
+                    for (int j = 0; j < 16; ++j) v[j] = tile[(hi4 * 16u + (uint32_t)j) * 16u + (lo4 ^ ((uint32_t)j & kSwz))];
                 } else if (round == 2) {   // registers: the row; thread: (A, B)
                     mine = here | spread(hi4, a.q[0]) | spread(lo4, a.q[1]);
 #pragma unroll
-                    for (int j = 0; j < 16; ++j) {
-                        const int4 q = tile[tid * 16u + ((uint32_t)j ^ (lo4 & 7u))];
-                        v[j] = Fx{q.x, q.y, q.z, q.w};
-                    }
+                    for (int j = 0; j < 16; ++j) v[j] = tile[tid * 16u + ((uint32_t)j ^ (lo4 & kSwz))];
                 }
 #pragma unroll 1
                 for (int k = k0; k < k1; ++k) {
                     const Term& t = a.term[k];
-                    {
-                        const Acc4 old = acc;
-                        const bool flip = t.flip;
-                        if (flip) acc = Acc4{};
-                        const uint32_t sel = t.sel;
-                        const bool im = t.im;
-                        switch (t.xt) {
-                            case 0: chain(v, acc); break;
-                            case 1: term<1>(v, sel, im, acc); break;
-                            case 2: term<2>(v, sel, im, acc); break;
-                            case 3: term<3>(v, sel, im, acc); break;
-                            case 4: term<4>(v, sel, im, acc); break;
-                            case 5: term<5>(v, sel, im, acc); break;
-                            case 6: term<6>(v, sel, im, acc); break;
-                            case 7: term<7>(v, sel, im, acc); break;
-                            case 8: term<8>(v, sel, im, acc); break;
-                            case 9: term<9>(v, sel, im, acc); break;
-                            case 10: term<10>(v, sel, im, acc); break;
-                            case 11: term<11>(v, sel, im, acc); break;
-                            case 12: term<12>(v, sel, im, acc); break;
-                            case 13: term<13>(v, sel, im, acc); break;
-                            case 14: term<14>(v, sel, im, acc); break;
-                            default: term<15>(v, sel, im, acc); break;
-                        }
-                        acc.m0 += acc.ll >> 28;   // at most 2^62
-                        acc.ll = 0;
-                        if (flip) {
-                            const long long f = -(long long)((__popcll(mine & t.zm) & 1) ^ (int)t.neg);
-                            acc.h0 = old.h0 + ((acc.h0 ^ f) - f);
-                            acc.h1 = old.h1 + ((acc.h1 ^ f) - f);
-                            acc.m0 = old.m0 + ((acc.m0 ^ f) - f);
-                            acc.m1 = old.m1 + ((acc.m1 ^ f) - f);
-                        }
+                    const typename P::Acc old = acc;
+                    const bool flip = t.flip;
+                    if (flip) acc = typename P::Acc{};
+                    const uint32_t sel = t.sel;
+                    const bool im = t.im;
+                    switch (t.xt) {
+                        case 0:
+                            if constexpr (P::kFixed) chain(v, acc);
+                            break;
+                        case 1: term<P, 1>(v, sel, im, acc); break;
+                        case 2: term<P, 2>(v, sel, im, acc); break;
+                        case 3: term<P, 3>(v, sel, im, acc); break;
+                        case 4: term<P, 4>(v, sel, im, acc); break;
+                        case 5: term<P, 5>(v, sel, im, acc); break;
+                        case 6: term<P, 6>(v, sel, im, acc); break;
+                        case 7: term<P, 7>(v, sel, im, acc); break;
+                        case 8: term<P, 8>(v, sel, im, acc); break;
+                        case 9: term<P, 9>(v, sel, im, acc); break;
+                        case 10: term<P, 10>(v, sel, im, acc); break;
+                        case 11: term<P, 11>(v, sel, im, acc); break;
+                        case 12: term<P, 12>(v, sel, im, acc); break;
+                        case 13: term<P, 13>(v, sel, im, acc); break;
+                        case 14: term<P, 14>(v, sel, im, acc); break;
+                        default: term<P, 15>(v, sel, im, acc); break;
+                    }
+                    P::term_end(acc);
+                    if (flip) {
+                        const typename P::Acc one = acc;
+                        acc = old;
+                        P::add(acc, one, (uint32_t)(__popcll(mine & t.zm) & 1) ^ t.neg);
                     }
                     if (t.fold) {
-                        fold(s, acc.h0 + acc.h1 + ((acc.m0 + acc.m1 + (1ll << 27)) >> 28), t.w, E);
-                        acc = Acc4{};
+                        P::fold(s, acc, t.w, E);
+                        acc = typename P::Acc{};
                     }
                 }
             }
         }
     }
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
-    if (lane == 0) sh[warp] = s;
+    double d = P::total(s);
+    for (int o = 16; o > 0; o >>= 1) d += __shfl_down_sync(0xffffffffu, d, o);
+    if (lane == 0) sh[warp] = d;
     __syncthreads();
     if (tid == 0) {
         double r = 0.0;
@@ -479,11 +635,18 @@ bool plan_sets(int n, int nterms, const uint64_t* xm, std::vector<PassPlan>& out
     return true;
 }
 
-template <class S>
+template <class P>
 class Launcher {
+    using S = typename P::S;
+
 public:
     Launcher(qe_state* s, const uint64_t* xm, const uint64_t* zm, const double* cf)
         : s_(s), xm_(xm), zm_(zm), cf_(cf) {}
+
+    // a power of two taken out of the weights (pairs of floats have a float's range)
+    int scale = 0;
+    // the weights' least and largest magnitude
+    double least = HUGE_VAL, most = 0.0;
 
     // launches: the passes, cut to the terms and masks of one
     void build(const std::vector<PassPlan>& plan, const std::vector<ZPlan>& z) {
@@ -507,7 +670,7 @@ public:
                 int nc = 0;
                 for (; zi < z.size() && g.nzg < kGroups && g.nz + z[zi].masks.size() <= kMasks; ++zi) {
                     ZGroup& zg = g.g[g.nzg++];
-                    zg.w = 2.0 * z[zi].w;
+                    zg.w = weight((P::kFixed ? 2.0 : 1.0) * z[zi].w);
                     zg.masks = (int)z[zi].masks.size();
                     zg.c0 = nc;
                     int at[16];
@@ -532,18 +695,25 @@ public:
         }
     }
 
-    double cost(double launch) const {
+    double cost(double unit) const {   // unit: launch times at n = 26 are those of n times this
         double c = 0.0;
         for (const auto& g : launches) {
-            c += 0.25 + launch + 0.06 * g.nzg;
-            for (int k = 0; k < g.t[3]; ++k) c += g.term[k].xt == 0 ? 0.06 : 0.034;
+            c += P::kCost.pass + unit * P::kCost.launch + P::kCost.masks * g.nzg;
+            for (int k = 0; k < g.t[3]; ++k) {
+                const Term& t = g.term[k];
+                int even = 0, odd = 0;   // pairs of the halves: half a term's cost each
+                for (uint32_t j = 0; j < 16; ++j)
+                    if ((t.sel >> j) & 1u) (__builtin_popcount(j & t.xt) & 1 ? odd : even) = 1;
+                const double parts = __builtin_popcount(t.xt) > 1 ? 0.5 * (even + odd) : 1.0;
+                c += t.xt == 0 ? 0.06 : P::kCost.term + P::kCost.pairs * parts;
+            }
         }
         return c;
     }
 
     double run() {
-        const size_t smem = sizeof(int4) << kTile;
-        QE_CUDA(cudaFuncSetAttribute(k_expect_sets<S>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        const size_t smem = sizeof(typename P::V) << kTile;
+        QE_CUDA(cudaFuncSetAttribute(k_expect_sets<P>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
         const unsigned most = (unsigned)(num_sms() * kPerSm);
         const unsigned grid = (unsigned)std::min<uint64_t>(most, launches[0].items);
         const size_t total = (size_t)grid * launches.size();
@@ -551,7 +721,7 @@ public:
         for (size_t i = 0; i < launches.size(); ++i) {
             launches[i].partial = scr + 1 + i * grid;
             Launch L(s_, sizeof(S) == 16 ? "expect_fx" : "expect_rounds", (double)dim(s_) * amp_bytes(s_));
-            k_expect_sets<S><<<grid, kThreads, smem, s_->stream>>>(launches[i]);
+            k_expect_sets<P><<<grid, kThreads, smem, s_->stream>>>(launches[i]);
             QE_CUDA(cudaGetLastError());
         }
         {
@@ -562,7 +732,7 @@ public:
         double e = 0.0;
         QE_CUDA(cudaMemcpyAsync(&e, scr, sizeof(double), cudaMemcpyDeviceToHost, s_->stream));
         QE_CUDA(cudaStreamSynchronize(s_->stream));
-        return e;
+        return std::ldexp(e, scale);
     }
 
 private:
@@ -571,6 +741,13 @@ private:
     const double* cf_;
     std::vector<Args<S>> launches;
 
+    double weight(double w) {
+        if (w != 0.0) {
+            least = std::min(least, std::fabs(w));
+            most = std::max(most, std::fabs(w));
+        }
+        return P::weight(std::ldexp(w, -scale));
+    }
     static uint32_t gather(uint64_t m, const uint8_t (&q)[4]) {
         uint32_t r = 0;
         for (int b = 0; b < 4; ++b) r |= (uint32_t)((m >> q[b]) & 1ull) << b;
@@ -583,7 +760,7 @@ private:
         std::vector<int> single[4], rest;
         for (int t : ts) {
             const uint32_t x = gather(xm_[t], q);
-            if (zm_[t] == 0 && !(x & (x - 1u))) single[__builtin_ctz(x)].push_back(t);
+            if (P::kFixed && zm_[t] == 0 && !(x & (x - 1u))) single[__builtin_ctz(x)].push_back(t);
             else rest.push_back(t);
         }
         for (size_t i = 0; i < single[0].size();) {
@@ -646,9 +823,9 @@ private:
         std::stable_sort(put.begin(), put.end(), [&](const Term& x, const Term& y) { return down ? x.w > y.w : x.w < y.w; });
         for (Term& t : put) {
             t.flip = t.neg || t.zm != 0;
-            // a fold's sums stay below 2^62: eight terms of eight pairs
+            // in fixed point a fold's sums stay below 2^62: eight terms of eight pairs
             const int u = t.xt == 0 ? 4 : 1;
-            if (k > 0 && (units + u > 8 || g.term[k - 1].w != t.w)) {
+            if (k > 0 && ((P::kFixed && units + u > 8) || g.term[k - 1].w != t.w)) {
                 g.term[k - 1].fold = 1;
                 units = 0;
             }
@@ -681,31 +858,33 @@ private:
         }
         g.t[3] = k;
         if (k > 0) g.term[k - 1].fold = 1;
+        for (int i = 0; i < k; ++i) g.term[i].w = weight(g.term[i].w);
     }
 };
 
-template <class S>
+template <class P>
 bool expect_impl(qe_state* s, int nterms, const uint64_t* xm, const uint64_t* zm, const double* cf, size_t other,
                  double* out) {
     std::vector<PassPlan> plan;
     if (!plan_sets(s->n, nterms, xm, plan)) return false;
     std::vector<ZPlan> z;
     plan_z(nterms, xm, zm, cf, z);
-    Launcher<S> l(s, xm, zm, cf);
+    Launcher<P> l(s, xm, zm, cf);
+    if (sizeof(typename P::S) == 8) {
+        double top = 0.0;
+        for (int t = 0; t < nterms; ++t) top = std::max(top, std::fabs(cf[t]));
+        if (top > 0.0) l.scale = std::ilogb(top);
+    }
     l.build(plan, z);
-    // The cheaper path, in ms at n = 26 and 5 us a launch at any size; constants
-    // from measurements of single terms, chains, all pairs, strings and masks
-    // (n = 26, this path and the other; complex128: Ising 1.2 / 2.3, Heisenberg
-    // 3.0 / 7.1, all X X pairs 26 / 42, X with random Z strings 2.5 / 3.3, 20 terms of
-    // four qubits 4.6 / 4.8; complex64: Ising 1.1 / 2.0, Heisenberg 2.9 / 3.9, nearest X X
-    // of different weights 2.1 / 1.9, strings 2.4 / 1.8, one X 0.25 / 0.24)
-    const double launch = std::ldexp(0.005, 26 - s->n);
+    if (sizeof(typename P::S) == 8 && l.least < std::ldexp(l.most, -40)) return false;   // weights beyond a float's range
+    const double unit = std::ldexp(1.0, 26 - s->n);
     int nx = 0;
     for (int t = 0; t < nterms; ++t) nx += xm[t] != 0;
-    const bool c128 = sizeof(S) == 16;
-    const double old = other * ((c128 ? 0.35 : 0.19) + launch) + nx * (c128 ? 0.045 : 0.04) +
-                       (nterms - nx) * (c128 ? 0.01 : 0.0045);
-    if (l.cost(launch) > old) return false;
+    Cost o = P::kOther;
+    if constexpr (std::is_same_v<P, Native>)
+        if (!c128_f64(s)) o = P::kOtherDf;
+    const double old = other * (o.pass + unit * o.launch) + nx * o.term + (nterms - nx) * o.masks;
+    if (l.cost(unit) > old) return false;
     *out = l.run();
     return true;
 }
@@ -713,10 +892,11 @@ bool expect_impl(qe_state* s, int nterms, const uint64_t* xm, const uint64_t* zm
 }  // namespace
 
 bool expect_sets(qe_state* s, int nterms, const uint64_t* xm, const uint64_t* zm, const double* cf, size_t other,
-                 double* out) {
+                 bool fixed, double* out) {
     if (s->n < kExpectSetsMin) return false;
-    if (s->dtype == QE_C128) return expect_impl<double2>(s, nterms, xm, zm, cf, other, out);
-    return expect_impl<float2>(s, nterms, xm, zm, cf, other, out);
+    if (s->dtype == QE_C64) return expect_impl<Pairs>(s, nterms, xm, zm, cf, other, out);
+    if (fixed) return expect_impl<Fixed>(s, nterms, xm, zm, cf, other, out);
+    return expect_impl<Native>(s, nterms, xm, zm, cf, other, out);
 }
 
 }  // namespace qe

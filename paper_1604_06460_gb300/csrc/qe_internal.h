@@ -177,9 +177,9 @@ int choose_fusion_width(qe_state* s, const std::vector<PendingGate>& queue);
 double reduce_norm2(qe_state* s);
 // expectation by passes over register sets of four qubits (large states, terms
 // of at most four X/Y qubits); false where another path has to take it.
-// `other`: the launches of that path
+// `other`: the launches of that path; `fixed`: it would be in fixed point
 bool expect_sets(qe_state* s, int nterms, const uint64_t* xm, const uint64_t* zm, const double* cf, size_t other,
-                 double* out);
+                 bool fixed, double* out);
 double reduce_expectation(qe_state* s, int nterms, const uint64_t* xm, const uint64_t* zm,
                           const double* cf);
 void reduce_probs(qe_state* s, int m, const int* qubits, double* out);

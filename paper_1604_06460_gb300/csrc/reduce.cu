@@ -1712,7 +1712,7 @@ double expect_impl(qe_state* s, int nterms, const uint64_t* xm, const uint64_t* 
         // large states by register sets, where that is cheaper
         double e = 0.0;
         const size_t other = sw == 3 ? SIZE_MAX : rounds ? rl.size() : plans.size() + (size_t)nwide;
-        if (sw != 2 && expect_sets(s, nterms, xm, zm, cf, other, &e)) return e;
+        if (sw != 2 && expect_sets(s, nterms, xm, zm, cf, other, kFx && rounds, &e)) return e;
         if (rounds) return expect_rounds<S, NAT>(s, rl, xm, zm, wv);
     }
     uint64_t max_grid = (uint64_t)num_sms() * 8;
