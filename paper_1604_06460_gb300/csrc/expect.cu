@@ -39,6 +39,8 @@
 #include <cmath>
 #include <cstring>
 #include <type_traits>
+#include <unordered_map>
+#include <unordered_set>
 #include <vector>
 
 #include "qe_arith.cuh"
@@ -55,6 +57,8 @@ constexpr int kTerms = 96, kMasks = 64, kGroups = 16;   // a pass: sums of pairs
 // register rounds, Heisenberg 0.097 against 0.142 by tiles; with fewer tiles
 // the launches decide and the other paths take as few
 constexpr int kExpectSetsMin = 17;
+constexpr size_t kHeld = kTerms * 3 / 8;   // terms of a pass: three make at most eight sums of pairs
+constexpr int kMany = 256;       // terms of a list that is worth tables and a first estimate
 constexpr uint32_t kZero = 64;   // biased FP64 exponent below which a tile's amplitudes count as zero
 
 // Some pairs (j, j ^ xt) of the register set, all of one weight: the terms of a
@@ -563,12 +567,15 @@ struct ZPlan {
 };
 
 void plan_z(int nterms, const uint64_t* xm, const uint64_t* zm, const double* cf, std::vector<ZPlan>& out) {
+    std::unordered_map<double, size_t> open;   // a weight's last group
     for (int t = 0; t < nterms; ++t) {
         if (xm[t] != 0) continue;
-        size_t g = 0;
-        while (g < out.size() && !(out[g].w == cf[t] && out[g].masks.size() < kMasks)) ++g;
-        if (g == out.size()) out.push_back(ZPlan{cf[t], {}});
-        out[g].masks.push_back(zm[t]);
+        const auto [at, fresh] = open.emplace(cf[t], out.size());
+        if (fresh || out[at->second].masks.size() == kMasks) {
+            at->second = out.size();
+            out.push_back(ZPlan{cf[t], {}});
+        }
+        out[at->second].masks.push_back(zm[t]);
     }
 }
 
@@ -593,15 +600,40 @@ bool plan_sets(int n, int nterms, const uint64_t* xm, std::vector<PassPlan>& out
     std::stable_sort(order.begin(), order.end(), [&](int x, int y) {
         return std::make_pair(__builtin_ctzll(xm[x]), xm[x]) < std::make_pair(__builtin_ctzll(xm[y]), xm[y]);
     });
+    // each term to the first set that contains it, else to the first with room;
+    // in long lists the first set of every subset is kept (of no fewer qubits
+    // than the terms have), and which sets have room
+    std::unordered_map<uint64_t, int> first;
+    std::vector<int> room;
+    int fewest = 4;
+    for (int t : order) fewest = std::min(fewest, __builtin_popcountll(xm[t]));
+    const bool many = (int)order.size() > kMany;
+    if (many) first.reserve(order.size());
     for (int t : order) {
-        size_t i = 0;
-        while (i < sets.size() && (sets[i].q & xm[t]) != xm[t]) ++i;
-        if (i == sets.size()) {
-            i = 0;
-            while (i < sets.size() && __builtin_popcountll(sets[i].q | xm[t]) > 4) ++i;
+        int i = -1;
+        if (many) {
+            const auto at = first.find(xm[t]);
+            if (at != first.end()) i = at->second;
+        } else {
+            for (size_t k = 0; k < sets.size() && i < 0; ++k)
+                if ((sets[k].q & xm[t]) == xm[t]) i = (int)k;
         }
-        if (i == sets.size()) sets.push_back(Set{});
-        sets[i].q |= xm[t];
+        if (i < 0) {
+            for (size_t r = 0; r < room.size() && i < 0; ++r)
+                if (__builtin_popcountll(sets[room[r]].q | xm[t]) <= 4) i = room[r];
+            if (i < 0) {
+                i = (int)sets.size();
+                sets.push_back(Set{});
+                room.push_back(i);
+            }
+            const uint64_t q = sets[i].q |= xm[t];
+            if (__builtin_popcountll(q) == 4) room.erase(std::find(room.begin(), room.end(), i));
+            for (uint64_t m = q; many && m != 0; m = (m - 1) & q) {
+                if (__builtin_popcountll(m) < fewest) continue;
+                int& f = first.emplace(m, i).first->second;
+                f = std::min(f, i);
+            }
+        }
         sets[i].terms.push_back(t);
     }
     std::vector<bool> done(sets.size(), false);
@@ -609,8 +641,15 @@ bool plan_sets(int n, int nterms, const uint64_t* xm, std::vector<PassPlan>& out
     for (size_t i = 0; i < sets.size(); ++i) {
         if (done[i]) continue;
         PassPlan p;
+        // a set beside it: the next one without its qubits, not looked for too long
         size_t k = i + 1;
-        while (k < sets.size() && (done[k] || (sets[k].q & sets[i].q))) ++k;
+        for (int tries = 0; k < sets.size() && (done[k] || (sets[k].q & sets[i].q)); ++k)
+            if (!done[k] && ++tries == 64) {
+                k = sets.size();
+                break;
+            }
+        for (size_t b = sets.size(); k >= sets.size() && sets.size() > i + 64 && b > std::max(sets.size() - 64, i + 1); --b)
+            if (!done[b - 1] && !(sets[b - 1].q & sets[i].q)) k = b - 1;
         p.q[0] = filled(n, sets[i].q, k < sets.size() ? sets[k].q : 0ull);
         p.terms[0] = sets[i].terms;
         if (k < sets.size()) {
@@ -660,7 +699,7 @@ public:
                 size_t held = 0;
                 more = false;
                 for (int r = 0; r < 3; ++r) {
-                    for (; at[r] < p.terms[r].size() && held < kTerms * 3 / 8; ++at[r], ++held)
+                    for (; at[r] < p.terms[r].size() && held < kHeld; ++at[r], ++held)
                         part.terms[r].push_back(p.terms[r][at[r]]);
                     more |= at[r] < p.terms[r].size();
                 }
@@ -862,6 +901,42 @@ private:
     }
 };
 
+// Cost of a plan's passes and of its different strings, each by itself: one term,
+// or two where Z bits in its set give its pairs both signs (each with half of the
+// pairs, of one parity or of both).
+template <class P>
+double rough_cost(const std::vector<PassPlan>& plan, const uint64_t* xm, const uint64_t* zm, double unit) {
+    struct Key {
+        uint64_t x, z;
+        bool operator==(const Key& k) const { return x == k.x && z == k.z; }
+    };
+    struct Hash {
+        size_t operator()(const Key& k) const { return (k.x * 0x9E3779B97F4A7C15ull ^ k.z) * 0xD6E8FEB86659FD93ull >> 16; }
+    };
+    std::unordered_set<Key, Hash> seen;
+    size_t count = 0, launches = 0;
+    for (const PassPlan& p : plan) {
+        size_t held = 0;
+        for (const auto& ts : p.terms) held += ts.size();
+        count += held;
+        launches += std::max<size_t>(1, (held + kHeld - 1) / kHeld);
+    }
+    seen.reserve(count);
+    double c = launches * (P::kCost.pass + unit * P::kCost.launch);
+    for (const PassPlan& p : plan)
+        for (int r = 0; r < 3; ++r) {
+            const uint64_t q = r == 0 ? p.q[0] : r == 1 ? p.q[1] : 15ull;
+            for (int t : p.terms[r]) {
+                if (!seen.insert(Key{xm[t], (zm[t] & ~q) << 1 | (__builtin_popcountll(xm[t] & zm[t]) & 1)}).second) continue;
+                const uint64_t low = xm[t] & (0ull - xm[t]), signs = zm[t] & q & ~low;
+                if (P::kFixed && zm[t] == 0 && xm[t] == low) c += 0.015;   // a quarter of a chain
+                else if (signs == 0) c += P::kCost.term + P::kCost.pairs;
+                else c += 2 * P::kCost.term + (signs == (xm[t] & ~low) ? 1 : 2) * P::kCost.pairs;
+            }
+        }
+    return c;
+}
+
 template <class P>
 bool expect_impl(qe_state* s, int nterms, const uint64_t* xm, const uint64_t* zm, const double* cf, size_t other,
                  double* out) {
@@ -869,6 +944,17 @@ bool expect_impl(qe_state* s, int nterms, const uint64_t* xm, const uint64_t* zm
     if (!plan_sets(s->n, nterms, xm, plan)) return false;
     std::vector<ZPlan> z;
     plan_z(nterms, xm, zm, cf, z);
+    const double unit = std::ldexp(1.0, 26 - s->n);
+    Cost o = P::kOther;
+    if constexpr (std::is_same_v<P, Native>)
+        if (!c128_f64(s)) o = P::kOtherDf;
+    int nx = 0;
+    for (int t = 0; t < nterms; ++t) nx += xm[t] != 0;
+    const double old = other * (o.pass + unit * o.launch) + nx * o.term + (nterms - nx) * o.masks;
+    // nothing is built for long sums that the passes and the different strings alone
+    // make too dear (10,000 random strings of four qubits at n = 20: 70 ms a call
+    // with all launches built, 53 so, 48 of them the other path's launches)
+    if (nterms > kMany && rough_cost<P>(plan, xm, zm, unit) > old) return false;
     Launcher<P> l(s, xm, zm, cf);
     if (sizeof(typename P::S) == 8) {
         double top = 0.0;
@@ -877,13 +963,6 @@ bool expect_impl(qe_state* s, int nterms, const uint64_t* xm, const uint64_t* zm
     }
     l.build(plan, z);
     if (sizeof(typename P::S) == 8 && l.least < std::ldexp(l.most, -40)) return false;   // weights beyond a float's range
-    const double unit = std::ldexp(1.0, 26 - s->n);
-    int nx = 0;
-    for (int t = 0; t < nterms; ++t) nx += xm[t] != 0;
-    Cost o = P::kOther;
-    if constexpr (std::is_same_v<P, Native>)
-        if (!c128_f64(s)) o = P::kOtherDf;
-    const double old = other * (o.pass + unit * o.launch) + nx * o.term + (nterms - nx) * o.masks;
     if (l.cost(unit) > old) return false;
     *out = l.run();
     return true;
