@@ -35,6 +35,7 @@
 #include <cooperative_groups.h>
 
 #include <algorithm>
+#include <atomic>
 #include <cstdlib>
 
 #include "qe_arith.cuh"
@@ -329,6 +330,42 @@ bool add_split(qe_state* s, int lo, int m, uint64_t c, int k, void (*rotate)(qe_
     return true;
 }
 
+// Whether the device runs clusters of sixteen blocks of k_add_bulk with `smem`
+// bytes each: more than the portable eight, and sixteen SMs of one GPC.  Asked
+// once a device and size.  QE_TEST_NO_CLUSTER16=1 (a test switch, read per call)
+// answers no.
+template <class S>
+bool sixteen_fit(size_t smem) {
+    const char* e = std::getenv("QE_TEST_NO_CLUSTER16");
+    if (e != nullptr && e[0] == '1') return false;
+    constexpr int kDevices = 64;
+    static std::atomic<int> known[kDevices][2];   // 0 not asked, 1 yes, 2 no
+    int dev = 0;
+    QE_CUDA(cudaGetDevice(&dev));
+    std::atomic<int>* const k = dev < kDevices ? &known[dev][smem > 64 * 1024] : nullptr;
+    if (k && k->load()) return k->load() == 1;
+    QE_CUDA(cudaFuncSetAttribute(k_add_bulk<S>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    QE_CUDA(cudaFuncSetAttribute(k_add_bulk<S>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(16);
+    cfg.blockDim = dim3(32);
+    cfg.dynamicSmemBytes = smem;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = 16;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    int clusters = 0;
+    if (cudaOccupancyMaxActiveClusters(&clusters, k_add_bulk<S>, &cfg) != cudaSuccess) {
+        cudaGetLastError();
+        clusters = 0;
+    }
+    if (k) k->store(clusters > 0 ? 1 : 2);
+    return clusters > 0;
+}
+
 template <class S>
 void add_impl(qe_state* s, int m, const int* qubits, uint64_t c) {
     const uint64_t mmask = (m >= 64) ? ~0ull : ((1ull << m) - 1ull);
@@ -352,10 +389,14 @@ void add_impl(qe_state* s, int m, const int* qubits, uint64_t c) {
     // SM where 128 KB leave room for one, and 16 of a GPC's 18 to 20 SMs for two
     // clusters of eight (1 MB slices at n = 29: 3.31 against 2.98 ms, 512 KB 2.76
     // against 2.96).  Slices of 2 MB: only where the walk's runs are at most 64
-    // bytes (complex128 lo = 2 5.6 -> 3.6 ms, lo = 3 3.2 and 3.6)
-    const int nblk = (contiguous && Sbits >= 3 && Sbits <= bulk_bits) ? 1 : Sbits <= bulk_bits + 2 ? 8 : 16;
-    const bool use_bulk = contiguous && lo < 5 && Sbits >= bulk_min && Sbits <= bulk_bits + ((sizeof(S) << lo) <= 64 ? 4 : 3) &&
-                          ((shift * sizeof(S)) % 16 == 0) && ((((uint64_t)sizeof(S) << Sbits) / nblk) % 16 == 0);
+    // bytes (complex128 lo = 2 5.6 -> 3.6 ms, lo = 3 3.2 and 3.6).  Where clusters of
+    // sixteen do not run, eight take 1 MB and the other paths 2 MB
+    const int bulk_most = bulk_bits + ((sizeof(S) << lo) <= 64 ? 4 : 3);
+    bool sixteen = contiguous && lo < 5 && Sbits > bulk_bits + 2 && Sbits <= bulk_most;
+    if (sixteen) sixteen = sixteen_fit<S>((sizeof(S) << Sbits) / 16);
+    const int nblk = (contiguous && Sbits >= 3 && Sbits <= bulk_bits) ? 1 : sixteen ? 16 : 8;
+    const bool use_bulk = contiguous && lo < 5 && Sbits >= bulk_min &&
+                          (sixteen || Sbits <= std::min(bulk_most, bulk_bits + 3)) && ((shift * sizeof(S)) % 16 == 0) && ((((uint64_t)sizeof(S) << Sbits) / nblk) % 16 == 0);
     if (use_bulk) {
         Launch L(s, nblk == 1 ? "add_bulk" : "add_bulk_cluster", 2.0 * dim(s) * amp_bytes(s));
         const uint64_t nslices = 1ull << (n - Sbits);
