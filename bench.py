@@ -73,6 +73,11 @@ KERNEL_CASES = {
     "tc64": "complex64 5-qubit block on qubits (3,7,11,15,19) of a 26-qubit state, 3 passes",
     "direct2": "complex128 2-qubit block on qubits (5,17) of a 26-qubit state (fusion width 2), 3 passes",
     "expect": "TFIM energy of a 26-qubit complex128 state (fixed point, register sets), 2 evaluations",
+    "heisenberg": "energy of a Heisenberg chain of unequal couplings, 26-qubit complex128 state (FP64 products on "
+                  "register sets), 2 evaluations",
+    "heisenberg64": "the same on a 26-qubit complex64 state (pairs of floats), 2 evaluations",
+    "sample": "4096 samples of a 26-qubit complex128 state (block masses, scan, shots), 2 draws",
+    "fft64": "emulated 26-qubit QFT of a complex64 state (radix-16 register passes), 2 transforms",
     "fft": "emulated 25-qubit QFT of a complex128 state, FP64 mode (5-qubit digit passes), 2 transforms",
     "fftdf": "emulated 26-qubit QFT of a complex128 state, double-float mode (digit passes), "
              "2 transforms",
@@ -80,6 +85,9 @@ KERNEL_CASES = {
                "2 products",
     "addc": "emulated add-constant on qubits [0,16) of a 26-qubit complex128 state (1 MiB slices, sixteen "
             "CTAs each, bulk copies), 2 additions",
+    "addwalk": "emulated add-constant on qubits 0, 2, .., 26 of a 27-qubit complex128 state (cycle walks), 2 additions",
+    "div": "emulated division by 8-qubit registers (index = a b c) of a 26-qubit complex128 state (planes of 1 MB "
+           "in batches through L2), 2 divisions",
     "mul": "emulated multiplication c += a b of 8-qubit registers (index = a b c) of a 26-qubit complex128 "
            "state (planes in shared memory), 2 multiplications",
     "batch": "512 ansatz circuits, n ~ U{10..20}, 8 layers, TFIM energy each, complex128 double-float, "
@@ -123,13 +131,41 @@ def run_kernel_case(qe, I, which):
             for _ in range(2):
                 st.add_const(list(range(16)), 40503)
             st.flush()
-    elif which == "mul":
+    elif which == "addwalk":
+        with qe.State(27, "c128") as st:
+            st.set_policy(qe.POLICY_EMULATE, 1)
+            st.init_random(2)
+            for _ in range(2):
+                st.add_const(list(range(0, 27, 2)), 4055)
+            st.flush()
+    elif which in ("mul", "div"):
         with qe.State(26, "c128") as st:
             st.set_policy(qe.POLICY_EMULATE, 1)
             st.init_random(2)
             for _ in range(2):
-                st.mul(list(range(16, 24)), list(range(8, 16)), list(range(8)))
+                (st.mul if which == "mul" else st.div)(list(range(16, 24)), list(range(8, 16)), list(range(8)))
             st.flush()
+    elif which == "sample":
+        with qe.State(26, "c128") as st:
+            st.init_random(2)
+            u = rng.random(4096)
+            for _ in range(2):
+                st.sample(u)
+    elif which == "fft64":
+        with qe.State(26, "c64") as st:
+            st.set_policy(qe.POLICY_EMULATE, 1)
+            st.init_random(2)
+            for _ in range(2):
+                st.apply_qft(0, 26)
+    elif which in ("heisenberg", "heisenberg64"):
+        with qe.State(26, "c64" if which.endswith("64") else "c128") as st:
+            st.init_random(2)
+            bonds = [3 << i for i in range(25)]
+            xm = np.array(bonds + bonds + [0] * 25, dtype=np.uint64)
+            zm = np.array([0] * 25 + bonds + bonds, dtype=np.uint64)
+            cf = np.repeat([1.0, 0.9, 1.1], 25)
+            for _ in range(2):
+                st.expectation(xm, zm, cf)
     elif which == "batch":
         ns = I.batch_sizes(512, 10, 20, 3)
         angles = [I.ansatz_angles(int(nq), 8, 300000 + i) for i, nq in enumerate(ns)]
@@ -346,12 +382,15 @@ KERNEL_SOURCES = {
     "oz_zgemm": ["oz_gemm.cu", "qe_oz.cuh", "qe_tc.cuh"],
     "add": ["perm.cu", "qe_arith.cuh"],
     "arith": ["arith.cu", "qe_arith.cuh"],
-    "batch": ["batch.cu", "qe_batch.h", "qe_arith.cuh"],
+    "batch": ["batch.cu", "qe_batch.h", "qe_f32x2.cuh", "qe_arith.cuh"],
+    "block_mass": ["sample.cu", "qe_arith.cuh"],
     "fft_twiddle": ["fft.cu", "qe_arith.cuh"],
     "digitrev": ["fft.cu", "qe_arith.cuh"],
     "gate_tc_k5": ["tcgen05.cu", "qe_tc.cuh", "qe_arith.cuh"],
     "gate_direct": ["gates.cu", "qe_arith.cuh"],
-    "expect_fx": ["reduce.cu", "expect.cu", "qe_oz.cuh", "qe_tc.cuh", "qe_arith.cuh"],
+    "expect_fx": ["reduce.cu", "expect.cu", "qe_f32x2.cuh", "qe_oz.cuh", "qe_tc.cuh", "qe_arith.cuh"],
+    "expect_native": ["expect.cu", "qe_f32x2.cuh", "qe_arith.cuh"],
+    "expect_pairs": ["expect.cu", "qe_f32x2.cuh", "qe_arith.cuh"],
     "fft": ["fft.cu", "qe_arith.cuh"],
 }
 

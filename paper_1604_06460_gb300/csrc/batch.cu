@@ -32,7 +32,7 @@
 //     tables with the factors (1, -kappa) folded in write it directly.
 // Double-float values keep (re, im) of the high and of the low words in packed
 // pairs, so that one f32x2 instruction serves both components.
-// 512 circuits of 10..22 qubits, 8 layers: complex128 double-float 242 ms with
+// 512 circuits of 10..22 qubits, 8 layers: complex128 double-float 252 ms with
 // the complex matrices, 74 ms so; FP64 1030 and 215 ms (its pipe's rate);
 // complex64 66 and 25 ms.
 //
@@ -885,9 +885,9 @@ void build_plan(qe_batch* b) {
     for (int c = 0; c < b->count; ++c)
         if (circ[c].n <= T) small.push_back(c);
     std::stable_sort(small.begin(), small.end(), [&](int x, int y) { return circ[x].n > circ[y].n; });
-    // Large circuits go in waves whose states together fit in the L2 cache,
-    // pass-major inside a wave, so that a circuit's passes find its state in
-    // L2 instead of HBM; the small circuits' items are spread evenly between
+    // Large circuits go in waves (kWaveBytes: complex64 ones fit in the L2 cache,
+    // so that a circuit's passes find its state there; complex128 ones exceed it
+    // on purpose), pass-major inside a wave; the small circuits' items are spread evenly between
     // the passes, where they occupy CTAs that would otherwise wait for a
     // pass to finish.  Every item's dependencies (its circuit's earlier
     // passes) come earlier in this order, so the claimed items never wait on

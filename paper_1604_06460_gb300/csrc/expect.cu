@@ -27,8 +27,9 @@
 //
 // Fixed point is bound by instruction issue at 16 warps an SM (registers), the
 // ALU pipe first: about 100 instructions an amplitude and pass, 36 of them the
-// limbs; FP64 products by their pipe; the pairs of floats by the FMA pipe (ten
-// packed instructions a pair, 60 % of its rate).  n = 28, against the other path
+// limbs; FP64 products by their pipe (90 % busy); the pairs of floats (ten packed
+// instructions a pair) by latency, the ALU pipe 46 and the FMA pipe 40 % busy at
+// 16 warps an SM.  n = 28, against the other path
 // (register rounds in fixed point, or tiles with FP64 or float-pair products):
 // transverse-field Ising complex128 9.42 -> 4.31 ms, complex64 8.31 -> 4.7;
 // Heisenberg chain with unequal couplings 33.3 -> 20.0 and 19.7 -> 6.4, with equal
