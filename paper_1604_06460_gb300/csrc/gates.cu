@@ -183,7 +183,10 @@ void dense_k(qe_state* s, int k, const int* qubits, const cd* U) {
 // a gate without overlap, 26.9 then, 11.5 now).  A gate of one qubit after another,
 // FP64 mode: n = 20 21.2 -> 19.8 us, n = 18 8.8 -> 6.6, n = 10 4.7 -> 4.2; CNOTs at
 // n = 20 6.9 -> 4.7.  Double-float loops lose 1 to 5 % at n = 28 to the statement at
-// their end: there the end of a block is the signal.
+// their end, complex64 ones up to 28 % (n = 28: a controlled phase 277 us without
+// overlap, 355 with the statement, 274 without it; a controlled gate 486, 608,
+// 484) except the one-qubit gate's (697, 650, 694): there the end of a block is the
+// signal.
 __device__ __forceinline__ void chain_begin() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void chain_end() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
@@ -247,7 +250,7 @@ __global__ void __launch_bounds__(kThreads) k_gate_direct(const __grid_constant_
             }
         }
     }
-    if constexpr (!std::is_same_v<P, DF>) chain_end();
+    if constexpr (std::is_same_v<P, F64> || (std::is_same_v<P, F32> && K == 1)) chain_end();
 }
 
 template <class P, int K>
@@ -296,7 +299,7 @@ __global__ void __launch_bounds__(kThreads) k_gate_diag(const __grid_constant__ 
         P::mac_first(acc, a.d[r], P::load(a.x[i]));
         a.x[i] = P::out(acc);
     }
-    if constexpr (!std::is_same_v<P, DF>) chain_end();
+    if constexpr (std::is_same_v<P, F64>) chain_end();
 }
 
 // --------------------------------------------- controlled / phase / permute
@@ -331,7 +334,7 @@ __global__ void __launch_bounds__(kThreads) k_controlled(const __grid_constant__
             a.x[base + a.tdep[r]] = P::out(acc);
         }
     }
-    if constexpr (!std::is_same_v<P, DF>) chain_end();
+    if constexpr (std::is_same_v<P, F64>) chain_end();
 }
 
 template <class P>
@@ -346,7 +349,7 @@ __global__ void __launch_bounds__(kThreads) k_permute(const __grid_constant__ Ct
         for (int r = 0; r < D; ++r)
             if (a.perm[r] != r) a.x[base + a.tdep[r]] = v[a.perm[r]];
     }
-    chain_end();
+    if constexpr (!std::is_same_v<P, F32>) chain_end();
 }
 
 unsigned flat_grid(uint64_t count) {
