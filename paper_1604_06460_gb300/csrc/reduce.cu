@@ -177,12 +177,11 @@ __device__ __forceinline__ double block_reduce_d(double a, double* sh) {
 // are fixed by the block (blockIdx / chunks), and the block walks a chunk of the
 // places of the other high bits, eight amplitudes at a time summed in fixed
 // point (mass_of), the eights in FP64.  The threads that differ only in bits
-// outside the register are then combined pairwise with Neumaier's
-// compensation.  Bound by HBM: n = 28, three qubits, complex128 0.67 ms (1.05
-// to 1.30 by FP64 products, two an amplitude; 0.71 at four blocks an SM, 0.80 at
-// six, whose registers spill), complex64 0.33 (0.44 to 0.92; 0.35 with five);
-// eight qubits on both sides of 8, read bin by bin with a stride before, 1.43 ->
-// 0.67 and 1.62 -> 0.32.
+// outside the register are then combined with Neumaier's compensation.  Bound by
+// HBM: n = 28, three qubits, complex128 0.67 ms (1.05 to 1.30 by FP64 products, two
+// an amplitude; 0.71 at four blocks an SM, 0.80 at six, whose registers spill),
+// complex64 0.33 (0.44 to 0.92; 0.35 with five); eight qubits on both sides of 8,
+// read bin by bin with a stride before, 1.43 -> 0.67 and 1.62 -> 0.32.
 constexpr int kLowBits = 8;
 template <class S>
 struct ProbArgs {
@@ -223,7 +222,7 @@ __device__ __forceinline__ double group_mass(const float2 (&v)[N]) {
 template <class S>
 __global__ void __launch_bounds__(1 << kLowBits, sizeof(S) == 16 ? 5 : 8) k_probs(const __grid_constant__ ProbArgs<S> a) {
     constexpr uint32_t T = 1u << kLowBits;
-    __shared__ double ss[T], sc[T];
+    __shared__ double ss[T];
     const uint32_t t = threadIdx.x;
     const uint64_t hv = blockIdx.x / a.chunks, ch = blockIdx.x % a.chunks;
     uint64_t dep = 0;   // hv's bits at the register's high qubits
@@ -256,23 +255,20 @@ __global__ void __launch_bounds__(1 << kLowBits, sizeof(S) == 16 ? 5 : 8) k_prob
             at = ((at | fixed) + 1ull) & ~fixed;
         }
     }
-    // pairwise over the thread bits outside the register
+    // the threads that differ only in bits outside the register: across warps in
+    // turn, by the warps that are left, then pairwise over their lanes (lanes
+    // first, in every warp, took four times as many steps of the FP64 pipe: 14 high
+    // qubits at n = 24 0.64 ms, 0.33 so)
+    ss[t] = s;
+    __syncthreads();
+    const uint32_t up = ~a.lowmask & (T - 32u);
+    if ((t & up) != 0u) return;
+    for (uint32_t u = (0u - up) & up; u != 0u; u = (u - up) & up) neumaier(s, c, ss[t | u]);
     for (int b = 0; b < 5; ++b) {
         if ((a.lowmask >> b) & 1u) continue;
         const double os = __shfl_down_sync(0xffffffffu, s, 1u << b), oc = __shfl_down_sync(0xffffffffu, c, 1u << b);
         neumaier(s, c, os);
         c += oc;
-    }
-    for (int b = 5; b < kLowBits; ++b) {
-        if ((a.lowmask >> b) & 1u) continue;
-        ss[t] = s;
-        sc[t] = c;
-        __syncthreads();
-        if (((t >> b) & 1u) == 0u) {
-            neumaier(s, c, ss[t + (1u << b)]);
-            c += sc[t + (1u << b)];
-        }
-        __syncthreads();
     }
     if (!in || (t & ~a.lowmask) != 0u) return;
     uint64_t bin = 0;
