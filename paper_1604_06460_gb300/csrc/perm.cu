@@ -389,9 +389,16 @@ void add_impl(qe_state* s, int m, const int* qubits, uint64_t c) {
     // SM where 128 KB leave room for one, and 16 of a GPC's 18 to 20 SMs for two
     // clusters of eight (1 MB slices at n = 29: 3.31 against 2.98 ms, 512 KB 2.76
     // against 2.96).  Slices of 2 MB: only where the walk's runs are at most 64
-    // bytes (complex128 lo = 2 5.6 -> 3.6 ms, lo = 3 3.2 and 3.6).  Where clusters of
+    // bytes (complex128 lo = 2 5.6 -> 3.6 ms, lo = 3 3.2 and 3.6), and on states below
+    // 23 qubits, which sit in the cache, at most 16 or, for an odd constant (a single
+    // cycle a column) of complex128, 32 (the walk and clusters: n = 22 complex128
+    // lo = 2 30.8 and 36 us, n = 21 lo = 1 22.7 and 27.0 with an even constant; n = 22
+    // complex64 lo = 3 20.6 and 28.2, lo = 2 23.4 and 27.8, lo = 1 48 and 27, n = 21 with an
+    // even constant 18.6 and 22.9).  Where clusters of
     // sixteen do not run, eight take 1 MB and the other paths 2 MB
-    const int bulk_most = bulk_bits + ((sizeof(S) << lo) <= 64 ? 4 : 3);
+    const bool wide = sizeof(S) == 16;
+    const size_t runs = n >= 23 ? 64 : (c & 1) ? (wide ? 32 : 16) : (wide || n >= 22) ? 16 : 0;
+    const int bulk_most = bulk_bits + ((sizeof(S) << lo) <= runs ? 4 : 3);
     bool sixteen = contiguous && lo < 5 && Sbits > bulk_bits + 2 && Sbits <= bulk_most;
     if (sixteen) sixteen = sixteen_fit<S>((sizeof(S) << Sbits) / 16);
     const int nblk = (contiguous && Sbits >= 3 && Sbits <= bulk_bits) ? 1 : sixteen ? 16 : 8;
