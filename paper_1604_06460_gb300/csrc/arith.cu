@@ -32,7 +32,7 @@ namespace qe {
 
 namespace {
 
-constexpr int kArithThreads = 512;
+constexpr int kArithThreads = 512, kWideThreads = 1024;   // of a tile of 64 KB, of 128 KB
 
 struct RegArg {
     int lo;            // qubit of bit 0
@@ -102,8 +102,8 @@ struct TileArgs {
 };
 
 // Whole planes in shared memory: one read and one write per amplitude.
-template <class S, int OP>
-__global__ void __launch_bounds__(kArithThreads) k_arith_plane(const __grid_constant__ TileArgs<S> a) {
+template <class S, int OP, int TH>
+__global__ void __launch_bounds__(TH) k_arith_plane(const __grid_constant__ TileArgs<S> a) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     S* buf = reinterpret_cast<S*>(smem_raw);
     __shared__ uint64_t offA[64], offB[256];
@@ -123,10 +123,10 @@ __global__ void __launch_bounds__(kArithThreads) k_arith_plane(const __grid_cons
         const uint64_t base = insert_zero_bits(t << a.L, a.hq, a.kh);
         auto at = [&](uint32_t i) { return base + (i & lowmask) + offA[(i >> a.L) & 63u] + offB[i >> a.L >> 6]; };
 #pragma unroll 8
-        for (uint32_t i = threadIdx.x; i < E; i += kArithThreads) buf[i] = a.x[at(i)];
+        for (uint32_t i = threadIdx.x; i < E; i += TH) buf[i] = a.x[at(i)];
         __syncthreads();
 #pragma unroll 4
-        for (uint32_t i = threadIdx.x; i < E; i += kArithThreads) {
+        for (uint32_t i = threadIdx.x; i < E; i += TH) {
             const uint64_t x = at(i);
             const uint32_t bv = reg_get(a.b, a.N, x);
             uint32_t av = OP == kDiv ? reg_get(a.la, a.N, i) : reg_get(a.a, a.N, x);
@@ -263,8 +263,15 @@ void arith_tiles(qe_state* s, int N, const int* qa, const int* qb, const int* qc
     a.a = make_reg(N, qa);
     a.b = make_reg(N, qb);
     // the tile's bits: the plane's qubits and the lowest others, 64 KB in all
-    // (less on small states, for at least 256 tiles)
-    a.T = std::min(s->n, std::max({P, std::min(sizeof(S) == 16 ? 12 : 13, s->n - 8), 5}));
+    // (less on small states, for at least 256 tiles).  Where a plane of 64 KB would
+    // fill a tile and leaves two qubits or more below it, twice that: whole sectors
+    // instead of 16 bytes (division of six-qubit complex128 registers at n = 26 from
+    // qubits 2, 3, 6 on 753, 1117, 1262 us in tiles of 64 KB, 661, 946, 1176 by planes
+    // one at a time, 617, 640, 689 so; from 0 and 1 on 457 and 540, 604 and 601 so)
+    int below = s->n;
+    for (int j = 0; j < N; ++j) below = std::min(below, OP == kDiv ? std::min(qa[j], qc[j]) : qc[j]);
+    const bool wide = sizeof(S) << P == 64 * 1024 && below >= 2;
+    a.T = wide ? std::min(P + 1, std::max(P, s->n - 8)) : std::min(s->n, std::max({P, std::min(sizeof(S) == 16 ? 12 : 13, s->n - 8), 5}));
     bool local[64] = {};
     for (int j = 0; j < N; ++j) {
         local[qc[j]] = true;
@@ -290,13 +297,14 @@ void arith_tiles(qe_state* s, int N, const int* qa, const int* qb, const int* qc
     if (OP == kDiv) a.la = make_reg(N, la);
     a.ntiles = 1ull << (s->n - a.T);
     const size_t smem = sizeof(S) << a.T;
-    auto fn = k_arith_plane<S, OP>;
+    const int threads = wide ? kWideThreads : kArithThreads;
+    auto fn = wide ? k_arith_plane<S, OP, kWideThreads> : k_arith_plane<S, OP, kArithThreads>;
     QE_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     int occ = 0;
-    QE_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fn, kArithThreads, smem));
+    QE_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fn, threads, smem));
     const uint64_t grid = std::min<uint64_t>(a.ntiles, (uint64_t)num_sms() * std::max(occ, 1));
     Launch L(s, tag, 2.0 * dim(s) * amp_bytes(s));
-    fn<<<(unsigned)grid, kArithThreads, smem, s->stream>>>(a);
+    fn<<<(unsigned)grid, threads, smem, s->stream>>>(a);
     QE_CUDA(cudaGetLastError());
 }
 

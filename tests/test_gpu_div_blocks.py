@@ -1,4 +1,4 @@
-"""Emulated division of planes above shared memory in blocks of one to eight
+"""Emulated division of planes at and above shared memory in blocks of one to eight
 planes (the qubits below those of a and c), registers interleaved and unordered,
 and blocks above a batch (nine complex128 qubits with three below).  Bit-exact
 against the definition in torch."""
@@ -26,7 +26,8 @@ def _mixed(n, N, lo, seed):
     return p[:N], b[:N], p[N:2 * N]
 
 
-REGS = [(22, (_run(1, 2, 7), _run(1, 1, 7), _run(1, 0, 7))), (23, (_run(2, 2, 7), _run(2, 1, 7), _run(2, 0, 7))),
+REGS = [(20, (_run(2, 2, 6), _run(2, 1, 6), _run(2, 0, 6))), (21, (_run(2, 2, 6), _run(2, 1, 6), _run(2, 0, 6))),
+        (22, (_run(4, 2, 6), _run(4, 1, 6), _run(4, 0, 6))), (22, _mixed(22, 6, 3, 4)), (22, (_run(1, 2, 7), _run(1, 1, 7), _run(1, 0, 7))), (23, (_run(2, 2, 7), _run(2, 1, 7), _run(2, 0, 7))),
         (24, (_run(3, 2, 7), _run(3, 1, 7), _run(3, 0, 7))), (21, (_run(7, 1, 7), _run(0, 0, 7), _run(7, 0, 7))),
         (22, _mixed(22, 7, 2, 1)), (23, _mixed(23, 7, 3, 2)), (25, _mixed(25, 8, 3, 3)),
         (27, (_run(9, 1, 9), _run(0, 0, 9), _run(9, 0, 9)))]
