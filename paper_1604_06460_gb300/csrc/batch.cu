@@ -37,6 +37,8 @@
 // complex64 66 and 25 ms.
 //
 // Work decomposition (one work queue, claimed in order with an atomic head):
+//   - circuits of at most seven or eight qubits go before, a warp each
+//     (k_batch_tiny);
 //   - a circuit with n <= T qubits is one item: its whole state lives in one
 //     CTA's shared memory, HBM is never touched;
 //   - a circuit with n > T qubits keeps its state in HBM and is processed in
@@ -61,6 +63,7 @@
 #include <algorithm>
 #include <cmath>
 #include <cstring>
+#include <type_traits>
 #include <vector>
 
 #include "qe_batch.h"
@@ -104,6 +107,7 @@ struct BF32 {
     __device__ __forceinline__ static F fmul(const F& a, const F& b) { return cmul(a, b); }
     __device__ __forceinline__ static V to_v(const F& f) { return f; }
     static constexpr int kGroup = 4;         // bits per register group
+    static constexpr int kTiny = 8;          // qubits of a circuit that one warp takes
     static constexpr int kSw = 4;            // swizzle: 16 8-byte slots a row
     struct R { f2 k, nk; };
     static K make_k(double k) { return (float)k; }
@@ -120,6 +124,10 @@ struct BF32 {
         const V p = fma2(r.k, b, a);
         b = fma2(r.nk, a, b);
         a = p;
+    }
+    // v + k u
+    __device__ __forceinline__ static V step(const V& v, K k, uint32_t minus, const V& u) {
+        return fma2(dup2(minus ? -k : k), u, v);
     }
     __device__ __forceinline__ static void norm(V&) {}
     __device__ __forceinline__ static V cmul(const V& w, const V& v) {
@@ -151,6 +159,7 @@ struct BDF {
         return V{pack2(x, y), pack2((float)__dsub_rn(f.x, (double)x), (float)__dsub_rn(f.y, (double)y))};
     }
     static constexpr int kGroup = 3;
+    static constexpr int kTiny = 7;
     static constexpr int kSw = 3;            // 8 16-byte slots a row
     struct R { f2 h, l; };
     static K make_k(double k) {
@@ -186,6 +195,10 @@ struct BDF {
         b = madd(b, nh, nl, r.h, a);
         a = p;
     }
+    __device__ __forceinline__ static V step(const V& v, K k, uint32_t minus, const V& u) {
+        const R r = expand(minus ? make_float2(-k.x, -k.y) : k);
+        return madd(v, r.h, r.l, neg2(r.h), u);
+    }
     __device__ __forceinline__ static void norm(V& v) {
         const f2 h = add2(v.h, v.l);
         v.l = sub2(v.l, sub2(h, v.h));
@@ -220,6 +233,7 @@ struct BF64 {
     using V = double2;
     using K = double;
     static constexpr int kGroup = 3;
+    static constexpr int kTiny = 7;
     static constexpr int kSw = 3;
     using R = double;
     static K make_k(double k) { return k; }
@@ -236,6 +250,10 @@ struct BF64 {
         const V p = make_double2(__fma_rn(k, b.x, a.x), __fma_rn(k, b.y, a.y));
         b = make_double2(__fma_rn(-k, a.x, b.x), __fma_rn(-k, a.y, b.y));
         a = p;
+    }
+    __device__ __forceinline__ static V step(const V& v, K k, uint32_t minus, const V& u) {
+        const double s = minus ? -k : k;
+        return make_double2(__fma_rn(s, u.x, v.x), __fma_rn(s, u.y, v.y));
     }
     __device__ __forceinline__ static void norm(V&) {}
     __device__ __forceinline__ static V cmul(const V& w, const V& v) {
@@ -522,6 +540,134 @@ __device__ void run_energy(Group<P> g, int b0, int cnt, bool z, int n, EAcc<P>& 
         if (g.dst & kToTile) __syncthreads();
         g.src = kFromTile;
     }
+}
+
+template <class T>
+__device__ __forceinline__ T shuffle_words(const T& v, uint32_t lane, bool flip) {
+    T r;
+    const uint32_t* s = reinterpret_cast<const uint32_t*>(&v);
+    uint32_t* d = reinterpret_cast<uint32_t*>(&r);
+#pragma unroll
+    for (int k = 0; k < (int)(sizeof(T) / 4); ++k)
+        d[k] = flip ? __shfl_xor_sync(0xffffffffu, s[k], lane) : __shfl_sync(0xffffffffu, s[k], lane);
+    return r;
+}
+
+// Circuits of at most P::kTiny qubits: a warp each, amplitude x in lane x & 31 and
+// register x >> 5, rotations of the low five qubits by shuffles, no barriers, the
+// next layer's factors loaded ahead.  One CTA a circuit, its amplitudes in
+// register groups, leaves most of its threads idle and waits at two barriers a
+// layer: 2000 circuits of six qubits, 40 layers, complex64 534 -> 42 us,
+// double-float 1188 -> 239, FP64 2050 -> 338 (367, 647 and 2098 a gate at a time); 256
+// of four qubits, 8 layers, 39 -> 27, 46 -> 31 and 52 -> 31 (29, 40 and 64).
+template <class P>
+struct TinyArgs {
+    const typename P::K* kap;
+    const typename P::F* fac;
+    const uint32_t* flips;
+    const Circ* circ;
+    const int* which;      // the circuits
+    int count, layers;
+    double hx;
+    double* energies;
+};
+
+template <class P, int E>
+__device__ void tiny_circuit(const TinyArgs<P>& a, int c) {
+    using V = typename P::V;
+    using F = typename P::F;
+    const Circ cc = a.circ[c];
+    const int n = cc.n;
+    const uint32_t lane = threadIdx.x & 31u;
+    const bool in = lane < (1u << n);
+    const uint32_t* flips = a.flips + cc.f_off;
+    const F* fac = a.fac + 2 * cc.u_off;
+    const typename P::K* kap = a.kap + cc.u_off;
+    // the diagonal (of layer 0: the product state): products over qubits 0..3 in
+    // lanes 0..15, over 4..7 in lanes 16..31
+    const int q0 = lane < 16u ? 0 : 4, nf = max(0, min(4, n - q0));
+    F f[4];
+    typename P::K kl{};
+    auto load = [&]() {
+#pragma unroll
+        for (int j = 0; j < 4; ++j) f[j] = j < nf ? fac[2 * (q0 + j) + ((lane >> j) & 1u)] : P::one();
+        if ((int)lane < n) kl = kap[lane];
+    };
+    load();
+    V v[E];
+    for (int l = 0; l < a.layers; ++l) {
+        F w = f[0];
+#pragma unroll
+        for (int j = 1; j < 4; ++j)
+            if (j < nf) w = P::fmul(f[j], w);
+        const typename P::K kk = kl;
+        fac += 2 * n;
+        kap += n;
+        if (l + 1 < a.layers) load();
+        if (l > 0) {
+            for (int q = 0; q < n; ++q) {
+                const typename P::K k = shuffle_words(kk, (uint32_t)q, false);
+                if (q < 5) {
+#pragma unroll
+                    for (int e = 0; e < E; ++e) v[e] = P::step(v[e], k, (lane >> q) & 1u, shuffle_words(v[e], 1u << q, true));
+                } else {
+                    const typename P::R r = P::expand(k);
+#pragma unroll
+                    for (int b = 1; b < E; b *= 2)
+                        if (q == 5 + (b > 1) + (b > 2))
+#pragma unroll
+                            for (int e = 0; e < E; ++e)
+                                if (!(e & b)) P::rot(v[e], v[e | b], r);
+                }
+                if (q % 3 == 2 || q == n - 1) {
+#pragma unroll
+                    for (int e = 0; e < E; ++e) P::norm(v[e]);
+                }
+            }
+        }
+        const F low = shuffle_words(w, lane & 15u, false);
+        const uint32_t flip = flips[l];
+#pragma unroll
+        for (int e = 0; e < E; ++e) {
+            const uint32_t x = lane | ((uint32_t)e << 5);
+            const F high = shuffle_words(w, 16u + (x >> 4), false);
+            const uint32_t y = x ^ flip;
+            const V d = P::neg(P::to_v(n > 4 ? P::fmul(high, low) : low), cz_odd<P>(y & ((1u << n) - 1u)));
+            v[e] = l == 0 ? d : P::cmul(d, v[e]);
+        }
+    }
+    EAcc<P> acc;
+    const uint32_t flip = flips[a.layers - 1], zmask = (1u << (n - 1)) - 1u;
+#pragma unroll
+    for (int e = 0; e < E; ++e) {
+        const uint32_t x = (lane | ((uint32_t)e << 5)) ^ flip;
+        if (in) acc.add_z(v[e], (float)((n - 1) - 2 * __popc((x ^ (x >> 1)) & zmask)));
+        for (int q = 0; q < min(n, 5); ++q) {
+            const V u = shuffle_words(v[e], 1u << q, true);
+            if (in && !((lane >> q) & 1u)) acc.add_x(u, v[e]);
+        }
+#pragma unroll
+        for (int b = 1; b < E; b *= 2)
+            if (!(e & b)) acc.add_x(v[e | b], v[e]);
+    }
+    double z = acc.z(), x = acc.x();
+    for (int o = 16; o > 0; o >>= 1) {
+        z += __shfl_down_sync(0xffffffffu, z, o);
+        x += __shfl_down_sync(0xffffffffu, x, o);
+    }
+    if (lane == 0) a.energies[c] = (z + 2.0 * a.hx * x) * cc.scale2;
+}
+
+constexpr int kTinyThreads = 128;
+template <class P>
+__global__ void __launch_bounds__(kTinyThreads) k_batch_tiny(const __grid_constant__ TinyArgs<P> a) {
+    const int i = (int)((blockIdx.x * (unsigned)kTinyThreads + threadIdx.x) >> 5);
+    if (i >= a.count) return;
+    const int c = a.which[i], n = a.circ[c].n;
+    if (n <= 5) tiny_circuit<P, 1>(a, c);
+    else if (n == 6) tiny_circuit<P, 2>(a, c);
+    else if (P::kTiny < 8 || n == 7) tiny_circuit<P, 4>(a, c);
+    else if constexpr (P::kTiny >= 8) tiny_circuit<P, 8>(a, c);
 }
 
 // Partial products of the factors (2 per qubit) over the local bits 0..5 and
@@ -819,6 +965,10 @@ void build_plan(qe_batch* b) {
     uint64_t state_off = 0;
     int slots = 0;
     std::vector<int> large;
+    // seven qubits in double-float take a warp longer than a CTA: only where the
+    // circuits outnumber the SMs
+    int tiny_bits = P::kTiny;
+    if (std::is_same<P, BDF>::value && std::count(b->n.begin(), b->n.end(), P::kTiny) < 2 * num_sms()) --tiny_bits;
     for (int c = 0; c < b->count; ++c) {
         Circ& cc = circ[c];
         cc.n = b->n[c];
@@ -826,7 +976,7 @@ void build_plan(qe_batch* b) {
         cc.scale2 = scale2[c];
         cc.f_off = (uint64_t)c * b->layers;
         cc.state_off = 0;
-        if (cc.n <= T) {
+        if (cc.n <= std::max(T, tiny_bits)) {
             cc.nitems = 1;
             cc.slot0 = 0;
             cc.nslots = 0;
@@ -881,9 +1031,10 @@ void build_plan(qe_batch* b) {
         items.push_back(it);
     };
     // small circuits (largest first): one item each, without dependencies
-    std::vector<int> small;
+    std::vector<int> small, tiny;
     for (int c = 0; c < b->count; ++c)
-        if (circ[c].n <= T) small.push_back(c);
+        if (circ[c].n <= tiny_bits) tiny.push_back(c);
+        else if (circ[c].n <= T) small.push_back(c);
     std::stable_sort(small.begin(), small.end(), [&](int x, int y) { return circ[x].n > circ[y].n; });
     // Large circuits go in waves (kWaveBytes: complex64 ones fit in the L2 cache,
     // so that a circuit's passes find its state there; complex128 ones exceed it
@@ -926,10 +1077,18 @@ void build_plan(qe_batch* b) {
     }
     if (b->items) cudaFree(b->items);
     if (b->circ) cudaFree(b->circ);
+    if (b->tiny) cudaFree(b->tiny);
+    b->tiny = nullptr;
+    b->ntiny = (int)tiny.size();
+    if (b->ntiny) {
+        std::stable_sort(tiny.begin(), tiny.end(), [&](int x, int y) { return circ[x].n > circ[y].n; });
+        QE_CUDA(cudaMalloc(&b->tiny, tiny.size() * sizeof(int)));
+        QE_CUDA(cudaMemcpy(b->tiny, tiny.data(), tiny.size() * sizeof(int), cudaMemcpyHostToDevice));
+    }
     if (b->partials) cudaFree(b->partials);
     b->items = b->circ = nullptr;
     b->partials = nullptr;
-    QE_CUDA(cudaMalloc(&b->items, items.size() * sizeof(Item)));
+    QE_CUDA(cudaMalloc(&b->items, std::max<size_t>(1, items.size()) * sizeof(Item)));
     QE_CUDA(cudaMemcpy(b->items, items.data(), items.size() * sizeof(Item), cudaMemcpyHostToDevice));
     QE_CUDA(cudaMalloc(&b->circ, circ.size() * sizeof(Circ)));
     QE_CUDA(cudaMemcpy(b->circ, circ.data(), circ.size() * sizeof(Circ), cudaMemcpyHostToDevice));
@@ -976,7 +1135,20 @@ void capture(qe_batch* b) {
     QE_CUDA(cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking));
     QE_CUDA(cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal));
     cudaMemsetAsync(b->sync, 0, (2 + b->count) * sizeof(unsigned), cs);
-    fn<<<grid, b->plan.threads, smem, cs>>>(a);
+    if (b->ntiny) {
+        TinyArgs<P> t;
+        t.kap = a.kap;
+        t.fac = a.fac;
+        t.flips = a.flips;
+        t.circ = a.circ;
+        t.which = b->tiny;
+        t.count = b->ntiny;
+        t.layers = b->layers;
+        t.hx = b->hx;
+        t.energies = b->energies;
+        k_batch_tiny<P><<<(b->ntiny * 32 + kTinyThreads - 1) / kTinyThreads, kTinyThreads, 0, cs>>>(t);
+    }
+    if (grid > 0) fn<<<grid, b->plan.threads, smem, cs>>>(a);
     cudaMemcpyAsync(b->host_energies, b->energies, b->count * sizeof(double), cudaMemcpyDeviceToHost, cs);
     cudaMemcpyAsync(b->host_status, b->sync + 1, sizeof(unsigned), cudaMemcpyDeviceToHost, cs);
     cudaError_t e = cudaStreamEndCapture(cs, &b->graph);
@@ -1037,7 +1209,7 @@ void batch_set_plan(qe_batch* b, int T, int tiles_per_item, int threads) {
 void batch_destroy(qe_batch* b) {
     if (b->exec) cudaGraphExecDestroy(b->exec);
     if (b->graph) cudaGraphDestroy(b->graph);
-    for (void* p : {b->states, b->fac, b->items, b->circ, (void*)b->sync, (void*)b->partials, (void*)b->energies})
+    for (void* p : {b->states, b->fac, b->items, b->circ, (void*)b->tiny, (void*)b->sync, (void*)b->partials, (void*)b->energies})
         if (p) cudaFree(p);
     if (b->host_energies) cudaFreeHost(b->host_energies);
     if (b->host_status) cudaFreeHost(b->host_status);

@@ -32,6 +32,8 @@ struct qe_batch {
     uint32_t* flips = nullptr;
     void* items = nullptr;
     void* circ = nullptr;
+    int* tiny = nullptr;        // circuits of a warp each
+    int ntiny = 0;
     unsigned* sync = nullptr;   // head, status, counters[count]
     double2* partials = nullptr;
     double* energies = nullptr;
