@@ -37,7 +37,7 @@
 // complex64 66 and 25 ms.
 //
 // Work decomposition (one work queue, claimed in order with an atomic head):
-//   - circuits of at most seven or eight qubits go before, a warp each
+//   - circuits of at most seven or eight qubits take a warp each, in a launch beside
 //     (k_batch_tiny);
 //   - a circuit with n <= T qubits is one item: its whole state lives in one
 //     CTA's shared memory, HBM is never touched;
@@ -557,9 +557,9 @@ __device__ __forceinline__ T shuffle_words(const T& v, uint32_t lane, bool flip)
 // register x >> 5, rotations of the low five qubits by shuffles, no barriers, the
 // next layer's factors loaded ahead.  One CTA a circuit, its amplitudes in
 // register groups, leaves most of its threads idle and waits at two barriers a
-// layer: 2000 circuits of six qubits, 40 layers, complex64 534 -> 42 us,
-// double-float 1188 -> 239, FP64 2050 -> 338 (367, 647 and 2098 a gate at a time); 256
-// of four qubits, 8 layers, 39 -> 27, 46 -> 31 and 52 -> 31 (29, 40 and 64).
+// layer: 2000 circuits of six qubits, 40 layers, complex64 535 -> 43 us,
+// double-float 1187 -> 281, FP64 2052 -> 388 (368, 648 and 2098 a gate at a time); 256
+// of four qubits, 8 layers, 39 -> 23, 46 -> 31 and 52 -> 31 (29, 40 and 64).
 template <class P>
 struct TinyArgs {
     const typename P::K* kap;
@@ -594,12 +594,21 @@ __device__ void tiny_circuit(const TinyArgs<P>& a, int c) {
         if ((int)lane < n) kl = kap[lane];
     };
     load();
+    // the last qubits of the register groups that a CTA would make (run_groups),
+    // where the amplitudes are renormalised
+    uint32_t ends = 0;
+    for (int m = 0, ng = (n + P::kGroup - 1) / P::kGroup, at = 0; m < ng; ++m) {
+        at += n / ng + (m >= ng - n % ng ? 1 : 0);
+        ends |= 1u << (at - 1);
+    }
     V v[E];
     for (int l = 0; l < a.layers; ++l) {
-        F w = f[0];
+        F w = f[0], mine[4];
 #pragma unroll
         for (int j = 1; j < 4; ++j)
             if (j < nf) w = P::fmul(f[j], w);
+#pragma unroll
+        for (int j = 0; j < 4; ++j) mine[j] = f[j];
         const typename P::K kk = kl;
         fac += 2 * n;
         kap += n;
@@ -619,7 +628,7 @@ __device__ void tiny_circuit(const TinyArgs<P>& a, int c) {
                             for (int e = 0; e < E; ++e)
                                 if (!(e & b)) P::rot(v[e], v[e | b], r);
                 }
-                if (q % 3 == 2 || q == n - 1) {
+                if (ends >> q & 1u) {
 #pragma unroll
                     for (int e = 0; e < E; ++e) P::norm(v[e]);
                 }
@@ -630,9 +639,22 @@ __device__ void tiny_circuit(const TinyArgs<P>& a, int c) {
 #pragma unroll
         for (int e = 0; e < E; ++e) {
             const uint32_t x = lane | ((uint32_t)e << 5);
-            const F high = shuffle_words(w, 16u + (x >> 4), false);
             const uint32_t y = x ^ flip;
-            const V d = P::neg(P::to_v(n > 4 ? P::fmul(high, low) : low), cz_odd<P>(y & ((1u << n) - 1u)));
+            // in the order of the tables' products, which rounds alike
+            F t = low;
+#pragma unroll
+            for (int j = 0; j < 2; ++j) {
+                const F h = shuffle_words(mine[j], 16u | (x >> 4 & (1u << j)), false);
+                if (n > 4 + j) t = P::fmul(h, t);
+            }
+            V d = P::to_v(t);
+            if (E > 2) {
+                F h = shuffle_words(mine[2], 16u | (x >> 4 & 4u), false);
+                const F h7 = shuffle_words(mine[3], 16u | (x >> 4 & 8u), false);
+                if (n > 7) h = P::fmul(h7, h);
+                d = P::cmul(d, P::to_v(h));
+            }
+            d = P::neg(d, cz_odd<P>(y & ((1u << n) - 1u)));
             v[e] = l == 0 ? d : P::cmul(d, v[e]);
         }
     }
@@ -965,10 +987,16 @@ void build_plan(qe_batch* b) {
     uint64_t state_off = 0;
     int slots = 0;
     std::vector<int> large;
-    // seven qubits in double-float take a warp longer than a CTA: only where the
-    // circuits outnumber the SMs
-    int tiny_bits = P::kTiny;
-    if (std::is_same<P, BDF>::value && std::count(b->n.begin(), b->n.end(), P::kTiny) < 2 * num_sms()) --tiny_bits;
+    // Beside circuits of several passes the tiny ones fill the gaps between those
+    // (200 circuits of 4..14 qubits 714 us as items, 722 beside).  Double-float: only
+    // where there are no others (4..8 qubits 64.3 and 65.3 us), and with seven
+    // qubits, which take a warp longer than a CTA, only where those outnumber the SMs
+    const int largest = *std::max_element(b->n.begin(), b->n.end());
+    int tiny_bits = largest > T ? 0 : P::kTiny;
+    if (std::is_same<P, BDF>::value) {
+        if (std::count(b->n.begin(), b->n.end(), P::kTiny) < 2 * num_sms()) --tiny_bits;
+        if (largest > tiny_bits) tiny_bits = 0;
+    }
     for (int c = 0; c < b->count; ++c) {
         Circ& cc = circ[c];
         cc.n = b->n[c];
@@ -1036,6 +1064,7 @@ void build_plan(qe_batch* b) {
         if (circ[c].n <= tiny_bits) tiny.push_back(c);
         else if (circ[c].n <= T) small.push_back(c);
     std::stable_sort(small.begin(), small.end(), [&](int x, int y) { return circ[x].n > circ[y].n; });
+    std::stable_sort(tiny.begin(), tiny.end(), [&](int x, int y) { return circ[x].n > circ[y].n; });
     // Large circuits go in waves (kWaveBytes: complex64 ones fit in the L2 cache,
     // so that a circuit's passes find its state there; complex128 ones exceed it
     // on purpose), pass-major inside a wave; the small circuits' items are spread evenly between
@@ -1081,7 +1110,6 @@ void build_plan(qe_batch* b) {
     b->tiny = nullptr;
     b->ntiny = (int)tiny.size();
     if (b->ntiny) {
-        std::stable_sort(tiny.begin(), tiny.end(), [&](int x, int y) { return circ[x].n > circ[y].n; });
         QE_CUDA(cudaMalloc(&b->tiny, tiny.size() * sizeof(int)));
         QE_CUDA(cudaMemcpy(b->tiny, tiny.data(), tiny.size() * sizeof(int), cudaMemcpyHostToDevice));
     }
@@ -1131,11 +1159,17 @@ void capture(qe_batch* b) {
     QE_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fn, b->plan.threads, smem));
     if (occ < 1) fail(QE_ERR_UNSUPPORTED, "batch tile does not fit on an SM");
     const unsigned grid = (unsigned)std::min<long long>((long long)num_sms() * occ, b->nitems);
-    cudaStream_t cs;
+    cudaStream_t cs, ts = nullptr;
+    cudaEvent_t fork = nullptr, join = nullptr;
     QE_CUDA(cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking));
-    QE_CUDA(cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal));
-    cudaMemsetAsync(b->sync, 0, (2 + b->count) * sizeof(unsigned), cs);
     if (b->ntiny) {
+        QE_CUDA(cudaStreamCreateWithFlags(&ts, cudaStreamNonBlocking));
+        QE_CUDA(cudaEventCreateWithFlags(&fork, cudaEventDisableTiming));
+        QE_CUDA(cudaEventCreateWithFlags(&join, cudaEventDisableTiming));
+    }
+    QE_CUDA(cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal));
+    if (b->ntiny) {
+        // a branch of its own: beside the others where they leave room
         TinyArgs<P> t;
         t.kap = a.kap;
         t.fac = a.fac;
@@ -1146,13 +1180,21 @@ void capture(qe_batch* b) {
         t.layers = b->layers;
         t.hx = b->hx;
         t.energies = b->energies;
-        k_batch_tiny<P><<<(b->ntiny * 32 + kTinyThreads - 1) / kTinyThreads, kTinyThreads, 0, cs>>>(t);
+        cudaEventRecord(fork, cs);
+        cudaStreamWaitEvent(ts, fork, 0);
+        k_batch_tiny<P><<<(unsigned)((b->ntiny * 32ll + kTinyThreads - 1) / kTinyThreads), kTinyThreads, 0, ts>>>(t);
+        cudaEventRecord(join, ts);
     }
+    cudaMemsetAsync(b->sync, 0, (2 + b->count) * sizeof(unsigned), cs);
     if (grid > 0) fn<<<grid, b->plan.threads, smem, cs>>>(a);
+    if (b->ntiny) cudaStreamWaitEvent(cs, join, 0);
     cudaMemcpyAsync(b->host_energies, b->energies, b->count * sizeof(double), cudaMemcpyDeviceToHost, cs);
     cudaMemcpyAsync(b->host_status, b->sync + 1, sizeof(unsigned), cudaMemcpyDeviceToHost, cs);
     cudaError_t e = cudaStreamEndCapture(cs, &b->graph);
     cudaStreamDestroy(cs);
+    if (ts) cudaStreamDestroy(ts);
+    if (fork) cudaEventDestroy(fork);
+    if (join) cudaEventDestroy(join);
     QE_CUDA(e);
     QE_CUDA(cudaGraphInstantiate(&b->exec, b->graph, 0));
 }

@@ -24,7 +24,8 @@ def _energy(n, angles, hx):
 
 
 @pytest.mark.parametrize("layers", [1, 2, 9])
-@pytest.mark.parametrize("ns", [[1], [7], [8], [1, 2, 3, 4, 5, 6, 7], [7, 8, 5, 13, 6, 3, 7, 7, 2, 8], [7] * 310])
+@pytest.mark.parametrize("ns", [[1], [7], [8], [1, 2, 3, 4, 5, 6, 7], [7, 8, 5, 13, 6, 3, 7, 7, 2, 8], [6, 1, 12, 8, 5],
+                                [7] * 310])
 @pytest.mark.parametrize("dtype,arith,tol", [("c128", 0, 2.0 ** -46), ("c128", 1, 1e-11), ("c64", None, 2e-4)])
 def test_tiny_circuits(ns, layers, dtype, arith, tol):
     from paper_1604_06460_gb300 import qe
