@@ -596,10 +596,10 @@ def main():
 
 
 ARITH_DESC = {
-    "fp64": ("complex128 in the FP64 mode: 3-5-qubit blocks as exact fp16-digit products of 56-bit "
-             "splittings on the tensor cores (each input rounded to 2^-56 of its 32-amplitude group's "
-             "scale, one rounding per output), everything else (FFT, reductions, smaller gates) in native "
-             "FP64"),
+    "fp64": ("complex128 in the FP64 mode: 3-5-qubit blocks and the QFT's digits as exact fp16-digit products "
+             "of 56-bit splittings on the tensor cores (each input rounded to 2^-56 of its 32-amplitude group's "
+             "scale, one rounding per output), twiddles between groups of digits and smaller gates in native FP64, "
+             "probabilities and the Ising energy in fixed point"),
     "df64": ("complex128 in the fast mode: 3-5-qubit blocks as exact fp16-digit products of 48-bit "
              "splittings on the tensor cores, smaller blocks and short FFTs in double-float (f32 pair, 47-bit) "
              "arithmetic, QFTs of several passes and sums as in the FP64 mode"),
